@@ -294,10 +294,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) prefill_attn_tc_kernel(const 
   // hold no attention CTA, and they take part in no cluster barrier.
   if ((int)blockIdx.y == a.Hkv) {
     pdl_launch_dependents();
-    for (int blk = (int)blockIdx.x; blk < a.bank_blocks; blk += (int)gridDim.x) {
-      bank_update_block(a.bank, bp, (int)blockIdx.z, blk);
-      __syncthreads();
-    }
+    if ((int)blockIdx.x < a.bank_ctas) bank_update_block<16, 256>(a.bank, bp, (int)blockIdx.z, (int)blockIdx.x, a.bank_ctas);
     pdl_wait();      // so that this launch has completed only once the kernel ahead of it has
     return;
   }
@@ -867,7 +864,7 @@ cudaError_t prefill_attention_tc_init() {
 cudaError_t launch_prefill_attention_tc(const AttnArgs& a, const BatchParams& bp, int* status, cudaStream_t st) {
   if (a.nsplit < 1 || a.nsplit > kMaxSplit) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(((bp.rows_per_stream + kTok - 1) / kTok) * a.nsplit, a.Hkv + (a.bank_blocks > 0 ? 1 : 0), bp.n_active);
+  cfg.gridDim = dim3(((bp.rows_per_stream + kTok - 1) / kTok) * a.nsplit, a.Hkv + (a.bank_ctas > 0 ? 1 : 0), bp.n_active);
   cfg.blockDim = dim3(kAttnThreads);
   cfg.stream = st;
   cudaLaunchAttribute attr[2];

@@ -13,18 +13,39 @@ __device__ __forceinline__ double warp_tree_sum(double v) {
   return v;
 }
 
-// cos(va, vb) over d elements by one warp: lane p sums elements k = p (mod 32) in ascending k in
-// fp64, then a butterfly 16, 8, 4, 2, 1; the result is the same in every lane
-__device__ __forceinline__ double warp_cosine(const bf16* va, const bf16* vb, int d, int lane) {
-  double dot = 0.0, na = 0.0, nb = 0.0;
-  for (int k = lane; k < d; k += 32) {
-    const double x = (double)__bfloat162float(va[k]);
-    const double y = (double)__bfloat162float(vb[k]);
-    dot = __dadd_rn(dot, __dmul_rn(x, y));
-    na = __dadd_rn(na, __dmul_rn(x, x));
-    nb = __dadd_rn(nb, __dmul_rn(y, y));
+// dot, |a|^2 and (kNormB) |b|^2 over d elements by one warp: lane p sums elements k = p (mod 32) in ascending k in fp64, then
+// a butterfly 16, 8, 4, 2, 1; the results are the same in every lane.  A product of two bf16 values is exact in fp64, so the
+// fused multiply-add rounds once, exactly where a separate addition would.  The loop is a chain of dependent fp64 adds fed
+// by 2-byte loads, so what it costs is load latency: kU elements of every lane are requested before any is used (one at a
+// time the scoring of a 1024-carrier bank took 33 us beside the attention of a one-layer frame step).
+template <bool kNormB, int kU>
+__device__ __forceinline__ void warp_dot_norms(const bf16* va, const bf16* vb, int d, int lane, double& dot, double& na, double& nb) {
+  dot = 0.0; na = 0.0;
+  if (kNormB) nb = 0.0;
+  const unsigned short* pa = reinterpret_cast<const unsigned short*>(va) + lane;
+  const unsigned short* pb = reinterpret_cast<const unsigned short*>(vb) + lane;
+  for (int k0 = 0; k0 < d; k0 += 32 * kU) {
+    unsigned short xa[kU], xb[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const int k = k0 + 32 * u;                     // d is a multiple of 64: uniform over the warp
+      xa[u] = (k < d) ? pa[k] : (unsigned short)0;   // (zeros add nothing: no sum is ever -0)
+      xb[u] = (k < d) ? pb[k] : (unsigned short)0;
+    }
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const double x = (double)__uint_as_float((uint32_t)xa[u] << 16);
+      const double y = (double)__uint_as_float((uint32_t)xb[u] << 16);
+      dot = __fma_rn(x, y, dot);
+      na = __fma_rn(x, x, na);
+      if (kNormB) nb = __fma_rn(y, y, nb);
+    }
   }
-  dot = warp_tree_sum(dot); na = warp_tree_sum(na); nb = warp_tree_sum(nb);
+  dot = warp_tree_sum(dot); na = warp_tree_sum(na);
+  if (kNormB) nb = warp_tree_sum(nb);
+}
+
+__device__ __forceinline__ double cosine_of(double dot, double na, double nb) {
   double s = 0.0;
   if (na != 0.0 && nb != 0.0) s = __ddiv_rn(dot, __dmul_rn(__dsqrt_rn(na), __dsqrt_rn(nb)));
   // a vector holding Inf or NaN has no cosine: counted as 0, like a zero vector
@@ -32,19 +53,14 @@ __device__ __forceinline__ double warp_cosine(const bf16* va, const bf16* vb, in
   return s;
 }
 
-// Block `block` of `n_blocks` (as the host sized them: one if no listed stream's bank is full,
-// else ceil(M / 8)) working on listed stream b.  Called by every thread of the CTA; threads
-// beyond the first 256 only keep the barriers company.
+// One of the `n_blocks` thread blocks (any number of them, whole warps) that update the bank of listed stream b.
 // Bank not full: block 0 appends; the other blocks return.
-// Bank full: one warp per temporal index j scores cos(e_j, e_other) -- e_other is the incoming
-// carrier (policy 0) or the next carrier in temporal order (policy 1).  Dot products are
-// accumulated in fp64 in a fixed order -- lane p sums elements k = p (mod 32) in ascending k,
-// then a butterfly 16, 8, 4, 2, 1 -- so that the score, and with it the argmax, is
-// reproducible bit for bit; products of two bf16 values are exact in fp64, so fused and
-// unfused accumulation agree.  The last block of a stream to finish picks the victim (largest
-// score, oldest on ties), closes the gap in the temporal order and appends.
-__device__ __forceinline__ void bank_update_block(const BankUpdateArgs& a, const BatchParams& bp, int b, int block) {
-  constexpr int NT = 256;
+// Bank full: the warps of all blocks deal the temporal indexes j among themselves and score cos(e_j, e_other) -- e_other is
+// the incoming carrier (policy 0) or the next carrier in temporal order (policy 1).  The fixed order of the fp64 sums makes
+// the score, and with it the argmax, reproducible bit for bit.  The last block of a stream to finish picks the victim
+// (largest score, oldest on ties), closes the gap in the temporal order and appends.
+template <int kU, int NT>   // kU: loads in flight (see above); NT: threads that take part in the argmax, at most the block's
+__device__ __forceinline__ void bank_update_block(const BankUpdateArgs& a, const BatchParams& bp, int b, int block, int n_blocks) {
   const int tid = threadIdx.x;
   const bool on = tid < NT;
   const int sid = bp.stream_id[b];
@@ -58,9 +74,9 @@ __device__ __forceinline__ void bank_update_block(const BankUpdateArgs& a, const
   int64_t* slot_pos = a.slot_pos + (size_t)sid * a.slots;
   const int count = bp.count[b];
   const int incoming = (a.incoming_emb != nullptr) ? meta->free_slot : a.step_slot[sid];
-  // chunked prefill: the incoming embedding is read from where it is parked and moved into its slot
+  // chunked prefill, a launch per frame: the incoming embedding is read from where it is parked and moved into its slot
   // by whoever commits
-  const bf16* emb_in = (a.incoming_emb != nullptr) ? a.incoming_emb + (size_t)b * a.d
+  const bf16* emb_in = (a.incoming_emb != nullptr) ? a.incoming_emb
                                                    : a.emb + ((size_t)sid * a.slots + incoming) * a.d;
   auto adopt = [&]() {      // all threads of the committing block
     if (a.incoming_emb != nullptr) {
@@ -86,42 +102,39 @@ __device__ __forceinline__ void bank_update_block(const BankUpdateArgs& a, const
   // ---- bank full: score, then the last block commits --------------------------------------
   double* scores = a.scores + (size_t)sid * a.slots;
   const int lane = tid & 31;
-  const int n_score_blocks = (a.M + 7) / 8;
-  const bool planned = a.pre_scores != nullptr;      // one block, scores already there: no ticket
-  if (!planned) {
-  if (block >= n_score_blocks) return;
-  const int j = block * 8 + (tid >> 5);
-  if (on && j < count && a.policy != 2) {
-    const int sa = order[j];
-    const int sb = (a.policy == 1 && j + 1 < count) ? order[j + 1] : incoming;
-    const bf16* va = a.emb + ((size_t)sid * a.slots + sa) * a.d;
-    const bf16* vb = (sb == incoming) ? emb_in : a.emb + ((size_t)sid * a.slots + sb) * a.d;
-    const double s = warp_cosine(va, vb, a.d, lane);
-    if (lane == 0 && VS_STORE_OK(bp, DR_SCORES, scores + j, 8)) scores[j] = s;
+  if (a.policy != 2) {
+    const int n_warps = (int)blockDim.x >> 5;
+    double nb = 0.0;                                  // policy 0: the incoming carrier's norm, worked out with the first row
+    bool first = true;
+    for (int j = block * n_warps + (tid >> 5); j < count; j += n_blocks * n_warps) {
+      const bf16* va = a.emb + ((size_t)sid * a.slots + order[j]) * a.d;
+      double dot, na;
+      if (a.policy == 1) {
+        const bf16* vb = (j + 1 < count) ? a.emb + ((size_t)sid * a.slots + order[j + 1]) * a.d : emb_in;
+        warp_dot_norms<true, kU>(va, vb, a.d, lane, dot, na, nb);
+      } else if (first) {
+        warp_dot_norms<true, kU>(va, emb_in, a.d, lane, dot, na, nb);
+        first = false;
+      } else {
+        warp_dot_norms<false, kU>(va, emb_in, a.d, lane, dot, na, nb);
+      }
+      const double s = cosine_of(dot, na, nb);
+      if (lane == 0 && VS_STORE_OK(bp, DR_SCORES, scores + j, 8)) scores[j] = s;
+    }
   }
   __shared__ int is_last;
   __threadfence();
   __syncthreads();
-  if (tid == 0) is_last = (atomicAdd(&meta->score_ticket, 1) == n_score_blocks - 1);
+  if (tid == 0) is_last = (atomicAdd(&meta->score_ticket, 1) == n_blocks - 1);
   __syncthreads();
   if (!is_last) return;
   __threadfence();
-  }
   __shared__ double best_s[NT];
   __shared__ int best_j[NT];
   double bs = -4.0; int bj = 0x7fffffff;   // every score lies in [-2, 2], so some thread takes an index < count
   if (on && a.policy != 2) {
     for (int i = tid; i < count; i += NT) {
-      double s;
-      if (planned) {
-        // the carrier at temporal index i, as an index on the chunk's bank axis
-        const int slot_i = order[i];
-        const long long fr = slot_frame[slot_i];
-        const int c = (fr >= a.chunk_first_frame) ? a.chunk_l1 + (int)(fr - a.chunk_first_frame) : slot_i;
-        s = a.pre_scores[(size_t)b * a.pre_stride + c];
-      } else {
-        s = __ldcg(scores + i);
-      }
+      const double s = __ldcg(scores + i);
       if (s > bs) { bs = s; bj = i; }                 // ascending i: first maximum kept
     }
   }
@@ -169,7 +182,7 @@ __device__ __forceinline__ void bank_update_block(const BankUpdateArgs& a, const
     meta->free_slot = victim_slot;
     meta->victim_logical = -1;
     meta->frames_seen += 1;
-    if (!planned) meta->score_ticket = 0;
+    meta->score_ticket = 0;
   }
 }
 

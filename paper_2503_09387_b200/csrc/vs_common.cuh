@@ -294,7 +294,7 @@ struct BankUpdateArgs {
   StreamMeta* meta;
   const int32_t* step_slot;      // [S] the slot the incoming carrier was written to
   // chunked prefill: the incoming carrier's embedding is still parked at `incoming_emb`; the slot
-  // is meta.free_slot, recorded in *record_slot, and the embedding moves into the bank here
+  // is meta.free_slot, recorded in *record_slot, and (adjacent-pair policy) the embedding moves into the bank here
   const bf16* incoming_emb;
   int32_t* record_slot;
   // ... and whom the update evicted, as an index on the chunk's bank axis: the slot for a carrier
@@ -348,9 +348,9 @@ struct AttnArgs {
   // whose members each take a contiguous run of key tiles and combine through distributed shared memory
   int nsplit;
   // frame steps, last layer: the bank update (it needs the carrier embeddings only) is done by the CTAs of one more
-  // plane of the grid (blockIdx.y == Hkv), which take its bank_blocks blocks of work in turn; 0: none
+  // plane of the grid (blockIdx.y == Hkv); 0: none.  bank_ctas: how many of the plane's CTAs per stream take part
   BankUpdateArgs bank;
-  int bank_blocks;
+  int bank_ctas;
   // chunk of frames in ONE launch (entry b = frame b): the bank segment is the bank as it was
   // before the chunk (chunk_count0 carriers) for every frame; what frame b must not see -- the slot
   // that was free, and whoever the updates of frames 0 .. b-1 evicted (chunk_victim) -- is masked
@@ -371,6 +371,8 @@ struct ChunkKvCommitArgs {
   bf16* bank_k; bf16* bank_v;              // this layer's bank [S][Hkv][slots][D]
   const int32_t* chunk_slot; const int32_t* chunk_victim;
   int F, N, Hkv, D, slots, sid, l1;
+  const bf16* emb_stage; bf16* emb;        // last layer: parked embeddings [F][d] and where they go [S][slots][d]; else null
+  int d;
 };
 cudaError_t launch_chunk_kv_commit(const ChunkKvCommitArgs& a, cudaStream_t st);
 constexpr int ATTN_EXCL_BITS = 8192;   // most (bank slots + chunk frames) the one-launch chunk attention can mask

@@ -121,7 +121,7 @@ void fill_layout(const Dims& D, Layout& Lo) {
   Lo.rope = reg(DR_ROPE, take((size_t)D.R_max * (D.D / 2) * 8));
   Lo.obuf = reg(DR_OBUF, take((size_t)D.R_max * D.Hq * D.D * 4));
   Lo.emb_stage = reg(DR_EMB_STAGE, take((size_t)D.maxChunk * D.d * 2));
-  Lo.chunk_scores = reg(DR_CHUNK_SCORES, take(D.maxChunk > 1 ? (size_t)D.maxChunk * (D.slots + D.maxChunk) * 8 : 8));
+  Lo.chunk_scores = reg(DR_CHUNK_SCORES, take((size_t)D.maxChunk * (D.slots + D.maxChunk) * 8));
   Lo.gemm_xchg = reg(DR_GEMM_XCHG, take((size_t)GEMM_XCHG_CTAS * 256 * GEMM_BLOCK_M * 4));
   Lo.scratch_end = off;
   Lo.total = off;
@@ -636,7 +636,12 @@ int vs_frame_prefill(vs_stream* h, const int32_t* stream_ids, int32_t n_active, 
       aa.nsplit = attn_split(h, bp, kl, 3);
     }
     // the bank update (Section 3.3, memory mechanism: evict if full, then append) rides in the last layer's launch
-    if (last) { aa.bank = ba; aa.bank_blocks = any_full ? (D.M + 7) / 8 : 1; }
+    // (a CTA scores a row per warp, 19 at a time; its plane is as wide as the attention's)
+    if (last) {
+      aa.bank = ba;
+      const int plane = (N + 1 + 15) / 16 * aa.nsplit, wanted = (D.M + 18) / 19;
+      aa.bank_ctas = !any_full ? 1 : (wanted < plane ? wanted : plane);
+    }
     aa.Hq = D.Hq; aa.Hkv = D.Hkv; aa.D = D.D; aa.slots = D.slots; aa.M = D.M;
     aa.scale_log2e = (float)(1.4426950408889634 / std::sqrt((double)D.D));
     VS_LAUNCH(h, st, KC_PREFILL_ATTN, launch_prefill_attention_tc(aa, bp, h->at<int>(lo.status), st));
@@ -732,6 +737,7 @@ int vs_frame_prefill_chunk(vs_stream* h, int32_t stream_id, const void* hidden, 
     VS_CK(cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming));
     VS_CK(cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming));
   }
+  const bool planned = D.evict_policy != 1;   // one plan for the whole chunk; else a bank update per frame, which moves its embedding itself
   const bool beside = !h->prof_on;           // the per-launch timing pass keeps everything on one stream
   cudaStream_t bst = beside ? h->side_stream : st;
   if (beside) {
@@ -749,7 +755,7 @@ int vs_frame_prefill_chunk(vs_stream* h, int32_t stream_id, const void* hidden, 
     ba.chunk_l1 = l1;
     ba.pre_scores = nullptr; ba.pre_stride = 0;
     const bool any_full = D.M > 0 && bp.count[F - 1] == D.M;
-    if (D.evict_policy != 1 && F > 1) {
+    if (planned) {
       // the updates score against their incoming carrier only (or not at all): every cosine of the
       // chunk in one launch, then all F updates in turn by one block
       ba.incoming_emb = h->at<bf16>(lo.emb_stage);
@@ -849,6 +855,8 @@ int vs_frame_prefill_chunk(vs_stream* h, int32_t stream_id, const void* hidden, 
         ca.kf = fa.kf; ca.vf = fa.vf; ca.bank_k = fa.bank_k; ca.bank_v = fa.bank_v;
         ca.chunk_slot = chunk_slot; ca.chunk_victim = chunk_victim;
         ca.F = F; ca.N = N; ca.Hkv = D.Hkv; ca.D = D.D; ca.slots = D.slots; ca.sid = stream_id; ca.l1 = l1;
+        ca.emb_stage = h->at<bf16>(lo.emb_stage); ca.d = D.d;
+        ca.emb = (last && planned) ? h->at<bf16>(lo.emb) : nullptr;
         VS_LAUNCH(h, st, KC_OTHER, launch_chunk_kv_commit(ca, st));
       }
     }

@@ -285,53 +285,157 @@ cudaError_t launch_argmax_rows(const float* logits, int32_t* token, unsigned lon
   return launch_pdl(argmax_rows_kernel, dim3(slices, rows), dim3(256), 0, st, logits, token, keys, tickets, vocab);
 }
 
-// The bank update of one frame as a launch of its own (chunked prefill).
-__global__ void __launch_bounds__(256, 8) bank_update_kernel(BankUpdateArgs a, BatchParams bp) {   // <= 32 registers: fits beside a projection CTA
+// The bank update of one frame as a launch of its own (chunked prefill, adjacent-pair policy).
+__global__ void __launch_bounds__(128, 8) bank_update_kernel(BankUpdateArgs a, BatchParams bp) {   // <= 64 registers: fits beside a projection CTA
   pdl_wait();
   pdl_launch_dependents();
-  bank_update_block(a, bp, (int)blockIdx.y, (int)blockIdx.x);
+  bank_update_block<8, 128>(a, bp, (int)blockIdx.y, (int)blockIdx.x, (int)gridDim.x);
 }
 
 cudaError_t launch_bank_update(const BankUpdateArgs& a, const BatchParams& bp, bool full, cudaStream_t st) {
-  dim3 grid(full ? (a.M + 7) / 8 : 1, bp.n_active);
-  return launch_pdl(bank_update_kernel, grid, dim3(256), 0, st, a, bp);
+  dim3 grid(full ? (a.M + 3) / 4 : 1, bp.n_active);
+  return launch_pdl(bank_update_kernel, grid, dim3(128), 0, st, a, bp);
 }
 
 // All cosines a chunk's bank updates can need when every update scores against its incoming carrier
 // (policy 0): frame b's carrier against bank slots 0 .. l1-1 as they were before the chunk and against
-// the chunk's carriers 0 .. b-1.  grid = (ceil((l1 + F) / 8), F), one warp per pair.
-__global__ void __launch_bounds__(256, 8) chunk_scores_kernel(BankUpdateArgs a, BatchParams bp, const bf16* emb_stage,
+// the chunk's carriers 0 .. b-1.  One warp per (candidate, frame) pair, four pairs to a block of 64 registers a thread,
+// which finds room beside a projection CTA.
+__global__ void __launch_bounds__(128, 8) chunk_scores_kernel(BankUpdateArgs a, BatchParams bp, const bf16* emb_stage,
                                                               double* out) {
   pdl_wait();                       // the pooled carriers are in place
   pdl_launch_dependents();
   const int b = blockIdx.y, lane = threadIdx.x & 31;
-  const int c = blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int c = blockIdx.x * 4 + (threadIdx.x >> 5);
   if (c >= a.chunk_l1 + b) return;                                 // uniform over the warp
   const int sid = bp.stream_id[b];
   const bf16* va = (c < a.chunk_l1) ? a.emb + ((size_t)sid * a.slots + c) * a.d : emb_stage + (size_t)(c - a.chunk_l1) * a.d;
-  const double s = warp_cosine(va, emb_stage + (size_t)b * a.d, a.d, lane);
-  if (lane == 0) out[(size_t)b * a.pre_stride + c] = s;
+  double dot, na, nb;
+  warp_dot_norms<true, 16>(va, emb_stage + (size_t)b * a.d, a.d, lane, dot, na, nb);
+  if (lane == 0) out[(size_t)b * a.pre_stride + c] = cosine_of(dot, na, nb);
 }
 
 cudaError_t launch_chunk_scores(const BankUpdateArgs& a, const BatchParams& bp, const bf16* emb_stage, double* out, cudaStream_t st) {
-  dim3 grid((a.chunk_l1 + bp.n_active + 7) / 8, bp.n_active);
-  return launch_pdl(chunk_scores_kernel, grid, dim3(256), 0, st, a, bp, emb_stage, out);
+  dim3 grid((a.chunk_l1 + bp.n_active + 3) / 4, bp.n_active);
+  return launch_pdl(chunk_scores_kernel, grid, dim3(128), 0, st, a, bp, emb_stage, out);
 }
 
-// The chunk's bank updates in turn by one block (the scores are looked up, the rest is the streaming
-// update): frame b finds the bank as frame b-1 left it.
-__global__ void __launch_bounds__(256, 8) chunk_plan_kernel(BankUpdateArgs a, BatchParams bp) {
+// The chunk's bank updates in turn by one block: frame b finds the bank as frame b-1 left it.  The temporal order lives in
+// shared memory as indexes on the chunk's bank axis (a slot for a carrier of before the chunk, l1 + i for the carrier of the
+// chunk's frame i), so an update is a gather of ready scores, an argmax (largest, oldest on ties) and a shift; metadata is
+// written once, after the last frame.  (Walking the streaming update's global arrays frame by frame took 6 us a frame, longer
+// than the projection it runs beside; this way it is about 1 us.)  The embeddings move into their slots with the K/V rows.
+__global__ void __launch_bounds__(256, 8) chunk_plan_kernel(BankUpdateArgs a, BatchParams bp) {   // <= 32 registers: fits beside a projection CTA
+  extern __shared__ unsigned short axis[];           // [M] carriers in temporal order (M + 1 + F <= 8192)
+  __shared__ double red_s[2][8];
+  __shared__ int red_i[2][8];
+  __shared__ int slot_of[VS_MAX_BATCH], victim[VS_MAX_BATCH];
   pdl_wait();
   pdl_launch_dependents();
-  for (int b = 0; b < bp.n_active; ++b) {
-    bank_update_block(a, bp, b, 0);
-    __threadfence_block();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int F = bp.n_active, sid = bp.stream_id[0], l1 = a.chunk_l1;
+  StreamMeta* meta = a.meta + sid;
+  int32_t* order = a.order + (size_t)sid * a.slots;
+  int32_t* slot_frame = a.slot_frame + (size_t)sid * a.slots;
+  int64_t* slot_pos = a.slot_pos + (size_t)sid * a.slots;
+  if (a.M == 0) {
+    if (tid == 0) { meta->frames_seen += F; meta->last_victim_frame = -1; }
+    return;
+  }
+  int count = bp.count[0], free_slot = meta->free_slot;
+  for (int i = tid; i < count; i += 256) axis[i] = (unsigned short)order[i];
+  __syncthreads();
+  int evicted = 0;
+  for (int b = 0; b < F; ++b) {
+    if (tid == 0) slot_of[b] = free_slot;
+    if (count < a.M) {
+      if (tid == 0) { axis[count] = (unsigned short)(l1 + b); victim[b] = -1; }
+      ++count;
+      free_slot = count;                             // slots fill in order until the bank is full
+      __syncthreads();
+      continue;
+    }
+    int v = 0;
+    if (a.policy != 2) {
+      double bs = -4.0; int bi = 0x7fffffff;         // every score lies in [-2, 2]
+      for (int i = tid; i < count; i += 256) {
+        const double s = __ldcg(a.pre_scores + (size_t)b * a.pre_stride + axis[i]);
+        if (s > bs) { bs = s; bi = i; }              // ascending i: the first maximum stays
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const double s2 = __shfl_xor_sync(0xffffffffu, bs, o);
+        const int i2 = __shfl_xor_sync(0xffffffffu, bi, o);
+        if (s2 > bs || (s2 == bs && i2 < bi)) { bs = s2; bi = i2; }
+      }
+      if (lane == 0) { red_s[b & 1][warp] = bs; red_i[b & 1][warp] = bi; }
+      __syncthreads();
+      bs = red_s[b & 1][0]; bi = red_i[b & 1][0];
+#pragma unroll
+      for (int w = 1; w < 8; ++w) {
+        const double s2 = red_s[b & 1][w]; const int i2 = red_i[b & 1][w];
+        if (s2 > bs || (s2 == bs && i2 < bi)) { bs = s2; bi = i2; }
+      }
+      v = ((unsigned)bi < (unsigned)count) ? bi : 0;
+    }
+    const int gone = axis[v];
+    free_slot = (gone < l1) ? gone : slot_of[gone - l1];
+    ++evicted;
+    // close the gap, 256 entries at a time in ascending order: a pass reads [base + 1, base + 256] before it writes
+    for (int base = v; base < count - 1; base += 256) {
+      const int i = base + tid;
+      const unsigned short next = (i < count - 1) ? axis[i + 1] : (unsigned short)0;
+      __syncthreads();
+      if (i < count - 1) axis[i] = next;
+    }
     __syncthreads();
+    if (tid == 0) { axis[count - 1] = (unsigned short)(l1 + b); victim[b] = gone; }
+    __syncthreads();
+  }
+  // what the updates leave behind
+  const int first_log = meta->log_count;
+  int my_victim_frame = -1;
+  if (tid < F) {
+    a.record_slot[tid] = slot_of[tid];
+    a.record_victim[tid] = victim[tid];
+    const int g = victim[tid];
+    if (g >= 0) my_victim_frame = (g >= l1) ? (int)(a.chunk_first_frame + (g - l1)) : slot_frame[g];
+  }
+  __syncthreads();
+  if (tid < F && victim[tid] >= 0) {
+    const int g = victim[tid], sl = (g < l1) ? g : slot_of[g - l1];
+    if (VS_STORE_OK(bp, DR_SLOT_FRAME, slot_frame + sl, 4)) slot_frame[sl] = -1;
+    if (a.log_cap > 0) {
+      // evictions start at the first frame that found the bank full and go on without a gap
+      const int n = evicted - (F - tid);
+      if (evicted - n <= a.log_cap) {
+        int32_t* e = a.evict_log + ((size_t)sid * a.log_cap + ((first_log + n) % a.log_cap)) * 2;
+        if (VS_STORE_OK(bp, DR_EVICT_LOG, e, 8)) { e[0] = (int32_t)bp.frame_id[tid]; e[1] = my_victim_frame; }
+      }
+    }
+  }
+  if (tid == F - 1) meta->last_victim_frame = my_victim_frame;
+  __syncthreads();
+  for (int i = tid; i < count; i += 256) {
+    const int c = axis[i], sl = (c < l1) ? c : slot_of[c - l1];
+    if (VS_STORE_OK(bp, DR_ORDER, order + i, 4)) order[i] = sl;
+    if (c >= l1) {
+      if (VS_STORE_OK(bp, DR_SLOT_FRAME, slot_frame + sl, 4)) slot_frame[sl] = (int32_t)bp.frame_id[c - l1];
+      if (VS_STORE_OK(bp, DR_SLOT_POS, slot_pos + sl, 8)) slot_pos[sl] = bp.pos_base[c - l1] + bp.rows_per_stream - 1;
+    }
+  }
+  if (tid == 0) {
+    meta->count = count;
+    meta->free_slot = free_slot;
+    meta->frames_seen += F;
+    meta->evictions += evicted;
+    meta->log_count += evicted;
+    meta->victim_logical = -1;
   }
 }
 
 cudaError_t launch_chunk_plan(const BankUpdateArgs& a, const BatchParams& bp, cudaStream_t st) {
-  return launch_pdl(chunk_plan_kernel, dim3(1), dim3(256), 0, st, a, bp);
+  return launch_pdl(chunk_plan_kernel, dim3(1), dim3(256), (size_t)(a.M > 0 ? a.M : 1) * 2, st, a, bp);
 }
 
 // grid = F CTAs of 128 threads: CTA i copies the carrier row of the chunk's frame i unless a later
@@ -350,6 +454,11 @@ __global__ void __launch_bounds__(128) chunk_kv_commit_kernel(ChunkKvCommitArgs 
     const size_t dst = (((size_t)a.sid * a.Hkv + hk) * a.slots + slot) * a.D + cc * 8;
     *reinterpret_cast<uint4*>(a.bank_k + dst) = *reinterpret_cast<const uint4*>(a.kf + src + hk * a.D + cc * 8);
     *reinterpret_cast<uint4*>(a.bank_v + dst) = *reinterpret_cast<const uint4*>(a.vf + src + hk * a.D + cc * 8);
+  }
+  if (a.emb != nullptr) {                                             // last layer: the parked embedding, too
+    const uint4* es = reinterpret_cast<const uint4*>(a.emb_stage + (size_t)i * a.d);
+    uint4* ed = reinterpret_cast<uint4*>(a.emb + ((size_t)a.sid * a.slots + slot) * a.d);
+    for (int c = threadIdx.x; c < a.d / 8; c += blockDim.x) ed[c] = es[c];
   }
 }
 
