@@ -2,14 +2,22 @@
 // query token per stream attends over [prompt prefix | carrier bank | text of the turn].  No
 // visual-token K/V exists at this point -- only carriers.
 //
-// grid = (key splits, query heads, streams), 256 threads.  A group of D/8 lanes owns one key
-// row and reads it with 128-bit loads; every lane issues the K and V loads of eight keys before
-// it uses any of them, so a warp has 16 key rows (8 KB) in flight.  Warps merge their running
-// (m, l, o) by shuffles and through shared memory.  The key splits of one (stream, query head)
-// form a thread-block cluster (1, 2, 4 or 8 CTAs): every CTA writes its partial triple into rank 0's
-// shared memory (distributed shared memory) and arrives at the cluster's hardware barrier; rank 0
-// alone waits there, combines and writes the row -- no global scratch, no atomics, no polling; the
-// co-scheduled cluster is what guarantees that the barrier completes.
+// Bound by reading the stored keys and values once and, for one stream, by the latency of that read
+// and of the merges behind it.  One CTA = one key split x one KV head x one stream, 8 warps; all
+// query heads of the group (at most 8) are the 8-column operand of mma.sync.m16n8k16, so K and V are
+// read once per group, straight from global memory into fragment registers:
+//   S^T = K Q^T   (16 keys x 8 heads; a lane's 16 contiguous bytes of a key row feed two MMAs, a
+//                  permutation of the dims that K and Q share; Q as its bf16 hi + lo pair)
+//   O^T += V^T P^T (16 dims x 8 heads; byte permutes pair the rows of four keys into the A operand, rows
+//                  of a tile being dims 8g + j; P, fp32, enters as a bf16 hi + lo pair -- 16 bits of
+//                  mantissa -- transposed by movmatrix)
+// A warp holds 16 keys (8 KB) of K and V in flight, two CTAs fit an SM.  Warps merge their (m, l, O)
+// through shared memory.  The key splits of one (stream, KV head) are a thread-block cluster (1, 2, 4
+// or 8 CTAs): each CTA pushes the slice of its partial rows that a peer finishes into that peer's
+// shared memory and arrives at the cluster's hardware barrier; every CTA then combines and stores its
+// own slice -- no global scratch, no atomics, no polling; the co-scheduled cluster is what guarantees
+// that the barrier completes.
+// (One CTA per query head, K and V read once per head: 53 us for 16 streams of 1150 keys.)
 #include "vs_common.cuh"
 
 namespace vs {
@@ -18,47 +26,60 @@ namespace {
 
 constexpr int kDecThreads = 256;
 constexpr int kDecWarps = kDecThreads / 32;
-constexpr int kBatch = 8;     // keys a lane group loads before computing
-constexpr int kMaxCluster = 8;  // portable cluster size: most key splits of one (stream, query head)
+constexpr int kTileKeys = 16;
+constexpr int kHeads = 8;       // query heads of a KV group, padded
+constexpr int kMaxCluster = DEC_SPLIT_MAX;
 
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 __device__ __forceinline__ uint32_t map_shared_rank(uint32_t addr, uint32_t rank) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
-__device__ __forceinline__ void st_shared_cluster_f32(uint32_t addr, float v) {
-  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+__device__ __forceinline__ void st_shared_cluster_f4(uint32_t addr, float4 v) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
+__device__ __forceinline__ void st_shared_cluster_f2(uint32_t addr, float2 v) {
+  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(v.x), "f"(v.y) : "memory");
 }
 __device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_arrive_release() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait_acquire() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ uint32_t transpose_8x8(uint32_t v) {
+  uint32_t r;
+  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(r) : "r"(v));
+  return r;
+}
+__device__ __forceinline__ uint32_t pack2(float lo, float hi) {
+  const __nv_bfloat162 t = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&t);
+}
+__device__ __forceinline__ uint32_t word(const uint4& v, int i) { return i == 0 ? v.x : (i == 1 ? v.y : (i == 2 ? v.z : v.w)); }
 
-// One CTA = one query head x one key split x one stream.  The heads of a KV group read the
-// same K/V rows from L2; spreading them over CTAs keeps every SM's instruction stream short,
-// which is what bounds this kernel (a few hundred keys of 256 bytes each).
 template <int D>
 __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(DecodeArgs a, BatchParams bp) {
-  constexpr int LPK = D / 8;            // lanes that share one key row (16 bytes each)
-  constexpr int KPW = 32 / LPK;         // lane groups (keys in parallel) per warp
-  __shared__ float st_m[kDecWarps];
-  __shared__ float st_l[kDecWarps];
-  __shared__ float st_o[kDecWarps][D];
-  __shared__ float peer_o[kMaxCluster][D];     // rank 0 only: the partial triples its peers (and itself) leave here
-  __shared__ float peer_ml[kMaxCluster][2];
+  constexpr int KC = D / 32;            // 16-byte pieces of a key row per lane (QK)
+  constexpr int VC = D / 64;            // 16-byte pieces of a value row per lane (PV)
+  constexpr int MT = D / 16;            // 16-dim tiles of O^T
+  __shared__ __align__(16) uint4 q_s[2][kHeads][D / 8];           // hi, lo; chunk index XOR 4 in odd rows
+  __shared__ __align__(16) float st_o[kDecWarps][kHeads][D];      // the warps' unnormalised rows
+  __shared__ float2 st_ml[kDecWarps][kHeads];                     // ... with their (max, denominator)
+  __shared__ __align__(16) float peer_o[kHeads * D];              // [split][slice]: what the cluster's CTAs leave for this one
+  __shared__ float2 peer_ml[kMaxCluster][kHeads];
 
   // what follows from the parameters alone comes before the wait on the stream's earlier kernels
-  const int split = blockIdx.x, qh = blockIdx.y, b = blockIdx.z;
+  const int split = blockIdx.x, hkv = blockIdx.y, b = blockIdx.z;
   const int sid = bp.stream_id[b];
-  const int hkv = qh / (a.Hq / a.Hkv);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int sub = lane / LPK, li = lane % LPK;
+  const int G = a.Hq / a.Hkv;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int g = lane >> 2, t4 = lane & 3;
   const int count = bp.count[b];
   const bool bank_full = (a.M > 0 && count == a.M);
   // first phase of the cluster's barrier: "this CTA runs", so that nobody writes into the shared memory of a
-  // CTA that has not started; everyone arrives here and waits only just before its one remote write
+  // CTA that has not started; everyone arrives here and waits only just before its remote writes
   if (a.nsplit > 1) cluster_arrive_relaxed();
 
   int P, NB, TL;
@@ -67,205 +88,221 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(DecodeArgs 
   const int Lv = P + NB + TL;
   const int begin = (int)(((long long)Lv * split) / a.nsplit);
   const int end = (int)(((long long)Lv * (split + 1)) / a.nsplit);
+  const int n_tiles = (end - begin + kTileKeys - 1) / kTileKeys;
 
   const size_t hoff = (size_t)sid * a.Hkv + hkv;
-  const bf16* pk = a.prefix_k + hoff * a.maxP * D + li * 8;
-  const bf16* pv = a.prefix_v + hoff * a.maxP * D + li * 8;
-  const bf16* bk = a.bank_k + hoff * a.slots * D + li * 8;
-  const bf16* bv = a.bank_v + hoff * a.slots * D + li * 8;
-  const bf16* tk = a.tail_k + hoff * a.maxT * D + li * 8;
-  const bf16* tv = a.tail_v + hoff * a.maxT * D + li * 8;
-
+  const size_t o_pre = hoff * a.maxP * D, o_bank = hoff * a.slots * D, o_tail = hoff * a.maxT * D;
+  // row v of the key axis, as an element offset, and which of the three stores it lies in
+  auto row_of = [&](int v, const bf16* p, const bf16* bk, const bf16* t) {
+    return v < P ? p + o_pre + (size_t)v * D : (v < P + NB ? bk + o_bank + (size_t)(v - P) * D : t + o_tail + (size_t)(v - P - NB) * D);
+  };
   // Only the step's own token (the last key) was written by the kernel just before this one; every
   // other key, and the bank's metadata, date from earlier steps, whose kernels had completed before
-  // that kernel let this one start.  So the first pass of K/V rows is fetched before the wait.
+  // that kernel let this one start.  So the first tile of K/V rows is fetched before the wait.
   // The slot being refilled holds no carrier: its key is fetched like any other (the row exists)
   // and masked when the scores are formed.
   const int hole = bank_full ? P + a.meta[sid].free_slot : -1;
   const int own_v = Lv - 1;
-  constexpr int kStride = kDecWarps * KPW;
-  // late == false: every key of the pass but the step's own; late == true: the step's own only
-  auto load_pass = [&](int wbase, uint4 (&kr)[kBatch], uint4 (&vr)[kBatch], bool late) {
+  uint4 kr[2][KC], vr[4][VC];
+  const int kofs = 4 * (g >> 1) + (g & 1);               // S^T rows g and g + 8 are keys kofs and kofs + 2 of the tile
+  // late == false: every key of the tile but the step's own; late == true: the step's own only
+  auto load_tile = [&](int v0, bool late) {
 #pragma unroll
-    for (int u = 0; u < kBatch; ++u) {
-      const int v = wbase + sub + u * kStride;
+    for (int i = 0; i < 2; ++i) {
+      const int v = v0 + kofs + 2 * i;
       if (v < end && ((v == own_v) == late)) {
-        const bf16* kp; const bf16* vp;
-        if (v < P) { kp = pk + (size_t)v * D; vp = pv + (size_t)v * D; }
-        else if (v < P + NB) { kp = bk + (size_t)(v - P) * D; vp = bv + (size_t)(v - P) * D; }
-        else { kp = tk + (size_t)(v - P - NB) * D; vp = tv + (size_t)(v - P - NB) * D; }
-        kr[u] = *reinterpret_cast<const uint4*>(kp);
-        vr[u] = *reinterpret_cast<const uint4*>(vp);
+        const uint4* kp = reinterpret_cast<const uint4*>(row_of(v, a.prefix_k, a.bank_k, a.tail_k));
+#pragma unroll
+        for (int c = 0; c < KC; ++c) kr[i][c] = kp[t4 + 4 * c];
       } else if (!late) {
-        kr[u] = make_uint4(0, 0, 0, 0); vr[u] = make_uint4(0, 0, 0, 0);
+#pragma unroll
+        for (int c = 0; c < KC; ++c) kr[i][c] = make_uint4(0, 0, 0, 0);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int v = v0 + 4 * t4 + r;
+      if (v < end && ((v == own_v) == late)) {
+        const uint4* vp = reinterpret_cast<const uint4*>(row_of(v, a.prefix_v, a.bank_v, a.tail_v));
+#pragma unroll
+        for (int c = 0; c < VC; ++c) vr[r][c] = vp[g + 8 * c];
+      } else if (!late) {
+#pragma unroll
+        for (int c = 0; c < VC; ++c) vr[r][c] = make_uint4(0, 0, 0, 0);
       }
     }
   };
-  const int wbase0 = begin + warp * KPW;                 // keys are dealt to (warp, lane group) round-robin
-  uint4 kr0[kBatch], vr0[kBatch];
-  load_pass(wbase0, kr0, vr0, false);
+  if (warp < n_tiles) load_tile(begin + warp * kTileKeys, false);
 
   VS_STAMP(bp, 5, 0);
   pdl_wait();
   pdl_launch_dependents();
   VS_STAMP(bp, 5, 1);
   // the step's own key and the query are both fresh: their loads go out together
-  if (wbase0 < end) load_pass(wbase0, kr0, vr0, true);
-
-  // this lane's 8 dims of the query (bf16 hi + lo pair), pre-scaled into the log2 domain
-  float q[8];
-  {
-    const size_t qo = (size_t)b * a.Hq * D + (size_t)qh * D + li * 8;
-    const uint4 raw = *reinterpret_cast<const uint4*>(a.q + qo);
-    const uint4 raw_lo = *reinterpret_cast<const uint4*>(a.q_lo + qo);
-    const __nv_bfloat162* h2 = reinterpret_cast<const __nv_bfloat162*>(&raw);
-    const __nv_bfloat162* l2 = reinterpret_cast<const __nv_bfloat162*>(&raw_lo);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float2 f = __bfloat1622float2(h2[i]);
-      const float2 fl = __bfloat1622float2(l2[i]);
-      q[2 * i] = (f.x + fl.x) * a.scale_log2e; q[2 * i + 1] = (f.y + fl.y) * a.scale_log2e;
-    }
-  }
-  float m = -INFINITY, l = 0.f, o[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) o[i] = 0.f;
-
-  auto compute_pass = [&](int wbase, const uint4 (&kr)[kBatch], const uint4 (&vr)[kBatch]) {
-    float s[kBatch];
-    float mx = m;
-#pragma unroll
-    for (int u = 0; u < kBatch; ++u) {
-      const int v = wbase + sub + u * kStride;
-      const __nv_bfloat162* k2 = reinterpret_cast<const __nv_bfloat162*>(&kr[u]);
-      float d = 0.f;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float2 f = __bfloat1622float2(k2[i]);
-        d = fmaf(q[2 * i], f.x, d); d = fmaf(q[2 * i + 1], f.y, d);
-      }
-#pragma unroll
-      for (int off = LPK / 2; off > 0; off >>= 1) d += __shfl_xor_sync(0xffffffffu, d, off);
-      s[u] = (v < end && v != hole) ? d : -INFINITY;
-      mx = fmaxf(mx, s[u]);
-    }
-    if (mx > -INFINITY) {
-      const float sc = exp2f(m - mx);                    // exp2f(-inf) = 0 on the first keys
-      l *= sc;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) o[i] *= sc;
-      m = mx;
-#pragma unroll
-      for (int u = 0; u < kBatch; ++u) {
-        const float p = exp2f(s[u] - mx);
-        l += p;
-        const __nv_bfloat162* v2 = reinterpret_cast<const __nv_bfloat162*>(&vr[u]);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float2 f = __bfloat1622float2(v2[i]);
-          o[2 * i] = fmaf(p, f.x, o[2 * i]);
-          o[2 * i + 1] = fmaf(p, f.y, o[2 * i + 1]);
-        }
-      }
-    }
-  };
-  if (wbase0 < end) compute_pass(wbase0, kr0, vr0);      // uniform over the warp
-  for (int wbase = wbase0 + kBatch * kStride; wbase < end; wbase += kBatch * kStride) {
-    uint4 kr[kBatch], vr[kBatch];
-    load_pass(wbase, kr, vr, false);
-    load_pass(wbase, kr, vr, true);
-    compute_pass(wbase, kr, vr);
-  }
-
-  // lane groups of a warp merge by shuffles (they own the same dims of different keys)
-#pragma unroll
-  for (int off = LPK; off < 32; off <<= 1) {
-    const float m2 = __shfl_xor_sync(0xffffffffu, m, off);
-    const float l2 = __shfl_xor_sync(0xffffffffu, l, off);
-    const float mn = fmaxf(m, m2);
-    const float w1 = (m == -INFINITY) ? 0.f : exp2f(m - mn);
-    const float w2 = (m2 == -INFINITY) ? 0.f : exp2f(m2 - mn);
-    l = l * w1 + l2 * w2;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const float o2 = __shfl_xor_sync(0xffffffffu, o[i], off);
-      o[i] = o[i] * w1 + o2 * w2;
-    }
-    m = mn;
-  }
-  if (sub == 0) {
-    if (li == 0) { st_m[warp] = m; st_l[warp] = l; }
-#pragma unroll
-    for (int i = 0; i < 8; ++i) st_o[warp][li * 8 + i] = o[i];
+  if (warp < n_tiles) load_tile(begin + warp * kTileKeys, true);
+  for (int i = tid; i < 2 * kHeads * (D / 8); i += kDecThreads) {
+    const int which = i / (kHeads * (D / 8)), r = i - which * (kHeads * (D / 8)), hd = r / (D / 8), c = r - hd * (D / 8);
+    uint4 v = make_uint4(0, 0, 0, 0);
+    if (hd < G) v = reinterpret_cast<const uint4*>((which ? a.q_lo : a.q) + ((size_t)b * a.Hq + (size_t)hkv * G + hd) * D)[c];
+    q_s[which][hd][c ^ ((hd & 1) << 2)] = v;
   }
   __syncthreads();
+  VS_STAMP(bp, 5, 2);
 
-  // warps -> CTA
-  const bool direct = a.nsplit == 1;
-  const size_t out_off = (size_t)b * a.Hq * D + (size_t)qh * D;
-  // the residual input is needed by whoever writes the row: fetched ahead of the cluster barrier
-  float h_res = 0.f;
-  if (a.h_out != nullptr && split == 0 && threadIdx.x < D) h_res = __bfloat162float(a.h_in[out_off + threadIdx.x]);
-  float M_cta = -INFINITY, L_cta = 0.f, O_cta = 0.f;      // this CTA's partial triple (threads below D)
-  if (threadIdx.x < D) {
-    const int c = threadIdx.x;
-    float M = -INFINITY;
+  float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};     // heads 2 * t4 and 2 * t4 + 1
+  float o[MT][4];
 #pragma unroll
-    for (int w = 0; w < kDecWarps; ++w) M = fmaxf(M, st_m[w]);
-    float L = 0.f, O = 0.f;
+  for (int j = 0; j < MT; ++j) { o[j][0] = 0.f; o[j][1] = 0.f; o[j][2] = 0.f; o[j][3] = 0.f; }
+
+  for (int ti = warp; ti < n_tiles; ti += kDecWarps) {
+    const int v0 = begin + ti * kTileKeys;
+    if (ti != warp) { load_tile(v0, false); load_tile(v0, true); }
+    float s[4] = {0.f, 0.f, 0.f, 0.f}, sl[4] = {0.f, 0.f, 0.f, 0.f};   // high and low query halves: two shorter chains
+#pragma unroll
+    for (int c = 0; c < KC; ++c) {
+      const int ch = (t4 + 4 * c) ^ ((g & 1) << 2);
+      const uint4 qh = q_s[0][g][ch], ql = q_s[1][g][ch];
+      mma_bf16(s, kr[0][c].x, kr[1][c].x, kr[0][c].y, kr[1][c].y, qh.x, qh.y);
+      mma_bf16(sl, kr[0][c].x, kr[1][c].x, kr[0][c].y, kr[1][c].y, ql.x, ql.y);
+      mma_bf16(s, kr[0][c].z, kr[1][c].z, kr[0][c].w, kr[1][c].w, qh.z, qh.w);
+      mma_bf16(sl, kr[0][c].z, kr[1][c].z, kr[0][c].w, kr[1][c].w, ql.z, ql.w);
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) s[e] += sl[e];
+    const int va = v0 + kofs, vb = va + 2;
+    const bool ina = va < end && va != hole, inb = vb < end && vb != hole;
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      s[e] = ina ? s[e] * a.scale_log2e : -INFINITY;
+      s[2 + e] = inb ? s[2 + e] * a.scale_log2e : -INFINITY;
+      float mx = fmaxf(s[e], s[2 + e]);
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 4));
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
+      const float mn = fmaxf(m[e], mx);
+      const float mu = (mn == -INFINITY) ? 0.f : mn;          // a tile of masked keys alone
+      const float sc = exp2f(m[e] - mu);                      // exp2f(-inf) = 0 on the first keys
+      s[e] = exp2f(s[e] - mu);
+      s[2 + e] = exp2f(s[2 + e] - mu);
+      l[e] = l[e] * sc + (s[e] + s[2 + e]);
+      m[e] = mn;
+#pragma unroll
+      for (int j = 0; j < MT; ++j) { o[j][e] *= sc; o[j][2 + e] *= sc; }
+    }
+    const uint32_t pa = pack2(s[0], s[1]), pb = pack2(s[2], s[3]);
+    const float2 fa = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&pa));
+    const float2 fb = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&pb));
+    const uint32_t ph0 = transpose_8x8(pa), ph1 = transpose_8x8(pb);
+    const uint32_t pl0 = transpose_8x8(pack2(s[0] - fa.x, s[1] - fa.y)), pl1 = transpose_8x8(pack2(s[2] - fb.x, s[3] - fb.y));
+#pragma unroll
+    for (int j = 0; j < MT; ++j) {
+      // tile j: row g = dim 8 g + j, row g + 8 = dim D / 2 + 8 g + j (D = 128) or 8 g + 4 + j (D = 64); k 2 t4, 2 t4 + 1 =
+      // keys 4 t4, 4 t4 + 1 of the tile, k 2 t4 + 8, + 9 = keys 4 t4 + 2, + 3
+      const int j2 = (D == 128) ? j : j + 4, c2 = (D == 128) ? VC - 1 : 0;
+      const uint32_t sel = (j & 1) ? 0x7632u : 0x5410u;
+      const uint32_t a0 = __byte_perm(word(vr[0][0], j >> 1), word(vr[1][0], j >> 1), sel);
+      const uint32_t a1 = __byte_perm(word(vr[0][c2], j2 >> 1), word(vr[1][c2], j2 >> 1), sel);
+      const uint32_t a2 = __byte_perm(word(vr[2][0], j >> 1), word(vr[3][0], j >> 1), sel);
+      const uint32_t a3 = __byte_perm(word(vr[2][c2], j2 >> 1), word(vr[3][c2], j2 >> 1), sel);
+      mma_bf16(o[j], a0, a1, a2, a3, ph0, ph1);
+      mma_bf16(o[j], a0, a1, a2, a3, pl0, pl1);
+    }
+  }
+
+  VS_STAMP(bp, 5, 3);
+  // warps -> CTA (a warp without a tile has nothing to leave)
+  const int n_used = min(n_tiles, kDecWarps);
+  if (warp < n_used) {
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+#pragma unroll
+      for (int off = 4; off < 32; off <<= 1) l[e] += __shfl_xor_sync(0xffffffffu, l[e], off);
+      if (g == 0) st_ml[warp][2 * t4 + e] = make_float2(m[e], l[e]);
+      float4* dst = reinterpret_cast<float4*>(st_o[warp][2 * t4 + e]);
+#pragma unroll
+      for (int hh = 0; hh < 2; ++hh)
+#pragma unroll
+        for (int j = 0; j < MT; j += 4)
+          dst[merge_unit(2 * t4 + e, (D == 128 ? hh * 16 + j / 4 : hh) + 2 * g)] =
+              make_float4(o[j][2 * hh + e], o[j + 1][2 * hh + e], o[j + 2][2 * hh + e], o[j + 3][2 * hh + e]);
+    }
+  }
+  const int nsplit = a.nsplit;
+  const int slice = G * D / nsplit;                      // outputs (head, dim) that one CTA of the cluster finishes
+  const size_t out_off = ((size_t)b * a.Hq + (size_t)hkv * G) * D;
+  // the residual input of what this thread stores: fetched ahead of the barriers
+  const int my = nsplit == 1 ? 4 * tid : split * slice + 4 * tid;
+  const bool mine = 4 * tid < slice;
+  uint2 h_res = make_uint2(0u, 0u);
+  if (a.h_out != nullptr && mine) h_res = *reinterpret_cast<const uint2*>(a.h_in + out_off + my);
+  __syncthreads();
+
+  auto store_row = [&](float4 v) {
+    if (a.out_fp32) *reinterpret_cast<float4*>(static_cast<float*>(a.out) + out_off + my) = v;
+    else *reinterpret_cast<uint2*>(static_cast<bf16*>(a.out) + out_off + my) = make_uint2(pack2(v.x, v.y), pack2(v.z, v.w));
+    if (a.h_out != nullptr && VS_STORE_OK(bp, a.h_out_region, a.h_out + out_off + my, 8)) {
+      const float2 h0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&h_res.x));
+      const float2 h1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&h_res.y));
+      *reinterpret_cast<uint2*>(a.h_out + out_off + my) = make_uint2(pack2(h0.x + v.x, h0.y + v.y), pack2(h1.x + v.z, h1.y + v.w));
+    }
+  };
+  // this CTA's partial of outputs 4 tid .. + 3 (G * D <= 1024 of them), all of one head
+  const int idx = 4 * tid, hd = idx / D, dim = idx - hd * D;
+  float M = -INFINITY, Lsum = 0.f;
+  float4 O = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (hd < G) {
+#pragma unroll
+    for (int w = 0; w < kDecWarps; ++w) if (w < n_used) M = fmaxf(M, st_ml[w][hd].x);
 #pragma unroll
     for (int w = 0; w < kDecWarps; ++w) {
-      const float wt = (st_m[w] == -INFINITY) ? 0.f : exp2f(st_m[w] - M);
-      L += st_l[w] * wt;
-      O += st_o[w][c] * wt;
-    }
-    if (direct) {
-      const float val = (L > 0.f) ? O / L : 0.f;
-      if (a.out_fp32) static_cast<float*>(a.out)[out_off + c] = val;
-      else static_cast<bf16*>(a.out)[out_off + c] = __float2bfloat16_rn(val);
-      if (a.h_out != nullptr && VS_STORE_OK(bp, a.h_out_region, a.h_out + out_off + c, 2)) a.h_out[out_off + c] = __float2bfloat16_rn(h_res + val);
-    } else {
-      M_cta = M; L_cta = L; O_cta = O;
-    }
-  }
-  if (direct) { VS_STAMP(bp, 5, 15); return; }
-
-  // Every CTA of the cluster (the key splits of this stream and query head) leaves its partial triple in rank 0's
-  // shared memory and arrives at the cluster's barrier; only rank 0 waits there, then combines what it was given.
-  // The other CTAs are done: nothing of theirs is read after they exit.
-  VS_STAMP(bp, 5, 4);
-  cluster_wait_acquire();                           // phase 1 (every CTA of the cluster has started) -- long since complete
-  if (threadIdx.x < D) {
-    const int c = threadIdx.x;
-    st_shared_cluster_f32(map_shared_rank(static_cast<uint32_t>(__cvta_generic_to_shared(&peer_o[split][c])), 0u), O_cta);
-    if (c == 0) {
-      const uint32_t ml = map_shared_rank(static_cast<uint32_t>(__cvta_generic_to_shared(&peer_ml[split][0])), 0u);
-      st_shared_cluster_f32(ml, M_cta);
-      st_shared_cluster_f32(ml + 4, L_cta);
-    }
-  }
-  cluster_arrive_release();                         // phase 2: "my triple is in place"
-  if (split != 0) { VS_STAMP(bp, 5, 15); return; }
-  cluster_wait_acquire();
-  VS_STAMP(bp, 5, 5);
-  if (threadIdx.x < D) {
-    const int c = threadIdx.x;
-    float M = -INFINITY;
-#pragma unroll
-    for (int r = 0; r < kMaxCluster; ++r) if (r < a.nsplit) M = fmaxf(M, peer_ml[r][0]);
-    float L = 0.f, val = 0.f;
-#pragma unroll
-    for (int r = 0; r < kMaxCluster; ++r) {
-      if (r < a.nsplit) {
-        const float wt = (peer_ml[r][0] == -INFINITY) ? 0.f : exp2f(peer_ml[r][0] - M);
-        L = fmaf(peer_ml[r][1], wt, L);
-        val = fmaf(peer_o[r][c], wt, val);
+      if (w < n_used) {
+        const float2 ml = st_ml[w][hd];
+        const float wt = (ml.x == -INFINITY) ? 0.f : exp2f(ml.x - M);
+        const float4 v = reinterpret_cast<const float4*>(st_o[w][hd])[merge_unit(hd, dim / 4)];
+        Lsum = fmaf(ml.y, wt, Lsum);
+        O.x = fmaf(v.x, wt, O.x); O.y = fmaf(v.y, wt, O.y); O.z = fmaf(v.z, wt, O.z); O.w = fmaf(v.w, wt, O.w);
       }
     }
-    val = (L > 0.f) ? val / L : 0.f;
-    if (a.out_fp32) static_cast<float*>(a.out)[out_off + c] = val;
-    else static_cast<bf16*>(a.out)[out_off + c] = __float2bfloat16_rn(val);
-    if (a.h_out != nullptr && VS_STORE_OK(bp, a.h_out_region, a.h_out + out_off + c, 2)) a.h_out[out_off + c] = __float2bfloat16_rn(h_res + val);
+  }
+  if (nsplit == 1) {
+    const float inv = (Lsum > 0.f) ? 1.f / Lsum : 0.f;
+    if (mine) store_row(make_float4(O.x * inv, O.y * inv, O.z * inv, O.w * inv));
+    VS_STAMP(bp, 5, 15);
+    return;
+  }
+
+  VS_STAMP(bp, 5, 4);
+  cluster_wait_acquire();                           // phase 1 (every CTA of the cluster has started) -- long since complete
+  if (hd < G) {
+    const int owner = idx / slice;                  // slice is a multiple of 4
+    const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(&peer_o[split * slice + idx - owner * slice]));
+    st_shared_cluster_f4(map_shared_rank(dst, (uint32_t)owner), O);
+    if (dim < 4 * nsplit) {                         // thread dim / 4 of the head tells rank dim / 4 the head's (max, denominator)
+      const uint32_t ml = static_cast<uint32_t>(__cvta_generic_to_shared(&peer_ml[split][hd]));
+      st_shared_cluster_f2(map_shared_rank(ml, (uint32_t)(dim >> 2)), make_float2(M, Lsum));
+    }
+  }
+  cluster_arrive_release();                         // phase 2: "my partials are in place"
+  cluster_wait_acquire();                           // nothing of a peer is read or written from here on
+  VS_STAMP(bp, 5, 5);
+  if (mine) {
+    const int h2 = my / D;
+    float Mx = -INFINITY;
+    for (int r = 0; r < nsplit; ++r) Mx = fmaxf(Mx, peer_ml[r][h2].x);
+    float den = 0.f;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int r = 0; r < kMaxCluster; ++r) {
+      if (r < nsplit) {
+        const float2 ml = peer_ml[r][h2];
+        const float wt = (ml.x == -INFINITY) ? 0.f : exp2f(ml.x - Mx);
+        const float4 p = *reinterpret_cast<const float4*>(&peer_o[r * slice + 4 * tid]);
+        den = fmaf(ml.y, wt, den);
+        v.x = fmaf(p.x, wt, v.x); v.y = fmaf(p.y, wt, v.y); v.z = fmaf(p.z, wt, v.z); v.w = fmaf(p.w, wt, v.w);
+      }
+    }
+    const float inv = (den > 0.f) ? 1.f / den : 0.f;
+    store_row(make_float4(v.x * inv, v.y * inv, v.z * inv, v.w * inv));
   }
   VS_STAMP(bp, 5, 15);
 }
@@ -275,7 +312,7 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(DecodeArgs 
 cudaError_t launch_decode_attention(const DecodeArgs& a, const BatchParams& bp, cudaStream_t st) {
   if (a.nsplit != 1 && a.nsplit != 2 && a.nsplit != 4 && a.nsplit != 8) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(a.nsplit, a.Hq, bp.n_active);
+  cfg.gridDim = dim3(a.nsplit, a.Hkv, bp.n_active);
   cfg.blockDim = dim3(kDecThreads);
   cfg.dynamicSmemBytes = 0;
   cfg.stream = st;

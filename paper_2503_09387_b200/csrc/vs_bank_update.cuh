@@ -106,7 +106,7 @@ __device__ __forceinline__ void bank_update_block(const BankUpdateArgs& a, const
     const int n_warps = (int)blockDim.x >> 5;
     double nb = 0.0;                                  // policy 0: the incoming carrier's norm, worked out with the first row
     bool first = true;
-    for (int j = block * n_warps + (tid >> 5); j < count; j += n_blocks * n_warps) {
+    for (int j = (tid >> 5) * n_blocks + block; j < count; j += n_blocks * n_warps) {
       const bf16* va = a.emb + ((size_t)sid * a.slots + order[j]) * a.d;
       double dot, na;
       if (a.policy == 1) {

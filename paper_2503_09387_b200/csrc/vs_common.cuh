@@ -55,7 +55,7 @@ struct BatchParams {
 enum DbgRegion { DR_BANK_K = 0, DR_BANK_V, DR_PREFIX_K, DR_PREFIX_V, DR_TAIL_K, DR_TAIL_V, DR_EMB, DR_META, DR_ORDER,
                  DR_SLOT_FRAME, DR_SLOT_POS, DR_EVICT_LOG, DR_SCORES, DR_STEP_SLOT, DR_CHUNK_SLOT, DR_CHUNK_VICTIM,
                  DR_GEMM_FLAGS, DR_HBUF0, DR_HBUF1, DR_XN, DR_ROW_SS, DR_Q, DR_Q_LO, DR_Q_TILED, DR_KF, DR_VF, DR_ROPE,
-                 DR_OBUF, DR_EMB_STAGE, DR_CHUNK_SCORES, DR_GEMM_XCHG, DR_ACT, DR_COUNT };
+                 DR_OBUF, DR_EMB_STAGE, DR_CHUNK_SCORES, DR_GEMM_XCHG, DR_ACT, DR_TOK, DR_COUNT };
 struct DebugTable {
   unsigned long long begin[DR_COUNT], end[DR_COUNT];   // device addresses
   int bad_region;                                      // -1, or the region of the first refused store
@@ -90,6 +90,8 @@ struct Dims {
 
 constexpr int KSPLIT_MAX = 4;   // CTAs sharing one output tile of the projection along K
 constexpr int DEC_SPLIT_MAX = 8;      // key splits of the decode attention = CTAs of one cluster
+constexpr int TOK_MAX_ROWS = 32;      // token rows of a step that the persistent kernel takes
+constexpr int TOK_MAX_CTAS = 160;     // ... one CTA per SM
 constexpr int GEMM_BLOCK_M = 128;
 constexpr int GEMM_BLOCK_K = 64;
 constexpr int GEMM_XCHG_CTAS = 160;   // most CTAs a K-split projection launches (one per SM)
@@ -113,6 +115,8 @@ struct Layout {
   size_t chunk_slot;            // int32 [VS_MAX_BATCH]  chunked prefill: slot each frame's carrier went to
   size_t chunk_victim;          // int32 [VS_MAX_BATCH]  ... and whom its bank update evicted (index on the bank axis)
   size_t gemm_flags;            // int32 [GEMM_XCHG_CTAS]  projection K split: partials delivered per slice owner
+  size_t tok_layers;            // TokLayer [L], then the vocabulary projection's tensor maps [2], as the token-step kernel reads them
+  size_t tok_sync;              // its counters, flags and tickets, zero between launches
   size_t lm_keys, lm_tickets;   // uint64 [256], int32 [256]  language-model head: greedy-choice keys and tickets per row
   size_t persistent_end;
   // per-step scratch
@@ -130,6 +134,7 @@ struct Layout {
   size_t emb_stage;             // bf16 [max_chunk][d]  chunked prefill: carrier embeddings before they have a slot
   size_t chunk_scores;          // f64  [max_chunk][slots + max_chunk]  chunked prefill: cosines of (frame, candidate) pairs
   size_t gemm_xchg;             // f32  [GEMM_XCHG_CTAS][256][128]  projection K split: partial tiles
+  size_t tok;                   // token-step kernel: partial sums of cut tiles, attention shares, row statistics
   size_t scratch_begin, scratch_end;
   size_t total;
   // checked build: the regions as the kernels name them, and the table the kernels read
@@ -184,6 +189,10 @@ __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepc
 __device__ __forceinline__ void prefetch_l2_bulk(const void* p, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
+// Decode attention, merging the warps of a CTA (rows of D fp32, one per query head of a group of up to 8):
+// 16-byte unit u of head hd's row in the merge buffer: spread so that the eight lanes that store side by side (two groups of dims,
+// four head pairs) and the eight that read side by side (one row) hit different banks
+__device__ __forceinline__ int merge_unit(int hd, int u) { return u ^ (((hd >> 1) & 1) | (((hd >> 2) & 1) << 2)); }
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
   cudaLaunchConfig_t cfg = {};
@@ -397,7 +406,49 @@ struct DecodeArgs {
   int to_prefix;                 // 1: the keys are the prefix alone (incl. the new token)
   float scale_log2e;
 };
+cudaError_t launch_decode_attention_heads(const DecodeArgs& a, const BatchParams& bp, cudaStream_t st);   // a CTA per query head
 cudaError_t launch_decode_attention(const DecodeArgs& a, const BatchParams& bp, cudaStream_t st);
+
+// A step of up to TOK_MAX_ROWS token rows through all layers, or the language-model head of as many rows: one persistent
+// kernel (vs_token.cu).
+struct TokLayer {
+  // the matrices as 4-D tensor maps {64 of K, rows, row groups, K blocks of 64}, 128-byte swizzle, one box = a stage (half of
+  // one for gate and up): 32 rows by [0] 512, [1] 256 elements
+  CUtensorMap tm_qkv[2], tm_o[2], tm_gate[2], tm_up[2], tm_down[2];
+  const bf16 *bias, *gain, *gain2;
+  const void* pad[13];           // (tensor maps start on multiples of 64 bytes)
+};
+static_assert(sizeof(TokLayer) % 128 == 0, "tensor maps of every layer stay aligned");
+struct TokArgs {
+  const TokLayer* layers;        // [L] in device memory
+  int L, rows, d, d_ff, full;    // full: the whole decoder block
+  int Hq, Hkv, D, slots, M, maxP, maxT, to_prefix;
+  int use_rmsnorm, residual, out_fp32, hidden_fp32;
+  int nsplit;                    // shares the keys of a (row, KV head) are cut into
+  float eps, scale_log2e;
+  const void* hidden;            // [rows][d]
+  void* out;                     // [rows][Hq * D]
+  bf16* hbuf[2]; bf16* xn; bf16* act; bf16* attn_rows; bf16* q; bf16* q_lo; bf16* kf; bf16* vf;
+  bf16 *prefix_k, *prefix_v, *bank_k, *bank_v, *tail_k, *tail_v;     // layer 0
+  size_t ls_prefix, ls_bank, ls_tail;                                // elements from layer to layer
+  const StreamMeta* meta;
+  const double* inv_freq;
+  float* ss; int ss_cap;         // [2][TOK_MAX_ROWS][ss_cap] parts of the rows' sums of squares (second half: post-attention norm)
+  float* part;                   // [CTA][8][32] float4: the end of a tile that another CTA began
+  float* att_part;               // [unit][8 * D + 16]: unnormalised rows of a share with their (max, denominator)
+  int *counters, *frag_flags, *tickets, *done;
+  int* status;
+  // language-model head (vocab > 0): rows of `hidden` -> fp32 logits and, if next_token, the greedy choice
+  int vocab;
+  const CUtensorMap* tm_lm;      // [2] in device memory
+  const bf16* gain_f;
+  float* logits; int32_t* next_token; unsigned long long* lm_keys;
+  int stages; uint32_t ring_bytes;                                   // set by the launch
+};
+inline size_t tok_sync_ints(int L, int Hkv) { return (size_t)(1 + 5 * L) * 32 + (size_t)TOK_MAX_CTAS * 8 + (size_t)TOK_MAX_ROWS * Hkv + 1; }
+cudaError_t token_step_init();   // opt-in shared memory attribute, once per process/device
+int token_step_split(int max_keys, int rows, int n_kv_heads, int n_sms);
+cudaError_t launch_token_step(const TokArgs& a, const BatchParams& bp, int n_sms, cudaStream_t st);
 
 
 // rows i < count of x = emb[sid][order[i]]: the bank's carrier embeddings in temporal order

@@ -76,6 +76,12 @@ constexpr size_t kGuardBytes = 0;
 #endif
 constexpr unsigned char kGuardByte = 0xC5;
 
+// scratch of the token-step kernel: partial sums of cut tiles, attention shares, parts of the rows' sums of squares
+size_t tok_part_bytes() { return (size_t)TOK_MAX_CTAS * 8 * 32 * 16; }
+size_t tok_att_bytes(const Dims& D) { return (size_t)TOK_MAX_CTAS * (8 * D.D + 16) * 4; }
+int tok_ss_cap(const Dims& D) { return D.d / 16 > D.Hkv ? D.d / 16 : D.Hkv; }
+size_t tok_ss_bytes(const Dims& D) { return (size_t)2 * TOK_MAX_ROWS * tok_ss_cap(D) * 4; }
+
 void fill_layout(const Dims& D, Layout& Lo) {
   size_t off = 0;
   size_t last_bytes = 0;
@@ -101,6 +107,8 @@ void fill_layout(const Dims& D, Layout& Lo) {
   Lo.chunk_slot = reg(DR_CHUNK_SLOT, take((size_t)VS_MAX_BATCH * 4));
   Lo.chunk_victim = reg(DR_CHUNK_VICTIM, take((size_t)VS_MAX_BATCH * 4));
   Lo.gemm_flags = reg(DR_GEMM_FLAGS, take((size_t)GEMM_XCHG_CTAS * 4));
+  Lo.tok_layers = take((size_t)D.L * sizeof(TokLayer) + 2 * sizeof(CUtensorMap));
+  Lo.tok_sync = take(tok_sync_ints(D.L, D.Hkv) * 4);
   Lo.lm_keys = take((size_t)256 * 8);          // language-model head: per-row argmax keys and tickets, zero between calls
   Lo.lm_tickets = take((size_t)256 * 4);
   Lo.dbg_table = take(sizeof(DebugTable));
@@ -122,6 +130,7 @@ void fill_layout(const Dims& D, Layout& Lo) {
   Lo.obuf = reg(DR_OBUF, take((size_t)D.R_max * D.Hq * D.D * 4));
   Lo.emb_stage = reg(DR_EMB_STAGE, take((size_t)D.maxChunk * D.d * 2));
   Lo.chunk_scores = reg(DR_CHUNK_SCORES, take((size_t)D.maxChunk * (D.slots + D.maxChunk) * 8));
+  Lo.tok = reg(DR_TOK, take(tok_part_bytes() + tok_att_bytes(D) + tok_ss_bytes(D)));
   Lo.gemm_xchg = reg(DR_GEMM_XCHG, take((size_t)GEMM_XCHG_CTAS * 256 * GEMM_BLOCK_M * 4));
   Lo.scratch_end = off;
   Lo.total = off;
@@ -180,6 +189,18 @@ int encode_2d(vs_stream* h, CUtensorMap* tm, const void* base, uint64_t inner, u
                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? VS_OK : VS_ERR_CUDA;
+}
+
+// A weight matrix [groups * rows][K] for the token-step kernel: dimensions {64, rows, groups, K / 64}, so that one copy brings
+// box_k blocks of 64 elements of box_rows rows of box_groups groups; blocks past the end of a row read as zeros.
+bool encode_weight(vs_stream* h, CUtensorMap* tm, const void* base, uint64_t K, uint64_t rows, uint64_t groups, uint32_t box_rows,
+                   uint32_t box_groups, uint32_t box_k) {
+  cuuint64_t dims[4] = {64, rows, groups, K / 64};
+  cuuint64_t strides[3] = {K * 2, rows * K * 2, 128};
+  cuuint32_t box[4] = {64, box_rows, box_groups, box_k};
+  cuuint32_t estr[4] = {1, 1, 1, 1};
+  return h->encode(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                   CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 // K or V rows for the attention kernel: dimensions {head_dim, rows, Z}, box {64, ATTN_KEY_BOX, 1}, 128-byte swizzle;
@@ -385,6 +406,53 @@ size_t layer_stride_bank(const Dims& D) { return (size_t)D.S * D.Hkv * D.slots *
 size_t layer_stride_prefix(const Dims& D) { return (size_t)D.S * D.Hkv * D.maxP * D.D; }
 size_t layer_stride_tail(const Dims& D) { return (size_t)D.S * D.Hkv * D.maxT * D.D; }
 
+// Whether a step of n_active x T rows goes to the persistent kernel (measured at the Qwen2-7B shape, us against the launches
+// layer by layer).  Full layers: up to 16 rows (3 layers and the head: 562 -> 437 for one row, 595 -> 549 for 16; 24 rows no
+// longer, their slabs leave the ring too few stages).  Attention alone: steps of several tokens (28 layers: 560 -> 443 for 2
+// rows, 795 -> 722 for 32) and single tokens of more streams than the matrix-vector kernel takes (579 -> 463 for 8), in a stack;
+// one to four single tokens are faster by launches (352 against 463: 11 us a layer is little more than the phases' own
+// synchronisation).  And not where a layer's projection holds less than 16 KB for every SM: there is then no weight stream to hide
+// that synchronisation behind.
+bool token_step_pays(const vs_stream* h, int n_active, int T, int matrix_rows, bool full) {
+  const int rows = n_active * T;
+  if (h->n_sms > TOK_MAX_CTAS || (size_t)matrix_rows * h->dm.d * 2 < (size_t)h->n_sms * 16384) return false;
+  if (full) return rows <= 16;
+  return rows <= TOK_MAX_ROWS && (T > 1 || (rows > 4 && h->dm.L > 1));
+}
+
+// what every launch of the token-step kernel gets
+TokArgs token_args(vs_stream* h, const void* hidden, int rows) {
+  const Dims& D = h->dm;
+  const Layout& lo = h->lo;
+  TokArgs a;
+  std::memset(&a, 0, sizeof(a));
+  a.layers = h->at<TokLayer>(lo.tok_layers);
+  a.L = D.L; a.rows = rows; a.d = D.d; a.d_ff = D.d_ff; a.full = D.d_ff > 0;
+  a.Hq = D.Hq; a.Hkv = D.Hkv; a.D = D.D; a.slots = D.slots; a.M = D.M; a.maxP = D.maxP; a.maxT = D.maxT;
+  a.use_rmsnorm = D.use_rmsnorm; a.residual = D.residual; a.out_fp32 = D.out_fp32;
+  a.nsplit = 1;
+  a.eps = D.rms_eps; a.scale_log2e = (float)(1.4426950408889634 / std::sqrt((double)D.D));
+  a.hidden = hidden;
+  a.hbuf[0] = h->at<bf16>(lo.hbuf[0]); a.hbuf[1] = h->at<bf16>(lo.hbuf[1]);
+  a.xn = h->at<bf16>(lo.xn); a.act = h->at<bf16>(lo.act); a.attn_rows = h->at<bf16>(lo.obuf);
+  a.q = h->at<bf16>(lo.q); a.q_lo = h->at<bf16>(lo.q_lo); a.kf = h->at<bf16>(lo.kf); a.vf = h->at<bf16>(lo.vf);
+  a.prefix_k = h->at<bf16>(lo.prefix_k); a.prefix_v = h->at<bf16>(lo.prefix_v);
+  a.bank_k = h->at<bf16>(lo.bank_k); a.bank_v = h->at<bf16>(lo.bank_v);
+  a.tail_k = h->at<bf16>(lo.tail_k); a.tail_v = h->at<bf16>(lo.tail_v);
+  a.ls_prefix = layer_stride_prefix(D); a.ls_bank = layer_stride_bank(D); a.ls_tail = layer_stride_tail(D);
+  a.meta = h->at<StreamMeta>(lo.meta);
+  a.inv_freq = h->at<double>(lo.inv_freq);
+  a.part = h->at<float>(lo.tok);
+  a.att_part = h->at<float>(lo.tok + tok_part_bytes());
+  a.ss = h->at<float>(lo.tok + tok_part_bytes() + tok_att_bytes(D)); a.ss_cap = tok_ss_cap(D);
+  a.counters = h->at<int>(lo.tok_sync);
+  a.frag_flags = a.counters + (size_t)(1 + 5 * D.L) * 32;
+  a.tickets = a.frag_flags + TOK_MAX_CTAS * 8;
+  a.done = a.tickets + (size_t)TOK_MAX_ROWS * D.Hkv;
+  a.status = h->at<int>(lo.status);
+  return a;
+}
+
 }  // namespace
 
 extern "C" {
@@ -481,10 +549,36 @@ int vs_create_stream(const vs_config* cfg, const vs_weights* weights, void* work
     h->gain_f = static_cast<const bf16*>(weights->norm_f_w);
     if (encode_2d(h, &h->tm_lm, weights->w_lm, (uint64_t)D.d, (uint64_t)D.vocab, GEMM_BLOCK_M) != VS_OK) return fail(VS_ERR_CUDA);
   }
-  if (qkv_gemm_init() != cudaSuccess || qkv_gemv_init() != cudaSuccess || prefill_attention_tc_init() != cudaSuccess) return fail(VS_ERR_CUDA);
+  if (qkv_gemm_init() != cudaSuccess || qkv_gemv_init() != cudaSuccess || token_step_init() != cudaSuccess || prefill_attention_tc_init() != cudaSuccess) return fail(VS_ERR_CUDA);
   for (int sp = 2; sp <= ATTN_MAX_SPLIT; ++sp) h->attn_clusters[sp] = prefill_attention_max_clusters(D.D, sp);
   // clear the whole workspace, then write the non-zero initial metadata
   if (cudaMemset(h->ws, 0, lo.total) != cudaSuccess) return fail(VS_ERR_CUDA);
+  {
+    std::vector<TokLayer> tl(D.L);
+    CUtensorMap lm[2];
+    std::memset(lm, 0, sizeof(lm));
+    bool ok = true;
+    for (int m = 0; m < 2 && ok; ++m) {
+      const uint32_t mt = 2, kb = m == 0 ? 8 : 4;  // 16-row sub-tiles of a weight tile, 64-element blocks of a stage
+      for (int l = 0; l < D.L && ok; ++l) {
+        TokLayer& t = tl[l];
+        if (m == 0) { std::memset(&t, 0, sizeof(TokLayer)); t.bias = h->bias[l]; t.gain = h->gain[l]; }
+        // (a head's halves apart: a tile holds both elements of its rotation pairs)
+        ok = encode_weight(h, &t.tm_qkv[m], h->w[l], D.d, D.D / 2, 2 * (D.Hq + 2 * D.Hkv), 8 * mt, 2, kb);
+        if (D.d_ff > 0) {
+          t.gain2 = h->gain2[l];
+          ok = ok && encode_weight(h, &t.tm_o[m], weights->w_o[l], D.d, D.d, 1, 16 * mt, 1, kb) &&
+               encode_weight(h, &t.tm_gate[m], weights->w_gate[l], D.d, D.d_ff, 1, 8 * mt, 1, kb) &&
+               encode_weight(h, &t.tm_up[m], weights->w_up[l], D.d, D.d_ff, 1, 8 * mt, 1, kb) &&
+               encode_weight(h, &t.tm_down[m], weights->w_down[l], D.d_ff, D.d, 1, 16 * mt, 1, kb);
+        }
+      }
+      if (D.vocab > 0) ok = ok && encode_weight(h, &lm[m], weights->w_lm, D.d, D.vocab, 1, 32, 1, m == 0 ? 8 : 4);
+    }
+    if (!ok || cudaMemcpy(h->ws + lo.tok_layers, tl.data(), tl.size() * sizeof(TokLayer), cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(h->ws + lo.tok_layers + tl.size() * sizeof(TokLayer), lm, sizeof(lm), cudaMemcpyHostToDevice) != cudaSuccess)
+      return fail(VS_ERR_CUDA);
+  }
   if (cudaMemset(h->ws + lo.slot_frame, 0xFF, (size_t)D.S * D.slots * 4) != cudaSuccess) return fail(VS_ERR_CUDA);
   std::vector<StreamMeta> metas(D.S);
   for (auto& m : metas) { std::memset(&m, 0, sizeof(m)); m.victim_logical = -1; m.last_victim_frame = -1; }
@@ -636,10 +730,11 @@ int vs_frame_prefill(vs_stream* h, const int32_t* stream_ids, int32_t n_active, 
       aa.nsplit = attn_split(h, bp, kl, 3);
     }
     // the bank update (Section 3.3, memory mechanism: evict if full, then append) rides in the last layer's launch
-    // (a CTA scores a row per warp, 19 at a time; its plane is as wide as the attention's)
+    // (a row per warp; four rows to a CTA, or as few as its plane, which is as wide as the attention's, allows: more rows on an
+    // SM wait for one another's fp64 conversions, 3 us longer with 19)
     if (last) {
       aa.bank = ba;
-      const int plane = (N + 1 + 15) / 16 * aa.nsplit, wanted = (D.M + 18) / 19;
+      const int plane = (N + 1 + 15) / 16 * aa.nsplit, wanted = (D.M + 3) / 4;
       aa.bank_ctas = !any_full ? 1 : (wanted < plane ? wanted : plane);
     }
     aa.Hq = D.Hq; aa.Hkv = D.Hkv; aa.D = D.D; aa.slots = D.slots; aa.M = D.M;
@@ -998,6 +1093,22 @@ int vs_decode_step(vs_stream* h, const int32_t* stream_ids, int32_t n_active, co
   const int rows = n_active * T;
   StreamMeta* meta = h->at<StreamMeta>(lo.meta);
 
+  if (token_step_pays(h, n_active, T, D.E_out, D.d_ff > 0)) {
+    // a few rows: one persistent launch for all layers
+    TokArgs ta = token_args(h, hidden, rows);
+    ta.out = out;
+    ta.to_prefix = to_prefix ? 1 : 0;
+    ta.nsplit = token_step_split(max_keys, rows, D.Hkv, h->n_sms);
+    VS_LAUNCH(h, st, KC_GEMV, launch_token_step(ta, bp, h->n_sms, st));
+    for (int i = 0; i < n_active; ++i) {
+      HostStream& s = h->hs[stream_ids[i]];
+      if (to_prefix) { s.prefix_len += T; s.next_pos += T; }
+      else s.text_len += T;
+    }
+    h->last_stream = st;
+    h->last_rows = rows;
+    return VS_OK;
+  }
   // a step of up to 16 rows needs no table: the projection works the rotation out itself
   const bool rope_inline = rows <= 16;
   if (!rope_inline) {
@@ -1061,15 +1172,23 @@ int vs_decode_step(vs_stream* h, const int32_t* stream_ids, int32_t n_active, co
       if (D.d_ff > 0) { da.out = h->at<void>(lo.obuf); da.out_fp32 = 0; da.h_in = nullptr; da.h_out = nullptr; }
       da.meta = meta;
       da.Hq = D.Hq; da.Hkv = D.Hkv; da.D = D.D; da.slots = D.slots; da.M = D.M; da.maxP = D.maxP; da.maxT = D.maxT;
-      // short contexts: one CTA per (stream, query head) writes the row directly; longer ones are
-      // split over a cluster of 2, 4 or 8 CTAs (a CTA then walks about 64 to 128 keys), fewer
-      // when many streams already fill the GPU
-      int ns = (max_keys <= 96) ? 1 : (max_keys <= 192 ? 2 : (max_keys <= 448 ? 4 : 8));
-      while (ns > 1 && (long long)ns * D.Hq * n_active > 4LL * h->n_sms) ns >>= 1;
+      // one stream: a CTA per query head, more: per KV head (K and V read once per group)
+      const bool by_head = n_active == 1;
+      int ns = 1;
+      if (by_head) {
+        // short contexts: the CTA writes the row directly; longer ones are split over a cluster of 2, 4 or 8 CTAs (a CTA
+        // then walks about 64 to 128 keys), fewer when the streams already fill the GPU
+        ns = (max_keys <= 96) ? 1 : (max_keys <= 192 ? 2 : (max_keys <= 448 ? 4 : 8));
+        while (ns > 1 && (long long)ns * D.Hq * n_active > 4LL * h->n_sms) ns >>= 1;
+      } else {
+        // a CTA's eight warps take 128 keys in one go: split the axis over a cluster of 2, 4 or 8 CTAs down to that,
+        // as long as all CTAs (two to an SM) run at once
+        while (ns < DEC_SPLIT_MAX && max_keys > 128 * ns && 2LL * ns * D.Hkv * n_active <= 2LL * h->n_sms) ns <<= 1;
+      }
       da.nsplit = ns;
       da.to_prefix = to_prefix ? 1 : 0;
       da.scale_log2e = scale_log2e;
-      VS_LAUNCH(h, st, KC_DECODE_ATTN, launch_decode_attention(da, bp, st));
+      VS_LAUNCH(h, st, KC_DECODE_ATTN, by_head ? launch_decode_attention_heads(da, bp, st) : launch_decode_attention(da, bp, st));
     } else {
       AttnArgs aa;
       std::memset(&aa, 0, sizeof(aa));
@@ -1197,6 +1316,14 @@ int vs_lm_head(vs_stream* h, const void* hidden, int32_t rows, void* logits, int
   bp.rows_per_stream = rows;
   VS_TRACE_NEXT(h, bp);
   bf16* xn = h->at<bf16>(lo.xn);
+  if (token_step_pays(h, rows, 1, D.vocab, true)) {
+    TokArgs ta = token_args(h, hidden, rows);
+    ta.full = 0; ta.hidden_fp32 = D.out_fp32;
+    ta.vocab = D.vocab; ta.tm_lm = reinterpret_cast<const CUtensorMap*>(ta.layers + D.L); ta.gain_f = h->gain_f;
+    ta.logits = static_cast<float*>(logits); ta.next_token = next_token; ta.lm_keys = h->at<unsigned long long>(lo.lm_keys);
+    VS_LAUNCH(h, st, KC_GEMV, launch_token_step(ta, bp, h->n_sms, st));
+    return VS_OK;
+  }
   float* ss = h->at<float>(lo.row_ss);
   VS_LAUNCH(h, st, KC_RMSNORM, launch_lm_norm(hidden, D.out_fp32, D.use_rmsnorm ? h->gain_f : nullptr, xn, ss, D.ss_parts, rows, D.d, st));
   ProjectionOut po;
