@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) prefill_attn_tc_kernel(const 
   // hold no attention CTA, and they take part in no cluster barrier.
   if ((int)blockIdx.y == a.Hkv) {
     pdl_launch_dependents();
-    if ((int)blockIdx.x < a.bank_ctas) bank_update_block<16, 256>(a.bank, bp, (int)blockIdx.z, (int)blockIdx.x, a.bank_ctas);
+    if ((int)blockIdx.x < a.bank_ctas) bank_update_block<16, 256>(a.bank, bp, (int)blockIdx.z, (int)blockIdx.x, a.bank_ctas, smem_raw, (uint32_t)L::kTotal);
     pdl_wait();      // so that this launch has completed only once the kernel ahead of it has
     return;
   }

@@ -13,15 +13,14 @@ __device__ __forceinline__ double warp_tree_sum(double v) {
   return v;
 }
 
-// dot, |a|^2 and (kNormB) |b|^2 over d elements by one warp: lane p sums elements k = p (mod 32) in ascending k in fp64, then
+// dot, |a|^2 and |b|^2 over d elements by one warp: lane p sums elements k = p (mod 32) in ascending k in fp64, then
 // a butterfly 16, 8, 4, 2, 1; the results are the same in every lane.  A product of two bf16 values is exact in fp64, so the
 // fused multiply-add rounds once, exactly where a separate addition would.  The loop is a chain of dependent fp64 adds fed
 // by 2-byte loads, so what it costs is load latency: kU elements of every lane are requested before any is used (one at a
 // time the scoring of a 1024-carrier bank took 33 us beside the attention of a one-layer frame step).
-template <bool kNormB, int kU>
+template <int kU>
 __device__ __forceinline__ void warp_dot_norms(const bf16* va, const bf16* vb, int d, int lane, double& dot, double& na, double& nb) {
-  dot = 0.0; na = 0.0;
-  if (kNormB) nb = 0.0;
+  dot = 0.0; na = 0.0; nb = 0.0;
   const unsigned short* pa = reinterpret_cast<const unsigned short*>(va) + lane;
   const unsigned short* pb = reinterpret_cast<const unsigned short*>(vb) + lane;
   for (int k0 = 0; k0 < d; k0 += 32 * kU) {
@@ -38,11 +37,11 @@ __device__ __forceinline__ void warp_dot_norms(const bf16* va, const bf16* vb, i
       const double y = (double)__uint_as_float((uint32_t)xb[u] << 16);
       dot = __fma_rn(x, y, dot);
       na = __fma_rn(x, x, na);
-      if (kNormB) nb = __fma_rn(y, y, nb);
+      nb = __fma_rn(y, y, nb);
     }
   }
   dot = warp_tree_sum(dot); na = warp_tree_sum(na);
-  if (kNormB) nb = warp_tree_sum(nb);
+  nb = warp_tree_sum(nb);
 }
 
 __device__ __forceinline__ double cosine_of(double dot, double na, double nb) {
@@ -53,18 +52,93 @@ __device__ __forceinline__ double cosine_of(double dot, double na, double nb) {
   return s;
 }
 
-// One of the `n_blocks` thread blocks (any number of them, whole warps) that update the bank of listed stream b.
+__device__ __forceinline__ void bank_cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))), "l"(src) : "memory");
+}
+
+// Scores bank rows j = first, first + step, ... < j1 against the incoming carrier (policy 0), a row per warp: the whole row is
+// fetched into shared memory at once (two buffers a warp, the next row on its way while this one is summed), so a row costs one
+// memory latency, and the incoming carrier is widened to fp64 once per block -- conversions to fp64 run at a sixteenth of
+// the fp32 rate.  (With 16 two-byte loads in flight a lane, 64 rows took 6.5 us beside the attention of a one-layer frame step,
+// longer than the attention; this way 3 us.)  Same sums in the same order as warp_dot_norms.
+__device__ __forceinline__ int staged_warps(int d, uint32_t bytes) {
+  const long long left = (long long)bytes - (long long)d * 8;
+  const int n = left > 0 ? (int)(left / (4LL * d)) : 0;
+  return min(n, (int)blockDim.x >> 5);
+}
+__device__ __forceinline__ void staged_scores(const BankUpdateArgs& a, const BatchParams& bp, const bf16* emb, const int32_t* order, const bf16* emb_in,
+                                              double* scores, int block, int n_blocks, int j1, uint8_t* smem, int n_warps) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, d = a.d;
+  double* ys = reinterpret_cast<double*>(smem);
+  uint8_t* rows = smem + (size_t)d * 8 + (size_t)warp * 4 * d;
+  const int step = n_blocks * n_warps;
+  int j = a.j0 + warp * n_blocks + block;
+  auto fetch = [&](int jj, int buf) {
+    if (jj < j1) {
+      const uint4* src = reinterpret_cast<const uint4*>(emb + (size_t)order[jj] * d);
+      uint4* dst = reinterpret_cast<uint4*>(rows + (size_t)buf * 2 * d);
+      for (int c = lane; c < d / 8; c += 32) bank_cp_async16(dst + c, src + c);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  if (warp < n_warps) { fetch(j, 0); fetch(j + step, 1); }
+  for (int c = tid; c < d / 8; c += (int)blockDim.x) {
+    const uint4 v = reinterpret_cast<const uint4*>(emb_in)[c];
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      ys[c * 8 + 2 * i] = (double)__uint_as_float(w[i] << 16);
+      ys[c * 8 + 2 * i + 1] = (double)__uint_as_float(w[i] & 0xffff0000u);
+    }
+  }
+  __syncthreads();
+  if (warp >= n_warps) return;
+  double nb = 0.0;                                    // the incoming carrier's norm, summed with the first row
+  bool first = true;
+  for (int buf = 0; j < j1; j += step, buf ^= 1) {
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncwarp();
+    const unsigned short* xs = reinterpret_cast<const unsigned short*>(rows + (size_t)buf * 2 * d);
+    double dot = 0.0, na = 0.0;
+    if (first) {
+#pragma unroll 8
+      for (int k = lane; k < d; k += 32) {
+        const double x = (double)__uint_as_float((uint32_t)xs[k] << 16), y = ys[k];
+        dot = __fma_rn(x, y, dot); na = __fma_rn(x, x, na); nb = __fma_rn(y, y, nb);
+      }
+      nb = warp_tree_sum(nb);
+      first = false;
+    } else {
+#pragma unroll 8
+      for (int k = lane; k < d; k += 32) {
+        const double x = (double)__uint_as_float((uint32_t)xs[k] << 16);
+        dot = __fma_rn(x, ys[k], dot); na = __fma_rn(x, x, na);
+      }
+    }
+    __syncwarp();
+    fetch(j + 2 * step, buf);
+    const double sc = cosine_of(warp_tree_sum(dot), warp_tree_sum(na), nb);
+    if (lane == 0 && VS_STORE_OK(bp, DR_SCORES, scores + j, 8)) scores[j] = sc;
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+// One of the `n_blocks` thread blocks (any number of them, whole warps) that update the bank of listed stream b.  smem:
+// `smem_bytes` of dynamic shared memory for the scoring, 16-byte aligned, or null.
 // Bank not full: block 0 appends; the other blocks return.
-// Bank full: the warps of all blocks deal the temporal indexes j among themselves and score cos(e_j, e_other) -- e_other is
-// the incoming carrier (policy 0) or the next carrier in temporal order (policy 1).  The fixed order of the fp64 sums makes
-// the score, and with it the argmax, reproducible bit for bit.  The last block of a stream to finish picks the victim
+// Bank full: the warps of all blocks deal the temporal indexes j0 .. j1 - 1 among themselves and score cos(e_j, e_other) --
+// e_other is the incoming carrier (policy 0) or the next carrier in temporal order (policy 1).  (A stack of layers shares
+// the scoring out over the layers' launches; the last one commits.)  The fixed order of the fp64 sums makes the score, and
+// with it the argmax, reproducible bit for bit.  The last block of a stream to finish picks the victim
 // (largest score, oldest on ties), closes the gap in the temporal order and appends.
-template <int kU, int NT>   // kU: loads in flight (see above); NT: threads that take part in the argmax, at most the block's
-__device__ __forceinline__ void bank_update_block(const BankUpdateArgs& a, const BatchParams& bp, int b, int block, int n_blocks) {
+template <int kU, int NT>   // kU: loads in flight where nothing is staged; NT: threads that take part in the argmax, at most the block's
+__device__ __forceinline__ void bank_update_block(const BankUpdateArgs& a, const BatchParams& bp, int b, int block, int n_blocks, uint8_t* smem,
+                                                  uint32_t smem_bytes) {
   const int tid = threadIdx.x;
   const bool on = tid < NT;
   const int sid = bp.stream_id[b];
   StreamMeta* meta = a.meta + sid;
+  if (!a.commit && (a.M == 0 || bp.count[b] < a.M)) return;           // nothing to score
   if (a.M == 0) {
     if (block == 0 && tid == 0) { meta->frames_seen += 1; meta->last_victim_frame = -1; }
     return;
@@ -102,26 +176,21 @@ __device__ __forceinline__ void bank_update_block(const BankUpdateArgs& a, const
   // ---- bank full: score, then the last block commits --------------------------------------
   double* scores = a.scores + (size_t)sid * a.slots;
   const int lane = tid & 31;
-  if (a.policy != 2) {
+  const int j1 = min(a.j1, count), staged = (smem != nullptr && a.policy == 0) ? staged_warps(a.d, smem_bytes) : 0;
+  if (staged > 0) {
+    staged_scores(a, bp, a.emb + (size_t)sid * a.slots * a.d, order, emb_in, scores, block, n_blocks, j1, smem, staged);
+  } else if (a.policy != 2) {
     const int n_warps = (int)blockDim.x >> 5;
-    double nb = 0.0;                                  // policy 0: the incoming carrier's norm, worked out with the first row
-    bool first = true;
-    for (int j = (tid >> 5) * n_blocks + block; j < count; j += n_blocks * n_warps) {
+    for (int j = a.j0 + (tid >> 5) * n_blocks + block; j < j1; j += n_blocks * n_warps) {
       const bf16* va = a.emb + ((size_t)sid * a.slots + order[j]) * a.d;
-      double dot, na;
-      if (a.policy == 1) {
-        const bf16* vb = (j + 1 < count) ? a.emb + ((size_t)sid * a.slots + order[j + 1]) * a.d : emb_in;
-        warp_dot_norms<true, kU>(va, vb, a.d, lane, dot, na, nb);
-      } else if (first) {
-        warp_dot_norms<true, kU>(va, emb_in, a.d, lane, dot, na, nb);
-        first = false;
-      } else {
-        warp_dot_norms<false, kU>(va, emb_in, a.d, lane, dot, na, nb);
-      }
+      const bf16* vb = (a.policy == 1 && j + 1 < count) ? a.emb + ((size_t)sid * a.slots + order[j + 1]) * a.d : emb_in;
+      double dot, na, nb;
+      warp_dot_norms<kU>(va, vb, a.d, lane, dot, na, nb);
       const double s = cosine_of(dot, na, nb);
       if (lane == 0 && VS_STORE_OK(bp, DR_SCORES, scores + j, 8)) scores[j] = s;
     }
   }
+  if (!a.commit) return;                             // (its scores are read by the last layer's launch)
   __shared__ int is_last;
   __threadfence();
   __syncthreads();

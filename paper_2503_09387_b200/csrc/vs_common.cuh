@@ -88,7 +88,7 @@ struct Dims {
   float rope_theta, rms_eps;
 };
 
-constexpr int KSPLIT_MAX = 4;   // CTAs sharing one output tile of the projection along K
+constexpr int KSPLIT_MAX = 5;   // CTAs sharing one output tile of a linear layer along K
 constexpr int DEC_SPLIT_MAX = 8;      // key splits of the decode attention = CTAs of one cluster
 constexpr int TOK_MAX_ROWS = 32;      // token rows of a step that the persistent kernel takes
 constexpr int TOK_MAX_CTAS = 160;     // ... one CTA per SM
@@ -279,11 +279,11 @@ struct ProjectionOut {
 struct GemmArgs {
   CUtensorMap tm_w2;             // mode 5: the up matrix (tm_w is then the gate matrix, both with boxes of 64 rows)
   CUtensorMap tm_w;              // [E_out, d] bf16, box 64 x 128, 128-byte swizzle
-  CUtensorMap tm_x;              // [rows, d] bf16, box 64 x tile_n, 128-byte swizzle
+  CUtensorMap tm_x;              // [rows, d] bf16, box 64 x tile_n (pairs: tile_n / 2), 128-byte swizzle
   ProjectionOut out;
   int rows, E_out, d;
-  int tile_n, n_tiles, ksplit;   // ksplit = CTAs per output tile along K: 1, 2 or 4
-  int m_sub;                     // 1: 128 weight rows per CTA; 2: 256 (two accumulators), only without a K split
+  int tile_n, n_tiles, ksplit;   // ksplit = CTAs per output tile along K (few rows)
+  bool pairs;                    // tiles of 256 rows on CTA pairs (vs_gemm_pair.cu) instead of 128 (vs_gemm_tcgen05.cu)
   float* xchg;                   // [m_tiles*n_tiles][ksplit][tile_n][128] fp32, needed when ksplit > 1
   int* flags;                    // [m_tiles*n_tiles][ksplit], zero between launches
   int n_sms;
@@ -291,6 +291,9 @@ struct GemmArgs {
 };
 cudaError_t launch_qkv_gemm(const GemmArgs& a, const BatchParams& bp, cudaStream_t st);
 cudaError_t qkv_gemm_init();     // opt-in shared memory attribute, once per process/device
+cudaError_t pair_gemm_init();
+int pair_gemm_max_pairs();       // CTA pairs that can be resident at once on the current device
+cudaError_t launch_pair_gemm(const GemmArgs& a, int max_pairs, const BatchParams& bp, cudaStream_t st);
 // Projection of one to four rows of a text step as a matrix-vector product (no RoPE table needed).
 bool qkv_gemv_supported(const ProjectionOut& o, int rows, int d);
 cudaError_t qkv_gemv_init();     // opt-in shared memory attribute, once per process/device
@@ -318,6 +321,7 @@ struct BankUpdateArgs {
   int pre_stride;
   int32_t* order; int32_t* slot_frame; int64_t* slot_pos; int32_t* evict_log; double* scores;
   int d, slots, M, policy, log_cap;
+  int j0, j1, commit;            // temporal indexes this launch scores; whether it also picks the victim and appends
 };
 // One segment of the attention's key axis.  Its K and V rows are reached through tensor maps with
 // dimensions {head_dim, rows, Z} and a box of {64, ATTN_KEY_BOX, 1} elements (128-byte swizzle):
@@ -356,7 +360,7 @@ struct AttnArgs {
   // CTAs that share the key tiles of one (row tile, KV head, batch entry): a thread-block cluster of 1 .. 4
   // whose members each take a contiguous run of key tiles and combine through distributed shared memory
   int nsplit;
-  // frame steps, last layer: the bank update (it needs the carrier embeddings only) is done by the CTAs of one more
+  // frame steps: the bank update (it needs the carrier embeddings only) is done by the CTAs of one more
   // plane of the grid (blockIdx.y == Hkv); 0: none.  bank_ctas: how many of the plane's CTAs per stream take part
   BankUpdateArgs bank;
   int bank_ctas;

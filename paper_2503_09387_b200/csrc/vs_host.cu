@@ -145,6 +145,7 @@ struct vs_stream {
   size_t ws_bytes = 0;
   int device = 0;
   int n_sms = 0;
+  int n_pairs = 0;                           // CTA pairs of the linear layers' kernel that can be resident at once
   // chunked prefill: the chunk's bank updates run on a stream of their own beside the projection
   cudaStream_t side_stream = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
@@ -255,33 +256,41 @@ void seg_step(AttnSegment& sg, const CUtensorMap& k, const CUtensorMap& v, int k
   sg.tk = k; sg.tv = v; sg.kind = kind; sg.rows_per_batch = rows_per_batch; sg.z0 = 0; sg.z_per_stream = 0;
 }
 
-// Token tiling of the projection.  Every CTA re-reads its weight rows and its token columns from
-// L2, (rows_w + tile_n) * (d / ksplit) * 2 bytes, and that traffic bounds the main loop.  The
-// choice minimises waves * ((rows_w + tile_n) / ksplit + the cost of summing a K split, about 40
-// row-equivalents) over 128- or 256-row weight tiles, the number of token tiles and the K split.
-// A K split needs the whole grid resident at once (its CTAs wait for one another), one CTA per SM.
-void choose_tiles(int K, int E, int n_sms, int rows, int& tile_n, int& n_tiles, int& ksplit, int& m_sub) {
-  const int total_kb = K / GEMM_BLOCK_K;
-  const int resident = n_sms < GEMM_XCHG_CTAS ? n_sms : GEMM_XCHG_CTAS;
+// Tiling of a linear layer: CTAs with 128 weight rows each and K cut into ksplit shares (few rows), or CTA pairs with 256
+// (many), and the token columns of a tile.  The choice minimises the clocks of the waves' main loops plus what their epilogues
+// add: a 64-element block of K costs a CTA the larger of its MMAs (tile_n columns, 2 clocks a column) and its operand
+// traffic from L2 at about 50 bytes a clock ((128 + tile_n) * 128 bytes, of a pair's CTA (128 + tile_n / 2) * 128).  The
+// epilogue of a tile costs about 4000 clocks, in a pair kernel only the last one counts; a K split 5000 more (partial tiles
+// through L2, a flag), and it needs its whole grid resident at once.
+struct Tiling { int tile_n, n_tiles, ksplit; bool pairs; };
+Tiling choose_tiles(int K, int E, int n_sms, int max_pairs, int rows, bool own_rope) {
+  const int kb = K / GEMM_BLOCK_K, resident = n_sms < GEMM_XCHG_CTAS ? n_sms : GEMM_XCHG_CTAS;
   const int nt_min = (rows + 255) / 256;
-  long long best = -1;
-  m_sub = 1; ksplit = 1; n_tiles = nt_min; tile_n = ((rows + nt_min - 1) / nt_min + 15) / 16 * 16;
-  for (int sub = 1; sub <= 2; ++sub) {
-    if (sub == 2 && E % (2 * GEMM_BLOCK_M) != 0) continue;
-    const int mt = (E + GEMM_BLOCK_M * sub - 1) / (GEMM_BLOCK_M * sub);
-    for (int nt = nt_min; nt <= nt_min + 32; ++nt) {
-      const int tn = ((rows + nt - 1) / nt + 15) / 16 * 16;
-      if ((long long)(nt - 1) * tn >= rows && nt > nt_min) continue;      // an empty last tile
-      if (tn < 64 && nt > nt_min) break;
-      for (int ks = 1; ks <= KSPLIT_MAX; ks *= 2) {
-        if (ks > 1 && (sub != 1 || total_kb % ks != 0 || mt * nt * ks > resident)) continue;
-        const long long waves = ((long long)mt * nt * ks + n_sms - 1) / n_sms;
-        const long long cost = waves * ((GEMM_BLOCK_M * sub + tn) * 4 / ks + (ks > 1 ? 160 : 0));   // in quarter rows
-        if (best < 0 || cost < best) { best = cost; m_sub = sub; n_tiles = nt; tile_n = tn; ksplit = ks; }
-      }
+  double best = -1.0;
+  Tiling t = {16, 1, 1, false};
+  for (int nt = nt_min; nt <= nt_min + 24; ++nt) {
+    const int tn = ((rows + nt - 1) / nt + 15) / 16 * 16;
+    if ((long long)(nt - 1) * tn >= rows && nt > nt_min) continue;      // an empty last tile
+    if (tn < 64 && nt > nt_min) break;
+    auto block = [&](int tn_own) { const double mma = 2.0 * tn, l2 = (128 + tn_own) * 2.56; return mma > l2 ? mma : l2; };
+    const int mt1 = (E + GEMM_BLOCK_M - 1) / GEMM_BLOCK_M, mt2 = (E + 2 * GEMM_BLOCK_M - 1) / (2 * GEMM_BLOCK_M);
+    for (int ks = 1; ks <= KSPLIT_MAX && ks <= kb; ++ks) {
+      const long long ctas = (long long)mt1 * nt * ks;
+      if (ks > 1 && ctas > resident) break;
+      const long long waves = (ctas + n_sms - 1) / n_sms;
+      const double cost = waves * (block(tn) * ((kb + ks - 1) / ks) + 4000.0) + (ks > 1 ? 5000.0 : 0.0);
+      if (best < 0 || cost < best) { best = cost; t = {tn, nt, ks, false}; }
     }
+    if (own_rope) continue;                                              // (the pair kernel reads a table)
+    const long long items = (long long)mt2 * nt, waves = (items + max_pairs - 1) / max_pairs;
+    const double cost = waves * (block(tn / 2) * kb + 500.0) + 4500.0;
+    if (best < 0 || cost < best) { best = cost; t = {tn, nt, 1, true}; }
   }
+  return t;
 }
+
+// launches the linear layer described by `g` (all but the tiling) on `src` [rows][K]
+int launch_linear(vs_stream* h, GemmArgs& g, const bf16* src, int rows, int K, int E, const BatchParams& bp, cudaStream_t st);
 
 int check_ids(vs_stream* h, const int32_t* ids, int32_t n) {
   if (h == nullptr || ids == nullptr || n < 1 || n > h->dm.S) return VS_ERR_INVALID_ARG;
@@ -334,16 +343,22 @@ int run_projection(vs_stream* h, int l, const bf16* src, int rows, const Project
     return VS_OK;
   }
   GemmArgs g;
-  choose_tiles(D.d, D.E_out, h->n_sms, rows, g.tile_n, g.n_tiles, g.ksplit, g.m_sub);
+  g.tm_w = h->tm_w[l]; g.tm_w2 = h->tm_w[l];
+  g.out = po;
+  return launch_linear(h, g, src, rows, D.d, D.E_out, bp, st);
+}
+
+int launch_linear(vs_stream* h, GemmArgs& g, const bf16* src, int rows, int K, int E, const BatchParams& bp, cudaStream_t st) {
+  const Tiling t = choose_tiles(K, E, h->n_sms, h->n_pairs, rows, g.out.mode < 4 && g.out.rope == nullptr);
+  g.tile_n = t.tile_n; g.n_tiles = t.n_tiles; g.ksplit = t.ksplit; g.pairs = t.pairs;
   g.xchg = h->at<float>(h->lo.gemm_xchg);
   g.flags = h->at<int>(h->lo.gemm_flags);
   g.n_sms = h->n_sms;
-  g.tm_w = h->tm_w[l]; g.tm_w2 = h->tm_w[l];
-  if (encode_2d(h, &g.tm_x, src, (uint64_t)D.d, (uint64_t)rows, (uint32_t)g.tile_n) != VS_OK) return VS_ERR_CUDA;
-  g.out = po;
-  g.rows = rows; g.E_out = D.E_out; g.d = D.d;
+  if (encode_2d(h, &g.tm_x, src, (uint64_t)K, (uint64_t)rows, (uint32_t)(t.pairs ? t.tile_n / 2 : t.tile_n)) != VS_OK) return VS_ERR_CUDA;
+  g.rows = rows; g.E_out = E; g.d = K;
   g.status = h->at<int>(h->lo.status);
-  VS_LAUNCH(h, st, KC_GEMM, launch_qkv_gemm(g, bp, st));
+  if (t.pairs) VS_LAUNCH(h, st, KC_GEMM, launch_pair_gemm(g, h->n_pairs, bp, st));
+  else VS_LAUNCH(h, st, KC_GEMM, launch_qkv_gemm(g, bp, st));
   return VS_OK;
 }
 
@@ -352,20 +367,10 @@ int run_projection(vs_stream* h, int l, const bf16* src, int rows, const Project
 int run_linear(vs_stream* h, const CUtensorMap& tm_w, const CUtensorMap& tm_w2, const bf16* src, int rows, int K, int E,
                ProjectionOut po, const BatchParams& bp, cudaStream_t st) {
   GemmArgs g;
-  choose_tiles(K, E, h->n_sms, rows, g.tile_n, g.n_tiles, g.ksplit, g.m_sub);
-  g.xchg = h->at<float>(h->lo.gemm_xchg);
-  g.flags = h->at<int>(h->lo.gemm_flags);
-  g.n_sms = h->n_sms;
   g.tm_w = tm_w; g.tm_w2 = tm_w2;
-  if (encode_2d(h, &g.tm_x, src, (uint64_t)K, (uint64_t)rows, (uint32_t)g.tile_n) != VS_OK) return VS_ERR_CUDA;
-  po.rope = h->at<float2>(h->lo.rope);      // (not read: nothing is rotated; selects the kernel variant that takes a table)
-  po.inv_freq = h->at<double>(h->lo.inv_freq);
   po.Hq = 0; po.Hkv = 0; po.D = 128; po.slots = 0; po.text_cap = 0; po.M = 0; po.norm_inline = 0;
   g.out = po;
-  g.rows = rows; g.E_out = E; g.d = K;
-  g.status = h->at<int>(h->lo.status);
-  VS_LAUNCH(h, st, KC_GEMM, launch_qkv_gemm(g, bp, st));
-  return VS_OK;
+  return launch_linear(h, g, src, rows, K, E, bp, st);
 }
 
 // The rest of decoder layer l (Section 4.1: Qwen2 backbone) after its attention: a_rows = the attention rows (bf16,
@@ -549,7 +554,9 @@ int vs_create_stream(const vs_config* cfg, const vs_weights* weights, void* work
     h->gain_f = static_cast<const bf16*>(weights->norm_f_w);
     if (encode_2d(h, &h->tm_lm, weights->w_lm, (uint64_t)D.d, (uint64_t)D.vocab, GEMM_BLOCK_M) != VS_OK) return fail(VS_ERR_CUDA);
   }
-  if (qkv_gemm_init() != cudaSuccess || qkv_gemv_init() != cudaSuccess || token_step_init() != cudaSuccess || prefill_attention_tc_init() != cudaSuccess) return fail(VS_ERR_CUDA);
+  if (pair_gemm_init() != cudaSuccess || qkv_gemm_init() != cudaSuccess || qkv_gemv_init() != cudaSuccess || token_step_init() != cudaSuccess || prefill_attention_tc_init() != cudaSuccess) return fail(VS_ERR_CUDA);
+  h->n_pairs = pair_gemm_max_pairs();
+  if (h->n_pairs < 1) return fail(VS_ERR_CUDA);
   for (int sp = 2; sp <= ATTN_MAX_SPLIT; ++sp) h->attn_clusters[sp] = prefill_attention_max_clusters(D.D, sp);
   // clear the whole workspace, then write the non-zero initial metadata
   if (cudaMemset(h->ws, 0, lo.total) != cudaSuccess) return fail(VS_ERR_CUDA);
@@ -657,6 +664,7 @@ int vs_frame_prefill(vs_stream* h, const int32_t* stream_ids, int32_t n_active, 
   ba.d = D.d; ba.slots = D.slots; ba.M = D.M; ba.policy = D.evict_policy; ba.log_cap = D.log_cap;
   ba.incoming_emb = nullptr; ba.record_slot = nullptr; ba.record_victim = nullptr; ba.chunk_first_frame = 0; ba.chunk_l1 = 0;
   ba.pre_scores = nullptr; ba.pre_stride = 0;
+  ba.j0 = 0; ba.j1 = D.M; ba.commit = 1;
 
   PoolArgs pa;
   pa.hidden = static_cast<const bf16*>(hidden);
@@ -729,13 +737,14 @@ int vs_frame_prefill(vs_stream* h, const int32_t* stream_ids, int32_t n_active, 
       }
       aa.nsplit = attn_split(h, bp, kl, 3);
     }
-    // the bank update (Section 3.3, memory mechanism: evict if full, then append) rides in the last layer's launch
-    // (a row per warp; four rows to a CTA, or as few as its plane, which is as wide as the attention's, allows: more rows on an
-    // SM wait for one another's fp64 conversions, 3 us longer with 19)
-    if (last) {
+    // the bank update (Section 3.3, memory mechanism: evict if full, then append) rides in the attention launches: each layer's
+    // scores a share of the bank (four rows to a CTA, or as few as its plane, which is as wide as the attention's, allows),
+    // the last one's commits
+    if (any_full || last) {
       aa.bank = ba;
-      const int plane = (N + 1 + 15) / 16 * aa.nsplit, wanted = (D.M + 3) / 4;
-      aa.bank_ctas = !any_full ? 1 : (wanted < plane ? wanted : plane);
+      aa.bank.j0 = (int)((int64_t)D.M * l / D.L); aa.bank.j1 = (int)((int64_t)D.M * (l + 1) / D.L); aa.bank.commit = last ? 1 : 0;
+      const int plane = (N + 1 + 15) / 16 * aa.nsplit, wanted = (aa.bank.j1 - aa.bank.j0 + 3) / 4;
+      aa.bank_ctas = !any_full || wanted < 1 ? 1 : (wanted < plane ? wanted : plane);
     }
     aa.Hq = D.Hq; aa.Hkv = D.Hkv; aa.D = D.D; aa.slots = D.slots; aa.M = D.M;
     aa.scale_log2e = (float)(1.4426950408889634 / std::sqrt((double)D.D));
@@ -849,6 +858,7 @@ int vs_frame_prefill_chunk(vs_stream* h, int32_t stream_id, const void* hidden, 
     ba.chunk_first_frame = bp.frame_id[0];
     ba.chunk_l1 = l1;
     ba.pre_scores = nullptr; ba.pre_stride = 0;
+  ba.j0 = 0; ba.j1 = D.M; ba.commit = 1;
     const bool any_full = D.M > 0 && bp.count[F - 1] == D.M;
     if (planned) {
       // the updates score against their incoming carrier only (or not at all): every cosine of the

@@ -289,7 +289,7 @@ cudaError_t launch_argmax_rows(const float* logits, int32_t* token, unsigned lon
 __global__ void __launch_bounds__(128, 8) bank_update_kernel(BankUpdateArgs a, BatchParams bp) {   // <= 64 registers: fits beside a projection CTA
   pdl_wait();
   pdl_launch_dependents();
-  bank_update_block<8, 128>(a, bp, (int)blockIdx.y, (int)blockIdx.x, (int)gridDim.x);
+  bank_update_block<8, 128>(a, bp, (int)blockIdx.y, (int)blockIdx.x, (int)gridDim.x, nullptr, 0);
 }
 
 cudaError_t launch_bank_update(const BankUpdateArgs& a, const BatchParams& bp, bool full, cudaStream_t st) {
@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(128, 8) chunk_scores_kernel(BankUpdateArgs a, 
   const int sid = bp.stream_id[b];
   const bf16* va = (c < a.chunk_l1) ? a.emb + ((size_t)sid * a.slots + c) * a.d : emb_stage + (size_t)(c - a.chunk_l1) * a.d;
   double dot, na, nb;
-  warp_dot_norms<true, 16>(va, emb_stage + (size_t)b * a.d, a.d, lane, dot, na, nb);
+  warp_dot_norms<16>(va, emb_stage + (size_t)b * a.d, a.d, lane, dot, na, nb);
   if (lane == 0) out[(size_t)b * a.pre_stride + c] = cosine_of(dot, na, nb);
 }
 
