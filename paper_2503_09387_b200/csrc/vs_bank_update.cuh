@@ -23,6 +23,7 @@ __device__ __forceinline__ void warp_dot_norms(const bf16* va, const bf16* vb, i
   dot = 0.0; na = 0.0; nb = 0.0;
   const unsigned short* pa = reinterpret_cast<const unsigned short*>(va) + lane;
   const unsigned short* pb = reinterpret_cast<const unsigned short*>(vb) + lane;
+#pragma unroll 1
   for (int k0 = 0; k0 < d; k0 += 32 * kU) {
     unsigned short xa[kU], xb[kU];
 #pragma unroll
@@ -44,7 +45,8 @@ __device__ __forceinline__ void warp_dot_norms(const bf16* va, const bf16* vb, i
   nb = warp_tree_sum(nb);
 }
 
-__device__ __forceinline__ double cosine_of(double dot, double na, double nb) {
+// (out of line: a square root, a division and their special cases, once per row)
+static __device__ __noinline__ double cosine_of(double dot, double na, double nb) {
   double s = 0.0;
   if (na != 0.0 && nb != 0.0) s = __ddiv_rn(dot, __dmul_rn(__dsqrt_rn(na), __dsqrt_rn(nb)));
   // a vector holding Inf or NaN has no cosine: counted as 0, like a zero vector
@@ -52,36 +54,55 @@ __device__ __forceinline__ double cosine_of(double dot, double na, double nb) {
   return s;
 }
 
+__host__ __device__ constexpr int bank_scratch_bytes(int nt) { return nt * 12 + 16; }
+
 __device__ __forceinline__ void bank_cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))), "l"(src) : "memory");
 }
 
-// Scores bank rows j = first, first + step, ... < j1 against the incoming carrier (policy 0), a row per warp: the whole row is
-// fetched into shared memory at once (two buffers a warp, the next row on its way while this one is summed), so a row costs one
-// memory latency, and the incoming carrier is widened to fp64 once per block -- conversions to fp64 run at a sixteenth of
-// the fp32 rate.  (With 16 two-byte loads in flight a lane, 64 rows took 6.5 us beside the attention of a one-layer frame step,
-// longer than the attention; this way 3 us.)  Same sums in the same order as warp_dot_norms.
+// Scores bank rows j0 .. j1 - 1 against the incoming carrier (policy 0), four rows to a warp: a lane's sum is a chain of d / 32
+// dependent fp64 operations, 9 clocks each at best, and every element costs a conversion of 9 to 14; four rows side by side fill
+// the one with the other.  The rows stream through shared memory, 512 elements of each at a time, two chunks ahead; the incoming carrier is
+// widened to fp64 once per block -- conversions to fp64 run at a sixteenth of the fp32 rate.  Same sums in the same order as
+// warp_dot_norms.  (One row a warp, staged whole: 16 banks of 1024 rows added 50 us to a batched frame step.)
+constexpr int kScoreRows = 4, kScoreChunk = 512, kScoreStages = 3, kScoreWarpBytes = kScoreRows * kScoreStages * kScoreChunk * 2;
 __device__ __forceinline__ int staged_warps(int d, uint32_t bytes) {
-  const long long left = (long long)bytes - (long long)d * 8;
-  const int n = left > 0 ? (int)(left / (4LL * d)) : 0;
-  return min(n, (int)blockDim.x >> 5);
+  const int left = (int)bytes - d * 8;
+  return left > 0 ? min(left / kScoreWarpBytes, (int)blockDim.x >> 5) : 0;
 }
 __device__ __forceinline__ void staged_scores(const BankUpdateArgs& a, const BatchParams& bp, const bf16* emb, const int32_t* order, const bf16* emb_in,
                                               double* scores, int block, int n_blocks, int j1, uint8_t* smem, int n_warps) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, d = a.d;
   double* ys = reinterpret_cast<double*>(smem);
-  uint8_t* rows = smem + (size_t)d * 8 + (size_t)warp * 4 * d;
-  const int step = n_blocks * n_warps;
-  int j = a.j0 + warp * n_blocks + block;
-  auto fetch = [&](int jj, int buf) {
-    if (jj < j1) {
-      const uint4* src = reinterpret_cast<const uint4*>(emb + (size_t)order[jj] * d);
-      uint4* dst = reinterpret_cast<uint4*>(rows + (size_t)buf * 2 * d);
-      for (int c = lane; c < d / 8; c += 32) bank_cp_async16(dst + c, src + c);
+  uint8_t* ring = smem + (size_t)d * 8 + (size_t)warp * kScoreWarpBytes;     // [stage][row][512]
+  const int step = n_blocks * n_warps, n_chunks = (d + kScoreChunk - 1) / kScoreChunk;
+  int j = a.j0 + warp * n_blocks + block;                                    // rows j, j + step, j + 2 step, j + 3 step side by side
+  const bf16* src[kScoreRows];
+  auto pick = [&]() {
+#pragma unroll
+    for (int r = 0; r < kScoreRows; ++r) src[r] = j + r * step < j1 ? emb + (size_t)order[j + r * step] * d : nullptr;
+  };
+  auto fetch = [&](int c) {
+    if (c < n_chunks) {
+#pragma unroll
+      for (int r = 0; r < kScoreRows; ++r) {
+        if (src[r] == nullptr) continue;
+        uint8_t* dst = ring + ((c % kScoreStages) * kScoreRows + r) * (kScoreChunk * 2);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const int k = c * kScoreChunk + (lane + 32 * i) * 8;
+          if (k < d) bank_cp_async16(dst + (lane + 32 * i) * 16, src[r] + k);
+        }
+      }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  if (warp < n_warps) { fetch(j, 0); fetch(j + step, 1); }
+  if (warp < n_warps) {
+    pick();
+#pragma unroll 1
+    for (int c = 0; c < kScoreStages - 1; ++c) fetch(c);
+  }
+#pragma unroll 1
   for (int c = tid; c < d / 8; c += (int)blockDim.x) {
     const uint4 v = reinterpret_cast<const uint4*>(emb_in)[c];
     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
@@ -93,38 +114,69 @@ __device__ __forceinline__ void staged_scores(const BankUpdateArgs& a, const Bat
   }
   __syncthreads();
   if (warp >= n_warps) return;
-  double nb = 0.0;                                    // the incoming carrier's norm, summed with the first row
-  bool first = true;
-  for (int buf = 0; j < j1; j += step, buf ^= 1) {
-    asm volatile("cp.async.wait_group 1;" ::: "memory");
-    __syncwarp();
-    const unsigned short* xs = reinterpret_cast<const unsigned short*>(rows + (size_t)buf * 2 * d);
-    double dot = 0.0, na = 0.0;
-    if (first) {
-#pragma unroll 8
-      for (int k = lane; k < d; k += 32) {
-        const double x = (double)__uint_as_float((uint32_t)xs[k] << 16), y = ys[k];
-        dot = __fma_rn(x, y, dot); na = __fma_rn(x, x, na); nb = __fma_rn(y, y, nb);
+#pragma unroll 1
+  while (j < j1) {
+    double dot[kScoreRows], na[kScoreRows], nb = 0.0;
+#pragma unroll
+    for (int r = 0; r < kScoreRows; ++r) { dot[r] = 0.0; na[r] = 0.0; }
+#pragma unroll 1
+    for (int c = 0; c < n_chunks; ++c) {
+      fetch(c + kScoreStages - 1);                     // into the stage that was read a chunk ago
+      asm volatile("cp.async.wait_group %0;" ::"n"(kScoreStages - 1) : "memory");
+      __syncwarp();
+      const unsigned short* xs = reinterpret_cast<const unsigned short*>(ring + (c % kScoreStages) * kScoreRows * (kScoreChunk * 2)) + lane;
+      const double* yc = ys + c * kScoreChunk + lane;
+      const int n = min(kScoreChunk, d - c * kScoreChunk);
+      // (64 elements a round: their twenty loads go out together -- one at a time the chain load, conversion, sum took 34 clocks a
+      // row and element where the conversion's rate allows 10)
+#pragma unroll 1
+      for (int k = 0; k < n; k += 128) {
+        double y[4];
+        unsigned short xr[kScoreRows][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const bool in = k + 32 * i < n;              // (n is a multiple of 64; zeros add nothing)
+          y[i] = in ? yc[k + 32 * i] : 0.0;
+#pragma unroll
+          for (int r = 0; r < kScoreRows; ++r) xr[r][i] = in ? xs[r * kScoreChunk + k + 32 * i] : (unsigned short)0;   // (a row that does not exist: whatever lies there)
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          nb = __fma_rn(y[i], y[i], nb);
+#pragma unroll
+          for (int r = 0; r < kScoreRows; ++r) {
+            const double x = (double)__uint_as_float((uint32_t)xr[r][i] << 16);
+            dot[r] = __fma_rn(x, y[i], dot[r]);
+            na[r] = __fma_rn(x, x, na[r]);
+          }
+        }
       }
-      nb = warp_tree_sum(nb);
-      first = false;
-    } else {
-#pragma unroll 8
-      for (int k = lane; k < d; k += 32) {
-        const double x = (double)__uint_as_float((uint32_t)xs[k] << 16);
-        dot = __fma_rn(x, ys[k], dot); na = __fma_rn(x, x, na);
-      }
+      __syncwarp();
     }
-    __syncwarp();
-    fetch(j + 2 * step, buf);
-    const double sc = cosine_of(warp_tree_sum(dot), warp_tree_sum(na), nb);
-    if (lane == 0 && VS_STORE_OK(bp, DR_SCORES, scores + j, 8)) scores[j] = sc;
+    nb = warp_tree_sum(nb);
+    const int j_done = j;
+    j += kScoreRows * step;
+    if (j < j1) {
+      pick();
+#pragma unroll 1
+      for (int c = 0; c < kScoreStages - 1; ++c) fetch(c);
+    }
+#pragma unroll 1
+    for (int r = 0; r < kScoreRows; ++r) {
+      // (row r's sums, picked without indexing registers)
+      const double dr = r == 0 ? dot[0] : (r == 1 ? dot[1] : (r == 2 ? dot[2] : dot[3]));
+      const double nr = r == 0 ? na[0] : (r == 1 ? na[1] : (r == 2 ? na[2] : na[3]));
+      const int jr = j_done + r * step;
+      if (jr >= j1) break;                             // uniform over the warp
+      const double sc = cosine_of(warp_tree_sum(dr), warp_tree_sum(nr), nb);
+      if (lane == 0 && VS_STORE_OK(bp, DR_SCORES, scores + jr, 8)) scores[jr] = sc;
+    }
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
-// One of the `n_blocks` thread blocks (any number of them, whole warps) that update the bank of listed stream b.  smem:
-// `smem_bytes` of dynamic shared memory for the scoring, 16-byte aligned, or null.
+// One of the `n_blocks` thread blocks (any number of them, whole warps) that update the bank of listed stream b.
+// scratch: 16-byte aligned shared memory, at least bank_scratch_bytes(NT); the more, the more rows are staged.
 // Bank not full: block 0 appends; the other blocks return.
 // Bank full: the warps of all blocks deal the temporal indexes j0 .. j1 - 1 among themselves and score cos(e_j, e_other) --
 // e_other is the incoming carrier (policy 0) or the next carrier in temporal order (policy 1).  (A stack of layers shares
@@ -132,8 +184,8 @@ __device__ __forceinline__ void staged_scores(const BankUpdateArgs& a, const Bat
 // with it the argmax, reproducible bit for bit.  The last block of a stream to finish picks the victim
 // (largest score, oldest on ties), closes the gap in the temporal order and appends.
 template <int kU, int NT>   // kU: loads in flight where nothing is staged; NT: threads that take part in the argmax, at most the block's
-__device__ __forceinline__ void bank_update_block(const BankUpdateArgs& a, const BatchParams& bp, int b, int block, int n_blocks, uint8_t* smem,
-                                                  uint32_t smem_bytes) {
+__device__ __forceinline__ void bank_update_block(const BankUpdateArgs& a, const BatchParams& bp, int b, int block, int n_blocks, void* scratch,
+                                                  uint32_t scratch_bytes) {
   const int tid = threadIdx.x;
   const bool on = tid < NT;
   const int sid = bp.stream_id[b];
@@ -155,6 +207,7 @@ __device__ __forceinline__ void bank_update_block(const BankUpdateArgs& a, const
   auto adopt = [&]() {      // all threads of the committing block
     if (a.incoming_emb != nullptr) {
       bf16* dst = const_cast<bf16*>(a.emb) + ((size_t)sid * a.slots + incoming) * a.d;
+#pragma unroll 1
       for (int k = tid; k < a.d; k += blockDim.x) if (VS_STORE_OK(bp, DR_EMB, dst + k, 2)) dst[k] = emb_in[k];
       if (tid == 0) { a.record_slot[b] = incoming; a.record_victim[b] = -1; }
     }
@@ -176,11 +229,12 @@ __device__ __forceinline__ void bank_update_block(const BankUpdateArgs& a, const
   // ---- bank full: score, then the last block commits --------------------------------------
   double* scores = a.scores + (size_t)sid * a.slots;
   const int lane = tid & 31;
-  const int j1 = min(a.j1, count), staged = (smem != nullptr && a.policy == 0) ? staged_warps(a.d, smem_bytes) : 0;
+  const int j1 = min(a.j1, count), staged = a.policy == 0 ? staged_warps(a.d, scratch_bytes) : 0;
   if (staged > 0) {
-    staged_scores(a, bp, a.emb + (size_t)sid * a.slots * a.d, order, emb_in, scores, block, n_blocks, j1, smem, staged);
+    staged_scores(a, bp, a.emb + (size_t)sid * a.slots * a.d, order, emb_in, scores, block, n_blocks, j1, static_cast<uint8_t*>(scratch), staged);
   } else if (a.policy != 2) {
     const int n_warps = (int)blockDim.x >> 5;
+#pragma unroll 1
     for (int j = a.j0 + (tid >> 5) * n_blocks + block; j < j1; j += n_blocks * n_warps) {
       const bf16* va = a.emb + ((size_t)sid * a.slots + order[j]) * a.d;
       const bf16* vb = (a.policy == 1 && j + 1 < count) ? a.emb + ((size_t)sid * a.slots + order[j + 1]) * a.d : emb_in;
@@ -191,17 +245,19 @@ __device__ __forceinline__ void bank_update_block(const BankUpdateArgs& a, const
     }
   }
   if (!a.commit) return;                             // (its scores are read by the last layer's launch)
-  __shared__ int is_last;
+  // (the staged rows and the carrier are done with when a block takes its ticket)
+  double* best_s = static_cast<double*>(scratch);                        // [NT]
+  int* best_j = reinterpret_cast<int*>(best_s + NT);                     // [NT]
+  int& is_last = best_j[NT];
   __threadfence();
   __syncthreads();
   if (tid == 0) is_last = (atomicAdd(&meta->score_ticket, 1) == n_blocks - 1);
   __syncthreads();
   if (!is_last) return;
   __threadfence();
-  __shared__ double best_s[NT];
-  __shared__ int best_j[NT];
   double bs = -4.0; int bj = 0x7fffffff;   // every score lies in [-2, 2], so some thread takes an index < count
   if (on && a.policy != 2) {
+#pragma unroll 1
     for (int i = tid; i < count; i += NT) {
       const double s = __ldcg(scores + i);
       if (s > bs) { bs = s; bj = i; }                 // ascending i: first maximum kept
@@ -209,6 +265,7 @@ __device__ __forceinline__ void bank_update_block(const BankUpdateArgs& a, const
   }
   if (on) { best_s[tid] = bs; best_j[tid] = bj; }
   __syncthreads();
+#pragma unroll 1
   for (int o = NT / 2; o > 0; o >>= 1) {
     if (tid < o) {
       const double s2 = best_s[tid + o]; const int j2 = best_j[tid + o];
@@ -226,6 +283,7 @@ __device__ __forceinline__ void bank_update_block(const BankUpdateArgs& a, const
   __syncthreads();
   // close the gap in the temporal order, one chunk of NT at a time in ascending order: a chunk
   // reads [base+1, base+NT] before anything at or above base is written
+#pragma unroll 1
   for (int base = v; base < count - 1; base += NT) {
     const int jj = base + tid;
     const int32_t next = (on && jj < count - 1) ? order[jj + 1] : 0;

@@ -183,6 +183,15 @@ __device__ __forceinline__ void vs_stamp(const BatchParams& bp, unsigned kernel,
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// One lane of a converged warp.  The warp that issues MMAs runs its loop as a whole, with this lane's predicate on the instructions
+// themselves: issued by one thread of a diverged warp they do not overlap one another (M 128 x N 128 x K 16: 106 clocks each
+// against 65, N 64: 95 against 49).
+__device__ __forceinline__ uint32_t elect_lane() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
+  return p;
+}
+
 // Asks the memory system to bring [p, p + bytes) into L2 (no destination, no completion to wait
 // for).  p 16-byte aligned, bytes a multiple of 16.  Used for weight rows: the matrices are
 // constant, so the request needs no ordering with any other kernel.
@@ -357,13 +366,13 @@ struct AttnArgs {
   int free_slot_stride;
   int Hq, Hkv, D, slots, M;
   float scale_log2e;
-  // CTAs that share the key tiles of one (row tile, KV head, batch entry): a thread-block cluster of 1 .. 4
+  // CTAs that share the key tiles of one (row tile, KV head, batch entry): a thread-block cluster of 1 .. 8
   // whose members each take a contiguous run of key tiles and combine through distributed shared memory
   int nsplit;
-  // frame steps: the bank update (it needs the carrier embeddings only) is done by the CTAs of one more
-  // plane of the grid (blockIdx.y == Hkv); 0: none.  bank_ctas: how many of the plane's CTAs per stream take part
+  // frame steps: the bank update (it needs the carrier embeddings only) is done by bank_grid CTAs of the grid (a multiple
+  // of nsplit; 0: none) from bank_pos (another) on, bank_ctas of them for each listed stream
   BankUpdateArgs bank;
-  int bank_ctas;
+  int bank_grid, bank_pos, bank_ctas;
   // chunk of frames in ONE launch (entry b = frame b): the bank segment is the bank as it was
   // before the chunk (chunk_count0 carriers) for every frame; what frame b must not see -- the slot
   // that was free, and whoever the updates of frames 0 .. b-1 evicted (chunk_victim) -- is masked
@@ -388,11 +397,12 @@ struct ChunkKvCommitArgs {
   int d;
 };
 cudaError_t launch_chunk_kv_commit(const ChunkKvCommitArgs& a, cudaStream_t st);
-constexpr int ATTN_EXCL_BITS = 8192;   // most (bank slots + chunk frames) the one-launch chunk attention can mask
+constexpr int ATTN_EXCL_BITS = 8192;   // most (bank slots + chunk frames) a chunk call takes
 cudaError_t launch_prefill_attention_tc(const AttnArgs& a, const BatchParams& bp, int* status, cudaStream_t st);
 cudaError_t prefill_attention_tc_init();
 int prefill_attention_max_clusters(int head_dim, int s);
-constexpr int ATTN_MAX_SPLIT = 2;   // clusters of 3 or 4 do not all fit on the GPU at once (one CTA per SM, clusters inside a GPC)
+bool prefill_attention_can_split(int head_dim, int group, int nsplit);
+constexpr int ATTN_MAX_SPLIT = 8;   // most CTAs sharing the key tiles of one row tile (one cluster)
 
 struct DecodeArgs {
   const bf16* q;                 // [n_active][Hq*D]

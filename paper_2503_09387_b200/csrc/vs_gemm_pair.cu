@@ -53,17 +53,18 @@ __device__ __forceinline__ void cluster_sync_all() {
 __device__ __forceinline__ uint32_t make_idesc_pair(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)((2 * GEMM_BLOCK_M) >> 4) << 24);
 }
-__device__ __forceinline__ void umma_bf16_pair(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t accumulate) {
+__device__ __forceinline__ void umma_bf16_pair(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t accumulate, uint32_t elected) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(tmem_d), "l"(da), "l"(db), "r"(idesc), "r"(accumulate) : "memory");
+      "{\n\t.reg .pred p, e;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\tsetp.ne.u32 e, %5, 0;\n\t"
+      "@e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(tmem_d), "l"(da), "l"(db), "r"(idesc), "r"(accumulate), "r"(elected) : "memory");
 }
 // arrives on the barrier at this offset in both CTAs once the MMAs issued so far have completed
-__device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-               ::"r"(bar), "h"((uint16_t)3) : "memory");
+__device__ __forceinline__ void umma_commit_pair(uint32_t bar, uint32_t elected) {
+  asm volatile("{\n\t.reg .pred e;\n\tsetp.ne.u32 e, %2, 0;\n\t"
+               "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}"
+               ::"r"(bar), "h"((uint16_t)3), "r"(elected) : "memory");
 }
 
 struct PairParams {
@@ -253,27 +254,27 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant
     }
   } else if (warp == 1) {
     pdl_wait();
-    if (lane == 0 && rank == 0) {
-      // ---- MMA issuer: one thread for both CTAs -------------------------------------------------------
-      const uint32_t idesc = make_idesc_pair(p.tile_n);
+    if (rank == 0) {
+      // ---- MMA issuer: one lane for both CTAs ---------------------------------------------------------
+      const uint32_t idesc = make_idesc_pair(p.tile_n), elected = elect_lane();
       int s = 0, j = 0;
       uint32_t par = 0;
       bool ok = true;
       for (int i = pair; i < n_items && ok; i += n_pairs, ++j) {
         const uint32_t acc = tmem + (uint32_t)((j & 1) * p.acc_cols);
-        ok = mbar_wait(acc_empty(j & 1), ((uint32_t)(j >> 1) & 1u) ^ 1u, abort_flag);
+        ok = __all_sync(0xffffffffu, mbar_wait(acc_empty(j & 1), ((uint32_t)(j >> 1) & 1u) ^ 1u, abort_flag));
         for (int kb = 0; kb < p.kblocks && ok; ++kb) {
-          ok = mbar_wait(full_bar(s), par, abort_flag);
+          ok = __all_sync(0xffffffffu, mbar_wait(full_bar(s), par, abort_flag));
           if (!ok) break;
           tcgen05_fence_after();
-          const uint32_t a_addr = base + (uint32_t)s * stage_bytes, b_addr = a_addr + kStageABytes;
+          const uint64_t da = make_smem_desc(base + (uint32_t)s * stage_bytes), db = make_smem_desc(base + (uint32_t)s * stage_bytes + kStageABytes);
 #pragma unroll
           for (int k = 0; k < GEMM_BLOCK_K / 16; ++k)      // 16 bf16 = 32 bytes further along K inside the 128-byte swizzle row
-            umma_bf16_pair(acc, make_smem_desc(a_addr + 32u * k), make_smem_desc(b_addr + 32u * k), idesc, (uint32_t)((kb | k) != 0));
-          umma_commit_pair(empty_bar(s));                  // frees the stage in both CTAs once these MMAs have read it
+            umma_bf16_pair(acc, da + 2u * k, db + 2u * k, idesc, (uint32_t)((kb | k) != 0), elected);
+          umma_commit_pair(empty_bar(s), elected);         // frees the stage in both CTAs once these MMAs have read it
           if (++s == p.stages) { s = 0; par ^= 1u; }
         }
-        if (ok) umma_commit_pair(acc_full(j & 1));
+        if (ok) umma_commit_pair(acc_full(j & 1), elected);
       }
     }
   } else {

@@ -1,6 +1,6 @@
 // QKV projection (Eq. 1: Q = X W_Q, K = X W_K, V = X W_V) on the 5th-generation tensor
 // cores: tcgen05.mma with the accumulator in tensor memory, operands staged in shared
-// memory by TMA, one elected thread issuing the MMAs.
+// memory by TMA, one elected lane issuing the MMAs.
 //
 // Orientation.  A frame brings only N + 1 (<= 256) token rows but E_out = (Hq + 2 Hkv) D
 // output features (4608 at the Qwen2-7B shape), so the *features* take the MMA's M axis
@@ -41,15 +41,15 @@ constexpr int kMaxThreads = 64 + 32 * kMaxEpiWarps;
 __device__ __forceinline__ uint32_t make_idesc(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(GEMM_BLOCK_M >> 4) << 24);
 }
-__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t accumulate) {
+__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t accumulate, uint32_t elected) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(tmem_d), "l"(da), "l"(db), "r"(idesc), "r"(accumulate) : "memory");
+      "{\n\t.reg .pred p, e;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\tsetp.ne.u32 e, %5, 0;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(tmem_d), "l"(da), "l"(db), "r"(idesc), "r"(accumulate), "r"(elected) : "memory");
 }
-__device__ __forceinline__ void umma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+__device__ __forceinline__ void umma_commit(uint32_t bar, uint32_t elected) {
+  asm volatile("{\n\t.reg .pred e;\n\tsetp.ne.u32 e, %1, 0;\n\t@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar), "r"(elected) : "memory");
 }
 struct KernelParams {
   ProjectionOut o;
@@ -160,26 +160,20 @@ qkv_gemm_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant_
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t idesc = make_idesc(p.tile_n);
-      bool ok = true;
-      for (int kb = 0; kb < kblocks; ++kb) {
-        const int s = kb % p.stages;
-        const uint32_t ph = (uint32_t)(kb / p.stages) & 1u;
-        ok = mbar_wait(full_bar(s), ph, abort_flag);
-        if (!ok) break;
-        tcgen05_fence_after();
-        const uint32_t a_addr = base + (uint32_t)s * stage_bytes;
-        const uint32_t b_addr = a_addr + kStageABytes;
+    const uint32_t idesc = make_idesc(p.tile_n), elected = elect_lane();
+    bool ok = true;
+    for (int kb = 0; kb < kblocks; ++kb) {
+      const int s = kb % p.stages;
+      ok = __all_sync(0xffffffffu, mbar_wait(full_bar(s), (uint32_t)(kb / p.stages) & 1u, abort_flag));
+      if (!ok) break;
+      tcgen05_fence_after();
+      const uint64_t da = make_smem_desc(base + (uint32_t)s * stage_bytes), db = make_smem_desc(base + (uint32_t)s * stage_bytes + kStageABytes);
 #pragma unroll
-        for (int k = 0; k < GEMM_BLOCK_K / 16; ++k) {
-          // 16 bf16 = 32 bytes further along K inside the 128-byte swizzle row
-          umma_bf16(tmem_acc, make_smem_desc(a_addr + 32u * k), make_smem_desc(b_addr + 32u * k), idesc, (uint32_t)((kb | k) != 0));
-        }
-        umma_commit(empty_bar(s));          // frees the stage once these MMAs have read it
-      }
-      if (ok) umma_commit(tmem_full_bar);   // accumulator complete
+      for (int k = 0; k < GEMM_BLOCK_K / 16; ++k)      // 16 bf16 = 32 bytes further along K inside the 128-byte swizzle row
+        umma_bf16(tmem_acc, da + 2u * k, db + 2u * k, idesc, (uint32_t)((kb | k) != 0), elected);
+      umma_commit(empty_bar(s), elected);              // frees the stage once these MMAs have read it
     }
+    if (ok) umma_commit(tmem_full_bar, elected);       // accumulator complete
   }
 
   // ---- epilogue ---------------------------------------------------------------------------

@@ -230,19 +230,21 @@ int ensure_step_maps(vs_stream* h, int rows) {
   return VS_OK;
 }
 
-// CTAs to spread the key tiles of a row tile over (one cluster): every CTA of the attention kernel takes
-// a whole SM, all clusters must be resident at once, and a split pays only while it shortens the longest
-// CTA's run of key tiles.  key_len[i]: segment lengths of the longest key axis among the listed entries.
+// CTAs to spread the key tiles of a row tile over (one cluster).  All clusters must be resident at once, with a little room for
+// the bank update's.  In key tiles (0.75 us each), measured on frames, clips and questions of 5 to 13 tiles: two CTAs an SM make
+// a tile a tenth longer, exchanging rows costs 2.2 and 0.3 for every CTA of the cluster.  key_len[i]: segment lengths of the
+// longest key axis among the listed entries.
 int attn_split(const vs_stream* h, const BatchParams& bp, const int* key_len, int n_len) {
-  int padded = 0;
-  for (int i = 0; i < n_len; ++i) padded += (key_len[i] + ATTN_KEY_BOX - 1) / ATTN_KEY_BOX * ATTN_KEY_BOX;
-  const int key_tiles = (padded + 127) / 128;
+  int key_tiles = 0;
+  for (int i = 0; i < n_len; ++i) key_tiles += (key_len[i] + ATTN_KEY_BOX - 1) / ATTN_KEY_BOX;
   const long long row_ctas = (long long)((bp.rows_per_stream + 15) / 16) * h->dm.Hkv * bp.n_active;
   int best = 1;
-  for (int s = 2; s <= ATTN_MAX_SPLIT; ++s) {
-    if (s > key_tiles || row_ctas * s > h->n_sms || h->attn_clusters[s] < row_ctas) break;
-    if ((key_tiles + s - 1) / s == (key_tiles + best - 1) / best) continue;
-    best = s;
+  double cost = 1e30;
+  for (int s = 1; s <= ATTN_MAX_SPLIT; ++s) {
+    if (s > 1 && (s > key_tiles || row_ctas * s > 2LL * h->n_sms || h->attn_clusters[s] < row_ctas + 4 ||
+                  !prefill_attention_can_split(h->dm.D, h->dm.G, s))) continue;
+    const double c = ((key_tiles + s - 1) / s) * (row_ctas * s > h->n_sms ? 1.1 : 1.0) + (s > 1 ? 2.2 + 0.3 * s : 0.0);
+    if (c < cost) { cost = c; best = s; }
   }
   return best;
 }
@@ -557,7 +559,7 @@ int vs_create_stream(const vs_config* cfg, const vs_weights* weights, void* work
   if (pair_gemm_init() != cudaSuccess || qkv_gemm_init() != cudaSuccess || qkv_gemv_init() != cudaSuccess || token_step_init() != cudaSuccess || prefill_attention_tc_init() != cudaSuccess) return fail(VS_ERR_CUDA);
   h->n_pairs = pair_gemm_max_pairs();
   if (h->n_pairs < 1) return fail(VS_ERR_CUDA);
-  for (int sp = 2; sp <= ATTN_MAX_SPLIT; ++sp) h->attn_clusters[sp] = prefill_attention_max_clusters(D.D, sp);
+  for (int sp = 2; sp <= ATTN_MAX_SPLIT; ++sp) h->attn_clusters[sp] = 2 * prefill_attention_max_clusters(D.D, sp);
   // clear the whole workspace, then write the non-zero initial metadata
   if (cudaMemset(h->ws, 0, lo.total) != cudaSuccess) return fail(VS_ERR_CUDA);
   {
@@ -738,13 +740,22 @@ int vs_frame_prefill(vs_stream* h, const int32_t* stream_ids, int32_t n_active, 
       aa.nsplit = attn_split(h, bp, kl, 3);
     }
     // the bank update (Section 3.3, memory mechanism: evict if full, then append) rides in the attention launches: each layer's
-    // scores a share of the bank (four rows to a CTA, or as few as its plane, which is as wide as the attention's, allows),
-    // the last one's commits
+    // scores a share of the bank, the last one's commits.  Five rows to a CTA (a row per warp) while the CTAs are few; at most one
+    // CTA for every two SMs, or for every SM where the attention comes in waves anyway: scoring is fp64 arithmetic and runs
+    // beside the tensor work of the SM's other CTA, but must not take the slots that the attention's clusters need
     if (any_full || last) {
       aa.bank = ba;
       aa.bank.j0 = (int)((int64_t)D.M * l / D.L); aa.bank.j1 = (int)((int64_t)D.M * (l + 1) / D.L); aa.bank.commit = last ? 1 : 0;
-      const int plane = (N + 1 + 15) / 16 * aa.nsplit, wanted = (aa.bank.j1 - aa.bank.j0 + 3) / 4;
-      aa.bank_ctas = !any_full || wanted < 1 ? 1 : (wanted < plane ? wanted : plane);
+      const int n_rows = aa.bank.j1 - aa.bank.j0, attn_ctas = (N + 16) / 16 * aa.nsplit * D.Hkv * n_active;
+      const int most = (attn_ctas > 2 * h->n_sms ? h->n_sms : h->n_sms / 2) / n_active;
+      int ctas = (n_rows + 4) / 5;
+      if (ctas > most) ctas = most;
+      aa.bank_ctas = !any_full || ctas < 1 ? 1 : ctas;
+      aa.bank_grid = (aa.bank_ctas * n_active + aa.nsplit - 1) / aa.nsplit * aa.nsplit;
+      // few of them start first (their chain is as long as the attention's); many would take slots that the attention's clusters
+      // need (a bank of 1024 carriers: 48 against 42 us a frame step) and come behind as many attention CTAs as run at once
+      const int ahead = aa.bank_grid <= h->n_sms / 4 ? 0 : 2 * h->n_sms - aa.bank_grid;
+      aa.bank_pos = (ahead < attn_ctas ? (ahead > 0 ? ahead : 0) : attn_ctas) / aa.nsplit * aa.nsplit;
     }
     aa.Hq = D.Hq; aa.Hkv = D.Hkv; aa.D = D.D; aa.slots = D.slots; aa.M = D.M;
     aa.scale_log2e = (float)(1.4426950408889634 / std::sqrt((double)D.D));

@@ -289,7 +289,8 @@ cudaError_t launch_argmax_rows(const float* logits, int32_t* token, unsigned lon
 __global__ void __launch_bounds__(128, 8) bank_update_kernel(BankUpdateArgs a, BatchParams bp) {   // <= 64 registers: fits beside a projection CTA
   pdl_wait();
   pdl_launch_dependents();
-  bank_update_block<8, 128>(a, bp, (int)blockIdx.y, (int)blockIdx.x, (int)gridDim.x, nullptr, 0);
+  __shared__ __align__(16) uint8_t scratch[bank_scratch_bytes(128)];
+  bank_update_block<8, 128>(a, bp, (int)blockIdx.y, (int)blockIdx.x, (int)gridDim.x, scratch, (uint32_t)sizeof(scratch));
 }
 
 cudaError_t launch_bank_update(const BankUpdateArgs& a, const BatchParams& bp, bool full, cudaStream_t st) {
