@@ -22,9 +22,9 @@
 // 64 keys x 64 dims through per-segment tensor maps, 128-byte swizzle as the MMA descriptors expect); tiles that hold only keys of
 // earlier steps (prefix, bank, tail) are requested before the wait on the stream's earlier kernels.
 // Few CTAs (a frame of one stream): the key tiles are shared by the CTAs of a thread-block cluster, each taking a contiguous run
-// of tiles.  Each CTA finishes the rows of some tokens: a softmax thread stores its unnormalised row with (max, denominator)
-// straight into the owner's shared memory (where the query was: dead once the owner's last S is there, which the first phase of
-// the cluster's barrier tells), and after the barrier's second phase the owner combines what it was given.
+// of tiles.  Each CTA finishes the rows of some tokens: the others send it theirs, unnormalised, with (max, denominator), by bulk
+// copies from shared memory to shared memory, counted on a barrier of the owner's (to where the query was: dead once the owner's
+// last S is there, which the first phase of the cluster's barrier tells).
 // All mbarrier waits are bounded.
 #include "vs_common.cuh"
 #include "vs_bank_update.cuh"
@@ -182,11 +182,14 @@ __device__ __forceinline__ uint32_t map_shared_rank(uint32_t addr, uint32_t rank
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
-__device__ __forceinline__ void st_cluster_f4(uint32_t addr, float4 v) {
-  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+// to a peer's shared memory, counted in bytes on a barrier of the peer's
+__device__ __forceinline__ void st_async_f2(uint32_t addr, float2 v, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];"
+               ::"r"(addr), "f"(v.x), "f"(v.y), "r"(bar) : "memory");
 }
-__device__ __forceinline__ void st_cluster_f2(uint32_t addr, float2 v) {
-  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(v.x), "f"(v.y) : "memory");
+__device__ __forceinline__ void bulk_to_peer(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(dst), "r"(src), "r"(bytes), "r"(bar) : "memory");
 }
 __device__ __forceinline__ void st_shared_f4(uint32_t addr, float4 v) {
   asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
@@ -224,8 +227,9 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
   const uint32_t bar_q = ctl + 40u;                                       // query copied row by row (128 arrivals)
   auto bar_full = [&](int s) { return ctl + 48u + 8u * (uint32_t)s; };    // ring stage landed (its bytes)
   auto bar_free = [&](int s) { return ctl + 96u + 8u * (uint32_t)s; };    // ring stage read (tcgen05.commit)
-  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(gbase + L::kCtl + 144);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(gbase + L::kCtl + 148);
+  const uint32_t bar_recv = ctl + 144u;                                   // the peers' parts of this CTA's rows have arrived (their bytes)
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(gbase + L::kCtl + 152);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(gbase + L::kCtl + 156);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // ---- bank update CTAs (frame steps), behind as many attention CTAs as run at once.  What they read -- carrier embeddings,
@@ -246,6 +250,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
     mbar_init(bar_o, 1);
     mbar_init(bar_qb, 1);
     mbar_init(bar_q, kSoftmaxThreads);
+    mbar_init(bar_recv, 1);
     for (int s = 0; s < NS; ++s) { mbar_init(bar_full(s), 1); mbar_init(bar_free(s), 1); }
     *abort_flag = (base & 1023u) != 0;      // (the swizzled layouts need the alignment that the declaration asks for)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -547,41 +552,43 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
     if (!ok) *abort_flag = 1;
   }
 
-  // ---- rows out: a warp per row, four rows in flight ----------------------------------------------------------
-  constexpr int F4 = D / 4, kWarps = kAttnThreads / 32;
-  constexpr uint32_t kMlOff = (uint32_t)L::kRowsOut * D * 4;          // (max, denominator) pairs behind the rows
+  // ---- rows out -----------------------------------------------------------------------------------------------
+  constexpr int F4 = D / 4, kWarps = kAttnThreads / 32, kRowBytes = D * 4;
+  constexpr uint32_t kMlOff = (uint32_t)L::kRowsOut * kRowBytes;      // (max, denominator) pairs behind the rows
   const int tok_per = (kTok + nsplit - 1) / nsplit;                   // CTA s of the cluster finishes tokens s * tok_per ...
-  const int my_rows = 8 * max(min(tok_per, kTok - split * tok_per), 0);   // row j: head j & 7 of token j >> 3 of those (none, perhaps)
+  auto tokens_of = [&](int s) { return max(min(tok_per, kTok - s * tok_per), 0); };   // ... this many of them (none, perhaps)
+  const int my_tok = tokens_of(split), my_rows = 8 * my_tok;          // row j: head j & 7 of token j >> 3
   uint8_t* res_s = gbase + L::kRing;                                  // [row j][D] bf16: residual input of the rows (the ring is dead by now)
-  float* ss_stage = reinterpret_cast<float*>(gbase + L::kRing + 128 * D * 2);   // [8 heads][16 tokens] sums of squares of stored residual rows
+  float* ss_stage = reinterpret_cast<float*>(gbase + L::kRing + (nsplit == 1 ? 128 * D * 2 : 0));   // [8 heads][16 tokens] sums of squares of stored residual rows
   VS_STAMP(bp, 2, 2);               // this CTA's tiles done
   __syncwarp();
-  if (warp < 4 && a.h_out != nullptr) {
+  if (warp < 4 && a.h_out != nullptr && nsplit == 1) {
+    // the residual input of the rows, into the ring (unless peers' rows are staged there)
     for (int i = tid; i < my_rows * CPR; i += kSoftmaxThreads) {
       const int j = i / CPR, c = i - j * CPR, gg = j & 7, tt = r0 + split * tok_per + (j >> 3);
-      if (gg < G && tt < rps)
-        cp_async16(base + L::kRing + (uint32_t)i * 16u, a.h_in + (((size_t)b * rps + tt) * a.Hq + (size_t)hkv * G + gg) * D + c * 8, true);
+      if (gg < G && tt < rps) {
+        const bf16* src = a.h_in + (((size_t)b * rps + tt) * a.Hq + (size_t)hkv * G + gg) * D + c * 8;
+        cp_async16(base + L::kRing + (uint32_t)i * 16u, src, true);
+      }
     }
     cp_async_commit();
   }
   if (nsplit > 1) {
     if (warp < 4 && n_tiles == 0) cluster_arrive();
-    cluster_wait();                 // every peer's query is dead
+    if (tid == 0) mbar_arrive_expect_tx(bar_recv, (uint32_t)((nsplit - 1) * G * my_tok * (kRowBytes + 8)));
+    cluster_wait();                 // every peer's query is dead, and its barriers exist
   }
   if (warp < 4) {
-    const int gg = tid >> 4, tk = tid & 15;
+    // Every thread's row: into this CTA's own area if it finishes the row (with 1 / denominator if there are no peers), else staged
+    // in the ring, from where it goes to the owner by bulk copies -- the rows of an owner's tokens lie side by side for every
+    // head.  (Stored straight into the peer's shared memory, 16 bytes a lane scattered over 32 rows, they took 4 us.)
+    const int gg = tid >> 4, tk = tid & 15, owner = nsplit == 1 ? 0 : tk / tok_per;
     const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
-    uint32_t dst = base + L::kQ;
-    int idx = tid;
-    float inv = 1.f;
-    if (nsplit == 1) {
-      inv = (l_run > 0.f) ? 1.f / l_run : 0.f;
-    } else {
-      const int owner = tk / tok_per;
-      idx = (split * G + gg) * tok_per + (tk - owner * tok_per);
-      dst = map_shared_rank(dst, (uint32_t)owner);
-      if (gg < G) st_cluster_f2(dst + kMlOff + (uint32_t)idx * 8u, make_float2(m_run, l_run));
-    }
+    const int theirs = kTok - my_tok;                                 // tokens of others, in order, numbered round this CTA's own
+    const int idx = nsplit == 1 ? tid : (owner == split ? (split * G + gg) * tok_per + (tk - owner * tok_per)
+                                                        : gg * theirs + (tk < split * tok_per ? tk : tk - my_tok));
+    const uint32_t dst = base + (owner == split ? L::kQ : L::kRing) + (uint32_t)idx * kRowBytes;
+    const float inv = nsplit > 1 ? 1.f : ((l_run > 0.f) ? 1.f / l_run : 0.f);
 #pragma unroll 1
     for (int c = 0; c < D; c += 32) {
       float ov[32];
@@ -593,78 +600,135 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
         for (int j = 0; j < 32; ++j) ov[j] = 0.f;
       }
       if (gg < G) {
+        // (16-byte units XOR-swizzled by 16 * (head & 1) + token)
 #pragma unroll
-        for (int j = 0; j < 32; j += 4) {
-          const uint32_t at = dst + (uint32_t)idx * (D * 4) + (uint32_t)((((c + j) >> 2) ^ (idx & (F4 - 1))) * 16);
-          const float4 v = make_float4(ov[j] * inv, ov[j + 1] * inv, ov[j + 2] * inv, ov[j + 3] * inv);
-          if (nsplit == 1) st_shared_f4(at, v); else st_cluster_f4(at, v);
-        }
+        for (int j = 0; j < 32; j += 4)
+          st_shared_f4(dst + (uint32_t)((((c + j) >> 2) ^ (tid & (F4 - 1))) * 16), make_float4(ov[j] * inv, ov[j + 1] * inv, ov[j + 2] * inv, ov[j + 3] * inv));
       }
       __syncwarp();
     }
     tc_fence_before();
+    if (nsplit > 1) {
+      if (gg < G) {
+        const uint32_t at = base + L::kQ + kMlOff + (uint32_t)((split * G + gg) * tok_per + (tk - owner * tok_per)) * 8u;
+        if (owner == split) *reinterpret_cast<float2*>(gbase + (at - base)) = make_float2(m_run, l_run);
+        else st_async_f2(map_shared_rank(at, (uint32_t)owner), make_float2(m_run, l_run), map_shared_rank(bar_recv, (uint32_t)owner));
+      }
+      // a warp's rows are those of two heads: it sends them on itself
+      fence_async_proxy();
+      __syncwarp();
+      const int o = lane >> 1, g = 2 * warp + (lane & 1);
+      if (o < nsplit && o != split && g < G) {
+        const int n = tokens_of(o), first = o * tok_per, src = g * theirs + (first < split * tok_per ? first : first - my_tok);
+        bulk_to_peer(map_shared_rank(base + L::kQ + (uint32_t)((split * G + g) * tok_per) * kRowBytes, (uint32_t)o),
+                     base + L::kRing + (uint32_t)src * kRowBytes, (uint32_t)(n * kRowBytes), map_shared_rank(bar_recv, (uint32_t)o));
+      }
+    }
+    cp_async_wait<0>();
   }
-  __syncwarp();
-  if (nsplit > 1) { cluster_arrive(); }
-  if (warp < 4) cp_async_wait<0>();
   {
-    if (nsplit > 1) cluster_wait();  // every part is in place, and nobody reads or writes a peer's memory from here on
+    if (nsplit > 1 && !mbar_wait(bar_recv, 0, abort_flag)) *abort_flag = 1;
     __syncthreads();
     VS_STAMP(bp, 2, 3);
-    // (a row at a time: this code runs once per CTA, and its size -- four rows unrolled: 25 KB -- cost more than the latency that
-    // unrolling hides)
-#pragma unroll 1
-    for (int j = warp; j < my_rows; j += kWarps) {
-      const int tl = j >> 3, gg = j & 7, tk = split * tok_per + tl, tt = r0 + tk, u = lane & (F4 - 1);
-      if (gg >= G || tt >= rps) continue;                              // uniform over the warp
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (nsplit == 1) {
-        const int idx = gg * 16 + tl;
-        v = *reinterpret_cast<const float4*>(gbase + L::kQ + (size_t)idx * (D * 4) + ((u ^ (idx & (F4 - 1))) * 16));
-      } else {
-        // (the running maximum and denominator as over key tiles)
+    if (nsplit > 1) {
+      // what each CTA's part of a row counts for, 2^(max_i - max) over the row's denominator: a thread per row, in place of the pairs
+      float2* mlp = reinterpret_cast<float2*>(gbase + L::kQ + kMlOff);
+      for (int i = tid; i < my_rows; i += kAttnThreads) {
+        const int tl = i >> 3, gg = i & 7;
+        if (gg >= G) continue;
+        float2 ml[ATTN_MAX_SPLIT];
         float mm = -INFINITY, den = 0.f;
-        const float2* mlp = reinterpret_cast<const float2*>(gbase + L::kQ + kMlOff);
-#pragma unroll 2
-        for (int s = 0; s < nsplit; ++s) {
-          const int idx = (s * G + gg) * tok_per + tl;
-          const float2 ml = mlp[idx];
-          const float4 o = *reinterpret_cast<const float4*>(gbase + L::kQ + (size_t)idx * (D * 4) + ((u ^ (idx & (F4 - 1))) * 16));
-          const float mn = fmaxf(mm, ml.x);
-          const float w0 = (mm == -INFINITY) ? 0.f : ex2_approx(mm - mn), w1 = (ml.x == -INFINITY) ? 0.f : ex2_approx(ml.x - mn);   // a CTA without visible keys adds nothing
-          mm = mn;
-          den = fmaf(den, w0, ml.y * w1);
-          v.x = fmaf(v.x, w0, o.x * w1); v.y = fmaf(v.y, w0, o.y * w1); v.z = fmaf(v.z, w0, o.z * w1); v.w = fmaf(v.w, w0, o.w * w1);
+#pragma unroll
+        for (int s = 0; s < ATTN_MAX_SPLIT; ++s) if (s < nsplit) { ml[s] = mlp[(s * G + gg) * tok_per + tl]; mm = fmaxf(mm, ml[s].x); }
+#pragma unroll
+        for (int s = 0; s < ATTN_MAX_SPLIT; ++s) if (s < nsplit) {
+          ml[s].x = (ml[s].x == -INFINITY) ? 0.f : ex2_approx(ml[s].x - mm);      // a CTA without visible keys adds nothing
+          den = fmaf(ml[s].y, ml[s].x, den);
         }
         const float inv = (den > 0.f) ? 1.f / den : 0.f;
-        v = make_float4(v.x * inv, v.y * inv, v.z * inv, v.w * inv);
+#pragma unroll
+        for (int s = 0; s < ATTN_MAX_SPLIT; ++s) if (s < nsplit) mlp[(s * G + gg) * tok_per + tl].x = ml[s].x * inv;
       }
-      const size_t obase = (((size_t)b * rps + tt) * a.Hq + (size_t)hkv * G + gg) * D + 4 * u;
+      __syncthreads();
+    }
+    // Half a warp per row (lane: units u and, with D = 128, u + 16), two heads of a token side by side, one pair at a time: this
+    // code runs once per CTA, and its size -- four rows unrolled: 25 KB -- cost more than the latency that unrolling hides.  The
+    // residual input is asked for three pairs ahead.
+    constexpr int NV = D / 64, kAhead = 3;
+    const int u = lane & 15, hv = lane >> 4;
+    struct Res { uint2 v[NV]; };
+    auto load_res = [&](int jp) {
+      const int j = 2 * jp + hv, gg = j & 7, tt = r0 + split * tok_per + (j >> 3);
+      Res r;
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        r.v[i] = make_uint2(0u, 0u);
+        if (a.h_out != nullptr && j < my_rows && gg < G && tt < rps)
+          r.v[i] = nsplit == 1 ? *reinterpret_cast<const uint2*>(res_s + (size_t)j * (D * 2) + (u + 16 * i) * 8)
+                               : *reinterpret_cast<const uint2*>(a.h_in + (((size_t)b * rps + tt) * a.Hq + (size_t)hkv * G + gg) * D + 4 * (u + 16 * i));
+      }
+      return r;
+    };
+    Res hq[kAhead];
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i) hq[i] = load_res(warp + i * kWarps);
+#pragma unroll 1
+    for (int jp = warp; 2 * jp < my_rows; jp += kWarps) {
+      const int j = 2 * jp + hv, tl = j >> 3, gg = j & 7, tk = split * tok_per + tl, tt = r0 + tk, sw = ((gg & 1) * 16 + tk) & (F4 - 1);
+      const Res h = hq[0];
+#pragma unroll
+      for (int i = 0; i + 1 < kAhead; ++i) hq[i] = hq[i + 1];
+      hq[kAhead - 1] = load_res(jp + kAhead * kWarps);
+      const bool valid = gg < G && tt < rps;
+      float4 v[NV];
+#pragma unroll
+      for (int i = 0; i < NV; ++i) v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (valid) {
+        const uint8_t* row0 = gbase + L::kQ + (size_t)(nsplit == 1 ? gg * 16 + tl : gg * tok_per + tl) * kRowBytes;
+        if (nsplit == 1) {
+#pragma unroll
+          for (int i = 0; i < NV; ++i) v[i] = *reinterpret_cast<const float4*>(row0 + (((u + 16 * i) ^ sw) * 16));
+        } else {
+          const float2* mlp = reinterpret_cast<const float2*>(gbase + L::kQ + kMlOff) + gg * tok_per + tl;
+#pragma unroll 2
+          for (int s = 0; s < nsplit; ++s) {
+            const float w = mlp[s * G * tok_per].x;
+#pragma unroll
+            for (int i = 0; i < NV; ++i) {
+              const float4 o = *reinterpret_cast<const float4*>(row0 + (size_t)(s * G * tok_per) * kRowBytes + (((u + 16 * i) ^ sw) * 16));
+              v[i].x = fmaf(o.x, w, v[i].x); v[i].y = fmaf(o.y, w, v[i].y); v[i].z = fmaf(o.z, w, v[i].z); v[i].w = fmaf(o.w, w, v[i].w);
+            }
+          }
+        }
+      }
+      const size_t orow = (((size_t)b * rps + tt) * a.Hq + (size_t)hkv * G + gg) * D + 4 * u;
       float ss = 0.f;
-      if (lane < F4) {
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        const size_t obase = orow + 64 * i;
+        if (!valid) continue;
         if (a.out != nullptr) {                                        // (null: a layer whose rows only feed the residual stream)
           if (a.out_fp32) {
-            *reinterpret_cast<float4*>(static_cast<float*>(a.out) + obase) = v;
+            *reinterpret_cast<float4*>(static_cast<float*>(a.out) + obase) = v[i];
           } else {
-            __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+            __nv_bfloat162 lo = __floats2bfloat162_rn(v[i].x, v[i].y), hi = __floats2bfloat162_rn(v[i].z, v[i].w);
             uint2 w; w.x = *reinterpret_cast<uint32_t*>(&lo); w.y = *reinterpret_cast<uint32_t*>(&hi);
             *reinterpret_cast<uint2*>(static_cast<bf16*>(a.out) + obase) = w;
           }
         }
         if (a.h_out != nullptr) {
-          const uint2 hraw = *reinterpret_cast<const uint2*>(res_s + (size_t)j * (D * 2) + u * 8);
-          const float2 h0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&hraw.x));
-          const float2 h1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&hraw.y));
-          __nv_bfloat162 lo = __floats2bfloat162_rn(h0.x + v.x, h0.y + v.y), hi = __floats2bfloat162_rn(h1.x + v.z, h1.y + v.w);
+          const float2 h0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&h.v[i].x));
+          const float2 h1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&h.v[i].y));
+          __nv_bfloat162 lo = __floats2bfloat162_rn(h0.x + v[i].x, h0.y + v[i].y), hi = __floats2bfloat162_rn(h1.x + v[i].z, h1.y + v[i].w);
           uint2 w; w.x = *reinterpret_cast<uint32_t*>(&lo); w.y = *reinterpret_cast<uint32_t*>(&hi);
           if (VS_STORE_OK(bp, a.h_out_region, a.h_out + obase, 8)) *reinterpret_cast<uint2*>(a.h_out + obase) = w;
           if (a.ss_out != nullptr) {
             // RMSNorm of the next layer: its statistics are those of the rows as stored (bf16)
             const float2 s0 = __bfloat1622float2(lo), s1 = __bfloat1622float2(hi);
-            ss = (s0.x * s0.x + s0.y * s0.y) + (s1.x * s1.x + s1.y * s1.y);
+            ss += (s0.x * s0.x + s0.y * s0.y) + (s1.x * s1.x + s1.y * s1.y);
             if (a.next_gain != nullptr) {
               // ... and, with a gain vector, the projection reads bf16(h * gain) instead of h
-              const uint2 graw = *reinterpret_cast<const uint2*>(a.next_gain + ((size_t)hkv * G + gg) * D + 4 * u);
+              const uint2 graw = *reinterpret_cast<const uint2*>(a.next_gain + ((size_t)hkv * G + gg) * D + 4 * u + 64 * i);
               const float2 g0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&graw.x));
               const float2 g1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&graw.y));
               __nv_bfloat162 x0 = __floats2bfloat162_rn(s0.x * g0.x, s0.y * g0.y), x1 = __floats2bfloat162_rn(s1.x * g1.x, s1.y * g1.y);
@@ -676,8 +740,8 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
       }
       if (a.ss_out != nullptr) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-        if (lane == 0) ss_stage[gg * 16 + tk] = ss;
+        for (int o = 8; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+        if (u == 0 && valid) ss_stage[gg * 16 + tk] = ss;
       }
     }
     if (a.ss_out != nullptr) {
@@ -692,6 +756,9 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
       }
     }
   }
+  // every CTA of the cluster has what it waited for: nobody's shared memory goes away while a copy may be reading it
+  __syncwarp();
+  if (nsplit > 1) { cluster_arrive(); cluster_wait(); }
   tc_fence_before();
   __syncthreads();
   if (warp == kIssuerWarp) {
@@ -715,9 +782,13 @@ cudaError_t prefill_attention_tc_init() {
   return e;
 }
 
-// whether `nsplit` CTAs can share a row tile's keys: the rows they leave one another have to fit where the query was
+// whether `nsplit` CTAs can share a row tile's keys: the rows they leave one another have to fit where the query was,
+// and those on their way in the ring
 bool prefill_attention_can_split(int head_dim, int group, int nsplit) {
-  return nsplit * group * ((kTok + nsplit - 1) / nsplit) <= (head_dim == 128 ? Smem<128>::kRowsOut : Smem<64>::kRowsOut);
+  const int tok_per = (kTok + nsplit - 1) / nsplit, last = kTok - (nsplit - 1) * tok_per;
+  const int room = head_dim == 128 ? Smem<128>::kRowsOut : Smem<64>::kRowsOut;
+  const int staged = head_dim == 128 ? Smem<128>::kStages * Smem<128>::kKVBytes / 512 : Smem<64>::kStages * Smem<64>::kKVBytes / 256;
+  return last > 0 && nsplit * group * tok_per <= room && group * (kTok - last) <= staged;
 }
 
 cudaError_t launch_prefill_attention_tc(const AttnArgs& a, const BatchParams& bp, int* status, cudaStream_t st) {

@@ -231,9 +231,9 @@ int ensure_step_maps(vs_stream* h, int rows) {
 }
 
 // CTAs to spread the key tiles of a row tile over (one cluster).  All clusters must be resident at once, with a little room for
-// the bank update's.  In key tiles (0.75 us each), measured on frames, clips and questions of 5 to 13 tiles: two CTAs an SM make
-// a tile a tenth longer, exchanging rows costs 2.2 and 0.3 for every CTA of the cluster.  key_len[i]: segment lengths of the
-// longest key axis among the listed entries.
+// the bank update's.  Cost in key tiles (about 1.7 us each when the CTA has its SM alone), fitted to frames, clips and questions of
+// 5 to 13 tiles: two CTAs an SM make a tile a tenth longer, a row tile's row stores cost three, shared by the CTAs of the
+// cluster, the exchange a half.  key_len[i]: segment lengths of the longest key axis among the listed entries.
 int attn_split(const vs_stream* h, const BatchParams& bp, const int* key_len, int n_len) {
   int key_tiles = 0;
   for (int i = 0; i < n_len; ++i) key_tiles += (key_len[i] + ATTN_KEY_BOX - 1) / ATTN_KEY_BOX;
@@ -243,7 +243,7 @@ int attn_split(const vs_stream* h, const BatchParams& bp, const int* key_len, in
   for (int s = 1; s <= ATTN_MAX_SPLIT; ++s) {
     if (s > 1 && (s > key_tiles || row_ctas * s > 2LL * h->n_sms || h->attn_clusters[s] < row_ctas + 4 ||
                   !prefill_attention_can_split(h->dm.D, h->dm.G, s))) continue;
-    const double c = ((key_tiles + s - 1) / s) * (row_ctas * s > h->n_sms ? 1.1 : 1.0) + (s > 1 ? 2.2 + 0.3 * s : 0.0);
+    const double c = ((key_tiles + s - 1) / s) * (row_ctas * s > h->n_sms ? 1.1 : 1.0) + 3.0 / s + (s > 1 ? 0.5 : 0.0);
     if (c < cost) { cost = c; best = s; }
   }
   return best;
