@@ -205,8 +205,8 @@ struct Smem {
   static constexpr int kKVBytes = kKeys * D * 2;          // a K or V tile
   static constexpr int kStages = D == 128 ? 3 : 6;
   static constexpr int kQ = 0;                            // [hi | lo]; at the end rows, fp32, and their (max, denominator)
-  static constexpr int kRowsOut = 2 * kQBytes / (D * 4 + 8);   // rows that fit there
   static constexpr int kRing = 2 * kQBytes;               // [stage] K or V tile; at the end (max, denominator) without a cluster, sums of squares
+  static constexpr int kRingRows = kStages * kKVBytes / (D * 4);   // fp32 rows that fit there
   static constexpr int kCtl = kRing + kStages * kKVBytes; // barriers, tmem slot, abort flag
   static constexpr int kTotal = kCtl + 256;
   static_assert(2 * (kTotal + 1024) <= 228 * 1024, "two CTAs an SM");
@@ -554,8 +554,9 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
 
   // ---- rows out -----------------------------------------------------------------------------------------------
   constexpr int F4 = D / 4, kWarps = kAttnThreads / 32, kRowBytes = D * 4;
-  constexpr uint32_t kMlOff = (uint32_t)L::kRowsOut * kRowBytes;      // (max, denominator) pairs behind the rows
   const int tok_per = (kTok + nsplit - 1) / nsplit;                   // CTA s of the cluster finishes tokens s * tok_per ...
+  const int n_recv = nsplit * G * tok_per;                            // rows that find a place where the query was: [CTA][head][token]
+  const uint32_t ml_off = (uint32_t)n_recv * kRowBytes;               // ... behind them their (max, denominator) pairs
   auto tokens_of = [&](int s) { return max(min(tok_per, kTok - s * tok_per), 0); };   // ... this many of them (none, perhaps)
   const int my_tok = tokens_of(split), my_rows = 8 * my_tok;          // row j: head j & 7 of token j >> 3
   uint8_t* res_s = gbase + L::kRing;                                  // [row j][D] bf16: residual input of the rows (the ring is dead by now)
@@ -578,6 +579,10 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
     if (tid == 0) mbar_arrive_expect_tx(bar_recv, (uint32_t)((nsplit - 1) * G * my_tok * (kRowBytes + 8)));
     cluster_wait();                 // every peer's query is dead, and its barriers exist
   }
+  // place of a staged row: the ring, the few that it has no room for behind the pairs
+  auto staged_at = [&](int i) {
+    return base + (i < L::kRingRows ? L::kRing + (uint32_t)i * kRowBytes : L::kQ + ml_off + (uint32_t)n_recv * 8u + (uint32_t)(i - L::kRingRows) * kRowBytes);
+  };
   if (warp < 4) {
     // Every thread's row: into this CTA's own area if it finishes the row (with 1 / denominator if there are no peers), else staged
     // in the ring, from where it goes to the owner by bulk copies -- the rows of an owner's tokens lie side by side for every
@@ -587,7 +592,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
     const int theirs = kTok - my_tok;                                 // tokens of others, in order, numbered round this CTA's own
     const int idx = nsplit == 1 ? tid : (owner == split ? (split * G + gg) * tok_per + (tk - owner * tok_per)
                                                         : gg * theirs + (tk < split * tok_per ? tk : tk - my_tok));
-    const uint32_t dst = base + (owner == split ? L::kQ : L::kRing) + (uint32_t)idx * kRowBytes;
+    const uint32_t dst = owner == split ? base + L::kQ + (uint32_t)idx * kRowBytes : staged_at(idx);
     const float inv = nsplit > 1 ? 1.f : ((l_run > 0.f) ? 1.f / l_run : 0.f);
 #pragma unroll 1
     for (int c = 0; c < D; c += 32) {
@@ -610,7 +615,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
     tc_fence_before();
     if (nsplit > 1) {
       if (gg < G) {
-        const uint32_t at = base + L::kQ + kMlOff + (uint32_t)((split * G + gg) * tok_per + (tk - owner * tok_per)) * 8u;
+        const uint32_t at = base + L::kQ + ml_off + (uint32_t)((split * G + gg) * tok_per + (tk - owner * tok_per)) * 8u;
         if (owner == split) *reinterpret_cast<float2*>(gbase + (at - base)) = make_float2(m_run, l_run);
         else st_async_f2(map_shared_rank(at, (uint32_t)owner), make_float2(m_run, l_run), map_shared_rank(bar_recv, (uint32_t)owner));
       }
@@ -621,7 +626,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
       if (o < nsplit && o != split && g < G) {
         const int n = tokens_of(o), first = o * tok_per, src = g * theirs + (first < split * tok_per ? first : first - my_tok);
         bulk_to_peer(map_shared_rank(base + L::kQ + (uint32_t)((split * G + g) * tok_per) * kRowBytes, (uint32_t)o),
-                     base + L::kRing + (uint32_t)src * kRowBytes, (uint32_t)(n * kRowBytes), map_shared_rank(bar_recv, (uint32_t)o));
+                     staged_at(src), (uint32_t)(n * kRowBytes), map_shared_rank(bar_recv, (uint32_t)o));
       }
     }
     cp_async_wait<0>();
@@ -632,7 +637,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
     VS_STAMP(bp, 2, 3);
     if (nsplit > 1) {
       // what each CTA's part of a row counts for, 2^(max_i - max) over the row's denominator: a thread per row, in place of the pairs
-      float2* mlp = reinterpret_cast<float2*>(gbase + L::kQ + kMlOff);
+      float2* mlp = reinterpret_cast<float2*>(gbase + L::kQ + ml_off);
       for (int i = tid; i < my_rows; i += kAttnThreads) {
         const int tl = i >> 3, gg = i & 7;
         if (gg >= G) continue;
@@ -689,7 +694,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
 #pragma unroll
           for (int i = 0; i < NV; ++i) v[i] = *reinterpret_cast<const float4*>(row0 + (((u + 16 * i) ^ sw) * 16));
         } else {
-          const float2* mlp = reinterpret_cast<const float2*>(gbase + L::kQ + kMlOff) + gg * tok_per + tl;
+          const float2* mlp = reinterpret_cast<const float2*>(gbase + L::kQ + ml_off) + gg * tok_per + tl;
 #pragma unroll 2
           for (int s = 0; s < nsplit; ++s) {
             const float w = mlp[s * G * tok_per].x;
@@ -782,13 +787,16 @@ cudaError_t prefill_attention_tc_init() {
   return e;
 }
 
-// whether `nsplit` CTAs can share a row tile's keys: the rows they leave one another have to fit where the query was,
-// and those on their way in the ring
+// Whether `nsplit` CTAs can share a row tile's keys: the rows they leave one another have to fit where the query was, those on
+// their way in the ring, with a few behind the others; and nobody may be without tokens.
 bool prefill_attention_can_split(int head_dim, int group, int nsplit) {
   const int tok_per = (kTok + nsplit - 1) / nsplit, last = kTok - (nsplit - 1) * tok_per;
-  const int room = head_dim == 128 ? Smem<128>::kRowsOut : Smem<64>::kRowsOut;
-  const int staged = head_dim == 128 ? Smem<128>::kStages * Smem<128>::kKVBytes / 512 : Smem<64>::kStages * Smem<64>::kKVBytes / 256;
-  return last > 0 && nsplit * group * tok_per <= room && group * (kTok - last) <= staged;
+  const int room = head_dim == 128 ? 2 * Smem<128>::kQBytes : 2 * Smem<64>::kQBytes, ring = head_dim == 128 ? Smem<128>::kRingRows : Smem<64>::kRingRows;
+  if (last < 1) return false;
+  const int received = nsplit * group * tok_per, staged = group * (kTok - last), over = staged > ring ? staged - ring : 0;
+  // (rows of one owner and head are sent as one run: none may lie on both sides of the ring's end)
+  if (over > 0 && (last != tok_per || ring % tok_per != 0)) return false;
+  return received * (head_dim * 4 + 8) + over * head_dim * 4 <= room;
 }
 
 cudaError_t launch_prefill_attention_tc(const AttnArgs& a, const BatchParams& bp, int* status, cudaStream_t st) {
