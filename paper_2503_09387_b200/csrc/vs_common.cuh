@@ -90,7 +90,7 @@ struct Dims {
 
 constexpr int KSPLIT_MAX = 5;   // CTAs sharing one output tile of a linear layer along K
 constexpr int DEC_SPLIT_MAX = 8;      // key splits of the decode attention = CTAs of one cluster
-constexpr int TOK_MAX_ROWS = 32;      // token rows of a step that the persistent kernel takes
+constexpr int TOK_MAX_ROWS = 16;      // token rows of a step that the persistent kernel takes
 constexpr int TOK_MAX_CTAS = 160;     // ... one CTA per SM
 constexpr int GEMM_BLOCK_M = 128;
 constexpr int GEMM_BLOCK_K = 64;
@@ -115,7 +115,7 @@ struct Layout {
   size_t chunk_slot;            // int32 [VS_MAX_BATCH]  chunked prefill: slot each frame's carrier went to
   size_t chunk_victim;          // int32 [VS_MAX_BATCH]  ... and whom its bank update evicted (index on the bank axis)
   size_t gemm_flags;            // int32 [GEMM_XCHG_CTAS]  projection K split: partials delivered per slice owner
-  size_t tok_layers;            // TokLayer [L], then the vocabulary projection's tensor maps [2], as the token-step kernel reads them
+  size_t tok_layers;            // TokLayer [L], then the vocabulary projection's tensor map, as the token-step kernel reads them
   size_t tok_sync;              // its counters, flags and tickets, zero between launches
   size_t lm_keys, lm_tickets;   // uint64 [256], int32 [256]  language-model head: greedy-choice keys and tickets per row
   size_t persistent_end;
@@ -427,10 +427,10 @@ cudaError_t launch_decode_attention(const DecodeArgs& a, const BatchParams& bp, 
 // kernel (vs_token.cu).
 struct TokLayer {
   // the matrices as 4-D tensor maps {64 of K, rows, row groups, K blocks of 64}, 128-byte swizzle, one box = a stage (half of
-  // one for gate and up): 32 rows by [0] 512, [1] 256 elements
-  CUtensorMap tm_qkv[2], tm_o[2], tm_gate[2], tm_up[2], tm_down[2];
+  // one for gate and up): 32 rows by 512 elements
+  CUtensorMap tm_qkv, tm_o, tm_gate, tm_up, tm_down;
   const bf16 *bias, *gain, *gain2;
-  const void* pad[13];           // (tensor maps start on multiples of 64 bytes)
+  const void* pad[13];          // (tensor maps start on multiples of 64 bytes)
 };
 static_assert(sizeof(TokLayer) % 128 == 0, "tensor maps of every layer stay aligned");
 struct TokArgs {
@@ -454,7 +454,7 @@ struct TokArgs {
   int* status;
   // language-model head (vocab > 0): rows of `hidden` -> fp32 logits and, if next_token, the greedy choice
   int vocab;
-  const CUtensorMap* tm_lm;      // [2] in device memory
+  const CUtensorMap* tm_lm;      // in device memory
   const bf16* gain_f;
   float* logits; int32_t* next_token; unsigned long long* lm_keys;
   int stages; uint32_t ring_bytes;                                   // set by the launch

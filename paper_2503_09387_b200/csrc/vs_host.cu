@@ -107,7 +107,7 @@ void fill_layout(const Dims& D, Layout& Lo) {
   Lo.chunk_slot = reg(DR_CHUNK_SLOT, take((size_t)VS_MAX_BATCH * 4));
   Lo.chunk_victim = reg(DR_CHUNK_VICTIM, take((size_t)VS_MAX_BATCH * 4));
   Lo.gemm_flags = reg(DR_GEMM_FLAGS, take((size_t)GEMM_XCHG_CTAS * 4));
-  Lo.tok_layers = take((size_t)D.L * sizeof(TokLayer) + 2 * sizeof(CUtensorMap));
+  Lo.tok_layers = take((size_t)D.L * sizeof(TokLayer) + sizeof(CUtensorMap));
   Lo.tok_sync = take(tok_sync_ints(D.L, D.Hkv) * 4);
   Lo.lm_keys = take((size_t)256 * 8);          // language-model head: per-row argmax keys and tickets, zero between calls
   Lo.lm_tickets = take((size_t)256 * 4);
@@ -414,16 +414,16 @@ size_t layer_stride_prefix(const Dims& D) { return (size_t)D.S * D.Hkv * D.maxP 
 size_t layer_stride_tail(const Dims& D) { return (size_t)D.S * D.Hkv * D.maxT * D.D; }
 
 // Whether a step of n_active x T rows goes to the persistent kernel (measured at the Qwen2-7B shape, us against the launches
-// layer by layer).  Full layers: up to 16 rows (3 layers and the head: 562 -> 437 for one row, 595 -> 549 for 16; 24 rows no
-// longer, their slabs leave the ring too few stages).  Attention alone: steps of several tokens (28 layers: 560 -> 443 for 2
-// rows, 795 -> 722 for 32) and single tokens of more streams than the matrix-vector kernel takes (579 -> 463 for 8), in a stack;
-// one to four single tokens are faster by launches (352 against 463: 11 us a layer is little more than the phases' own
-// synchronisation).  And not where a layer's projection holds less than 16 KB for every SM: there is then no weight stream to hide
-// that synchronisation behind.
+// layer by layer).  Full layers and the head: up to 8 rows (3 layers and the head: 455 -> 437 for one row, 336 -> 303 for 8
+// without the head; at 16 the slabs leave the ring too few stages, 344 -> 362).  Attention alone: steps of several tokens up to
+// 16 rows (28 layers: 589 -> 474 for 2 rows, 783 -> 559 for 16; 32 rows 770 -> 842) and single tokens of more streams than the
+// matrix-vector kernel takes (545 -> 460 for 8, 588 -> 517 for 16), in a stack; one to four single tokens are faster by launches
+// (352 against 463: 11 us a layer is little more than the phases' own synchronisation).  And not where a layer's projection holds
+// less than 16 KB for every SM: there is then no weight stream to hide that synchronisation behind.
 bool token_step_pays(const vs_stream* h, int n_active, int T, int matrix_rows, bool full) {
   const int rows = n_active * T;
   if (h->n_sms > TOK_MAX_CTAS || (size_t)matrix_rows * h->dm.d * 2 < (size_t)h->n_sms * 16384) return false;
-  if (full) return rows <= 16;
+  if (full) return rows <= 8;
   return rows <= TOK_MAX_ROWS && (T > 1 || (rows > 4 && h->dm.L > 1));
 }
 
@@ -564,28 +564,26 @@ int vs_create_stream(const vs_config* cfg, const vs_weights* weights, void* work
   if (cudaMemset(h->ws, 0, lo.total) != cudaSuccess) return fail(VS_ERR_CUDA);
   {
     std::vector<TokLayer> tl(D.L);
-    CUtensorMap lm[2];
-    std::memset(lm, 0, sizeof(lm));
+    CUtensorMap lm;
+    std::memset(&lm, 0, sizeof(lm));
     bool ok = true;
-    for (int m = 0; m < 2 && ok; ++m) {
-      const uint32_t mt = 2, kb = m == 0 ? 8 : 4;  // 16-row sub-tiles of a weight tile, 64-element blocks of a stage
-      for (int l = 0; l < D.L && ok; ++l) {
-        TokLayer& t = tl[l];
-        if (m == 0) { std::memset(&t, 0, sizeof(TokLayer)); t.bias = h->bias[l]; t.gain = h->gain[l]; }
-        // (a head's halves apart: a tile holds both elements of its rotation pairs)
-        ok = encode_weight(h, &t.tm_qkv[m], h->w[l], D.d, D.D / 2, 2 * (D.Hq + 2 * D.Hkv), 8 * mt, 2, kb);
-        if (D.d_ff > 0) {
-          t.gain2 = h->gain2[l];
-          ok = ok && encode_weight(h, &t.tm_o[m], weights->w_o[l], D.d, D.d, 1, 16 * mt, 1, kb) &&
-               encode_weight(h, &t.tm_gate[m], weights->w_gate[l], D.d, D.d_ff, 1, 8 * mt, 1, kb) &&
-               encode_weight(h, &t.tm_up[m], weights->w_up[l], D.d, D.d_ff, 1, 8 * mt, 1, kb) &&
-               encode_weight(h, &t.tm_down[m], weights->w_down[l], D.d_ff, D.d, 1, 16 * mt, 1, kb);
-        }
+    for (int l = 0; l < D.L && ok; ++l) {
+      TokLayer& t = tl[l];
+      std::memset(&t, 0, sizeof(TokLayer));
+      t.bias = h->bias[l]; t.gain = h->gain[l];
+      // boxes of 8 64-element blocks of 32 rows (a head's halves apart: a tile holds both elements of its rotation pairs)
+      ok = encode_weight(h, &t.tm_qkv, h->w[l], D.d, D.D / 2, 2 * (D.Hq + 2 * D.Hkv), 16, 2, 8);
+      if (D.d_ff > 0) {
+        t.gain2 = h->gain2[l];
+        ok = ok && encode_weight(h, &t.tm_o, weights->w_o[l], D.d, D.d, 1, 32, 1, 8) &&
+             encode_weight(h, &t.tm_gate, weights->w_gate[l], D.d, D.d_ff, 1, 16, 1, 8) &&
+             encode_weight(h, &t.tm_up, weights->w_up[l], D.d, D.d_ff, 1, 16, 1, 8) &&
+             encode_weight(h, &t.tm_down, weights->w_down[l], D.d_ff, D.d, 1, 32, 1, 8);
       }
-      if (D.vocab > 0) ok = ok && encode_weight(h, &lm[m], weights->w_lm, D.d, D.vocab, 1, 32, 1, m == 0 ? 8 : 4);
     }
+    if (D.vocab > 0) ok = ok && encode_weight(h, &lm, weights->w_lm, D.d, D.vocab, 1, 32, 1, 8);
     if (!ok || cudaMemcpy(h->ws + lo.tok_layers, tl.data(), tl.size() * sizeof(TokLayer), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(h->ws + lo.tok_layers + tl.size() * sizeof(TokLayer), lm, sizeof(lm), cudaMemcpyHostToDevice) != cudaSuccess)
+        cudaMemcpy(h->ws + lo.tok_layers + tl.size() * sizeof(TokLayer), &lm, sizeof(lm), cudaMemcpyHostToDevice) != cudaSuccess)
       return fail(VS_ERR_CUDA);
   }
   if (cudaMemset(h->ws + lo.slot_frame, 0xFF, (size_t)D.S * D.slots * 4) != cudaSuccess) return fail(VS_ERR_CUDA);

@@ -177,10 +177,8 @@ struct Phase {
   int K, kst, tiles;            // reduction length, stages per tile, tiles
   int s0, s1;                   // this CTA's stages
 };
-// K elements of a stage: 512 (32 KB of weights); 256 where the rows' slabs leave room for no more
-__host__ __device__ constexpr int stage_k(int nt) { return nt <= 2 ? 512 : 256; }
+constexpr int KS = 512;                           // K elements of a stage (32 KB of weights)
 constexpr int MT = 2;                             // 16-row sub-tiles of a weight tile
-template <int KS>
 __device__ __noinline__ Phase make_phase(const TokArgs& a, int kind, int cta, int ncta) {
   Phase p;
   int rows = 0;
@@ -339,7 +337,7 @@ __device__ __forceinline__ void finish_item(const TokArgs& a, const BatchParams&
     bf16* out = kind == PH_WO ? a.hbuf[1] : a.hbuf[0];
     const bool last = kind == PH_DN && l + 1 == a.L;
     const bf16* gain = kind == PH_WO ? a.layers[l].gain2 : (last ? nullptr : a.layers[l + 1].gain);
-    float* ss = a.ss + (kind == PH_WO ? (size_t)32 * a.ss_cap : 0);
+    float* ss = a.ss + (kind == PH_WO ? (size_t)TOK_MAX_ROWS * a.ss_cap : 0);
     const int f1 = mt * 16 + pg, reg = kind == PH_WO ? DR_HBUF1 : DR_HBUF0;
     (void)reg;
 #pragma unroll
@@ -374,10 +372,9 @@ __device__ __forceinline__ void finish_item(const TokArgs& a, const BatchParams&
 
 template <int D, int NT>   // head size; 8-token columns
 __global__ void __launch_bounds__(kThreads, 1) token_kernel(const __grid_constant__ TokArgs a, const __grid_constant__ BatchParams bp) {
-  constexpr int TM = 16 * MT, KS = stage_k(NT);   // a stage: 32 weight rows x KS elements, and KS elements of every token row
+  constexpr int TM = 16 * MT;                     // a stage: 32 weight rows x KS elements, and KS elements of every token row
   constexpr uint32_t kStageW = TM * KS * 2;       // the weights of a stage; behind them the token rows, RS bytes apart (64 more than
   constexpr int RS = KS * 2 + 64;                 // their slab: two neighbouring rows lie in different banks)
-  constexpr int kMap = KS == 512 ? 0 : 1;
   constexpr int ITEMS = MT * NT;                  // 16 x 8 accumulators of a tile
   constexpr int KC = D / 32, VC = D / 64, OT = D / 16;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -432,10 +429,10 @@ __global__ void __launch_bounds__(kThreads, 1) token_kernel(const __grid_constan
     if (lane == 0)
       for_phases([&](int l, int kind) {
         if (kind == PH_ATT) return;
-        const Phase p = make_phase<KS>(a, kind, cta, ncta);
+        const Phase p = make_phase(a, kind, cta, ncta);
         const TokLayer* ly = a.layers + l;
-        const CUtensorMap* tm = kind == PH_QKV ? &ly->tm_qkv[kMap] : kind == PH_WO ? &ly->tm_o[kMap] : kind == PH_GU ? &ly->tm_gate[kMap]
-                              : kind == PH_DN ? &ly->tm_down[kMap] : a.tm_lm + kMap;
+        const CUtensorMap* tm = kind == PH_QKV ? &ly->tm_qkv : kind == PH_WO ? &ly->tm_o : kind == PH_GU ? &ly->tm_gate
+                              : kind == PH_DN ? &ly->tm_down : a.tm_lm;
         asm volatile("prefetch.tensormap [%0];" ::"l"(tm) : "memory");
         int tile = p.s0 / p.kst, kk = p.s0 - tile * p.kst;
 #pragma unroll 1
@@ -449,7 +446,7 @@ __global__ void __launch_bounds__(kThreads, 1) token_kernel(const __grid_constan
             tma_load_4d(dst, tm, 0, pb * 8, 2 * hs, kb, full(slot));
           } else if (kind == PH_GU) {
             tma_load_4d(dst, tm, 0, tile * MT * 8, 0, kb, full(slot));
-            tma_load_4d(dst + kStageW / 2, &ly->tm_up[kMap], 0, tile * MT * 8, 0, kb, full(slot));
+            tma_load_4d(dst + kStageW / 2, &ly->tm_up, 0, tile * MT * 8, 0, kb, full(slot));
           } else {
             tma_load_4d(dst, tm, 0, tile * TM, 0, kb, full(slot));
           }
@@ -471,7 +468,7 @@ __global__ void __launch_bounds__(kThreads, 1) token_kernel(const __grid_constan
     uint32_t par = 1;
     for_phases([&](int l, int kind) {
       if (kind == PH_ATT) return;
-      const Phase p = make_phase<KS>(a, kind, cta, ncta);
+      const Phase p = make_phase(a, kind, cta, ncta);
       const bf16* x = phase_rows(a, l, kind);
       if (p.s0 < p.s1) {
         if (lane == 0) wait_input(a, l, kind, ncta, abort_flag);
@@ -512,12 +509,12 @@ __global__ void __launch_bounds__(kThreads, 1) token_kernel(const __grid_constan
     if (a.use_rmsnorm)
       for_phases([&](int l, int kind) {
         if (kind != PH_QKV && kind != PH_GU && kind != PH_LM) return;
-        const Phase p = make_phase<KS>(a, kind, cta, ncta);
+        const Phase p = make_phase(a, kind, cta, ncta);
         if (p.s0 >= p.s1) return;
         if (lane == 0) wait_input(a, l, kind, ncta, abort_flag);
         __syncwarp();
         const int parts = (kind == PH_LM || (kind == PH_QKV && l == 0)) ? 1 : (a.full ? a.d / 16 : a.Hkv);
-        const float* ss = a.ss + (kind == PH_GU ? (size_t)32 * a.ss_cap : 0);
+        const float* ss = a.ss + (kind == PH_GU ? (size_t)TOK_MAX_ROWS * a.ss_cap : 0);
         // lanes of a row: as many as it has parts (up to 32), so that few-part rows are summed side by side
         int lpr = 1;
         while (lpr < parts && lpr < 32) lpr <<= 1;
@@ -598,7 +595,7 @@ __global__ void __launch_bounds__(kThreads, 1) token_kernel(const __grid_constan
     int slot = 0;
     uint32_t par = 0, rs_parity = 0;
     auto weight_phase = [&](int l, int kind) {
-      const Phase p = make_phase<KS>(a, kind, cta, ncta);
+      const Phase p = make_phase(a, kind, cta, ncta);
       const int seq = 1 + l * 5 + kind;
       if (warp == 0 && kind == PH_QKV) TOK_STAMP(0, l);
       const bool normed = a.use_rmsnorm && (kind == PH_QKV || kind == PH_GU || kind == PH_LM);
@@ -623,15 +620,15 @@ __global__ void __launch_bounds__(kThreads, 1) token_kernel(const __grid_constan
         FinishIn in = {};
         if (part_ends && item < ITEMS && kk_begin == 0) in = finish_in<D>(a, l, kind, tile * MT + item / NT, item % NT, lane);
         const uint32_t xb = ring + slot * stage_bytes + kStageW;
-        // the stage's weights: [K block of 64][rows][128 bytes, swizzled]; each warp takes 64 (or 32) of K
-        constexpr int KW = KS / kCW / 32;
-        const uint32_t wb = ring + slot * stage_bytes + (uint32_t)(warp * KW / 2) * kb_stride + (uint32_t)pg * 128;
+        // the stage's weights: [K block of 64][rows][128 bytes, swizzled]; each warp takes 64 of K
+        constexpr int KW = KS / kCW / 32;                              // 32s of K
+        static_assert(KW == 2, "a warp takes a 64-element block");
+        const uint32_t wb = ring + slot * stage_bytes + (uint32_t)warp * kb_stride + (uint32_t)pg * 128;
         if (warp * KW * 32 < len) {                                    // (a multiple of 64; what is left of KW 32s is zeros)
           uint4 xv[KW][NT], w0[KW][MT], w1[KW][MT];
 #pragma unroll
           for (int kb = 0; kb < KW; ++kb) {
-            const int half32 = KW == 2 ? kb : (warp & 1);              // which 32 of the 64-element block
-            const uint32_t cb = (uint32_t)(((half32 * 4 + t4) ^ pg) << 4);
+            const uint32_t cb = (uint32_t)(((kb * 4 + t4) ^ pg) << 4);
 #pragma unroll
             for (int mt = 0; mt < MT; ++mt) {
               w0[kb][mt] = lds128(wb + (uint32_t)mt * m_off + cb);
@@ -1030,7 +1027,7 @@ constexpr size_t kMaxDynSmem = 227 * 1024;
 constexpr size_t kCtlBytes = 6144;
 template <int D, int NT>
 struct TokShape {
-  static constexpr size_t kRS = (size_t)stage_k(NT) * 2 + 64, kW = (size_t)16 * MT * stage_k(NT) * 2;   // bytes of a token row and of the weights in a stage
+  static constexpr size_t kRS = (size_t)KS * 2 + 64, kW = (size_t)16 * MT * KS * 2;   // bytes of a token row and of the weights in a stage
   static constexpr size_t kRed = (size_t)kCW * MT * NT * 512, kO = (size_t)kCW * kHeads * D * 4;
   static constexpr size_t kFixed = (kRed > kO ? kRed : kO) + (size_t)NT * 8 * (D / 2) * 8 + kCtlBytes;
 };
@@ -1051,7 +1048,6 @@ template <int D>
 cudaError_t init_head() {
   cudaError_t e = cudaFuncSetAttribute(token_kernel<D, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynSmem);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(token_kernel<D, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynSmem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(token_kernel<D, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynSmem);
   return e;
 }
 }  // namespace
@@ -1072,13 +1068,11 @@ cudaError_t launch_token_step(const TokArgs& a, const BatchParams& bp, int n_sms
   const int D = a.vocab > 0 ? 128 : a.D;
   if (D == 128) {
     if (a.rows <= 8) return launch_shape<128, 1>(a, bp, n_sms, st);
-    if (a.rows <= 16) return launch_shape<128, 2>(a, bp, n_sms, st);
-    return launch_shape<128, 4>(a, bp, n_sms, st);
+    return launch_shape<128, 2>(a, bp, n_sms, st);
   }
   if (D != 64) return cudaErrorInvalidValue;
   if (a.rows <= 8) return launch_shape<64, 1>(a, bp, n_sms, st);
-  if (a.rows <= 16) return launch_shape<64, 2>(a, bp, n_sms, st);
-  return launch_shape<64, 4>(a, bp, n_sms, st);
+  return launch_shape<64, 2>(a, bp, n_sms, st);
 }
 
 }  // namespace vs
