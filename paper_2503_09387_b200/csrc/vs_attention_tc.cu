@@ -554,10 +554,11 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
 
   // ---- rows out -----------------------------------------------------------------------------------------------
   constexpr int F4 = D / 4, kWarps = kAttnThreads / 32, kRowBytes = D * 4;
-  const int tok_per = (kTok + nsplit - 1) / nsplit;                   // CTA s of the cluster finishes tokens s * tok_per ...
+  const int n_tok = min(kTok, rps - r0);                              // tokens of this row tile
+  const int tok_per = (n_tok + nsplit - 1) / nsplit;                  // CTA s of the cluster finishes tokens s * tok_per ...
   const int n_recv = nsplit * G * tok_per;                            // rows that find a place where the query was: [CTA][head][token]
   const uint32_t ml_off = (uint32_t)n_recv * kRowBytes;               // ... behind them their (max, denominator) pairs
-  auto tokens_of = [&](int s) { return max(min(tok_per, kTok - s * tok_per), 0); };   // ... this many of them (none, perhaps)
+  auto tokens_of = [&](int s) { return max(min(tok_per, n_tok - s * tok_per), 0); };   // ... this many of them (none, perhaps)
   const int my_tok = tokens_of(split), my_rows = 8 * my_tok;          // row j: head j & 7 of token j >> 3
   uint8_t* res_s = gbase + L::kRing;                                  // [row j][D] bf16: residual input of the rows (the ring is dead by now)
   float* ss_stage = reinterpret_cast<float*>(gbase + L::kRing + (nsplit == 1 ? 128 * D * 2 : 0));   // [8 heads][16 tokens] sums of squares of stored residual rows
@@ -589,7 +590,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
     // head.  (Stored straight into the peer's shared memory, 16 bytes a lane scattered over 32 rows, they took 4 us.)
     const int gg = tid >> 4, tk = tid & 15, owner = nsplit == 1 ? 0 : tk / tok_per;
     const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
-    const int theirs = kTok - my_tok;                                 // tokens of others, in order, numbered round this CTA's own
+    const int theirs = n_tok - my_tok;                                // tokens of others, in order, numbered round this CTA's own
     const int idx = nsplit == 1 ? tid : (owner == split ? (split * G + gg) * tok_per + (tk - owner * tok_per)
                                                         : gg * theirs + (tk < split * tok_per ? tk : tk - my_tok));
     const uint32_t dst = owner == split ? base + L::kQ + (uint32_t)idx * kRowBytes : staged_at(idx);
@@ -604,7 +605,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
 #pragma unroll
         for (int j = 0; j < 32; ++j) ov[j] = 0.f;
       }
-      if (gg < G) {
+      if (gg < G && tk < n_tok) {
         // (16-byte units XOR-swizzled by 16 * (head & 1) + token)
 #pragma unroll
         for (int j = 0; j < 32; j += 4)
@@ -614,7 +615,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
     }
     tc_fence_before();
     if (nsplit > 1) {
-      if (gg < G) {
+      if (gg < G && tk < n_tok) {
         const uint32_t at = base + L::kQ + ml_off + (uint32_t)((split * G + gg) * tok_per + (tk - owner * tok_per)) * 8u;
         if (owner == split) *reinterpret_cast<float2*>(gbase + (at - base)) = make_float2(m_run, l_run);
         else st_async_f2(map_shared_rank(at, (uint32_t)owner), make_float2(m_run, l_run), map_shared_rank(bar_recv, (uint32_t)owner));
@@ -625,7 +626,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
       const int o = lane >> 1, g = 2 * warp + (lane & 1);
       if (o < nsplit && o != split && g < G) {
         const int n = tokens_of(o), first = o * tok_per, src = g * theirs + (first < split * tok_per ? first : first - my_tok);
-        bulk_to_peer(map_shared_rank(base + L::kQ + (uint32_t)((split * G + g) * tok_per) * kRowBytes, (uint32_t)o),
+        if (n > 0) bulk_to_peer(map_shared_rank(base + L::kQ + (uint32_t)((split * G + g) * tok_per) * kRowBytes, (uint32_t)o),
                      staged_at(src), (uint32_t)(n * kRowBytes), map_shared_rank(bar_recv, (uint32_t)o));
       }
     }
@@ -634,6 +635,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
   {
     if (nsplit > 1 && !mbar_wait(bar_recv, 0, abort_flag)) *abort_flag = 1;
     __syncthreads();
+    if (nsplit > 1) cluster_arrive();   // this CTA has what it waited for
     VS_STAMP(bp, 2, 3);
     if (nsplit > 1) {
       // what each CTA's part of a row counts for, 2^(max_i - max) over the row's denominator: a thread per row, in place of the pairs
@@ -763,7 +765,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
   }
   // every CTA of the cluster has what it waited for: nobody's shared memory goes away while a copy may be reading it
   __syncwarp();
-  if (nsplit > 1) { cluster_arrive(); cluster_wait(); }
+  if (nsplit > 1) cluster_wait();
   tc_fence_before();
   __syncthreads();
   if (warp == kIssuerWarp) {
