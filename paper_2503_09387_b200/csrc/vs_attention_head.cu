@@ -1,4 +1,4 @@
-// Decode attention, one CTA per query head: the variant for one stream (see vs_attention.cu for the grouped one).  There
+// Decode attention, one CTA per query head: the variant for few streams (see vs_attention.cu for the grouped one).  There
 // the step is a chain of latencies -- a key range's scores, the merges, the store -- and 28 short chains beat four that do
 // seven heads each (11.5 against 13.1 us per layer of the 28-layer token step at the Qwen2-7B shape, bank 512); reading K and V once
 // per head costs nothing while they are few.

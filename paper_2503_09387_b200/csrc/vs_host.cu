@@ -230,18 +230,19 @@ int ensure_step_maps(vs_stream* h, int rows) {
   return VS_OK;
 }
 
-// CTAs to spread the key tiles of a row tile over (one cluster).  All clusters must be resident at once, with a little room for
-// the bank update's.  Cost in key tiles (about 1.7 us each when the CTA has its SM alone), fitted to frames, clips and questions of
+// CTAs to spread the key tiles of a row tile over (one cluster).  All must be resident at once, beside bank_ctas for the bank
+// update (39 of those behind 264 of 296 made a frame step of three streams 61 us a layer, not 50).  Cost in key tiles (about 1.7
+// us each when the CTA has its SM alone), fitted to frames, clips and questions of
 // 5 to 13 tiles: two CTAs an SM make a tile a tenth longer, a row tile's row stores cost three, shared by the CTAs of the
 // cluster, the exchange a half.  key_len[i]: segment lengths of the longest key axis among the listed entries.
-int attn_split(const vs_stream* h, const BatchParams& bp, const int* key_len, int n_len) {
+int attn_split(const vs_stream* h, const BatchParams& bp, const int* key_len, int n_len, int bank_ctas) {
   int key_tiles = 0;
   for (int i = 0; i < n_len; ++i) key_tiles += (key_len[i] + ATTN_KEY_BOX - 1) / ATTN_KEY_BOX;
   const long long row_ctas = (long long)((bp.rows_per_stream + 15) / 16) * h->dm.Hkv * bp.n_active;
   int best = 1;
   double cost = 1e30;
   for (int s = 1; s <= ATTN_MAX_SPLIT; ++s) {
-    if (s > 1 && (s > key_tiles || row_ctas * s > 2LL * h->n_sms || h->attn_clusters[s] < row_ctas + 4 ||
+    if (s > 1 && (s > key_tiles || row_ctas * s + bank_ctas > 2LL * h->n_sms || h->attn_clusters[s] < row_ctas + (bank_ctas + s - 1) / s ||
                   !prefill_attention_can_split(h->dm.D, h->dm.G, s))) continue;
     const double c = ((key_tiles + s - 1) / s) * (row_ctas * s > h->n_sms ? 1.1 : 1.0) + 3.0 / s + (s > 1 ? 0.5 : 0.0);
     if (c < cost) { cost = c; best = s; }
@@ -260,10 +261,12 @@ void seg_step(AttnSegment& sg, const CUtensorMap& k, const CUtensorMap& v, int k
 
 // Tiling of a linear layer: CTAs with 128 weight rows each and K cut into ksplit shares (few rows), or CTA pairs with 256
 // (many), and the token columns of a tile.  The choice minimises the clocks of the waves' main loops plus what their epilogues
-// add: a 64-element block of K costs a CTA the larger of its MMAs (tile_n columns, 2 clocks a column) and its operand
-// traffic from L2 at about 50 bytes a clock ((128 + tile_n) * 128 bytes, of a pair's CTA (128 + tile_n / 2) * 128).  The
-// epilogue of a tile costs about 4000 clocks, in a pair kernel only the last one counts; a K split 5000 more (partial tiles
-// through L2, a flag), and it needs its whole grid resident at once.
+// add.  The main loops run at the operands' rate from L2, about 47 bytes a clock of an SM (the MMAs need less: 2 clocks a token
+// column): a 64-element block of K is (128 + tile_n) * 128 bytes to a CTA, (128 + tile_n / 2) * 128 to a CTA of a pair.  A tile's
+// epilogue costs 900 clocks and 14 a column, in a pair kernel only the last one counts, with 3100 clocks for the longer start;
+// a K split 1000 and 3.5 a column more (partial tiles through L2, a flag), and it needs its whole grid resident at once.
+// Fitted to whole steps of 17 to 1280 rows at the shapes of two backbones, K 1024 to 18944: the chosen tiling is 0.3 % slower
+// than the best one on average (a split costed at 5000 clocks whatever its tile left 1.2 %, at K = 18944 and 480 rows 10 %).
 struct Tiling { int tile_n, n_tiles, ksplit; bool pairs; };
 Tiling choose_tiles(int K, int E, int n_sms, int max_pairs, int rows, bool own_rope) {
   const int kb = K / GEMM_BLOCK_K, resident = n_sms < GEMM_XCHG_CTAS ? n_sms : GEMM_XCHG_CTAS;
@@ -274,18 +277,19 @@ Tiling choose_tiles(int K, int E, int n_sms, int max_pairs, int rows, bool own_r
     const int tn = ((rows + nt - 1) / nt + 15) / 16 * 16;
     if ((long long)(nt - 1) * tn >= rows && nt > nt_min) continue;      // an empty last tile
     if (tn < 64 && nt > nt_min) break;
-    auto block = [&](int tn_own) { const double mma = 2.0 * tn, l2 = (128 + tn_own) * 2.56; return mma > l2 ? mma : l2; };
+    auto block = [&](int tn_own) { return (128 + tn_own) * 2.7; };
+    const double epilogue = 900.0 + 14.0 * tn;
     const int mt1 = (E + GEMM_BLOCK_M - 1) / GEMM_BLOCK_M, mt2 = (E + 2 * GEMM_BLOCK_M - 1) / (2 * GEMM_BLOCK_M);
     for (int ks = 1; ks <= KSPLIT_MAX && ks <= kb; ++ks) {
       const long long ctas = (long long)mt1 * nt * ks;
       if (ks > 1 && ctas > resident) break;
       const long long waves = (ctas + n_sms - 1) / n_sms;
-      const double cost = waves * (block(tn) * ((kb + ks - 1) / ks) + 4000.0) + (ks > 1 ? 5000.0 : 0.0);
+      const double cost = waves * (block(tn) * ((kb + ks - 1) / ks) + epilogue) + (ks > 1 ? 1000.0 + 3.5 * tn : 0.0);
       if (best < 0 || cost < best) { best = cost; t = {tn, nt, ks, false}; }
     }
     if (own_rope) continue;                                              // (the pair kernel reads a table)
     const long long items = (long long)mt2 * nt, waves = (items + max_pairs - 1) / max_pairs;
-    const double cost = waves * (block(tn / 2) * kb + 500.0) + 4500.0;
+    const double cost = waves * (block(tn / 2) * kb + 100.0) + epilogue + 3100.0;
     if (best < 0 || cost < best) { best = cost; t = {tn, nt, 1, true}; }
   }
   return t;
@@ -418,13 +422,14 @@ size_t layer_stride_tail(const Dims& D) { return (size_t)D.S * D.Hkv * D.maxT * 
 // without the head; at 16 the slabs leave the ring too few stages, 344 -> 362).  Attention alone: steps of several tokens up to
 // 16 rows (28 layers: 589 -> 474 for 2 rows, 783 -> 559 for 16; 32 rows 770 -> 842) and single tokens of more streams than the
 // matrix-vector kernel takes (545 -> 460 for 8, 588 -> 517 for 16), in a stack; one to four single tokens are faster by launches
-// (352 against 463: 11 us a layer is little more than the phases' own synchronisation).  And not where a layer's projection holds
+// (352 against 463: 11 us a layer is little more than the phases' own synchronisation), and so are two to four rows in a single
+// layer (17.7 against 19.4).  And not where a layer's projection holds
 // less than 16 KB for every SM: there is then no weight stream to hide that synchronisation behind.
 bool token_step_pays(const vs_stream* h, int n_active, int T, int matrix_rows, bool full) {
   const int rows = n_active * T;
   if (h->n_sms > TOK_MAX_CTAS || (size_t)matrix_rows * h->dm.d * 2 < (size_t)h->n_sms * 16384) return false;
   if (full) return rows <= 8;
-  return rows <= TOK_MAX_ROWS && (T > 1 || (rows > 4 && h->dm.L > 1));
+  return rows <= TOK_MAX_ROWS && (T > 1) + (rows > 4) + (h->dm.L > 1) >= 2;
 }
 
 // what every launch of the token-step kernel gets
@@ -729,14 +734,6 @@ int vs_frame_prefill(vs_stream* h, const int32_t* stream_ids, int32_t n_active, 
       aa.h_in = nullptr; aa.h_out = nullptr; aa.ss_out = nullptr; aa.next_gain = nullptr; aa.xn_out = nullptr;
     }
     aa.free_slot = h->at<int32_t>(lo.step_slot); aa.free_slot_stride = 1;
-    {
-      int kl[3] = {0, 0, N + 1};
-      for (int i = 0; i < n_active; ++i) {
-        const int bl = D.M == 0 ? 0 : (bp.count[i] == D.M ? D.M + 1 : bp.count[i]);
-        if (bp.prefix_len[i] + bl > kl[0] + kl[1]) { kl[0] = bp.prefix_len[i]; kl[1] = bl; }
-      }
-      aa.nsplit = attn_split(h, bp, kl, 3);
-    }
     // the bank update (Section 3.3, memory mechanism: evict if full, then append) rides in the attention launches: each layer's
     // scores a share of the bank, the last one's commits.  Five rows to a CTA (a row per warp) while the CTAs are few; at most one
     // CTA for every two SMs, or for every SM where the attention comes in waves anyway: scoring is fp64 arithmetic and runs
@@ -744,11 +741,21 @@ int vs_frame_prefill(vs_stream* h, const int32_t* stream_ids, int32_t n_active, 
     if (any_full || last) {
       aa.bank = ba;
       aa.bank.j0 = (int)((int64_t)D.M * l / D.L); aa.bank.j1 = (int)((int64_t)D.M * (l + 1) / D.L); aa.bank.commit = last ? 1 : 0;
-      const int n_rows = aa.bank.j1 - aa.bank.j0, attn_ctas = (N + 16) / 16 * aa.nsplit * D.Hkv * n_active;
-      const int most = (attn_ctas > 2 * h->n_sms ? h->n_sms : h->n_sms / 2) / n_active;
+      const int n_rows = aa.bank.j1 - aa.bank.j0, most = ((N + 16) / 16 * D.Hkv * n_active > 2 * h->n_sms ? h->n_sms : h->n_sms / 2) / n_active;
       int ctas = (n_rows + 4) / 5;
       if (ctas > most) ctas = most;
       aa.bank_ctas = !any_full || ctas < 1 ? 1 : ctas;
+    }
+    {
+      int kl[3] = {0, 0, N + 1};
+      for (int i = 0; i < n_active; ++i) {
+        const int bl = D.M == 0 ? 0 : (bp.count[i] == D.M ? D.M + 1 : bp.count[i]);
+        if (bp.prefix_len[i] + bl > kl[0] + kl[1]) { kl[0] = bp.prefix_len[i]; kl[1] = bl; }
+      }
+      aa.nsplit = attn_split(h, bp, kl, 3, aa.bank_ctas * n_active);
+    }
+    if (aa.bank_ctas > 0) {
+      const int attn_ctas = (N + 16) / 16 * aa.nsplit * D.Hkv * n_active;
       aa.bank_grid = (aa.bank_ctas * n_active + aa.nsplit - 1) / aa.nsplit * aa.nsplit;
       // few of them start first (their chain is as long as the attention's); many would take slots that the attention's clusters
       // need (a bank of 1024 carriers: 48 against 42 us a frame step) and come behind as many attention CTAs as run at once
@@ -959,7 +966,7 @@ int vs_frame_prefill_chunk(vs_stream* h, int32_t stream_id, const void* hidden, 
       aa.chunk_mode = 1; aa.chunk_count0 = count0; aa.chunk_victim = chunk_victim;
       {
         const int kl[4] = {bp.prefix_len[0], D.M == 0 ? 0 : l1, D.M == 0 ? 0 : F - 1, N + 1};
-        aa.nsplit = attn_split(h, bp, kl, 4);
+        aa.nsplit = attn_split(h, bp, kl, 4, 0);
       }
       aa.Hq = D.Hq; aa.Hkv = D.Hkv; aa.D = D.D; aa.slots = D.slots; aa.M = D.M;
       aa.scale_log2e = (float)(1.4426950408889634 / std::sqrt((double)D.D));
@@ -1060,7 +1067,7 @@ int vs_bank_forward(vs_stream* h, int32_t stream_id, void* out, void* cuda_strea
     aa.Hq = D.Hq; aa.Hkv = D.Hkv; aa.D = D.D; aa.slots = D.slots; aa.M = 0;      // no bank segment on this key axis
     {
       const int kl[2] = {bp.prefix_len[0], rows};
-      aa.nsplit = attn_split(h, bp, kl, 2);
+      aa.nsplit = attn_split(h, bp, kl, 2, 0);
     }
     aa.scale_log2e = (float)(1.4426950408889634 / std::sqrt((double)D.D));
     VS_LAUNCH(h, st, KC_PREFILL_ATTN, launch_prefill_attention_tc(aa, bp, h->at<int>(lo.status), st));
@@ -1191,17 +1198,19 @@ int vs_decode_step(vs_stream* h, const int32_t* stream_ids, int32_t n_active, co
       if (D.d_ff > 0) { da.out = h->at<void>(lo.obuf); da.out_fp32 = 0; da.h_in = nullptr; da.h_out = nullptr; }
       da.meta = meta;
       da.Hq = D.Hq; da.Hkv = D.Hkv; da.D = D.D; da.slots = D.slots; da.M = D.M; da.maxP = D.maxP; da.maxT = D.maxT;
-      // one stream: a CTA per query head, more: per KV head (K and V read once per group)
-      const bool by_head = n_active == 1;
-      int ns = 1;
+      // A CTA per query head, or per KV head (K and V read once per group).  The first for one stream, and for two to four in large
+      // groups where all its CTAs, two to an SM, run at once: its chains are shorter (two streams of 250 keys: 96 against 110 us
+      // for 8 layers at the Qwen2-7B shape, groups of seven; of 640 keys, more CTAs than that: 135 against 109; groups of four: 61
+      // either way or 8 % slower).  There short contexts are written by the CTA directly, longer ones split over a cluster of 2, 4
+      // or 8 CTAs (a CTA then walks about 64 to 128 keys)
+      int ns = (max_keys <= 96) ? 1 : (max_keys <= 192 ? 2 : (max_keys <= 448 ? 4 : 8));
+      const bool by_head = n_active == 1 || (n_active <= 4 && D.G > 4 && (long long)ns * D.Hq * n_active <= 2LL * h->n_sms);
       if (by_head) {
-        // short contexts: the CTA writes the row directly; longer ones are split over a cluster of 2, 4 or 8 CTAs (a CTA
-        // then walks about 64 to 128 keys), fewer when the streams already fill the GPU
-        ns = (max_keys <= 96) ? 1 : (max_keys <= 192 ? 2 : (max_keys <= 448 ? 4 : 8));
         while (ns > 1 && (long long)ns * D.Hq * n_active > 4LL * h->n_sms) ns >>= 1;
       } else {
         // a CTA's eight warps take 128 keys in one go: split the axis over a cluster of 2, 4 or 8 CTAs down to that,
         // as long as all CTAs (two to an SM) run at once
+        ns = 1;
         while (ns < DEC_SPLIT_MAX && max_keys > 128 * ns && 2LL * ns * D.Hkv * n_active <= 2LL * h->n_sms) ns <<= 1;
       }
       da.nsplit = ns;
@@ -1227,7 +1236,7 @@ int vs_decode_step(vs_stream* h, const int32_t* stream_ids, int32_t n_active, co
           const int tl = to_prefix ? 0 : bp.text_len[i];
           if (bp.prefix_len[i] + bl + tl > kl[0] + kl[1] + kl[2]) { kl[0] = bp.prefix_len[i]; kl[1] = bl; kl[2] = tl; }
         }
-        aa.nsplit = attn_split(h, bp, kl, 4);
+        aa.nsplit = attn_split(h, bp, kl, 4, 0);
       }
       aa.out = (l == D.L - 1) ? out : (D.residual ? nullptr : h->at<void>(lo.obuf));
       aa.out_fp32 = D.out_fp32;
