@@ -175,6 +175,84 @@ __device__ __forceinline__ void staged_scores(const BankUpdateArgs& a, const Bat
   asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
+// Scores bank rows j0 .. j1 - 1 against their successors (policy 1; the last one's is the incoming carrier): a warp takes four
+// neighbours and the row behind them, so that a row is read, widened and squared once for the two scores it has a part in (a
+// score at a time: twice the conversions, and their latency bare -- a frame step with a bank of 22 rows took 65 us, not 56).
+// Rows stream through shared memory as above; same sums in the same order as warp_dot_norms.
+constexpr int kAdjWarpBytes = (kScoreRows + 1) * kScoreStages * kScoreChunk * 2;
+__device__ __forceinline__ void staged_adjacent_scores(const BankUpdateArgs& a, const BatchParams& bp, const bf16* emb, const int32_t* order,
+                                                       const bf16* emb_in, double* scores, int block, int n_blocks, int j1, int count, uint8_t* smem,
+                                                       int n_warps) {
+  constexpr int R = kScoreRows + 1;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, d = a.d;
+  if (warp >= n_warps) return;
+  uint8_t* ring = smem + (size_t)warp * kAdjWarpBytes;                       // [stage][row][512]
+  const int n_chunks = (d + kScoreChunk - 1) / kScoreChunk;
+#pragma unroll 1
+  for (int j = a.j0 + (warp * n_blocks + block) * kScoreRows; j < j1; j += n_blocks * n_warps * kScoreRows) {
+    const bf16* src[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) src[r] = j + r > j1 ? nullptr : (j + r < count ? emb + (size_t)order[j + r] * d : emb_in);
+    auto fetch = [&](int c) {
+      if (c < n_chunks) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          if (src[r] == nullptr) continue;
+          uint8_t* dst = ring + ((c % kScoreStages) * R + r) * (kScoreChunk * 2);
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const int k = c * kScoreChunk + (lane + 32 * i) * 8;
+            if (k < d) bank_cp_async16(dst + (lane + 32 * i) * 16, src[r] + k);
+          }
+        }
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+#pragma unroll 1
+    for (int c = 0; c < kScoreStages - 1; ++c) fetch(c);
+    double dot[kScoreRows], sq[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) { sq[r] = 0.0; if (r < kScoreRows) dot[r] = 0.0; }
+#pragma unroll 1
+    for (int c = 0; c < n_chunks; ++c) {
+      fetch(c + kScoreStages - 1);                     // into the stage that was read a chunk ago
+      asm volatile("cp.async.wait_group %0;" ::"n"(kScoreStages - 1) : "memory");
+      __syncwarp();
+      const unsigned short* xs = reinterpret_cast<const unsigned short*>(ring + (c % kScoreStages) * R * (kScoreChunk * 2)) + lane;
+      const int n = min(kScoreChunk, d - c * kScoreChunk);
+#pragma unroll 1
+      for (int k = 0; k < n; k += 64) {                // (n is a multiple of 64)
+        unsigned short xr[2][R];
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+          for (int r = 0; r < R; ++r) xr[i][r] = xs[r * kScoreChunk + k + 32 * i];    // (a row that does not exist: whatever lies there)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          double x[R];
+#pragma unroll
+          for (int r = 0; r < R; ++r) { x[r] = (double)__uint_as_float((uint32_t)xr[i][r] << 16); sq[r] = __fma_rn(x[r], x[r], sq[r]); }
+#pragma unroll
+          for (int r = 0; r < kScoreRows; ++r) dot[r] = __fma_rn(x[r], x[r + 1], dot[r]);
+        }
+      }
+      __syncwarp();
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) sq[r] = warp_tree_sum(sq[r]);
+#pragma unroll 1
+    for (int r = 0; r < kScoreRows; ++r) {
+      if (j + r >= j1) break;                          // uniform over the warp
+      const double sc = cosine_of(warp_tree_sum(dot[0]), sq[0], sq[1]);
+      if (lane == 0 && VS_STORE_OK(bp, DR_SCORES, scores + j + r, 8)) scores[j + r] = sc;
+      // (the next row's sums move up: registers are not indexed)
+      dot[0] = dot[1]; dot[1] = dot[2]; dot[2] = dot[3];
+      sq[0] = sq[1]; sq[1] = sq[2]; sq[2] = sq[3]; sq[3] = sq[4];
+    }
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
 // One of the `n_blocks` thread blocks (any number of them, whole warps) that update the bank of listed stream b.
 // scratch: 16-byte aligned shared memory, at least bank_scratch_bytes(NT); the more, the more rows are staged.
 // Bank not full: block 0 appends; the other blocks return.
@@ -229,8 +307,11 @@ __device__ __forceinline__ void bank_update_block(const BankUpdateArgs& a, const
   // ---- bank full: score, then the last block commits --------------------------------------
   double* scores = a.scores + (size_t)sid * a.slots;
   const int lane = tid & 31;
-  const int j1 = min(a.j1, count), staged = a.policy == 0 ? staged_warps(a.d, scratch_bytes) : 0;
-  if (staged > 0) {
+  const int j1 = min(a.j1, count);
+  const int staged = a.policy == 0 ? staged_warps(a.d, scratch_bytes) : (a.policy == 1 ? min((int)scratch_bytes / kAdjWarpBytes, (int)blockDim.x >> 5) : 0);
+  if (staged > 0 && a.policy == 1) {
+    staged_adjacent_scores(a, bp, a.emb + (size_t)sid * a.slots * a.d, order, emb_in, scores, block, n_blocks, j1, count, static_cast<uint8_t*>(scratch), staged);
+  } else if (staged > 0) {
     staged_scores(a, bp, a.emb + (size_t)sid * a.slots * a.d, order, emb_in, scores, block, n_blocks, j1, static_cast<uint8_t*>(scratch), staged);
   } else if (a.policy != 2) {
     const int n_warps = (int)blockDim.x >> 5;

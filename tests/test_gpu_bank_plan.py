@@ -24,3 +24,16 @@ def test_chunks_across_the_fill_of_the_bank(M, policy):
     assert p.ora[0].evictions == w.n_frames - M
     p.text([0], [w.decode_hidden(0)], "decode")
     p.close()
+
+
+@pytest.mark.parametrize("M,L,heads", [(1, 1, 2), (2, 1, 9), (4, 2, 9), (5, 1, 17), (13, 2, 9), (140, 1, 9)])
+def test_neighbours_scored_in_groups(M, L, heads):
+    w = synth.workload("long" if L == 1 else "deep", n_layers=L, d_model=64 * heads, n_q_heads=heads, n_kv_heads=1 if heads < 9 else heads, head_dim=64, tokens_per_frame=3,
+                       n_frames=M + 9, bank_capacity=M, prefix_len=2, question_len=0, decode_tokens=0, frame_model="iid", seed=53)
+    p = Pair(w, evict_policy=1)
+    p.text([0], [w.prefix_hidden()], "prefix")
+    for t in range(w.n_frames):
+        p.frame([0], [w.frame_hidden(t)], f"frame {t}", mode="full" if L > 1 or t + 3 > w.n_frames else "carrier")
+        if t + 1 >= M:
+            p.check_bank(0)
+    p.close()
