@@ -178,9 +178,10 @@ __device__ __forceinline__ void staged_scores(const BankUpdateArgs& a, const Bat
 // Scores bank rows j0 .. j1 - 1 against their successors (policy 1; the last one's is the incoming carrier): a warp takes four
 // neighbours and the row behind them, so that a row is read, widened and squared once for the two scores it has a part in (a
 // score at a time: twice the conversions, and their latency bare -- a frame step with a bank of 22 rows took 65 us, not 56).
-// Rows stream through shared memory as above; same sums in the same order as warp_dot_norms.
+// Rows stream through shared memory as above; same sums in the same order as warp_dot_norms.  (Out of line: inlined, it cost the
+// attention kernel's own code 2 %.)
 constexpr int kAdjWarpBytes = (kScoreRows + 1) * kScoreStages * kScoreChunk * 2;
-__device__ __forceinline__ void staged_adjacent_scores(const BankUpdateArgs& a, const BatchParams& bp, const bf16* emb, const int32_t* order,
+static __device__ __noinline__ void staged_adjacent_scores(const BankUpdateArgs& a, const BatchParams& bp, const bf16* emb, const int32_t* order,
                                                        const bf16* emb_in, double* scores, int block, int n_blocks, int j1, int count, uint8_t* smem,
                                                        int n_warps) {
   constexpr int R = kScoreRows + 1;
