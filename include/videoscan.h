@@ -21,8 +21,8 @@
  *    VS_ERR_DEVICE_TIMEOUT in a device status word that vs_bank_state reports.
  *    A handle that has reported it holds unspecified state: destroy it.
  *  - The projection of a step whose K split spans several thread blocks lets those
- *    blocks wait for one another, which needs all of them on the GPU at once: a
- *    handle expects the whole GPU while a step runs.  In particular the steps of two
+ *    blocks wait for one another, and so does the persistent kernel that takes steps of
+ *    a few token rows, which needs all of them on the GPU at once: a handle expects the whole GPU while a step runs.  In particular the steps of two
  *    handles on one GPU must not overlap (same stream, or ordered by events): two such
  *    projections holding half the SMs each would wait for blocks that cannot start,
  *    and both would end with VS_ERR_DEVICE_TIMEOUT.

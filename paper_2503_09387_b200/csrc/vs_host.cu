@@ -1,9 +1,9 @@
 // Host layer of the C ABI: argument checks, workspace carve-up, launch sequencing.
-// Per frame (Section 3.3, prefilling): pool -> per layer [norm] -> QKV GEMM (epilogue: RoPE,
-// carrier K/V into the bank's free slot) -> attention [-> residual] -> bank update (eviction
-// scoring when the bank is full, then append).  Per text step (Section 3.3, decoding): RoPE
-// table -> per layer [norm] -> GEMM (epilogue: K/V appended to prefix or tail) -> attention.  Nothing here allocates device memory or synchronises, except
-// create / bank_state / last_step_kv.
+// Per frame (Section 3.3, prefilling): pool -> per layer QKV GEMM (epilogue: RoPE, carrier K/V into the bank's free slot) ->
+// attention [-> residual, the next layer's norm], in whose launches spare CTAs update the bank (eviction scoring when it is full,
+// then append) [-> W_o -> gate and up -> W_down].  Per text step (Section 3.3, decoding): one persistent kernel for a few rows, else
+// [RoPE table ->] per layer GEMM or matrix-vector kernel (epilogue: K/V appended to prefix or tail) -> attention [-> the rest].
+// Nothing here allocates device memory or synchronises, except create / bank_state / last_step_kv.
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
