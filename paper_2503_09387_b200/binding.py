@@ -119,9 +119,12 @@ def _check(code: int, what: str) -> None:
         raise VsError(code, what)
 
 
+_id_arrays = {n: C.c_int32 * n for n in range(65)}       # (making the type takes longer than filling an array of it)
+
+
 def _ids(stream_ids: Sequence[int]):
-    arr = (C.c_int32 * len(stream_ids))(*stream_ids)
-    return arr, len(stream_ids)
+    n = len(stream_ids)
+    return (_id_arrays.get(n) or C.c_int32 * n)(*stream_ids), n
 
 
 # ---- C-named entry points (thin) ----------------------------------------------------------
@@ -280,6 +283,7 @@ class StreamBatch:
         self.torch = torch
         self.cfg = cfg
         self.device = torch.device("cuda", cfg.device)
+        self.device_index = int(cfg.device)
         self.weights = [w.contiguous() for w in weights]
         self.biases = biases
         self.norm_weights = norm_weights
@@ -302,7 +306,8 @@ class StreamBatch:
         self.out_torch_dtype = torch.float32 if cfg.out_dtype == 1 else torch.bfloat16
 
     def _stream(self) -> int:
-        return self.torch.cuda.current_stream(self.device).cuda_stream
+        # (current_stream(device).cuda_stream without the Stream object: a token step of one layer is bound by the host)
+        return self.torch._C._cuda_getCurrentRawStream(self.device_index)
 
     def lm_head(self, hidden, logits=None, want_token=True):
         """hidden: [rows, d_model] of the handle's output dtype -> (logits fp32 [rows, vocab], next tokens int32 [rows] or None)."""
