@@ -212,6 +212,36 @@ struct Smem {
   static_assert(2 * (kTotal + 1024) <= 228 * 1024, "two CTAs an SM");
 };
 
+// Where a row tile's rows lie in the shared memory of CTA `split` of its cluster once the CTA's key tiles are done: byte offsets.
+// The tile has n_tok tokens; CTA s finishes tokens s * tok_per ..., tok_per of them or what is left (without a cluster: all, 16 places).
+template <int D>
+struct Exchange {
+  int G, nsplit, n_tok, split, tok_per, my_tok;
+  static constexpr int kRowBytes = D * 4;
+  __host__ __device__ Exchange(int group, int nsplit_, int n_tok_, int split_)
+      : G(group), nsplit(nsplit_), n_tok(n_tok_), split(split_), tok_per(nsplit_ == 1 ? kTok : (n_tok_ + nsplit_ - 1) / nsplit_) { my_tok = tokens_of(split_); }
+  __host__ __device__ int tokens_of(int s) const {      // (none, perhaps)
+    const int n = n_tok - s * tok_per;
+    return n < 0 ? 0 : (n < tok_per ? n : tok_per);
+  }
+  // a row that this CTA finishes, as CTA s left it: where the query was; behind them their (max, denominator) pairs
+  __host__ __device__ int rows() const { return nsplit * G * tok_per; }
+  __host__ __device__ uint32_t row(int s, int g, int tl) const { return (uint32_t)(Smem<D>::kQ + ((s * G + g) * tok_per + tl) * kRowBytes); }
+  __host__ __device__ uint32_t pair(int s, int g, int tl) const { return (uint32_t)(Smem<D>::kQ + rows() * kRowBytes + ((s * G + g) * tok_per + tl) * 8); }
+  // row `i` of those that are on their way to the peers, which may be read until the cluster's last barrier: the ring, the few that
+  // it has no room for behind the pairs
+  static constexpr int ring_rows() { return Smem<D>::kRingRows; }
+  __host__ __device__ int staged_rows() const { return nsplit == 1 ? 0 : G * (n_tok - my_tok); }
+  __host__ __device__ uint32_t staged(int i) const {
+    return (uint32_t)(i < Smem<D>::kRingRows ? Smem<D>::kRing + i * kRowBytes : Smem<D>::kQ + rows() * (kRowBytes + 8) + (i - Smem<D>::kRingRows) * kRowBytes);
+  }
+  // sum of squares of a stored residual row: behind the residual input in the ring; in a cluster, where the ring holds rows on their
+  // way, the dead half of the row's first pair (a pair's denominator has gone into the weight that stands in its first half)
+  __host__ __device__ uint32_t sum_of_squares(int g, int tl) const {
+    return nsplit == 1 ? (uint32_t)(Smem<D>::kRing + kRows * D * 2 + (g * kTok + tl) * 4) : pair(0, g, tl) + 4u;
+  }
+};
+
 template <int D>
 __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const __grid_constant__ AttnArgs a,
                                                                           const __grid_constant__ BatchParams bp, int* status) {
@@ -555,13 +585,9 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
   // ---- rows out -----------------------------------------------------------------------------------------------
   constexpr int F4 = D / 4, kWarps = kAttnThreads / 32, kRowBytes = D * 4;
   const int n_tok = min(kTok, rps - r0);                              // tokens of this row tile
-  const int tok_per = (n_tok + nsplit - 1) / nsplit;                  // CTA s of the cluster finishes tokens s * tok_per ...
-  const int n_recv = nsplit * G * tok_per;                            // rows that find a place where the query was: [CTA][head][token]
-  const uint32_t ml_off = (uint32_t)n_recv * kRowBytes;               // ... behind them their (max, denominator) pairs
-  auto tokens_of = [&](int s) { return max(min(tok_per, n_tok - s * tok_per), 0); };   // ... this many of them (none, perhaps)
-  const int my_tok = tokens_of(split), my_rows = 8 * my_tok;          // row j: head j & 7 of token j >> 3
+  const Exchange<D> ex(G, nsplit, n_tok, split);
+  const int tok_per = ex.tok_per, my_tok = ex.my_tok, my_rows = 8 * my_tok;   // row j: head j & 7 of token j >> 3
   uint8_t* res_s = gbase + L::kRing;                                  // [row j][D] bf16: residual input of the rows (the ring is dead by now)
-  float* ss_stage = reinterpret_cast<float*>(gbase + L::kRing + (nsplit == 1 ? 128 * D * 2 : 0));   // [8 heads][16 tokens] sums of squares of stored residual rows
   VS_STAMP(bp, 2, 2);               // this CTA's tiles done
   __syncwarp();
   if (warp < 4 && a.h_out != nullptr && nsplit == 1) {
@@ -580,10 +606,6 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
     if (tid == 0) mbar_arrive_expect_tx(bar_recv, (uint32_t)((nsplit - 1) * G * my_tok * (kRowBytes + 8)));
     cluster_wait();                 // every peer's query is dead, and its barriers exist
   }
-  // place of a staged row: the ring, the few that it has no room for behind the pairs
-  auto staged_at = [&](int i) {
-    return base + (i < L::kRingRows ? L::kRing + (uint32_t)i * kRowBytes : L::kQ + ml_off + (uint32_t)n_recv * 8u + (uint32_t)(i - L::kRingRows) * kRowBytes);
-  };
   if (warp < 4) {
     // Every thread's row: into this CTA's own area if it finishes the row (with 1 / denominator if there are no peers), else staged
     // in the ring, from where it goes to the owner by bulk copies -- the rows of an owner's tokens lie side by side for every
@@ -591,9 +613,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
     const int gg = tid >> 4, tk = tid & 15, owner = nsplit == 1 ? 0 : tk / tok_per;
     const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
     const int theirs = n_tok - my_tok;                                // tokens of others, in order, numbered round this CTA's own
-    const int idx = nsplit == 1 ? tid : (owner == split ? (split * G + gg) * tok_per + (tk - owner * tok_per)
-                                                        : gg * theirs + (tk < split * tok_per ? tk : tk - my_tok));
-    const uint32_t dst = owner == split ? base + L::kQ + (uint32_t)idx * kRowBytes : staged_at(idx);
+    const uint32_t dst = base + (owner == split ? ex.row(split, gg, tk - owner * tok_per) : ex.staged(gg * theirs + (tk < split * tok_per ? tk : tk - my_tok)));
     const float inv = nsplit > 1 ? 1.f : ((l_run > 0.f) ? 1.f / l_run : 0.f);
 #pragma unroll 1
     for (int c = 0; c < D; c += 32) {
@@ -616,7 +636,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
     tc_fence_before();
     if (nsplit > 1) {
       if (gg < G && tk < n_tok) {
-        const uint32_t at = base + L::kQ + ml_off + (uint32_t)((split * G + gg) * tok_per + (tk - owner * tok_per)) * 8u;
+        const uint32_t at = base + ex.pair(split, gg, tk - owner * tok_per);
         if (owner == split) *reinterpret_cast<float2*>(gbase + (at - base)) = make_float2(m_run, l_run);
         else st_async_f2(map_shared_rank(at, (uint32_t)owner), make_float2(m_run, l_run), map_shared_rank(bar_recv, (uint32_t)owner));
       }
@@ -625,9 +645,9 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
       __syncwarp();
       const int o = lane >> 1, g = 2 * warp + (lane & 1);
       if (o < nsplit && o != split && g < G) {
-        const int n = tokens_of(o), first = o * tok_per, src = g * theirs + (first < split * tok_per ? first : first - my_tok);
-        if (n > 0) bulk_to_peer(map_shared_rank(base + L::kQ + (uint32_t)((split * G + g) * tok_per) * kRowBytes, (uint32_t)o),
-                     staged_at(src), (uint32_t)(n * kRowBytes), map_shared_rank(bar_recv, (uint32_t)o));
+        const int n = ex.tokens_of(o), first = o * tok_per, src = g * theirs + (first < split * tok_per ? first : first - my_tok);
+        if (n > 0) bulk_to_peer(map_shared_rank(base + ex.row(split, g, 0), (uint32_t)o), base + ex.staged(src), (uint32_t)(n * kRowBytes),
+                                map_shared_rank(bar_recv, (uint32_t)o));
       }
     }
     cp_async_wait<0>();
@@ -639,7 +659,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
     VS_STAMP(bp, 2, 3);
     if (nsplit > 1) {
       // what each CTA's part of a row counts for, 2^(max_i - max) over the row's denominator: a thread per row, in place of the pairs
-      float2* mlp = reinterpret_cast<float2*>(gbase + L::kQ + ml_off);
+      float2* mlp = reinterpret_cast<float2*>(gbase + ex.pair(0, 0, 0));
       for (int i = tid; i < my_rows; i += kAttnThreads) {
         const int tl = i >> 3, gg = i & 7;
         if (gg >= G) continue;
@@ -691,12 +711,12 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
 #pragma unroll
       for (int i = 0; i < NV; ++i) v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (valid) {
-        const uint8_t* row0 = gbase + L::kQ + (size_t)(nsplit == 1 ? gg * 16 + tl : gg * tok_per + tl) * kRowBytes;
+        const uint8_t* row0 = gbase + ex.row(0, gg, tl);
         if (nsplit == 1) {
 #pragma unroll
           for (int i = 0; i < NV; ++i) v[i] = *reinterpret_cast<const float4*>(row0 + (((u + 16 * i) ^ sw) * 16));
         } else {
-          const float2* mlp = reinterpret_cast<const float2*>(gbase + L::kQ + ml_off) + gg * tok_per + tl;
+          const float2* mlp = reinterpret_cast<const float2*>(gbase + ex.pair(0, gg, tl));
 #pragma unroll 2
           for (int s = 0; s < nsplit; ++s) {
             const float w = mlp[s * G * tok_per].x;
@@ -748,7 +768,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
       if (a.ss_out != nullptr) {
 #pragma unroll
         for (int o = 8; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-        if (u == 0 && valid) ss_stage[gg * 16 + tk] = ss;
+        if (u == 0 && valid) *reinterpret_cast<float*>(gbase + ex.sum_of_squares(gg, tl)) = ss;
       }
     }
     if (a.ss_out != nullptr) {
@@ -757,7 +777,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
       __syncthreads();
       if (tid < kTok && tid / tok_per == split && r0 + tid < rps) {
         float tot = 0.f;
-        for (int gg = 0; gg < G; ++gg) tot += ss_stage[gg * 16 + tid];
+        for (int gg = 0; gg < G; ++gg) tot += *reinterpret_cast<const float*>(gbase + ex.sum_of_squares(gg, tid - split * tok_per));
         float* sp = a.ss_out + ((size_t)b * rps + r0 + tid) * a.Hkv + hkv;
         if (VS_STORE_OK(bp, DR_ROW_SS, sp, 4)) *sp = tot;
       }
@@ -787,6 +807,24 @@ cudaError_t prefill_attention_tc_init() {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k[i], cudaFuncAttributePreferredSharedMemoryCarveout, 100);   // two CTAs an SM
   }
   return e;
+}
+
+// The byte ranges of the above in CTA `split`, as (begin, end) pairs for a check on the host: its rows and their pairs, the rows on
+// their way to the peers (the ring's, those behind the pairs), its sums of squares; the end of the query's place and of all.
+void prefill_attention_ranges(int head_dim, int group, int nsplit, int n_tok, int split, int32_t* r) {
+  auto fill = [&](auto ex, int q_end, int total) {
+    const int n = ex.staged_rows(), in_ring = n < ex.ring_rows() ? n : ex.ring_rows(), last = ex.my_tok - 1;
+    const int row = ex.kRowBytes, none = 0;
+    const bool own = ex.my_tok > 0;
+    const int v[] = {own ? (int)ex.row(0, 0, 0) : none, own ? (int)ex.row(nsplit - 1, group - 1, last) + row : none,
+                     own ? (int)ex.pair(0, 0, 0) : none, own ? (int)ex.pair(nsplit - 1, group - 1, last) + 8 : none,
+                     in_ring > 0 ? (int)ex.staged(0) : none, in_ring > 0 ? (int)ex.staged(in_ring - 1) + row : none,
+                     n > in_ring ? (int)ex.staged(in_ring) : none, n > in_ring ? (int)ex.staged(n - 1) + row : none,
+                     own ? (int)ex.sum_of_squares(0, 0) : none, own ? (int)ex.sum_of_squares(group - 1, last) + 4 : none, q_end, total};
+    for (int i = 0; i < 12; ++i) r[i] = v[i];
+  };
+  if (head_dim == 128) fill(Exchange<128>(group, nsplit, n_tok, split), 2 * Smem<128>::kQBytes, Smem<128>::kTotal);
+  else fill(Exchange<64>(group, nsplit, n_tok, split), 2 * Smem<64>::kQBytes, Smem<64>::kTotal);
 }
 
 // Whether `nsplit` CTAs can share a row tile's keys: the rows they leave one another have to fit where the query was, those on
