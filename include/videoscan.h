@@ -100,7 +100,8 @@ typedef struct {
                                     E_out = (Hq + 2*Hkv) * D, rows ordered Q heads, K heads, V heads;
                                     16-byte aligned                                                  */
   const void* const* b_qkv;      /* [n_layers] each [E_out], or NULL (whole array or any entry)      */
-  const void* const* norm_w;     /* [n_layers] each [d_model] RMSNorm gain, or NULL = all ones       */
+  const void* const* norm_w;     /* [n_layers] each [d_model] RMSNorm gain, or NULL = all ones; keep it
+                                    16-byte aligned (some step sizes load it that way)               */
   /* the rest of the decoder block, read only when d_ff > 0 (all "out x in", row-major, 16-byte aligned):
    *   h1 = h + A W_o^T (A: the layer's attention rows),  h2 = h1 + (SiLU(n W_gate^T) * (n W_up^T)) W_down^T,
    *   n = RMSNorm(h1) when use_rmsnorm.  A step's `out` then receives the last layer's h2 ([..][d_model]). */
@@ -147,15 +148,15 @@ int vs_create_stream(const vs_config* cfg, const vs_weights* weights,
  *   then the carrier's K/V of every layer enters the bank (evicting first when the bank is
  *   full) and everything else of the frame is dropped.
  * stream_ids: HOST [n_active], distinct ids in [0, n_streams).
- * hidden:     DEVICE bf16 [n_active][N][d_model].
+ * hidden:     DEVICE bf16 [n_active][N][d_model], 16-byte aligned.
  * carrier_override: DEVICE bf16 [n_active][d_model] used as the carrier token instead of
  *             the mean (e.g. projector(mean) computed by the caller), or NULL.
- * out:        DEVICE [n_active][N+1][Hq*D] of `out_dtype`, last layer's attention output, row N
- *             being the carrier's; may be NULL.  On a handle with d_ff > 0: the hidden state that
+ * out:        DEVICE [n_active][N+1][Hq*D] of `out_dtype`, 16-byte (fp32) or 8-byte (bf16) aligned: the
+ *             last layer's attention output, row N being the carrier's; may be NULL.  On a handle with d_ff > 0: the hidden state that
  *             leaves the last decoder block (Hq*D == d_model there), a bf16 storage point widened
  *             to `out_dtype`.
  * Errors: VS_ERR_STATE if a listed stream has an open text turn (call vs_end_turn first);
- *         VS_ERR_CAPACITY if N > max_tokens_per_frame. */
+ *         VS_ERR_CAPACITY if N > max_tokens_per_frame; VS_ERR_INVALID_ARG for a misaligned pointer. */
 int vs_frame_prefill(vs_stream* h, const int32_t* stream_ids, int32_t n_active,
                      const void* hidden, int32_t N, const void* carrier_override,
                      void* out, void* cuda_stream);
@@ -167,7 +168,7 @@ int vs_frame_prefill(vs_stream* h, const int32_t* stream_ids, int32_t n_active,
  * only at carrier embeddings, which are all known once the frames are pooled.  Per layer the
  * Q/K/V projection of all F*(N+1) rows is one GEMM and the attention of all F frames is one launch
  * (each frame with its own view of the bank).
- * hidden: DEVICE bf16 [F][N][d_model];  out: DEVICE [F][N+1][Hq*D] of `out_dtype`, or NULL.
+ * hidden: DEVICE bf16 [F][N][d_model];  out: DEVICE [F][N+1][Hq*D] of `out_dtype`, or NULL; aligned as there.
  * The chunk's bank updates are enqueued on a stream that the handle owns, forked from and joined
  * back into `cuda_stream` by events, so that they run beside the projection; the handle's first
  * call of this function creates that stream and its two events (no device memory).
@@ -181,7 +182,8 @@ int vs_frame_prefill_chunk(vs_stream* h, int32_t stream_id, const void* hidden, 
  * the stored carrier embeddings of ONE stream, in temporal order, one token per frame at
  * positions prefix_len + i, go through the layers, each attending over the prompt prefix and the
  * carriers up to itself.  Reads the bank, changes nothing.
- * out: DEVICE [count][Hq*D] of `out_dtype` (count = carriers in the bank; vs_bank_state tells).
+ * out: DEVICE [count][Hq*D] of `out_dtype`, aligned as vs_frame_prefill's (count = carriers in the bank;
+ * vs_bank_state tells).
  * count = 0 is not an error: nothing is launched. */
 int vs_bank_forward(vs_stream* h, int32_t stream_id, void* out, void* cuda_stream);
 
@@ -190,9 +192,12 @@ int vs_bank_forward(vs_stream* h, int32_t stream_id, void* out, void* cuda_strea
  * itself]; no visual-token K/V exists any more.  Before a stream's first frame the tokens
  * extend the prompt prefix instead (the system instruction comes first, Section 3.3) and
  * stay for the life of the stream.
- * hidden: DEVICE bf16 [n_active][T][d_model];  out: DEVICE [n_active][T][Hq*D] of `out_dtype`.
+ * hidden: DEVICE bf16 [n_active][T][d_model], 16-byte aligned;  out: DEVICE [n_active][T][Hq*D] of
+ * `out_dtype`, 16-byte (fp32) or 8-byte (bf16) aligned.  With T = 1 and d_ff = 0 any element-aligned `out` will do
+ * (several streams are served faster when it is aligned as above).
  * All listed streams must be in the same phase (all before or all after their first frame).
- * Errors: VS_ERR_CAPACITY on prefix / tail overflow or T > max_step_tokens. */
+ * Errors: VS_ERR_CAPACITY on prefix / tail overflow or T > max_step_tokens; VS_ERR_INVALID_ARG for a
+ *         misaligned pointer. */
 int vs_decode_step(vs_stream* h, const int32_t* stream_ids, int32_t n_active,
                    const void* hidden, int32_t T, void* out, void* cuda_stream);
 

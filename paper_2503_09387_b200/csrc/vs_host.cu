@@ -435,6 +435,9 @@ bool token_step_pays(const vs_stream* h, int n_active, int T, int matrix_rows, b
   return rows <= TOK_MAX_ROWS && (T > 1) + (rows > 4) + (h->dm.L > 1) >= 2;
 }
 
+// Whether `p` can take a step's rows as most kernels store them, four elements at a time.
+bool takes_rows(const void* p, const Dims& D) { return (reinterpret_cast<uintptr_t>(p) & (D.out_fp32 ? 15u : 7u)) == 0; }
+
 // what every launch of the token-step kernel gets
 TokArgs token_args(vs_stream* h, const void* hidden, int rows) {
   const Dims& D = h->dm;
@@ -637,6 +640,7 @@ int vs_frame_prefill(vs_stream* h, const int32_t* stream_ids, int32_t n_active, 
   int rc = check_ids(h, stream_ids, n_active);
   if (rc != VS_OK) return rc;
   if (hidden == nullptr || N < 1) return VS_ERR_INVALID_ARG;
+  if ((reinterpret_cast<uintptr_t>(hidden) & 15u) != 0 || !takes_rows(out, h->dm)) return VS_ERR_INVALID_ARG;
   const Dims& D = h->dm;
   const Layout& lo = h->lo;
   if (N > D.maxN) return VS_ERR_CAPACITY;
@@ -790,7 +794,7 @@ int vs_frame_prefill_chunk(vs_stream* h, int32_t stream_id, const void* hidden, 
   int rc = check_ids(h, &stream_id, 1);
   if (rc != VS_OK) return rc;
   if (hidden == nullptr || N < 1 || F < 1) return VS_ERR_INVALID_ARG;
-  if ((reinterpret_cast<uintptr_t>(hidden) & 15u) != 0) return VS_ERR_INVALID_ARG;
+  if ((reinterpret_cast<uintptr_t>(hidden) & 15u) != 0 || !takes_rows(out, h->dm)) return VS_ERR_INVALID_ARG;
   const Dims& D = h->dm;
   const Layout& lo = h->lo;
   if (N > D.maxN || F > D.maxChunk) return VS_ERR_CAPACITY;
@@ -1007,7 +1011,7 @@ int vs_bank_forward(vs_stream* h, int32_t stream_id, void* out, void* cuda_strea
   const HostStream& hs = h->hs[stream_id];
   const int count = (int)(hs.frames_seen < D.M ? hs.frames_seen : D.M);
   if (count == 0) return VS_OK;
-  if (out == nullptr) return VS_ERR_INVALID_ARG;
+  if (out == nullptr || !takes_rows(out, D)) return VS_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   VS_CK(cudaSetDevice(h->device));
 
@@ -1093,6 +1097,11 @@ int vs_decode_step(vs_stream* h, const int32_t* stream_ids, int32_t n_active, co
   const Dims& D = h->dm;
   const Layout& lo = h->lo;
   if (T > D.maxStepT) return VS_ERR_CAPACITY;
+  // rows at any address: the persistent kernel stores a full layer's element by element, and so does the attention by query head,
+  // which takes a single token per stream
+  const bool wide = takes_rows(out, D);
+  const bool persistent = token_step_pays(h, n_active, T, D.E_out, D.d_ff > 0) && (wide || D.d_ff > 0);
+  if (!wide && !persistent && (T > 1 || D.d_ff > 0)) return VS_ERR_INVALID_ARG;
   const bool to_prefix = h->hs[stream_ids[0]].frames_seen == 0;
   for (int i = 0; i < n_active; ++i) {
     const HostStream& s = h->hs[stream_ids[i]];
@@ -1122,7 +1131,7 @@ int vs_decode_step(vs_stream* h, const int32_t* stream_ids, int32_t n_active, co
   const int rows = n_active * T;
   StreamMeta* meta = h->at<StreamMeta>(lo.meta);
 
-  if (token_step_pays(h, n_active, T, D.E_out, D.d_ff > 0)) {
+  if (persistent) {
     // a few rows: one persistent launch for all layers
     TokArgs ta = token_args(h, hidden, rows);
     ta.out = out;
@@ -1207,7 +1216,7 @@ int vs_decode_step(vs_stream* h, const int32_t* stream_ids, int32_t n_active, co
       // either way or 8 % slower).  There short contexts are written by the CTA directly, longer ones split over a cluster of 2, 4
       // or 8 CTAs (a CTA then walks about 64 to 128 keys)
       int ns = (max_keys <= 96) ? 1 : (max_keys <= 192 ? 2 : (max_keys <= 448 ? 4 : 8));
-      const bool by_head = n_active == 1 || (n_active <= 4 && D.G > 4 && (long long)ns * D.Hq * n_active <= 2LL * h->n_sms);
+      const bool by_head = n_active == 1 || !wide || (n_active <= 4 && D.G > 4 && (long long)ns * D.Hq * n_active <= 2LL * h->n_sms);
       if (by_head) {
         while (ns > 1 && (long long)ns * D.Hq * n_active > 4LL * h->n_sms) ns >>= 1;
       } else {

@@ -853,7 +853,7 @@ __global__ void __launch_bounds__(kThreads, 1) token_kernel(const __grid_constan
       const bf16* gain = (a.use_rmsnorm && !a.full && l + 1 < a.L) ? a.layers[l + 1].gain : nullptr;
       if (mine && a.residual && !a.full) {
         hr = __ldcg(reinterpret_cast<const uint2*>(layer_input(a, l) + off));
-        if (gain != nullptr) gw = *reinterpret_cast<const uint2*>(gain + (size_t)hkv * G * D + idx);
+        if (gain != nullptr) { const uint32_t* gp = reinterpret_cast<const uint32_t*>(gain + (size_t)hkv * G * D + idx); gw = make_uint2(gp[0], gp[1]); }   // (4-byte aligned, like every reader of a gain on this path)
       }
       const int n_used = min(n_tiles, kCW);
       if (warp < n_used) {
