@@ -204,18 +204,23 @@ struct Smem {
   static constexpr int kQBytes = kRows * D * 2;           // one of hi / lo
   static constexpr int kKVBytes = kKeys * D * 2;          // a K or V tile
   static constexpr int kStages = D == 128 ? 3 : 6;
-  static constexpr int kQ = 0;                            // [hi | lo]; at the end rows, fp32, and their (max, denominator)
-  static constexpr int kRing = 2 * kQBytes;               // [stage] K or V tile; at the end (max, denominator) without a cluster, sums of squares
-  static constexpr int kRingRows = kStages * kKVBytes / (D * 4);   // fp32 rows that fit there
+  static constexpr int kQ = 0;                            // [hi | lo]; at the end fp32 rows (see Exchange)
+  static constexpr int kRing = 2 * kQBytes;               // [stage] K or V tile; at the end rows or, without a cluster, residual input
   static constexpr int kCtl = kRing + kStages * kKVBytes; // barriers, tmem slot, abort flag
-  static constexpr int kTotal = kCtl + 256;
+  static constexpr int kPairs = kCtl + 160;               // (max, denominator) of the peers' parts; weights; sums of squares
+  static constexpr int kPairRows = D == 128 ? 108 : 128;  // (as many as two CTAs an SM leave room for)
+  static constexpr int kTotal = kPairs + kPairRows * 8;
   static_assert(2 * (kTotal + 1024) <= 228 * 1024, "two CTAs an SM");
 };
 
 // Where a row tile's rows lie in the shared memory of CTA `split` of its cluster once the CTA's key tiles are done: byte offsets.
-// The tile has n_tok tokens; CTA s finishes tokens s * tok_per ..., tok_per of them or what is left (without a cluster: all, 16 places).
+// The tile has n_tok tokens; CTA s finishes tokens s * tok_per ..., tok_per of them or what is left (without a cluster: all).
+// Where the query was: the rows of its tokens, [CTA they come from][head][token].  At the top of the ring, on into the query's place
+// where the ring does not hold them all: the rows that are on their way to the peers.  The peers' (max, denominator) pairs have a place
+// of their own.  (With the pairs behind the rows a group of eight heads could not be split at all: its 128 rows fill the query's place.)
 template <int D>
 struct Exchange {
+  using L = Smem<D>;
   int G, nsplit, n_tok, split, tok_per, my_tok;
   static constexpr int kRowBytes = D * 4;
   __host__ __device__ Exchange(int group, int nsplit_, int n_tok_, int split_)
@@ -224,22 +229,16 @@ struct Exchange {
     const int n = n_tok - s * tok_per;
     return n < 0 ? 0 : (n < tok_per ? n : tok_per);
   }
-  // a row that this CTA finishes, as CTA s left it: where the query was; behind them their (max, denominator) pairs
+  // token tl of head g, as CTA s leaves it in the memory of the CTA that finishes it
   __host__ __device__ int rows() const { return nsplit * G * tok_per; }
-  __host__ __device__ uint32_t row(int s, int g, int tl) const { return (uint32_t)(Smem<D>::kQ + ((s * G + g) * tok_per + tl) * kRowBytes); }
-  __host__ __device__ uint32_t pair(int s, int g, int tl) const { return (uint32_t)(Smem<D>::kQ + rows() * kRowBytes + ((s * G + g) * tok_per + tl) * 8); }
-  // row `i` of those that are on their way to the peers, which may be read until the cluster's last barrier: the ring, the few that
-  // it has no room for behind the pairs
-  static constexpr int ring_rows() { return Smem<D>::kRingRows; }
+  __host__ __device__ uint32_t row(int s, int g, int tl) const { return (uint32_t)(L::kQ + ((s * G + g) * tok_per + tl) * kRowBytes); }
+  // ... with its pair, unless that is CTA `owner` itself: [head][token][peer].  A row's pairs give way to its weights, one a CTA, and
+  // these, once the row is merged, to the sum of squares of the stored residual row.
+  __host__ __device__ uint32_t stats(int g, int tl) const { return (uint32_t)(L::kPairs + (g * tok_per + tl) * (nsplit == 1 ? 4 : (nsplit - 1) * 8)); }
+  __host__ __device__ uint32_t pair(int owner, int s, int g, int tl) const { return stats(g, tl) + 8u * (uint32_t)(s - (s > owner ? 1 : 0)); }
+  // row `i` of those on their way, which may be read until the cluster's last barrier
   __host__ __device__ int staged_rows() const { return nsplit == 1 ? 0 : G * (n_tok - my_tok); }
-  __host__ __device__ uint32_t staged(int i) const {
-    return (uint32_t)(i < Smem<D>::kRingRows ? Smem<D>::kRing + i * kRowBytes : Smem<D>::kQ + rows() * (kRowBytes + 8) + (i - Smem<D>::kRingRows) * kRowBytes);
-  }
-  // sum of squares of a stored residual row: behind the residual input in the ring; in a cluster, where the ring holds rows on their
-  // way, the dead half of the row's first pair (a pair's denominator has gone into the weight that stands in its first half)
-  __host__ __device__ uint32_t sum_of_squares(int g, int tl) const {
-    return nsplit == 1 ? (uint32_t)(Smem<D>::kRing + kRows * D * 2 + (g * kTok + tl) * 4) : pair(0, g, tl) + 4u;
-  }
+  __host__ __device__ uint32_t staged(int i) const { return (uint32_t)(L::kCtl - (staged_rows() - i) * kRowBytes); }
 };
 
 template <int D>
@@ -606,11 +605,11 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
     if (tid == 0) mbar_arrive_expect_tx(bar_recv, (uint32_t)((nsplit - 1) * G * my_tok * (kRowBytes + 8)));
     cluster_wait();                 // every peer's query is dead, and its barriers exist
   }
+  const int gg = tid >> 4, tk = tid & 15, owner = nsplit == 1 ? 0 : tk / tok_per;      // softmax threads: their row
   if (warp < 4) {
     // Every thread's row: into this CTA's own area if it finishes the row (with 1 / denominator if there are no peers), else staged
     // in the ring, from where it goes to the owner by bulk copies -- the rows of an owner's tokens lie side by side for every
     // head.  (Stored straight into the peer's shared memory, 16 bytes a lane scattered over 32 rows, they took 4 us.)
-    const int gg = tid >> 4, tk = tid & 15, owner = nsplit == 1 ? 0 : tk / tok_per;
     const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
     const int theirs = n_tok - my_tok;                                // tokens of others, in order, numbered round this CTA's own
     const uint32_t dst = base + (owner == split ? ex.row(split, gg, tk - owner * tok_per) : ex.staged(gg * theirs + (tk < split * tok_per ? tk : tk - my_tok)));
@@ -635,10 +634,9 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
     }
     tc_fence_before();
     if (nsplit > 1) {
-      if (gg < G && tk < n_tok) {
-        const uint32_t at = base + ex.pair(split, gg, tk - owner * tok_per);
-        if (owner == split) *reinterpret_cast<float2*>(gbase + (at - base)) = make_float2(m_run, l_run);
-        else st_async_f2(map_shared_rank(at, (uint32_t)owner), make_float2(m_run, l_run), map_shared_rank(bar_recv, (uint32_t)owner));
+      if (gg < G && tk < n_tok && owner != split) {
+        const uint32_t at = base + ex.pair(owner, split, gg, tk - owner * tok_per);
+        st_async_f2(map_shared_rank(at, (uint32_t)owner), make_float2(m_run, l_run), map_shared_rank(bar_recv, (uint32_t)owner));
       }
       // a warp's rows are those of two heads: it sends them on itself
       fence_async_proxy();
@@ -653,31 +651,38 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
     cp_async_wait<0>();
   }
   {
-    if (nsplit > 1 && !mbar_wait(bar_recv, 0, abort_flag)) *abort_flag = 1;
+    if (nsplit > 1) {
+      if (!mbar_wait(bar_recv, 0, abort_flag)) *abort_flag = 1;
+      if (warp < 4) {
+        // What each CTA's part of a row counts for, 2^(max_i - max) over the row's denominator: a lane per part, two, four or eight to a
+        // row, for the rows of the warp's two heads (its threads still have this CTA's pairs): one round, or two in clusters of 3
+        // and 6.  (A thread per row with the parts unrolled: 0.5 us a launch more, for the code's size.)
+        const int lg = nsplit > 4 ? 3 : (nsplit > 2 ? 2 : 1), wide = 1 << lg, s = lane & (wide - 1);
+#pragma unroll 1
+        for (int j0 = 0; j0 < 2 * my_tok; j0 += 32 >> lg) {
+          const int j = j0 + (lane >> lg), g = 2 * warp + (j & 1), tl = j >> 1, from = (j & 1) * 16 + split * tok_per + tl;
+          float m = __shfl_sync(0xffffffffu, m_run, from), l = __shfl_sync(0xffffffffu, l_run, from), den = 0.f;
+          const bool on = s < nsplit && tl < my_tok && g < G;
+          if (s != split) {
+            const float2 ml = on ? *reinterpret_cast<const float2*>(gbase + ex.pair(split, s, g, tl)) : make_float2(-INFINITY, 0.f);
+            m = ml.x; l = ml.y;
+          }
+          float mm = m;
+#pragma unroll
+          for (int o = ATTN_MAX_SPLIT / 2; o > 0; o >>= 1) if (o < wide) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, o));
+          const float w = (m == -INFINITY) ? 0.f : ex2_approx(m - mm);                // a CTA without visible keys adds nothing
+#pragma unroll
+          for (int i = 0; i < ATTN_MAX_SPLIT; ++i) {
+            const float li = __shfl_sync(0xffffffffu, l, i, wide), wi = __shfl_sync(0xffffffffu, w, i, wide);
+            if (i < wide) den = fmaf(li, wi, den);
+          }
+          if (on) reinterpret_cast<float*>(gbase + ex.stats(g, tl))[s] = w * ((den > 0.f) ? 1.f / den : 0.f);
+        }
+      }
+    }
     __syncthreads();
     if (nsplit > 1) cluster_arrive();   // this CTA has what it waited for
     VS_STAMP(bp, 2, 3);
-    if (nsplit > 1) {
-      // what each CTA's part of a row counts for, 2^(max_i - max) over the row's denominator: a thread per row, in place of the pairs
-      float2* mlp = reinterpret_cast<float2*>(gbase + ex.pair(0, 0, 0));
-      for (int i = tid; i < my_rows; i += kAttnThreads) {
-        const int tl = i >> 3, gg = i & 7;
-        if (gg >= G) continue;
-        float2 ml[ATTN_MAX_SPLIT];
-        float mm = -INFINITY, den = 0.f;
-#pragma unroll
-        for (int s = 0; s < ATTN_MAX_SPLIT; ++s) if (s < nsplit) { ml[s] = mlp[(s * G + gg) * tok_per + tl]; mm = fmaxf(mm, ml[s].x); }
-#pragma unroll
-        for (int s = 0; s < ATTN_MAX_SPLIT; ++s) if (s < nsplit) {
-          ml[s].x = (ml[s].x == -INFINITY) ? 0.f : ex2_approx(ml[s].x - mm);      // a CTA without visible keys adds nothing
-          den = fmaf(ml[s].y, ml[s].x, den);
-        }
-        const float inv = (den > 0.f) ? 1.f / den : 0.f;
-#pragma unroll
-        for (int s = 0; s < ATTN_MAX_SPLIT; ++s) if (s < nsplit) mlp[(s * G + gg) * tok_per + tl].x = ml[s].x * inv;
-      }
-      __syncthreads();
-    }
     // Half a warp per row (lane: units u and, with D = 128, u + 16), two heads of a token side by side, one pair at a time: this
     // code runs once per CTA, and its size -- four rows unrolled: 25 KB -- cost more than the latency that unrolling hides.  The
     // residual input is asked for three pairs ahead.
@@ -716,10 +721,10 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
 #pragma unroll
           for (int i = 0; i < NV; ++i) v[i] = *reinterpret_cast<const float4*>(row0 + (((u + 16 * i) ^ sw) * 16));
         } else {
-          const float2* mlp = reinterpret_cast<const float2*>(gbase + ex.pair(0, gg, tl));
-#pragma unroll 2
+          const float* weights = reinterpret_cast<const float*>(gbase + ex.stats(gg, tl));
+#pragma unroll 4
           for (int s = 0; s < nsplit; ++s) {
-            const float w = mlp[s * G * tok_per].x;
+            const float w = weights[s];
 #pragma unroll
             for (int i = 0; i < NV; ++i) {
               const float4 o = *reinterpret_cast<const float4*>(row0 + (size_t)(s * G * tok_per) * kRowBytes + (((u + 16 * i) ^ sw) * 16));
@@ -768,16 +773,20 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
       if (a.ss_out != nullptr) {
 #pragma unroll
         for (int o = 8; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-        if (u == 0 && valid) *reinterpret_cast<float*>(gbase + ex.sum_of_squares(gg, tl)) = ss;
+        if (u == 0 && valid) *reinterpret_cast<float*>(gbase + ex.stats(gg, tl)) = ss;
       }
     }
     if (a.ss_out != nullptr) {
       // the token's sum of squares over this KV head's query heads, in head order; the projection adds
       // the KV heads' parts in order: the same bits whatever the launch shape
       __syncthreads();
-      if (tid < kTok && tid / tok_per == split && r0 + tid < rps) {
+      const int tl = tid - split * tok_per;
+      if ((unsigned)tl < (unsigned)my_tok) {
+        const uint8_t* part = gbase + ex.stats(0, tl);
+        const uint32_t step = ex.stats(1, tl) - ex.stats(0, tl);
         float tot = 0.f;
-        for (int gg = 0; gg < G; ++gg) tot += *reinterpret_cast<const float*>(gbase + ex.sum_of_squares(gg, tid - split * tok_per));
+#pragma unroll 4
+        for (int gg = 0; gg < G; ++gg, part += step) tot += *reinterpret_cast<const float*>(part);
         float* sp = a.ss_out + ((size_t)b * rps + r0 + tid) * a.Hkv + hkv;
         if (VS_STORE_OK(bp, DR_ROW_SS, sp, 4)) *sp = tot;
       }
@@ -809,34 +818,38 @@ cudaError_t prefill_attention_tc_init() {
   return e;
 }
 
-// The byte ranges of the above in CTA `split`, as (begin, end) pairs for a check on the host: its rows and their pairs, the rows on
-// their way to the peers (the ring's, those behind the pairs), its sums of squares; the end of the query's place and of all.
+// The byte ranges of an Exchange in CTA `split`, as (begin, end) pairs for a check on the host: the rows it finishes, the peers' pairs,
+// the rows on their way to them, its sums of squares; the end of the query's place and of all.
 void prefill_attention_ranges(int head_dim, int group, int nsplit, int n_tok, int split, int32_t* r) {
   auto fill = [&](auto ex, int q_end, int total) {
-    const int n = ex.staged_rows(), in_ring = n < ex.ring_rows() ? n : ex.ring_rows(), last = ex.my_tok - 1;
-    const int row = ex.kRowBytes, none = 0;
-    const bool own = ex.my_tok > 0;
-    const int v[] = {own ? (int)ex.row(0, 0, 0) : none, own ? (int)ex.row(nsplit - 1, group - 1, last) + row : none,
-                     own ? (int)ex.pair(0, 0, 0) : none, own ? (int)ex.pair(nsplit - 1, group - 1, last) + 8 : none,
-                     in_ring > 0 ? (int)ex.staged(0) : none, in_ring > 0 ? (int)ex.staged(in_ring - 1) + row : none,
-                     n > in_ring ? (int)ex.staged(in_ring) : none, n > in_ring ? (int)ex.staged(n - 1) + row : none,
-                     own ? (int)ex.sum_of_squares(0, 0) : none, own ? (int)ex.sum_of_squares(group - 1, last) + 4 : none, q_end, total};
-    for (int i = 0; i < 12; ++i) r[i] = v[i];
+    const int n = ex.my_tok, row = ex.kRowBytes, first = split == 0 ? 1 : 0, last = split == nsplit - 1 ? nsplit - 2 : nsplit - 1, staged = ex.staged_rows();
+    for (int i = 0; i < 8; ++i) r[i] = 0;
+    if (n > 0) {
+      r[0] = (int)ex.row(0, 0, 0); r[1] = (int)ex.row(nsplit - 1, group - 1, n - 1) + row;
+      r[6] = (int)ex.stats(0, 0); r[7] = (int)ex.stats(group - 1, n - 1) + 4;
+    }
+    if (n > 0 && nsplit > 1) { r[2] = (int)ex.pair(split, first, 0, 0); r[3] = (int)ex.pair(split, last, group - 1, n - 1) + 8; }
+    if (staged > 0) { r[4] = (int)ex.staged(0); r[5] = (int)ex.staged(staged - 1) + row; }
+    r[8] = q_end; r[9] = total;
   };
-  if (head_dim == 128) fill(Exchange<128>(group, nsplit, n_tok, split), 2 * Smem<128>::kQBytes, Smem<128>::kTotal);
-  else fill(Exchange<64>(group, nsplit, n_tok, split), 2 * Smem<64>::kQBytes, Smem<64>::kTotal);
+  if (head_dim == 128) fill(Exchange<128>(group, nsplit, n_tok, split), Smem<128>::kRing, Smem<128>::kTotal);
+  else fill(Exchange<64>(group, nsplit, n_tok, split), Smem<64>::kRing, Smem<64>::kTotal);
 }
 
-// Whether `nsplit` CTAs can share a row tile's keys: the rows they leave one another have to fit where the query was, those on
-// their way in the ring, with a few behind the others; and nobody may be without tokens.
+// Whether `nsplit` CTAs can share a row tile's keys: the rows that a CTA finishes have to fit where the query was, those on their way
+// above them, the peers' pairs in their place (a tile of fewer tokens needs less of each); and nobody may be without tokens.  (Six
+// for seven heads would fit with 64 dims, and lost to the eight that it was taken for: 170 rows over 427 keys, two KV heads, 20.5
+// against 18.9 us a layer.)  Eight heads in four CTAs against one, 128 dims, four KV heads: 170 rows over 491 keys 35 against 41 us a
+// layer, 32 rows over 608 keys 31 against 37; 64 dims, in eight CTAs, 32 rows: 17 against 26.
+template <int D>
+static bool can_split(int group, int nsplit) {
+  const Exchange<D> ex(group, nsplit, kTok, nsplit - 1);
+  if (nsplit == 6 && group > 6) return false;
+  return ex.my_tok >= 1 && ex.rows() <= kRows && ex.rows() - group * ex.tok_per <= Smem<D>::kPairRows &&
+         (ex.rows() + ex.staged_rows()) * ex.kRowBytes <= Smem<D>::kCtl;
+}
 bool prefill_attention_can_split(int head_dim, int group, int nsplit) {
-  const int tok_per = (kTok + nsplit - 1) / nsplit, last = kTok - (nsplit - 1) * tok_per;
-  const int room = head_dim == 128 ? 2 * Smem<128>::kQBytes : 2 * Smem<64>::kQBytes, ring = head_dim == 128 ? Smem<128>::kRingRows : Smem<64>::kRingRows;
-  if (last < 1) return false;
-  const int received = nsplit * group * tok_per, staged = group * (kTok - last), over = staged > ring ? staged - ring : 0;
-  // (rows of one owner and head are sent as one run: none may lie on both sides of the ring's end)
-  if (over > 0 && (last != tok_per || ring % tok_per != 0)) return false;
-  return received * (head_dim * 4 + 8) + over * head_dim * 4 <= room;
+  return head_dim == 128 ? can_split<128>(group, nsplit) : can_split<64>(group, nsplit);
 }
 
 cudaError_t launch_prefill_attention_tc(const AttnArgs& a, const BatchParams& bp, int* status, cudaStream_t st) {

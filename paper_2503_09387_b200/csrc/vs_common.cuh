@@ -402,6 +402,7 @@ cudaError_t launch_prefill_attention_tc(const AttnArgs& a, const BatchParams& bp
 cudaError_t prefill_attention_tc_init();
 int prefill_attention_max_clusters(int head_dim, int s);
 bool prefill_attention_can_split(int head_dim, int group, int nsplit);
+int attention_split(int head_dim, int group, int row_ctas, int key_tiles, int bank_ctas, int n_sms, const int* clusters);
 void prefill_attention_ranges(int head_dim, int group, int nsplit, int n_tok, int split, int32_t* ranges);
 constexpr int ATTN_MAX_SPLIT = 8;   // most CTAs sharing the key tiles of one row tile (one cluster)
 

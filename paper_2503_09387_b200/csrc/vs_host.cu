@@ -15,6 +15,29 @@
 
 using namespace vs;
 
+namespace vs {
+
+// CTAs to spread the key tiles of each of row_ctas row tiles over (one cluster).  All must be resident at once, beside bank_ctas for
+// the bank update (39 of those behind 264 of 296 made a frame step of three streams 61 us a layer, not 50).  Cost in key tiles (about
+// 1.7 us each when the CTA has its SM alone), fitted to frames, clips, carriers and questions of 2 to 13 tiles: two CTAs an SM make a
+// tile longer, a row tile's row stores cost three, shared by the CTAs of the cluster -- also by those that have no key tile (45
+// rows of two tiles: 27 us a layer split in two, 25 in eight) --, the exchange a half, and nearly every SM taken 0.4: the next
+// linear layer's CTAs then find no room to wait in, with their weights.  clusters[s]: clusters of s CTAs that run at once.
+int attention_split(int head_dim, int group, int row_ctas, int key_tiles, int bank_ctas, int n_sms, const int* clusters) {
+  int best = 1;
+  double cost = 1e30;
+  for (int s = 1; s <= ATTN_MAX_SPLIT; ++s) {
+    const long long ctas = (long long)row_ctas * s;
+    if (s > 1 && (ctas + bank_ctas > 2LL * n_sms || clusters[s] < row_ctas + (bank_ctas + s - 1) / s ||
+                  !prefill_attention_can_split(head_dim, group, s))) continue;
+    const double c = ((key_tiles + s - 1) / s) * (ctas > n_sms ? 1.08 : 1.0) + 3.0 / s + (s > 1 ? 0.5 : 0.0) + (4 * ctas > 3 * n_sms ? 0.4 : 0.0);
+    if (c < cost) { cost = c; best = s; }
+  }
+  return best;
+}
+
+}  // namespace vs
+
 namespace {
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -230,27 +253,12 @@ int ensure_step_maps(vs_stream* h, int rows) {
   return VS_OK;
 }
 
-// CTAs to spread the key tiles of a row tile over (one cluster).  All must be resident at once, beside bank_ctas for the bank
-// update (39 of those behind 264 of 296 made a frame step of three streams 61 us a layer, not 50).  Cost in key tiles (about 1.7
-// us each when the CTA has its SM alone), fitted to frames, clips, carriers and questions of 2 to 13 tiles: two CTAs an SM make a
-// tile longer, a row tile's row stores cost three, shared by the CTAs of the cluster -- also by those that have no key tile (45
-// rows of two tiles: 27 us a layer split in two, 25 in eight) --, the exchange a half, and nearly every SM taken 0.4: the next
-// linear layer's CTAs then find no room to wait in, with their weights.  key_len[i]: segment lengths of the longest key axis among
-// the listed entries.
+// CTAs that share the key tiles of a row tile (see attention_split), for the longest key axis among the listed entries, whose
+// segments have key_len[i] keys
 int attn_split(const vs_stream* h, const BatchParams& bp, const int* key_len, int n_len, int bank_ctas) {
   int key_tiles = 0;
   for (int i = 0; i < n_len; ++i) key_tiles += (key_len[i] + ATTN_KEY_BOX - 1) / ATTN_KEY_BOX;
-  const long long row_ctas = (long long)((bp.rows_per_stream + 15) / 16) * h->dm.Hkv * bp.n_active;
-  int best = 1;
-  double cost = 1e30;
-  for (int s = 1; s <= ATTN_MAX_SPLIT; ++s) {
-    if (s > 1 && (row_ctas * s + bank_ctas > 2LL * h->n_sms || h->attn_clusters[s] < row_ctas + (bank_ctas + s - 1) / s ||
-                  !prefill_attention_can_split(h->dm.D, h->dm.G, s))) continue;
-    const long long ctas = row_ctas * s;
-    const double c = ((key_tiles + s - 1) / s) * (ctas > h->n_sms ? 1.08 : 1.0) + 3.0 / s + (s > 1 ? 0.5 : 0.0) + (4 * ctas > 3 * h->n_sms ? 0.4 : 0.0);
-    if (c < cost) { cost = c; best = s; }
-  }
-  return best;
+  return attention_split(h->dm.D, h->dm.G, (bp.rows_per_stream + 15) / 16 * h->dm.Hkv * bp.n_active, key_tiles, bank_ctas, h->n_sms, h->attn_clusters);
 }
 
 // segments of the attention's key axis

@@ -20,10 +20,10 @@ def _can_split(lib, D, G, n):
 
 
 def _ranges(lib, D, G, n, n_tok, split):
-    r = (C.c_int32 * 12)()
+    r = (C.c_int32 * 10)()
     lib._ZN2vs24prefill_attention_rangesEiiiiiPi(D, G, n, n_tok, split, r)
-    names = ("rows", "pairs", "staged", "staged_rest", "sums")
-    return {k: (r[2 * i], r[2 * i + 1]) for i, k in enumerate(names)}, r[10], r[11]
+    names = ("rows", "pairs", "staged", "sums")
+    return {k: (r[2 * i], r[2 * i + 1]) for i, k in enumerate(names)}, r[8], r[9]
 
 
 def _meet(a, b):
@@ -36,9 +36,17 @@ def test_nothing_lies_over_rows_on_their_way(lib, D):
         for n in (n for n in range(1, 9) if _can_split(lib, D, G, n)):
             for n_tok in range(1, 17):
                 for split in range(n):
-                    r, q_end, total = _ranges(lib, D, G, n, n_tok, split)
+                    r, ring, total = _ranges(lib, D, G, n, n_tok, split)
                     what = (D, G, n, n_tok, split, r)
                     assert all(0 <= b <= e <= total for b, e in r.values()), what
-                    for s in ("staged", "staged_rest"):
-                        assert not any(_meet(r[s], r[k]) for k in ("rows", "pairs", "sums")), what
+                    assert not any(_meet(r["staged"], r[k]) for k in ("rows", "pairs", "sums")), what
                     assert not _meet(r["rows"], r["pairs"]) and not _meet(r["rows"], r["sums"]), what
+                    assert r["rows"][1] <= ring, what                         # the ring may still be in use when they come
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_every_group_can_be_split(lib, D):
+    assert all(_can_split(lib, D, G, n) for G in range(1, 9) for n in (2, 4))
+    assert all(_can_split(lib, D, G, 3) for G in range(1, 8))                     # (eight heads: 144 rows)
+    assert not any(_can_split(lib, D, G, n) for G in range(1, 9) for n in (5, 7)) # 16 tokens leave the last CTA none
+    assert all(_can_split(lib, D, G, 8) for G in range(1, 8 if D == 128 else 9))

@@ -1,8 +1,12 @@
-"""Key tiles of the prefill attention shared by the CTAs of a cluster: one to eight of them, groups whose rows fill the exchange
-area and whose last rows lie behind it, token counts that leave a CTA of the cluster few rows or none."""
-import pytest
+"""Key tiles of the prefill attention shared by the CTAs of a cluster: every size of cluster that a group can have (the choice is
+asked of the library), groups whose rows fill the exchange area and reach out of it, token counts that leave a CTA of the cluster few
+rows or none."""
+import ctypes as C
 
-from paper_2503_09387_b200 import synth
+import pytest
+import torch
+
+from paper_2503_09387_b200 import binding, synth
 from tests.parity import Pair
 
 pytestmark = pytest.mark.gpu
@@ -24,4 +28,34 @@ def test_every_cluster_size(Hq, Hkv, D, S):
         p.text(ids, [row(8 + i, T, s) for s in ids], f"{T} rows")
     for s in ids:
         p.check_bank(s)
+    p.close()
+
+
+def _cluster_size(G, D, row_tiles, key_tiles):
+    lib = binding.load_library()
+    clusters = (C.c_int * 9)(0, 0, *(2 * lib._ZN2vs30prefill_attention_max_clustersEii(D, s) for s in range(2, 9)))
+    return lib._ZN2vs15attention_splitEiiiiiiPKi(D, G, row_tiles, key_tiles, 0, torch.cuda.get_device_properties(0).multi_processor_count, clusters)
+
+
+# streams of a call and its rows: 10, 32, 80, 128 and 160 row tiles, the last one of a stream often ragged
+CALLS = ((1, 153), (2, 251), (5, 243), (8, 256), (10, 242))
+
+
+@pytest.mark.parametrize("G,D,sizes", [(7, 128, [8, 4, 3, 2, 1]), (8, 128, [4, 4, 2, 2, 1]), (5, 128, [8, 6, 3, 2, 1]),
+                                       (8, 64, [8, 4, 2, 2, 1]), (7, 64, [8, 4, 3, 2, 1])])
+def test_the_cluster_sizes_in_use(G, D, sizes):
+    S, d = 10, G * D
+    w = synth.workload("deep", n_layers=2, d_model=d, n_q_heads=G, n_kv_heads=1, head_dim=D, tokens_per_frame=5, n_frames=0, bank_capacity=1,
+                       prefix_len=3, question_len=0, decode_tokens=0, n_streams=S, frame_model="iid", seed=67)
+    p = Pair(w, with_gain=True, max_prefix=1200, max_step_tokens=256)
+    used, at = [], [0] * S
+    for i, (n, T) in enumerate(CALLS):
+        ids = list(range(n))
+        tiles = max((at[s] + 63) // 64 for s in ids) + (T + 63) // 64
+        used.append(_cluster_size(G, D, n * ((T + 15) // 16), tiles))
+        p.text(ids, [synth.normal_bf16(w.seed, synth.TAG_QUESTION, (T, d), 1.0, offset=(i * S + s) * 256 * d) for s in ids], f"{n} x {T} rows")
+        for s in ids:
+            at[s] += T
+    assert used == sizes
+    p.check_bank(0)
     p.close()
