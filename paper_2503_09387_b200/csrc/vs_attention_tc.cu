@@ -654,30 +654,37 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
     if (nsplit > 1) {
       if (!mbar_wait(bar_recv, 0, abort_flag)) *abort_flag = 1;
       if (warp < 4) {
-        // What each CTA's part of a row counts for, 2^(max_i - max) over the row's denominator: a lane per part, two, four or eight to a
-        // row, for the rows of the warp's two heads (its threads still have this CTA's pairs): one round, or two in clusters of 3
-        // and 6.  (A thread per row with the parts unrolled: 0.5 us a launch more, for the code's size.)
-        const int lg = nsplit > 4 ? 3 : (nsplit > 2 ? 2 : 1), wide = 1 << lg, s = lane & (wide - 1);
-#pragma unroll 1
-        for (int j0 = 0; j0 < 2 * my_tok; j0 += 32 >> lg) {
-          const int j = j0 + (lane >> lg), g = 2 * warp + (j & 1), tl = j >> 1, from = (j & 1) * 16 + split * tok_per + tl;
-          float m = __shfl_sync(0xffffffffu, m_run, from), l = __shfl_sync(0xffffffffu, l_run, from), den = 0.f;
-          const bool on = s < nsplit && tl < my_tok && g < G;
-          if (s != split) {
-            const float2 ml = on ? *reinterpret_cast<const float2*>(gbase + ex.pair(split, s, g, tl)) : make_float2(-INFINITY, 0.f);
-            m = ml.x; l = ml.y;
-          }
-          float mm = m;
+        // What each CTA's part of a row counts for, 2^(max_i - max) over the row's denominator: two parts a lane (s and s + wide), so that
+        // the rows of the warp's two heads, whose threads still have this CTA's pairs, are done in one round.  (A thread per row, the
+        // parts unrolled: 0.5 us a launch more, for the code's size; a part a lane: as much in clusters of 3 and 6, for a second round.)
+        const int lg = nsplit > 4 ? 2 : (nsplit > 2 ? 1 : 0), wide = 1 << lg;
+        const int j = lane >> lg, g = 2 * warp + (j & 1), tl = j >> 1, from = (j & 1) * 16 + split * tok_per + tl;
+        const float m_own = __shfl_sync(0xffffffffu, m_run, from), l_own = __shfl_sync(0xffffffffu, l_run, from);
+        const bool row_on = tl < my_tok && g < G;
+        float2 ml[2];
+        float den = 0.f;
 #pragma unroll
-          for (int o = ATTN_MAX_SPLIT / 2; o > 0; o >>= 1) if (o < wide) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, o));
-          const float w = (m == -INFINITY) ? 0.f : ex2_approx(m - mm);                // a CTA without visible keys adds nothing
+        for (int k = 0; k < 2; ++k) {
+          const int s = (lane & (wide - 1)) + k * wide;
+          ml[k] = make_float2(m_own, l_own);
+          if (s != split) ml[k] = (row_on && s < nsplit) ? *reinterpret_cast<const float2*>(gbase + ex.pair(split, s, g, tl)) : make_float2(-INFINITY, 0.f);
+        }
+        float mm = fmaxf(ml[0].x, ml[1].x);
+        if (wide > 2) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, 2));
+        if (wide > 1) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, 1));
 #pragma unroll
-          for (int i = 0; i < ATTN_MAX_SPLIT; ++i) {
-            const float li = __shfl_sync(0xffffffffu, l, i, wide), wi = __shfl_sync(0xffffffffu, w, i, wide);
+        for (int k = 0; k < 2; ++k) ml[k].x = (ml[k].x == -INFINITY) ? 0.f : ex2_approx(ml[k].x - mm);      // a CTA without visible keys adds nothing
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float li = __shfl_sync(0xffffffffu, ml[k].y, i, wide), wi = __shfl_sync(0xffffffffu, ml[k].x, i, wide);
             if (i < wide) den = fmaf(li, wi, den);
           }
-          if (on) reinterpret_cast<float*>(gbase + ex.stats(g, tl))[s] = w * ((den > 0.f) ? 1.f / den : 0.f);
-        }
+        const float inv = (den > 0.f) ? 1.f / den : 0.f;
+        float* weights = reinterpret_cast<float*>(gbase + ex.stats(g, tl)) + (lane & (wide - 1));
+#pragma unroll
+        for (int k = 0; k < 2; ++k) if (row_on && (lane & (wide - 1)) + k * wide < nsplit) weights[k * wide] = ml[k].x * inv;
       }
     }
     __syncthreads();
