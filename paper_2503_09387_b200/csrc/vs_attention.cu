@@ -238,6 +238,7 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(DecodeArgs 
   __syncthreads();
 
   auto store_row = [&](float4 v) {
+    if (!VS_STORE_OK(bp, a.out_region, static_cast<uint8_t*>(a.out) + (out_off + my) * (a.out_fp32 ? 4 : 2), a.out_fp32 ? 16 : 8)) return;
     if (a.out_fp32) *reinterpret_cast<float4*>(static_cast<float*>(a.out) + out_off + my) = v;
     else *reinterpret_cast<uint2*>(static_cast<bf16*>(a.out) + out_off + my) = make_uint2(pack2(v.x, v.y), pack2(v.z, v.w));
     if (a.h_out != nullptr && VS_STORE_OK(bp, a.h_out_region, a.h_out + out_off + my, 8)) {

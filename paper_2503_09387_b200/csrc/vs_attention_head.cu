@@ -222,6 +222,7 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_head_kernel(Decode
     }
     if (direct) {
       const float val = (L > 0.f) ? O / L : 0.f;
+      if (!VS_STORE_OK(bp, a.out_region, static_cast<uint8_t*>(a.out) + (out_off + c) * (a.out_fp32 ? 4 : 2), a.out_fp32 ? 4 : 2)) return;
       if (a.out_fp32) static_cast<float*>(a.out)[out_off + c] = val;
       else static_cast<bf16*>(a.out)[out_off + c] = __float2bfloat16_rn(val);
       if (a.h_out != nullptr && VS_STORE_OK(bp, a.h_out_region, a.h_out + out_off + c, 2)) a.h_out[out_off + c] = __float2bfloat16_rn(h_res + val);
@@ -264,6 +265,7 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_head_kernel(Decode
       }
     }
     val = (L > 0.f) ? val / L : 0.f;
+    if (!VS_STORE_OK(bp, a.out_region, static_cast<uint8_t*>(a.out) + (out_off + c) * (a.out_fp32 ? 4 : 2), a.out_fp32 ? 4 : 2)) return;
     if (a.out_fp32) static_cast<float*>(a.out)[out_off + c] = val;
     else static_cast<bf16*>(a.out)[out_off + c] = __float2bfloat16_rn(val);
     if (a.h_out != nullptr && VS_STORE_OK(bp, a.h_out_region, a.h_out + out_off + c, 2)) a.h_out[out_off + c] = __float2bfloat16_rn(h_res + val);

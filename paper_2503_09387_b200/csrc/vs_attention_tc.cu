@@ -748,11 +748,11 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
         if (!valid) continue;
         if (a.out != nullptr) {                                        // (null: a layer whose rows only feed the residual stream)
           if (a.out_fp32) {
-            *reinterpret_cast<float4*>(static_cast<float*>(a.out) + obase) = v[i];
+            if (VS_STORE_OK(bp, a.out_region, static_cast<float*>(a.out) + obase, 16)) *reinterpret_cast<float4*>(static_cast<float*>(a.out) + obase) = v[i];
           } else {
             __nv_bfloat162 lo = __floats2bfloat162_rn(v[i].x, v[i].y), hi = __floats2bfloat162_rn(v[i].z, v[i].w);
             uint2 w; w.x = *reinterpret_cast<uint32_t*>(&lo); w.y = *reinterpret_cast<uint32_t*>(&hi);
-            *reinterpret_cast<uint2*>(static_cast<bf16*>(a.out) + obase) = w;
+            if (VS_STORE_OK(bp, a.out_region, static_cast<bf16*>(a.out) + obase, 8)) *reinterpret_cast<uint2*>(static_cast<bf16*>(a.out) + obase) = w;
           }
         }
         if (a.h_out != nullptr) {

@@ -269,9 +269,10 @@ __device__ __forceinline__ void bank_update_block(const BankUpdateArgs& a, const
   const bool on = tid < NT;
   const int sid = bp.stream_id[b];
   StreamMeta* meta = a.meta + sid;
+  const bool meta_ok = VS_STORE_OK(bp, DR_META, meta, sizeof(StreamMeta));
   if (!a.commit && (a.M == 0 || bp.count[b] < a.M)) return;           // nothing to score
   if (a.M == 0) {
-    if (block == 0 && tid == 0) { meta->frames_seen += 1; meta->last_victim_frame = -1; }
+    if (block == 0 && tid == 0 && meta_ok) { meta->frames_seen += 1; meta->last_victim_frame = -1; }
     return;
   }
   int32_t* order = a.order + (size_t)sid * a.slots;
@@ -288,7 +289,8 @@ __device__ __forceinline__ void bank_update_block(const BankUpdateArgs& a, const
       bf16* dst = const_cast<bf16*>(a.emb) + ((size_t)sid * a.slots + incoming) * a.d;
 #pragma unroll 1
       for (int k = tid; k < a.d; k += blockDim.x) if (VS_STORE_OK(bp, DR_EMB, dst + k, 2)) dst[k] = emb_in[k];
-      if (tid == 0) { a.record_slot[b] = incoming; a.record_victim[b] = -1; }
+      if (tid == 0 && VS_STORE_OK(bp, DR_CHUNK_SLOT, a.record_slot + b, 4)) a.record_slot[b] = incoming;
+      if (tid == 0 && VS_STORE_OK(bp, DR_CHUNK_VICTIM, a.record_victim + b, 4)) a.record_victim[b] = -1;
     }
   };
   const int64_t carrier_pos = bp.pos_base[b] + bp.rows_per_stream - 1;
@@ -298,10 +300,12 @@ __device__ __forceinline__ void bank_update_block(const BankUpdateArgs& a, const
       if (VS_STORE_OK(bp, DR_ORDER, order + count, 4)) order[count] = incoming;
       if (VS_STORE_OK(bp, DR_SLOT_FRAME, slot_frame + incoming, 4)) slot_frame[incoming] = (int32_t)bp.frame_id[b];
       if (VS_STORE_OK(bp, DR_SLOT_POS, slot_pos + incoming, 8)) slot_pos[incoming] = carrier_pos;
-      meta->count = count + 1;
-      meta->free_slot = count + 1;          // slots fill in order until the bank is full
-      meta->last_victim_frame = -1;
-      meta->frames_seen += 1;
+      if (meta_ok) {
+        meta->count = count + 1;
+        meta->free_slot = count + 1;        // slots fill in order until the bank is full
+        meta->last_victim_frame = -1;
+        meta->frames_seen += 1;
+      }
     }
     return;
   }
@@ -333,7 +337,7 @@ __device__ __forceinline__ void bank_update_block(const BankUpdateArgs& a, const
   int& is_last = best_j[NT];
   __threadfence();
   __syncthreads();
-  if (tid == 0) is_last = (atomicAdd(&meta->score_ticket, 1) == n_blocks - 1);
+  if (tid == 0) is_last = meta_ok && (atomicAdd(&meta->score_ticket, 1) == n_blocks - 1);
   __syncthreads();
   if (!is_last) return;
   __threadfence();
@@ -385,7 +389,7 @@ __device__ __forceinline__ void bank_update_block(const BankUpdateArgs& a, const
     meta->log_count += 1;
     meta->evictions += 1;
     meta->last_victim_frame = victim_frame;
-    if (a.incoming_emb != nullptr)
+    if (a.incoming_emb != nullptr && VS_STORE_OK(bp, DR_CHUNK_VICTIM, a.record_victim + b, 4))
       a.record_victim[b] = (victim_frame >= a.chunk_first_frame) ? a.chunk_l1 + (int)(victim_frame - a.chunk_first_frame)
                                                                  : victim_slot;
     meta->free_slot = victim_slot;

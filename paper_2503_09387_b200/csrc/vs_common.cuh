@@ -48,28 +48,34 @@ struct BatchParams {
 };
 
 // ---- checked stores (only in a -DVS_DEBUG_BOUNDS build; the product build compiles none of it) ----
-// Stand-in for a memory checker: every store of a kernel into the workspace names the region it
-// means to write; a store outside that region is skipped and the first one is recorded (region,
+// Stand-in for a memory checker: every store or atomic of a kernel into the workspace (but for the status word and
+// the scratch-poisoning test aid) names the region it means to write; a store outside that region is skipped and the first one is recorded (region,
 // byte offset from the region's start) -- no trap.  Behind every region lie 256 guard bytes that
 // vs_bank_state verifies.  Either finding is reported as VS_ERR_BOUNDS.
 enum DbgRegion { DR_BANK_K = 0, DR_BANK_V, DR_PREFIX_K, DR_PREFIX_V, DR_TAIL_K, DR_TAIL_V, DR_EMB, DR_META, DR_ORDER,
                  DR_SLOT_FRAME, DR_SLOT_POS, DR_EVICT_LOG, DR_SCORES, DR_STEP_SLOT, DR_CHUNK_SLOT, DR_CHUNK_VICTIM,
                  DR_GEMM_FLAGS, DR_HBUF0, DR_HBUF1, DR_XN, DR_ROW_SS, DR_Q, DR_Q_LO, DR_Q_TILED, DR_KF, DR_VF, DR_ROPE,
-                 DR_OBUF, DR_EMB_STAGE, DR_CHUNK_SCORES, DR_GEMM_XCHG, DR_ACT, DR_TOK, DR_COUNT };
+                 DR_OBUF, DR_EMB_STAGE, DR_CHUNK_SCORES, DR_GEMM_XCHG, DR_ACT, DR_TOK, DR_INV_FREQ, DR_STATUS, DR_TOK_LAYERS, DR_TOK_SYNC,
+                 DR_LM_KEYS, DR_LM_TICKETS, DR_COUNT };
 struct DebugTable {
   unsigned long long begin[DR_COUNT], end[DR_COUNT];   // device addresses
   int bad_region;                                      // -1, or the region of the first refused store
   long long bad_offset;
 };
+struct DebugRef {                                      // the table, for kernels that get no BatchParams
+#ifdef VS_DEBUG_BOUNDS
+  DebugTable* dbg;
+#endif
+};
 #if defined(VS_DEBUG_BOUNDS) && defined(__CUDACC__)
-__device__ __forceinline__ bool vs_store_ok(const BatchParams& bp, int region, const void* p, size_t bytes) {
-  if (bp.dbg == nullptr) return true;
+__device__ __forceinline__ bool vs_store_ok(DebugTable* dbg, int region, const void* p, size_t bytes) {
+  if (dbg == nullptr || region < 0) return true;
   const unsigned long long a = reinterpret_cast<unsigned long long>(p);
-  if (a >= bp.dbg->begin[region] && a + bytes <= bp.dbg->end[region]) return true;
-  if (atomicCAS(&bp.dbg->bad_region, -1, region) == -1) bp.dbg->bad_offset = (long long)(a - bp.dbg->begin[region]);
+  if (a >= dbg->begin[region] && a + bytes <= dbg->end[region]) return true;
+  if (atomicCAS(&dbg->bad_region, -1, region) == -1) dbg->bad_offset = (long long)(a - dbg->begin[region]);
   return false;
 }
-#define VS_STORE_OK(bp, region, p, bytes) vs_store_ok(bp, region, p, bytes)
+#define VS_STORE_OK(bp, region, p, bytes) vs_store_ok((bp).dbg, region, p, bytes)
 #else
 #define VS_STORE_OK(bp, region, p, bytes) true
 #endif
@@ -238,16 +244,16 @@ struct RopeArgs {
 cudaError_t launch_rope_table(const RopeArgs& a, const BatchParams& bp, cudaStream_t st);
 
 // sum of squares of every row -> row_ss[row][parts] (part 0; the other parts zero); with a gain vector hg = bf16(h * gain)
-cudaError_t launch_rms_stats(const bf16* h, const bf16* gain, bf16* hg, float* row_ss, int parts, int rows, int d,
+cudaError_t launch_rms_stats(const bf16* h, const bf16* gain, bf16* hg, float* row_ss, int parts, int rows, int d, DebugRef dr,
                              cudaStream_t st);
 // Input of the language-model head: xn[row] = bf16(h[row]) (times gain, rounded again, with a gain vector), the
 // sum of squares of bf16(h[row]) in part 0 of row_ss[row][parts].  h is fp32 or bf16.
 cudaError_t launch_lm_norm(const void* h, int h_fp32, const bf16* gain, bf16* xn, float* row_ss, int parts, int rows, int d,
-                           cudaStream_t st);
+                           DebugRef dr, cudaStream_t st);
 // token[row] = index of the largest of logits[row][0..vocab), the lowest index among equals, NaN below everything.
 // keys[rows] and tickets[rows] are scratch that is zero between calls (the kernel leaves it so).
 cudaError_t launch_argmax_rows(const float* logits, int32_t* token, unsigned long long* keys, int* tickets, int rows, int vocab,
-                               cudaStream_t st);
+                               DebugRef dr, cudaStream_t st);
 
 // What the projection epilogue writes (finished rows: bias, RoPE, bf16) and where rows persist.
 struct ProjectionOut {
@@ -354,6 +360,7 @@ struct AttnArgs {
   int n_seg;
   void* out;                     // [rows][Hq*D], bf16 or fp32
   int out_fp32;
+  int out_region;                // checked build: the workspace region that out lies in, or -1 (the caller's buffer)
   const bf16* h_in;              // residual input [rows][d] or null
   bf16* h_out;                   // residual output or null
   // RMSNorm of the layer that follows (needs h_out): the sum of squares of every stored residual row over this KV
@@ -395,6 +402,7 @@ struct ChunkKvCommitArgs {
   int F, N, Hkv, D, slots, sid, l1;
   const bf16* emb_stage; bf16* emb;        // last layer: parked embeddings [F][d] and where they go [S][slots][d]; else null
   int d;
+  DebugRef dr;
 };
 cudaError_t launch_chunk_kv_commit(const ChunkKvCommitArgs& a, cudaStream_t st);
 constexpr int ATTN_EXCL_BITS = 8192;   // most (bank slots + chunk frames) a chunk call takes
@@ -414,6 +422,7 @@ struct DecodeArgs {
   const bf16* tail_k;   const bf16* tail_v;    // [S][Hkv][maxT][D]
   void* out;                     // [n_active][Hq*D], bf16 or fp32
   int out_fp32;
+  int out_region;                // checked build: the workspace region that out lies in, or -1 (the caller's buffer)
   const bf16* h_in; bf16* h_out;
   int h_out_region;              // checked build: which residual buffer h_out is (DR_HBUF0 / DR_HBUF1)
   const StreamMeta* meta;
@@ -469,7 +478,7 @@ cudaError_t launch_token_step(const TokArgs& a, const BatchParams& bp, int n_sms
 
 // rows i < count of x = emb[sid][order[i]]: the bank's carrier embeddings in temporal order
 cudaError_t launch_gather_carriers(const bf16* emb, const int32_t* order, bf16* x, int sid, int slots, int d, int count,
-                                   cudaStream_t st);
+                                   DebugRef dr, cudaStream_t st);
 cudaError_t launch_poison(void* p, size_t bytes, cudaStream_t st);
 cudaError_t launch_reset(StreamMeta* meta, int32_t* slot_frame, int slots, const BatchParams& bp, cudaStream_t st);
 

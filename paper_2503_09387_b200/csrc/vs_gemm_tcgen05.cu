@@ -255,7 +255,8 @@ qkv_gemm_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant_
       // then orders them before the flag increments for whoever acquires a flag
       __threadfence();
       for (int s = 0; s < p.ksplit; ++s)
-        if (s != rank && first_block(s, n_blk, p.ksplit) < first_block(s + 1, n_blk, p.ksplit)) atomicAdd(p.flags + group * p.ksplit + s, 1);
+        if (s != rank && first_block(s, n_blk, p.ksplit) < first_block(s + 1, n_blk, p.ksplit) &&
+            VS_STORE_OK(bp, DR_GEMM_FLAGS, p.flags + group * p.ksplit + s, 4)) atomicAdd(p.flags + group * p.ksplit + s, 1);
     }
   }
   if (warp >= 2 && acc_ok) {
@@ -280,7 +281,7 @@ qkv_gemm_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant_
         else if (now - t0 > kWaitLimitNs) *abort_flag = 1;
       }
     }
-    *mine = 0;                                                 // next launch starts from zero
+    if (VS_STORE_OK(bp, DR_GEMM_FLAGS, mine, 4)) *mine = 0;                                                 // next launch starts from zero
   }
   tcgen05_fence_before();
   __syncthreads();

@@ -124,16 +124,16 @@ void fill_layout(const Dims& D, Layout& Lo) {
   Lo.slot_pos = reg(DR_SLOT_POS, take((size_t)D.S * D.slots * 8));
   Lo.evict_log = reg(DR_EVICT_LOG, take((size_t)D.S * (D.log_cap > 0 ? D.log_cap : 1) * 8));
   Lo.scores = reg(DR_SCORES, take((size_t)D.S * D.slots * 8));
-  Lo.inv_freq = take((size_t)(D.D / 2) * 8);
-  Lo.status = take(8 * 4);
+  Lo.inv_freq = reg(DR_INV_FREQ, take((size_t)(D.D / 2) * 8));
+  Lo.status = reg(DR_STATUS, take(8 * 4));
   Lo.step_slot = reg(DR_STEP_SLOT, take((size_t)D.S * 4));
   Lo.chunk_slot = reg(DR_CHUNK_SLOT, take((size_t)VS_MAX_BATCH * 4));
   Lo.chunk_victim = reg(DR_CHUNK_VICTIM, take((size_t)VS_MAX_BATCH * 4));
   Lo.gemm_flags = reg(DR_GEMM_FLAGS, take((size_t)GEMM_XCHG_CTAS * 4));
-  Lo.tok_layers = take((size_t)D.L * sizeof(TokLayer) + sizeof(CUtensorMap));
-  Lo.tok_sync = take(tok_sync_ints(D.L, D.Hkv) * 4);
-  Lo.lm_keys = take((size_t)256 * 8);          // language-model head: per-row argmax keys and tickets, zero between calls
-  Lo.lm_tickets = take((size_t)256 * 4);
+  Lo.tok_layers = reg(DR_TOK_LAYERS, take((size_t)D.L * sizeof(TokLayer) + sizeof(CUtensorMap)));
+  Lo.tok_sync = reg(DR_TOK_SYNC, take(tok_sync_ints(D.L, D.Hkv) * 4));
+  Lo.lm_keys = reg(DR_LM_KEYS, take((size_t)256 * 8));          // language-model head: per-row argmax keys and tickets, zero between calls
+  Lo.lm_tickets = reg(DR_LM_TICKETS, take((size_t)256 * 4));
   Lo.dbg_table = take(sizeof(DebugTable));
   Lo.persistent_end = off;
   Lo.scratch_begin = off;
@@ -329,6 +329,20 @@ int check_ids(vs_stream* h, const int32_t* ids, int32_t n) {
 #define VS_BP_INIT(h, bp) std::memset(&(bp), 0, sizeof(bp))
 #define VS_TRACE_NEXT(h, bp)
 #endif
+
+// checked build: whether a launch's rows go to the workspace
+int rows_region(const vs_stream* h, const void* out) { return out == h->ws + h->lo.obuf ? DR_OBUF : -1; }
+
+DebugRef debug_ref(const vs_stream* h) {
+  DebugRef r;
+  std::memset(&r, 0, sizeof(r));
+#ifdef VS_DEBUG_BOUNDS
+  r.dbg = h->at<DebugTable>(h->lo.dbg_table);
+#else
+  (void)h;
+#endif
+  return r;
+}
 
 #define VS_CK(expr) do { if ((expr) != cudaSuccess) return VS_ERR_CUDA; } while (0)
 
@@ -709,7 +723,7 @@ int vs_frame_prefill(vs_stream* h, const int32_t* stream_ids, int32_t n_active, 
     if (D.use_rmsnorm) {
       // layer 0: a launch of its own; deeper layers: the attention kernel that stored h_in left the statistics
       if (l == 0) VS_LAUNCH(h, st, KC_RMSNORM, launch_rms_stats(h_in, h->gain[l], h->at<bf16>(lo.xn), h->at<float>(lo.row_ss),
-                                                                D.ss_parts, rows, D.d, st));
+                                                                D.ss_parts, rows, D.d, debug_ref(h), st));
       if (h->gain[l] != nullptr) src = h->at<bf16>(lo.xn);
     }
     ProjectionOut fa;
@@ -779,6 +793,7 @@ int vs_frame_prefill(vs_stream* h, const int32_t* stream_ids, int32_t n_active, 
     }
     aa.Hq = D.Hq; aa.Hkv = D.Hkv; aa.D = D.D; aa.slots = D.slots; aa.M = D.M;
     aa.scale_log2e = (float)(1.4426950408889634 / std::sqrt((double)D.D));
+    aa.out_region = rows_region(h, aa.out);
     VS_LAUNCH(h, st, KC_PREFILL_ATTN, launch_prefill_attention_tc(aa, bp, h->at<int>(lo.status), st));
     if (D.d_ff > 0) {
       // h2 lands in hbuf[0] again: the layer input of every layer is hbuf[0]
@@ -934,7 +949,7 @@ int vs_frame_prefill_chunk(vs_stream* h, int32_t stream_id, const void* hidden, 
     if (D.use_rmsnorm) {
       // layer 0: a launch of its own; deeper layers: the attention kernel that stored h_in left the statistics
       if (l == 0) VS_LAUNCH(h, st, KC_RMSNORM, launch_rms_stats(h_in, h->gain[l], h->at<bf16>(lo.xn), h->at<float>(lo.row_ss),
-                                                                D.ss_parts, rows, D.d, st));
+                                                                D.ss_parts, rows, D.d, debug_ref(h), st));
       if (h->gain[l] != nullptr) src = h->at<bf16>(lo.xn);
     }
     ProjectionOut fa;
@@ -985,6 +1000,7 @@ int vs_frame_prefill_chunk(vs_stream* h, int32_t stream_id, const void* hidden, 
       }
       aa.Hq = D.Hq; aa.Hkv = D.Hkv; aa.D = D.D; aa.slots = D.slots; aa.M = D.M;
       aa.scale_log2e = (float)(1.4426950408889634 / std::sqrt((double)D.D));
+      aa.out_region = rows_region(h, aa.out);
       VS_LAUNCH(h, st, KC_PREFILL_ATTN, launch_prefill_attention_tc(aa, bp, h->at<int>(lo.status), st));
       if (D.M > 0) {
         ChunkKvCommitArgs ca;
@@ -993,6 +1009,7 @@ int vs_frame_prefill_chunk(vs_stream* h, int32_t stream_id, const void* hidden, 
         ca.F = F; ca.N = N; ca.Hkv = D.Hkv; ca.D = D.D; ca.slots = D.slots; ca.sid = stream_id; ca.l1 = l1;
         ca.emb_stage = h->at<bf16>(lo.emb_stage); ca.d = D.d;
         ca.emb = (last && planned) ? h->at<bf16>(lo.emb) : nullptr;
+        ca.dr = debug_ref(h);
         VS_LAUNCH(h, st, KC_OTHER, launch_chunk_kv_commit(ca, st));
       }
     }
@@ -1033,7 +1050,7 @@ int vs_bank_forward(vs_stream* h, int32_t stream_id, void* out, void* cuda_strea
   bp.pos_base[0] = hs.prefix_len;
   const int rows = count;
   VS_LAUNCH(h, st, KC_OTHER, launch_gather_carriers(h->at<bf16>(lo.emb), h->at<int32_t>(lo.order), h->at<bf16>(lo.hbuf[0]),
-                                                    stream_id, D.slots, D.d, count, st));
+                                                    stream_id, D.slots, D.d, count, debug_ref(h), st));
   RopeArgs ra;
   ra.inv_freq = h->at<double>(lo.inv_freq); ra.rope = h->at<float2>(lo.rope); ra.D = D.D;
   VS_LAUNCH(h, st, KC_ROPE, launch_rope_table(ra, bp, st));
@@ -1046,7 +1063,7 @@ int vs_bank_forward(vs_stream* h, int32_t stream_id, void* out, void* cuda_strea
     if (D.use_rmsnorm) {
       // layer 0: a launch of its own; deeper layers: the attention kernel that stored h_in left the statistics
       if (l == 0) VS_LAUNCH(h, st, KC_RMSNORM, launch_rms_stats(h_in, h->gain[l], h->at<bf16>(lo.xn), h->at<float>(lo.row_ss),
-                                                                D.ss_parts, rows, D.d, st));
+                                                                D.ss_parts, rows, D.d, debug_ref(h), st));
       if (h->gain[l] != nullptr) src = h->at<bf16>(lo.xn);
     }
     ProjectionOut fa;
@@ -1085,6 +1102,7 @@ int vs_bank_forward(vs_stream* h, int32_t stream_id, void* out, void* cuda_strea
       aa.nsplit = attn_split(h, bp, kl, 2, 0);
     }
     aa.scale_log2e = (float)(1.4426950408889634 / std::sqrt((double)D.D));
+    aa.out_region = rows_region(h, aa.out);
     VS_LAUNCH(h, st, KC_PREFILL_ATTN, launch_prefill_attention_tc(aa, bp, h->at<int>(lo.status), st));
     if (D.d_ff > 0) {
       rc = run_block_rest(h, l, rows, h_in, h->at<bf16>(lo.obuf), (l == D.L - 1) ? out : nullptr, bp, st);
@@ -1178,7 +1196,7 @@ int vs_decode_step(vs_stream* h, const int32_t* stream_ids, int32_t n_active, co
       // layer 0, and every layer of a single-token step (its attention kernel leaves no statistics): a launch of
       // its own; else the tensor-core attention that stored h_in left them
       if (l == 0 || (T == 1 && D.d_ff == 0)) VS_LAUNCH(h, st, KC_RMSNORM, launch_rms_stats(h_in, h->gain[l], h->at<bf16>(lo.xn), h->at<float>(lo.row_ss),
-                                                                          D.ss_parts, rows, D.d, st));
+                                                                          D.ss_parts, rows, D.d, debug_ref(h), st));
       if (h->gain[l] != nullptr) src = h->at<bf16>(lo.xn);
     }
     bf16* pk = h->at<bf16>(lo.prefix_k) + (size_t)l * layer_stride_prefix(D);
@@ -1236,6 +1254,7 @@ int vs_decode_step(vs_stream* h, const int32_t* stream_ids, int32_t n_active, co
       da.nsplit = ns;
       da.to_prefix = to_prefix ? 1 : 0;
       da.scale_log2e = scale_log2e;
+      da.out_region = rows_region(h, da.out);
       VS_LAUNCH(h, st, KC_DECODE_ATTN, by_head ? launch_decode_attention_heads(da, bp, st) : launch_decode_attention(da, bp, st));
     } else {
       AttnArgs aa;
@@ -1270,6 +1289,7 @@ int vs_decode_step(vs_stream* h, const int32_t* stream_ids, int32_t n_active, co
         aa.out = h->at<void>(lo.obuf); aa.out_fp32 = 0;
         aa.h_in = nullptr; aa.h_out = nullptr; aa.ss_out = nullptr; aa.next_gain = nullptr; aa.xn_out = nullptr;
       }
+      aa.out_region = rows_region(h, aa.out);
       VS_LAUNCH(h, st, KC_PREFILL_ATTN, launch_prefill_attention_tc(aa, bp, h->at<int>(lo.status), st));
     }
     if (D.d_ff > 0) {
@@ -1373,7 +1393,7 @@ int vs_lm_head(vs_stream* h, const void* hidden, int32_t rows, void* logits, int
     return VS_OK;
   }
   float* ss = h->at<float>(lo.row_ss);
-  VS_LAUNCH(h, st, KC_RMSNORM, launch_lm_norm(hidden, D.out_fp32, D.use_rmsnorm ? h->gain_f : nullptr, xn, ss, D.ss_parts, rows, D.d, st));
+  VS_LAUNCH(h, st, KC_RMSNORM, launch_lm_norm(hidden, D.out_fp32, D.use_rmsnorm ? h->gain_f : nullptr, xn, ss, D.ss_parts, rows, D.d, debug_ref(h), st));
   ProjectionOut po;
   std::memset(&po, 0, sizeof(po));
   po.mode = 6; po.final_out = logits; po.final_fp32 = 1;
@@ -1381,7 +1401,7 @@ int vs_lm_head(vs_stream* h, const void* hidden, int32_t rows, void* logits, int
   int rc = run_linear(h, h->tm_lm, h->tm_lm, xn, rows, D.d, D.vocab, po, bp, st);
   if (rc != VS_OK) return rc;
   if (next_token != nullptr) VS_LAUNCH(h, st, KC_OTHER, launch_argmax_rows(static_cast<const float*>(logits), next_token, h->at<unsigned long long>(lo.lm_keys),
-                                                                    h->at<int>(lo.lm_tickets), rows, D.vocab, st));
+                                                                    h->at<int>(lo.lm_tickets), rows, D.vocab, debug_ref(h), st));
   return VS_OK;
 }
 

@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(256) pool_kernel(PoolArgs a, BatchParams bp, i
       if (VS_STORE_OK(bp, DR_EMB, ep, 2)) *ep = cv;
       // the step's other kernels take the slot from this copy: the bank update, which moves
       // meta.free_slot on, runs beside the last attention kernel
-      if (blockIdx.x == 0 && threadIdx.x == 0) a.step_slot[sid] = slot;
+      if (blockIdx.x == 0 && threadIdx.x == 0 && VS_STORE_OK(bp, DR_STEP_SLOT, a.step_slot + sid, 4)) a.step_slot[sid] = slot;
     }
   }
   VS_STAMP(bp, 0, 15);
@@ -127,7 +127,8 @@ __global__ void __launch_bounds__(256) rope_table_kernel(RopeArgs a, BatchParams
   const double ang = (double)(bp.pos_base[b] + r) * a.inv_freq[k];
   double s, c;
   sincos(ang, &s, &c);
-  a.rope[((size_t)b * T + r) * half + k] = make_float2((float)c, (float)s);
+  float2* rp = a.rope + ((size_t)b * T + r) * half + k;
+  if (VS_STORE_OK(bp, DR_ROPE, rp, 8)) *rp = make_float2((float)c, (float)s);
 }
 
 cudaError_t launch_rope_table(const RopeArgs& a, const BatchParams& bp, cudaStream_t st) {
@@ -146,7 +147,7 @@ cudaError_t launch_rope_table(const RopeArgs& a, const BatchParams& bp, cudaStre
 // ------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) rms_stats_kernel(const bf16* __restrict__ h, const bf16* __restrict__ gain,
                                                         bf16* __restrict__ hg, float* __restrict__ row_ss,
-                                                        int parts, int d) {
+                                                        int parts, int d, DebugRef dr) {
   pdl_wait();
   pdl_launch_dependents();
   const size_t row = blockIdx.x;
@@ -157,7 +158,7 @@ __global__ void __launch_bounds__(256) rms_stats_kernel(const bf16* __restrict__
     ss += v.x * v.x + v.y * v.y;
     if (gain != nullptr) {
       const float2 g = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(gain + c));
-      *reinterpret_cast<__nv_bfloat162*>(hg + row * d + c) = __floats2bfloat162_rn(v.x * g.x, v.y * g.y);
+      if (VS_STORE_OK(dr, DR_XN, hg + row * d + c, 4)) *reinterpret_cast<__nv_bfloat162*>(hg + row * d + c) = __floats2bfloat162_rn(v.x * g.x, v.y * g.y);
     }
   }
   __shared__ float red[8];
@@ -165,7 +166,7 @@ __global__ void __launch_bounds__(256) rms_stats_kernel(const bf16* __restrict__
   for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == 0 && VS_STORE_OK(dr, DR_ROW_SS, row_ss + row * parts, (size_t)parts * 4)) {
     float tot = 0.f;
 #pragma unroll
     for (int i = 0; i < 8; ++i) tot += red[i];
@@ -174,9 +175,9 @@ __global__ void __launch_bounds__(256) rms_stats_kernel(const bf16* __restrict__
   }
 }
 
-cudaError_t launch_rms_stats(const bf16* h, const bf16* gain, bf16* hg, float* row_ss, int parts, int rows, int d,
+cudaError_t launch_rms_stats(const bf16* h, const bf16* gain, bf16* hg, float* row_ss, int parts, int rows, int d, DebugRef dr,
                              cudaStream_t st) {
-  return launch_pdl(rms_stats_kernel, dim3(rows), dim3(256), 0, st, h, gain, hg, row_ss, parts, d);
+  return launch_pdl(rms_stats_kernel, dim3(rows), dim3(256), 0, st, h, gain, hg, row_ss, parts, d, dr);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -186,7 +187,7 @@ cudaError_t launch_rms_stats(const bf16* h, const bf16* gain, bf16* hg, float* r
 // projection reads xn and applies the row scale from the sum of squares left here.  One block per row.
 // ------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) lm_norm_kernel(const void* __restrict__ h, int h_fp32, const bf16* __restrict__ gain,
-                                                      bf16* __restrict__ xn, float* __restrict__ row_ss, int parts, int d) {
+                                                      bf16* __restrict__ xn, float* __restrict__ row_ss, int parts, int d, DebugRef dr) {
   pdl_wait();
   pdl_launch_dependents();
   const size_t row = blockIdx.x;
@@ -205,14 +206,14 @@ __global__ void __launch_bounds__(256) lm_norm_kernel(const void* __restrict__ h
       const float2 g = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(gain + c));
       hv = __floats2bfloat162_rn(v.x * g.x, v.y * g.y);
     }
-    *reinterpret_cast<__nv_bfloat162*>(xn + row * d + c) = hv;
+    if (VS_STORE_OK(dr, DR_XN, xn + row * d + c, 4)) *reinterpret_cast<__nv_bfloat162*>(xn + row * d + c) = hv;
   }
   __shared__ float red[8];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == 0 && VS_STORE_OK(dr, DR_ROW_SS, row_ss + row * parts, (size_t)parts * 4)) {
     float tot = 0.f;
 #pragma unroll
     for (int i = 0; i < 8; ++i) tot += red[i];
@@ -222,8 +223,8 @@ __global__ void __launch_bounds__(256) lm_norm_kernel(const void* __restrict__ h
 }
 
 cudaError_t launch_lm_norm(const void* h, int h_fp32, const bf16* gain, bf16* xn, float* row_ss, int parts, int rows, int d,
-                           cudaStream_t st) {
-  return launch_pdl(lm_norm_kernel, dim3(rows), dim3(256), 0, st, h, h_fp32, gain, xn, row_ss, parts, d);
+                           DebugRef dr, cudaStream_t st) {
+  return launch_pdl(lm_norm_kernel, dim3(rows), dim3(256), 0, st, h, h_fp32, gain, xn, row_ss, parts, d, dr);
 }
 
 // Greedy choice.  (value, index) pairs are compared as "larger value, else equal value and lower
@@ -240,7 +241,7 @@ __device__ __forceinline__ unsigned long long argmax_key(float v, int i) {
 }
 
 __global__ void __launch_bounds__(256) argmax_rows_kernel(const float* __restrict__ logits, int32_t* __restrict__ token,
-                                                          unsigned long long* __restrict__ keys, int* __restrict__ tickets, int vocab) {
+                                                          unsigned long long* __restrict__ keys, int* __restrict__ tickets, int vocab, DebugRef dr) {
   pdl_wait();
   pdl_launch_dependents();
   const int row = blockIdx.y;
@@ -267,6 +268,7 @@ __global__ void __launch_bounds__(256) argmax_rows_kernel(const float* __restric
   if (threadIdx.x == 0) {
     for (int w = 1; w < 8; ++w)
       if (better(sv[w], si[w], bv, bi)) { bv = sv[w]; bi = si[w]; }
+    if (!VS_STORE_OK(dr, DR_LM_KEYS, keys + row, 8) || !VS_STORE_OK(dr, DR_LM_TICKETS, tickets + row, 4)) return;
     if (bi != 0x7fffffff) atomicMax(keys + row, argmax_key(bv, bi));      // a slice without a number offers nothing
     __threadfence();
     if (atomicAdd(tickets + row, 1) == (int)gridDim.x - 1) {
@@ -279,10 +281,10 @@ __global__ void __launch_bounds__(256) argmax_rows_kernel(const float* __restric
 }
 
 cudaError_t launch_argmax_rows(const float* logits, int32_t* token, unsigned long long* keys, int* tickets, int rows, int vocab,
-                               cudaStream_t st) {
+                               DebugRef dr, cudaStream_t st) {
   int slices = (vocab + 4095) / 4096;
   if (slices > 64) slices = 64;
-  return launch_pdl(argmax_rows_kernel, dim3(slices, rows), dim3(256), 0, st, logits, token, keys, tickets, vocab);
+  return launch_pdl(argmax_rows_kernel, dim3(slices, rows), dim3(256), 0, st, logits, token, keys, tickets, vocab, dr);
 }
 
 // The bank update of one frame as a launch of its own (chunked prefill, adjacent-pair policy).
@@ -313,7 +315,8 @@ __global__ void __launch_bounds__(128, 8) chunk_scores_kernel(BankUpdateArgs a, 
   const bf16* va = (c < a.chunk_l1) ? a.emb + ((size_t)sid * a.slots + c) * a.d : emb_stage + (size_t)(c - a.chunk_l1) * a.d;
   double dot, na, nb;
   warp_dot_norms<16>(va, emb_stage + (size_t)b * a.d, a.d, lane, dot, na, nb);
-  if (lane == 0) out[(size_t)b * a.pre_stride + c] = cosine_of(dot, na, nb);
+  double* op = out + (size_t)b * a.pre_stride + c;
+  if (lane == 0 && VS_STORE_OK(bp, DR_CHUNK_SCORES, op, 8)) *op = cosine_of(dot, na, nb);
 }
 
 cudaError_t launch_chunk_scores(const BankUpdateArgs& a, const BatchParams& bp, const bf16* emb_stage, double* out, cudaStream_t st) {
@@ -336,11 +339,12 @@ __global__ void __launch_bounds__(256, 8) chunk_plan_kernel(BankUpdateArgs a, Ba
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int F = bp.n_active, sid = bp.stream_id[0], l1 = a.chunk_l1;
   StreamMeta* meta = a.meta + sid;
+  const bool meta_ok = VS_STORE_OK(bp, DR_META, meta, sizeof(StreamMeta));
   int32_t* order = a.order + (size_t)sid * a.slots;
   int32_t* slot_frame = a.slot_frame + (size_t)sid * a.slots;
   int64_t* slot_pos = a.slot_pos + (size_t)sid * a.slots;
   if (a.M == 0) {
-    if (tid == 0) { meta->frames_seen += F; meta->last_victim_frame = -1; }
+    if (tid == 0 && meta_ok) { meta->frames_seen += F; meta->last_victim_frame = -1; }
     return;
   }
   int count = bp.count[0], free_slot = meta->free_slot;
@@ -397,8 +401,8 @@ __global__ void __launch_bounds__(256, 8) chunk_plan_kernel(BankUpdateArgs a, Ba
   const int first_log = meta->log_count;
   int my_victim_frame = -1;
   if (tid < F) {
-    a.record_slot[tid] = slot_of[tid];
-    a.record_victim[tid] = victim[tid];
+    if (VS_STORE_OK(bp, DR_CHUNK_SLOT, a.record_slot + tid, 4)) a.record_slot[tid] = slot_of[tid];
+    if (VS_STORE_OK(bp, DR_CHUNK_VICTIM, a.record_victim + tid, 4)) a.record_victim[tid] = victim[tid];
     const int g = victim[tid];
     if (g >= 0) my_victim_frame = (g >= l1) ? (int)(a.chunk_first_frame + (g - l1)) : slot_frame[g];
   }
@@ -415,7 +419,7 @@ __global__ void __launch_bounds__(256, 8) chunk_plan_kernel(BankUpdateArgs a, Ba
       }
     }
   }
-  if (tid == F - 1) meta->last_victim_frame = my_victim_frame;
+  if (tid == F - 1 && meta_ok) meta->last_victim_frame = my_victim_frame;
   __syncthreads();
   for (int i = tid; i < count; i += 256) {
     const int c = axis[i], sl = (c < l1) ? c : slot_of[c - l1];
@@ -425,7 +429,7 @@ __global__ void __launch_bounds__(256, 8) chunk_plan_kernel(BankUpdateArgs a, Ba
       if (VS_STORE_OK(bp, DR_SLOT_POS, slot_pos + sl, 8)) slot_pos[sl] = bp.pos_base[c - l1] + bp.rows_per_stream - 1;
     }
   }
-  if (tid == 0) {
+  if (tid == 0 && meta_ok) {
     meta->count = count;
     meta->free_slot = free_slot;
     meta->frames_seen += F;
@@ -453,13 +457,13 @@ __global__ void __launch_bounds__(128) chunk_kv_commit_kernel(ChunkKvCommitArgs 
   for (int c = threadIdx.x; c < a.Hkv * per_head; c += blockDim.x) {
     const int hk = c / per_head, cc = c - hk * per_head;
     const size_t dst = (((size_t)a.sid * a.Hkv + hk) * a.slots + slot) * a.D + cc * 8;
-    *reinterpret_cast<uint4*>(a.bank_k + dst) = *reinterpret_cast<const uint4*>(a.kf + src + hk * a.D + cc * 8);
-    *reinterpret_cast<uint4*>(a.bank_v + dst) = *reinterpret_cast<const uint4*>(a.vf + src + hk * a.D + cc * 8);
+    if (VS_STORE_OK(a.dr, DR_BANK_K, a.bank_k + dst, 16)) *reinterpret_cast<uint4*>(a.bank_k + dst) = *reinterpret_cast<const uint4*>(a.kf + src + hk * a.D + cc * 8);
+    if (VS_STORE_OK(a.dr, DR_BANK_V, a.bank_v + dst, 16)) *reinterpret_cast<uint4*>(a.bank_v + dst) = *reinterpret_cast<const uint4*>(a.vf + src + hk * a.D + cc * 8);
   }
   if (a.emb != nullptr) {                                             // last layer: the parked embedding, too
     const uint4* es = reinterpret_cast<const uint4*>(a.emb_stage + (size_t)i * a.d);
     uint4* ed = reinterpret_cast<uint4*>(a.emb + ((size_t)a.sid * a.slots + slot) * a.d);
-    for (int c = threadIdx.x; c < a.d / 8; c += blockDim.x) ed[c] = es[c];
+    for (int c = threadIdx.x; c < a.d / 8; c += blockDim.x) if (VS_STORE_OK(a.dr, DR_EMB, ed + c, 16)) ed[c] = es[c];
   }
 }
 
@@ -468,18 +472,18 @@ cudaError_t launch_chunk_kv_commit(const ChunkKvCommitArgs& a, cudaStream_t st) 
 }
 
 __global__ void __launch_bounds__(256) gather_carriers_kernel(const bf16* __restrict__ emb, const int32_t* __restrict__ order,
-                                                             bf16* __restrict__ x, int sid, int slots, int d) {
+                                                             bf16* __restrict__ x, int sid, int slots, int d, DebugRef dr) {
   pdl_wait();
   pdl_launch_dependents();
   const int i = blockIdx.x;
   const uint4* src = reinterpret_cast<const uint4*>(emb + ((size_t)sid * slots + order[(size_t)sid * slots + i]) * d);
   uint4* dst = reinterpret_cast<uint4*>(x + (size_t)i * d);
-  for (int c = threadIdx.x; c < d / 8; c += blockDim.x) dst[c] = src[c];
+  for (int c = threadIdx.x; c < d / 8; c += blockDim.x) if (VS_STORE_OK(dr, DR_HBUF0, dst + c, 16)) dst[c] = src[c];
 }
 
 cudaError_t launch_gather_carriers(const bf16* emb, const int32_t* order, bf16* x, int sid, int slots, int d, int count,
-                                   cudaStream_t st) {
-  return launch_pdl(gather_carriers_kernel, dim3(count), dim3(256), 0, st, emb, order, x, sid, slots, d);
+                                   DebugRef dr, cudaStream_t st) {
+  return launch_pdl(gather_carriers_kernel, dim3(count), dim3(256), 0, st, emb, order, x, sid, slots, d, dr);
 }
 
 __global__ void poison_kernel(uint32_t* p, size_t n) {
@@ -498,8 +502,9 @@ cudaError_t launch_poison(void* p, size_t bytes, cudaStream_t st) {
 __global__ void reset_kernel(StreamMeta* meta, int32_t* slot_frame, int slots, BatchParams bp) {
   pdl_wait();
   const int sid = bp.stream_id[blockIdx.x];
-  for (int i = threadIdx.x; i < slots; i += blockDim.x) slot_frame[(size_t)sid * slots + i] = -1;
-  if (threadIdx.x == 0) {
+  for (int i = threadIdx.x; i < slots; i += blockDim.x)
+    if (VS_STORE_OK(bp, DR_SLOT_FRAME, slot_frame + (size_t)sid * slots + i, 4)) slot_frame[(size_t)sid * slots + i] = -1;
+  if (threadIdx.x == 0 && VS_STORE_OK(bp, DR_META, meta + sid, sizeof(StreamMeta))) {
     StreamMeta m;
     m.count = 0; m.free_slot = 0; m.victim_logical = -1; m.last_victim_frame = -1;
     m.frames_seen = 0; m.evictions = 0; m.log_count = 0; m.score_ticket = 0;

@@ -587,7 +587,7 @@ __global__ void __launch_bounds__(kThreads, 1) token_kernel(const __grid_constan
           for (int i = 0; i < kCW; ++i) t += sum_s[i];
           float* sp = a.ss + (size_t)r * a.ss_cap;
           if (VS_STORE_OK(bp, DR_TOK, sp, 4)) *sp = t;
-          add_release(a.counters, 1);
+          if (VS_STORE_OK(bp, DR_TOK_SYNC, a.counters, 4)) add_release(a.counters, 1);
         }
         compute_bar();
       }
@@ -676,7 +676,7 @@ __global__ void __launch_bounds__(kThreads, 1) token_kernel(const __grid_constan
             float4* dst = reinterpret_cast<float4*>(a.part) + ((size_t)cta * ITEMS + item) * 32 + lane;
             if (VS_STORE_OK(bp, DR_TOK, dst, 16)) __stcg(dst, v);
             __syncwarp();
-            if (lane == 0) st_release(a.frag_flags + cta * 8 + item, seq);
+            if (lane == 0 && VS_STORE_OK(bp, DR_TOK_SYNC, a.frag_flags + cta * 8 + item, 4)) st_release(a.frag_flags + cta * 8 + item, seq);
           } else {
           if (kk + 1 < p.kst) {
             const uint32_t total = (uint32_t)(p.tiles * p.kst);
@@ -701,7 +701,7 @@ __global__ void __launch_bounds__(kThreads, 1) token_kernel(const __grid_constan
       if (warp == 0 && kind == PH_QKV) TOK_STAMP(3, l);
       compute_bar();                                                   // every finisher's stores come before this point
       if (warp == 0 && kind == PH_QKV) TOK_STAMP(4, l);
-      if (tid == 0) add_release(counter(a, l, kind), 1);
+      if (tid == 0 && VS_STORE_OK(bp, DR_TOK_SYNC, counter(a, l, kind), 4)) add_release(counter(a, l, kind), 1);
     };
 
     // ---- attention of layer l: unit = (token row, KV head, share of the keys) ------------------------------
@@ -898,7 +898,7 @@ __global__ void __launch_bounds__(kThreads, 1) token_kernel(const __grid_constan
         }
         compute_bar();
         if (tid == 0) {
-          const int t = add_acq_rel(a.tickets + rh, 1);
+          const int t = VS_STORE_OK(bp, DR_TOK_SYNC, a.tickets + rh, 4) ? add_acq_rel(a.tickets + rh, 1) : 0;
           if (t == a.nsplit - 1) a.tickets[rh] = 0;                          // (the next layer's units start after this one's)
           *bcast = t;
         }
@@ -972,7 +972,7 @@ __global__ void __launch_bounds__(kThreads, 1) token_kernel(const __grid_constan
           float* sp = a.ss + (size_t)row * a.ss_cap + hkv;
           if (VS_STORE_OK(bp, DR_TOK, sp, 4)) *sp = t;
         }
-        add_release(counter(a, l, PH_ATT), 1);
+        if (VS_STORE_OK(bp, DR_TOK_SYNC, counter(a, l, PH_ATT), 4)) add_release(counter(a, l, PH_ATT), 1);
       }
       if (warp == 0) TOK_STAMP(12, l);
     };
@@ -993,7 +993,7 @@ __global__ void __launch_bounds__(kThreads, 1) token_kernel(const __grid_constan
     });
     if (a.vocab > 0) {
       compute_bar();
-      if (tid < rows && a.next_token != nullptr && best_s[tid] != 0ull) atomicMax(a.lm_keys + tid, best_s[tid]);
+      if (tid < rows && a.next_token != nullptr && best_s[tid] != 0ull && VS_STORE_OK(bp, DR_LM_KEYS, a.lm_keys + tid, 8)) atomicMax(a.lm_keys + tid, best_s[tid]);
     }
   }
 
@@ -1002,16 +1002,18 @@ __global__ void __launch_bounds__(kThreads, 1) token_kernel(const __grid_constan
   if (tid == 0) {
     if (*abort_flag) atomicExch(a.status, VS_ERR_DEVICE_TIMEOUT);
     __threadfence();
-    *bcast = atomicAdd(a.done, 1);
+    *bcast = VS_STORE_OK(bp, DR_TOK_SYNC, a.done, 4) ? atomicAdd(a.done, 1) : 0;
     __threadfence();
   }
   __syncthreads();
   if (*bcast == ncta - 1) {
     const int n_counters = 1 + 5 * a.L;
 #pragma unroll 1
-    for (int i = tid; i < n_counters; i += kThreads) a.counters[(size_t)i * kCntStride] = 0;
+    for (int i = tid; i < n_counters; i += kThreads)
+      if (VS_STORE_OK(bp, DR_TOK_SYNC, a.counters + (size_t)i * kCntStride, 4)) a.counters[(size_t)i * kCntStride] = 0;
 #pragma unroll 1
-    for (int i = tid; i < ncta * 8; i += kThreads) a.frag_flags[i] = 0;
+    for (int i = tid; i < ncta * 8; i += kThreads)
+      if (VS_STORE_OK(bp, DR_TOK_SYNC, a.frag_flags + i, 4)) a.frag_flags[i] = 0;
     if (tid == 0) *a.done = 0;
     if (a.vocab > 0 && a.next_token != nullptr && tid < rows) {
       const unsigned long long k = atomicExch(a.lm_keys + tid, 0ull);

@@ -3,6 +3,8 @@ every kernel store into the workspace is tested against the region it names (a s
 skipped and recorded, nothing traps), and 256 guard bytes lie behind every workspace region;
 vs_bank_state reports either finding as VS_ERR_BOUNDS.  The small odd-shaped cases run through it
 against the oracle: parity must hold and no finding may be reported."""
+import os
+
 import numpy as np
 import pytest
 
@@ -97,6 +99,27 @@ def test_the_guard_check_is_alive(checked_library):
     with pytest.raises(binding.VsError) as err:
         p.gpu.bank_state(0)
     assert err.value.code == binding.VS_ERR_BOUNDS
+    p.close()
+
+
+def test_guard_bytes_lie_behind_every_region(checked_library):
+    """As many runs of guard bytes as the layout takes regions (but the table of regions itself), and each of them is watched."""
+    source = open(os.path.join(os.path.dirname(build.__file__), "csrc", "vs_host.cu")).read()
+    layout = source[source.index("void fill_layout("):source.index("struct vs_stream {")]
+    n_regions = layout.count("take(") - layout.count("take(sizeof(DebugTable))")
+    w = synth.workload("tiny", n_frames=2)
+    p = Pair(w, max_chunk_frames=2)
+    off = p.gpu._ws_ptr - p.gpu.workspace.data_ptr()
+    blocks = p.gpu.workspace[off:off + p.gpu.workspace_bytes // 256 * 256].view(-1, 256)
+    guards = (blocks == 0xC5).all(dim=1).nonzero().flatten().tolist()
+    assert len(guards) == n_regions
+    for g in guards:
+        assert p.check_bank(0)["device_status"] == 0
+        blocks[g, 255] = 0
+        with pytest.raises(binding.VsError) as err:
+            p.gpu.bank_state(0)
+        assert err.value.code == binding.VS_ERR_BOUNDS
+        blocks[g, 255] = 0xC5
     p.close()
 
 
