@@ -284,6 +284,7 @@ class StreamBatch:
         self.cfg = cfg
         self.device = torch.device("cuda", cfg.device)
         self.device_index = int(cfg.device)
+        self._raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)      # (not part of torch's public API)
         self.weights = [w.contiguous() for w in weights]
         self.biases = biases
         self.norm_weights = norm_weights
@@ -306,8 +307,10 @@ class StreamBatch:
         self.out_torch_dtype = torch.float32 if cfg.out_dtype == 1 else torch.bfloat16
 
     def _stream(self) -> int:
-        # (current_stream(device).cuda_stream without the Stream object: a token step of one layer is bound by the host)
-        return self.torch._C._cuda_getCurrentRawStream(self.device_index)
+        # without the Stream object where this torch has the call: a token step of one layer is bound by the host
+        if self._raw_stream is not None:
+            return self._raw_stream(self.device_index)
+        return self.torch.cuda.current_stream(self.device).cuda_stream
 
     def lm_head(self, hidden, logits=None, want_token=True):
         """hidden: [rows, d_model] of the handle's output dtype -> (logits fp32 [rows, vocab], next tokens int32 [rows] or None)."""

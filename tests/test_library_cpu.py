@@ -68,3 +68,12 @@ def test_null_arguments_are_rejected(lib):
 def test_missing_library_fails_loudly(tmp_path):
     with pytest.raises(FileNotFoundError):
         binding.load_library(str(tmp_path / "nope.so"))
+
+
+def test_current_stream_with_and_without_torchs_private_call():
+    import types
+    public = types.SimpleNamespace(cuda=types.SimpleNamespace(current_stream=lambda device: types.SimpleNamespace(cuda_stream=0x70 + device)))
+    for raw, want in ((None, 0x73), (lambda index: 0x90 + index, 0x93)):
+        b = binding.StreamBatch.__new__(binding.StreamBatch)
+        b.handle, b.torch, b.device, b.device_index, b._raw_stream = None, public, 3, 3, raw
+        assert b._stream() == want
