@@ -1236,13 +1236,15 @@ int vs_decode_step(vs_stream* h, const int32_t* stream_ids, int32_t n_active, co
       if (D.d_ff > 0) { da.out = h->at<void>(lo.obuf); da.out_fp32 = 0; da.h_in = nullptr; da.h_out = nullptr; }
       da.meta = meta;
       da.Hq = D.Hq; da.Hkv = D.Hkv; da.D = D.D; da.slots = D.slots; da.M = D.M; da.maxP = D.maxP; da.maxT = D.maxT;
-      // A CTA per query head, or per KV head (K and V read once per group).  The first for one stream, and for two to four in large
-      // groups where all its CTAs, two to an SM, run at once: its chains are shorter (two streams of 250 keys: 96 against 110 us
-      // for 8 layers at the Qwen2-7B shape, groups of seven; of 640 keys, more CTAs than that: 135 against 109; groups of four: 61
-      // either way or 8 % slower).  There short contexts are written by the CTA directly, longer ones split over a cluster of 2, 4
-      // or 8 CTAs (a CTA then walks about 64 to 128 keys)
+      // A CTA per query head, or per KV head (K and V read once per group).  The first for one stream, and for two to four in groups of
+      // more than four where its CTAs, two to an SM, take no more than seven eighths of the places: its chains are shorter (8 layers,
+      // head size 128, us against by KV head: groups of seven, two streams, 246 keys 94 / 117; of six, three streams, 166 keys
+      // 88 / 98; of five, three streams, 246 keys 83 / 89; of five, four streams, 166 keys 90 / 86 is the one found the other
+      // way; groups of four: 61 either way or 8 % slower).  Beyond that its clusters no longer all fit (256 CTAs in clusters of four
+      // 146 / 147, 288 of 296: 120 / 100).  There short contexts are written by the CTA directly, longer ones split over a cluster of
+      // 2, 4 or 8 CTAs (a CTA then walks about 64 to 128 keys)
       int ns = (max_keys <= 96) ? 1 : (max_keys <= 192 ? 2 : (max_keys <= 448 ? 4 : 8));
-      const bool by_head = n_active == 1 || !wide || (n_active <= 4 && D.G > 4 && (long long)ns * D.Hq * n_active <= 2LL * h->n_sms);
+      const bool by_head = n_active == 1 || !wide || (n_active <= 4 && D.G > 4 && 4LL * ns * D.Hq * n_active <= 7LL * h->n_sms);
       if (by_head) {
         while (ns > 1 && (long long)ns * D.Hq * n_active > 4LL * h->n_sms) ns >>= 1;
       } else {
