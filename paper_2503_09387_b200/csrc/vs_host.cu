@@ -442,19 +442,27 @@ size_t layer_stride_bank(const Dims& D) { return (size_t)D.S * D.Hkv * D.slots *
 size_t layer_stride_prefix(const Dims& D) { return (size_t)D.S * D.Hkv * D.maxP * D.D; }
 size_t layer_stride_tail(const Dims& D) { return (size_t)D.S * D.Hkv * D.maxT * D.D; }
 
-// Whether a step of n_active x T rows goes to the persistent kernel (measured at the Qwen2-7B shape, us against the launches
-// layer by layer).  Full layers and the head: up to 8 rows (3 layers and the head: 455 -> 437 for one row, 336 -> 303 for 8
-// without the head; at 16 the slabs leave the ring too few stages, 344 -> 362).  Attention alone: steps of several tokens up to
-// 16 rows (28 layers: 589 -> 474 for 2 rows, 783 -> 559 for 16; 32 rows 770 -> 842) and single tokens of more streams than the
-// matrix-vector kernel takes (545 -> 460 for 8, 588 -> 517 for 16), in a stack; one to four single tokens are faster by launches
-// (352 against 463: 11 us a layer is little more than the phases' own synchronisation), and so are two to four rows in a single
-// layer (17.7 against 19.4).  And not where a layer's projection holds
-// less than 16 KB for every SM: there is then no weight stream to hide that synchronisation behind.
-bool token_step_pays(const vs_stream* h, int n_active, int T, int matrix_rows, bool full) {
+// Whether a step of n_active x T rows goes to the persistent kernel.  Both sides measured (us, persistent against launches layer by
+// layer); the number of keys moves them alike (64 to 1024 carriers).
+// Full layers and the head, up to 8 rows (at 16 the slabs leave the ring too few stages: 3 layers at the Qwen2-7B shape 362 against
+// 344).  Where a layer's projection holds 223 KB for every SM (that shape, 2 layers): one row 181 against 184, eight 199 against 213.
+// Narrower layers hide less of the phases' synchronisation behind weights, and single tokens of several streams, whose launches are
+// the cheapest (matrix-vector kernel, attention by head), go there from three rows on: 6 layers of width 1536 (42 KB an SM) 237
+// against 242 for two streams, 260 against 246 for four, 300 against 272 for eight; 1024 (21 KB) 168 / 181, 188 / 179, 227 / 210;
+// 2048 (85 KB) 272 / 263, 287 / 268, 330 / 295.  One stream's several tokens stay: 239 / 273 for two, 302 / 306 for eight at 1536.
+// Attention alone: steps of several tokens up to 16 rows (8 layers over 564 keys: width 1024 79 / 84 for two tokens, 82 / 118 for
+// five; 2048 108 / 113, 101 / 148; 3584 138 / 132, 129 / 174; 16 rows 192 / 206, 32 rows 842 against 770 for 28 layers) and single
+// tokens of more streams than the matrix-vector kernel takes (8 streams 180 / 251, 16 209 / 249), in a stack; one to four single
+// tokens are faster by launches (28 layers 463 against 352), and so are two to four rows in a single layer (19.4 against 17.7).
+// And not where a layer's projection holds less than 16 KB for every SM: there is then no weight stream to hide the
+// synchronisation behind.
+// wide: the rows' address takes four elements at a time; else the kernel takes what no other can store, a full layer's rows.
+bool token_step_pays(const vs_stream* h, int n_active, int T, int matrix_rows, bool full, bool wide) {
   const int rows = n_active * T;
-  if (h->n_sms > TOK_MAX_CTAS || (size_t)matrix_rows * h->dm.d * 2 < (size_t)h->n_sms * 16384) return false;
-  if (full) return rows <= 8;
-  return rows <= TOK_MAX_ROWS && (T > 1) + (rows > 4) + (h->dm.L > 1) >= 2;
+  const size_t per_sm = (size_t)matrix_rows * h->dm.d * 2 / h->n_sms;
+  if (h->n_sms > TOK_MAX_CTAS || per_sm < 16384) return false;
+  if (full) return rows <= (T > 1 || per_sm >= 131072 || !wide ? 8 : 2);
+  return wide && rows <= TOK_MAX_ROWS && (T > 1) + (rows > 4) + (h->dm.L > 1) >= 2;
 }
 
 // Whether `p` can take a step's rows as most kernels store them, four elements at a time.
@@ -1126,7 +1134,7 @@ int vs_decode_step(vs_stream* h, const int32_t* stream_ids, int32_t n_active, co
   // rows at any address: the persistent kernel stores a full layer's element by element, and so does the attention by query head,
   // which takes a single token per stream
   const bool wide = takes_rows(out, D);
-  const bool persistent = token_step_pays(h, n_active, T, D.E_out, D.d_ff > 0) && (wide || D.d_ff > 0);
+  const bool persistent = token_step_pays(h, n_active, T, D.E_out, D.d_ff > 0, wide);
   if (!wide && !persistent && (T > 1 || D.d_ff > 0)) return VS_ERR_INVALID_ARG;
   const bool to_prefix = h->hs[stream_ids[0]].frames_seen == 0;
   for (int i = 0; i < n_active; ++i) {
@@ -1386,7 +1394,7 @@ int vs_lm_head(vs_stream* h, const void* hidden, int32_t rows, void* logits, int
   bp.rows_per_stream = rows;
   VS_TRACE_NEXT(h, bp);
   bf16* xn = h->at<bf16>(lo.xn);
-  if (token_step_pays(h, rows, 1, D.vocab, true)) {
+  if (token_step_pays(h, rows, 1, D.vocab, true, true)) {
     TokArgs ta = token_args(h, hidden, rows);
     ta.full = 0; ta.hidden_fp32 = D.out_fp32;
     ta.vocab = D.vocab; ta.tm_lm = reinterpret_cast<const CUtensorMap*>(ta.layers + D.L); ta.gain_f = h->gain_f;

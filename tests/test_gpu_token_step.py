@@ -35,6 +35,20 @@ def test_steps_of_every_tile_shape(d, Hq, Hkv, D, d_ff, L, prefix):
     p.close()
 
 
+@pytest.mark.parametrize("d_ff,one_launch", [(704, [(1, 1), (2, 1), (1, 2), (1, 8), (3, 2)]), (0, [(1, 2), (1, 8), (1, 9), (3, 2), (3, 3)])])
+def test_which_steps_are_one_launch(d_ff, one_launch):
+    """Narrow layers (24 KB of projection an SM): single tokens of three streams on are launches, several tokens are not."""
+    w = synth.workload("deep", n_layers=2, d_model=1152, n_q_heads=18, n_kv_heads=3, head_dim=64, tokens_per_frame=5, n_frames=1, bank_capacity=2,
+                       prefix_len=3, question_len=0, decode_tokens=0, n_streams=3, frame_model="iid", seed=71)
+    p = Pair(w, max_prefix=64, max_text=16, max_step_tokens=32, **({"d_ff": d_ff} if d_ff else {}))
+    for n, T in ((1, 1), (2, 1), (3, 1), (1, 2), (1, 8), (1, 9), (3, 2), (3, 3), (1, 17)):
+        p.gpu.profile_read()
+        p.text(list(range(n)), [synth.normal_bf16(w.seed, synth.TAG_QUESTION, (T, 1152), 1.0, offset=(T * 4 + s) * 32 * 1152) for s in range(n)], f"{n} x {T}")
+        launches = sum(v[2] for v in p.gpu.profile_read().values())
+        assert (launches == 1) == ((n, T) in one_launch), (n, T, launches)
+    p.close()
+
+
 @pytest.mark.parametrize("d,vocab,rows,norm,gain,out_dtype", [(1152, 1280, 1, True, True, 1), (1088, 1280, 8, True, False, 0), (1088, 1280, 9, True, False, 0),
                                                               (1088, 1280, 32, False, False, 1)])
 def test_lm_head_of_a_few_rows(d, vocab, rows, norm, gain, out_dtype):
