@@ -304,6 +304,8 @@ struct GemmArgs {
   int n_sms;
   int* status;
 };
+struct Tiling { int tile_n, n_tiles, ksplit, pairs; };
+Tiling choose_tiles(int K, int E, int n_sms, int max_pairs, int rows, bool own_rope);
 cudaError_t launch_qkv_gemm(const GemmArgs& a, const BatchParams& bp, cudaStream_t st);
 cudaError_t qkv_gemm_init();     // opt-in shared memory attribute, once per process/device
 cudaError_t pair_gemm_init();
@@ -405,7 +407,7 @@ struct ChunkKvCommitArgs {
   DebugRef dr;
 };
 cudaError_t launch_chunk_kv_commit(const ChunkKvCommitArgs& a, cudaStream_t st);
-constexpr int ATTN_EXCL_BITS = 8192;   // most (bank slots + chunk frames) a chunk call takes
+constexpr int CHUNK_AXIS_MAX = 8192;   // most (bank slots + chunk frames) a chunk call takes: the plan keeps the bank's order in shared memory
 cudaError_t launch_prefill_attention_tc(const AttnArgs& a, const BatchParams& bp, int* status, cudaStream_t st);
 cudaError_t prefill_attention_tc_init();
 int prefill_attention_max_clusters(int head_dim, int s);

@@ -36,6 +36,41 @@ int attention_split(int head_dim, int group, int row_ctas, int key_tiles, int ba
   return best;
 }
 
+// Tiling of a linear layer: CTAs with 128 weight rows each and K cut into ksplit shares (few rows), or CTA pairs with 256
+// (many), and the token columns of a tile.  The choice minimises the clocks of the waves' main loops plus what their epilogues
+// add.  The main loops run at the operands' rate from L2, about 47 bytes a clock of an SM (the MMAs need less: 2 clocks a token
+// column): a 64-element block of K is (128 + tile_n) * 128 bytes to a CTA, (128 + tile_n / 2) * 128 to a CTA of a pair.  A tile's
+// epilogue costs 900 clocks and 14 a column, in a pair kernel only the last one counts, with 3100 clocks for the longer start;
+// a K split 1000 and 3.5 a column more (partial tiles through L2, a flag), and it needs its whole grid resident at once.
+// Fitted to whole steps of 17 to 1280 rows at the shapes of two backbones, K 1024 to 18944: the chosen tiling is 0.3 % slower
+// than the best one on average (a split costed at 5000 clocks whatever its tile left 1.2 %, at K = 18944 and 480 rows 10 %).
+Tiling choose_tiles(int K, int E, int n_sms, int max_pairs, int rows, bool own_rope) {
+  const int kb = K / GEMM_BLOCK_K, resident = n_sms < GEMM_XCHG_CTAS ? n_sms : GEMM_XCHG_CTAS;
+  const int nt_min = (rows + 255) / 256;
+  double best = -1.0;
+  Tiling t = {16, 1, 1, 0};
+  for (int nt = nt_min; nt <= nt_min + 24; ++nt) {
+    const int tn = ((rows + nt - 1) / nt + 15) / 16 * 16;
+    if ((long long)(nt - 1) * tn >= rows && nt > nt_min) continue;      // an empty last tile
+    if (tn < 64 && nt > nt_min) break;
+    auto block = [&](int tn_own) { return (128 + tn_own) * 2.7; };
+    const double epilogue = 900.0 + 14.0 * tn;
+    const int mt1 = (E + GEMM_BLOCK_M - 1) / GEMM_BLOCK_M, mt2 = (E + 2 * GEMM_BLOCK_M - 1) / (2 * GEMM_BLOCK_M);
+    for (int ks = 1; ks <= KSPLIT_MAX && ks <= kb; ++ks) {
+      const long long ctas = (long long)mt1 * nt * ks;
+      if (ks > 1 && ctas > resident) break;
+      const long long waves = (ctas + n_sms - 1) / n_sms;
+      const double cost = waves * (block(tn) * ((kb + ks - 1) / ks) + epilogue) + (ks > 1 ? 1000.0 + 3.5 * tn : 0.0);
+      if (best < 0 || cost < best) { best = cost; t = {tn, nt, ks, 0}; }
+    }
+    if (own_rope) continue;                                              // (the pair kernel reads a table)
+    const long long items = (long long)mt2 * nt, waves = (items + max_pairs - 1) / max_pairs;
+    const double cost = waves * (block(tn / 2) * kb + 100.0) + epilogue + 3100.0;
+    if (best < 0 || cost < best) { best = cost; t = {tn, nt, 1, 1}; }
+  }
+  return t;
+}
+
 }  // namespace vs
 
 namespace {
@@ -270,42 +305,6 @@ void seg_step(AttnSegment& sg, const CUtensorMap& k, const CUtensorMap& v, int k
   sg.tk = k; sg.tv = v; sg.kind = kind; sg.rows_per_batch = rows_per_batch; sg.z0 = 0; sg.z_per_stream = 0;
 }
 
-// Tiling of a linear layer: CTAs with 128 weight rows each and K cut into ksplit shares (few rows), or CTA pairs with 256
-// (many), and the token columns of a tile.  The choice minimises the clocks of the waves' main loops plus what their epilogues
-// add.  The main loops run at the operands' rate from L2, about 47 bytes a clock of an SM (the MMAs need less: 2 clocks a token
-// column): a 64-element block of K is (128 + tile_n) * 128 bytes to a CTA, (128 + tile_n / 2) * 128 to a CTA of a pair.  A tile's
-// epilogue costs 900 clocks and 14 a column, in a pair kernel only the last one counts, with 3100 clocks for the longer start;
-// a K split 1000 and 3.5 a column more (partial tiles through L2, a flag), and it needs its whole grid resident at once.
-// Fitted to whole steps of 17 to 1280 rows at the shapes of two backbones, K 1024 to 18944: the chosen tiling is 0.3 % slower
-// than the best one on average (a split costed at 5000 clocks whatever its tile left 1.2 %, at K = 18944 and 480 rows 10 %).
-struct Tiling { int tile_n, n_tiles, ksplit; bool pairs; };
-Tiling choose_tiles(int K, int E, int n_sms, int max_pairs, int rows, bool own_rope) {
-  const int kb = K / GEMM_BLOCK_K, resident = n_sms < GEMM_XCHG_CTAS ? n_sms : GEMM_XCHG_CTAS;
-  const int nt_min = (rows + 255) / 256;
-  double best = -1.0;
-  Tiling t = {16, 1, 1, false};
-  for (int nt = nt_min; nt <= nt_min + 24; ++nt) {
-    const int tn = ((rows + nt - 1) / nt + 15) / 16 * 16;
-    if ((long long)(nt - 1) * tn >= rows && nt > nt_min) continue;      // an empty last tile
-    if (tn < 64 && nt > nt_min) break;
-    auto block = [&](int tn_own) { return (128 + tn_own) * 2.7; };
-    const double epilogue = 900.0 + 14.0 * tn;
-    const int mt1 = (E + GEMM_BLOCK_M - 1) / GEMM_BLOCK_M, mt2 = (E + 2 * GEMM_BLOCK_M - 1) / (2 * GEMM_BLOCK_M);
-    for (int ks = 1; ks <= KSPLIT_MAX && ks <= kb; ++ks) {
-      const long long ctas = (long long)mt1 * nt * ks;
-      if (ks > 1 && ctas > resident) break;
-      const long long waves = (ctas + n_sms - 1) / n_sms;
-      const double cost = waves * (block(tn) * ((kb + ks - 1) / ks) + epilogue) + (ks > 1 ? 1000.0 + 3.5 * tn : 0.0);
-      if (best < 0 || cost < best) { best = cost; t = {tn, nt, ks, false}; }
-    }
-    if (own_rope) continue;                                              // (the pair kernel reads a table)
-    const long long items = (long long)mt2 * nt, waves = (items + max_pairs - 1) / max_pairs;
-    const double cost = waves * (block(tn / 2) * kb + 100.0) + epilogue + 3100.0;
-    if (best < 0 || cost < best) { best = cost; t = {tn, nt, 1, true}; }
-  }
-  return t;
-}
-
 // launches the linear layer described by `g` (all but the tiling) on `src` [rows][K]
 int launch_linear(vs_stream* h, GemmArgs& g, const bf16* src, int rows, int K, int E, const BatchParams& bp, cudaStream_t st);
 
@@ -381,7 +380,7 @@ int run_projection(vs_stream* h, int l, const bf16* src, int rows, const Project
 
 int launch_linear(vs_stream* h, GemmArgs& g, const bf16* src, int rows, int K, int E, const BatchParams& bp, cudaStream_t st) {
   const Tiling t = choose_tiles(K, E, h->n_sms, h->n_pairs, rows, g.out.mode < 4 && g.out.rope == nullptr);
-  g.tile_n = t.tile_n; g.n_tiles = t.n_tiles; g.ksplit = t.ksplit; g.pairs = t.pairs;
+  g.tile_n = t.tile_n; g.n_tiles = t.n_tiles; g.ksplit = t.ksplit; g.pairs = t.pairs != 0;
   g.xchg = h->at<float>(h->lo.gemm_xchg);
   g.flags = h->at<int>(h->lo.gemm_flags);
   g.n_sms = h->n_sms;
@@ -865,9 +864,8 @@ int vs_frame_prefill_chunk(vs_stream* h, int32_t stream_id, const void* hidden, 
   // before the chunk (all M + 1 slots once the bank is full)
   const int count0 = bp.count[0];
   const int l1 = (D.M > 0 && count0 == D.M) ? D.M + 1 : count0;
-  // the attention launch's mask of hidden bank keys; refused on the bank's capacity, not on its fill, so that a
-  // stream does not run into the limit only once its bank is full
-  if ((D.M > 0 ? D.M + 1 : 0) + F > ATTN_EXCL_BITS) return VS_ERR_CAPACITY;
+  // refused on the bank's capacity, not on its fill, so that a stream does not run into the limit only once its bank is full
+  if ((D.M > 0 ? D.M + 1 : 0) + F > CHUNK_AXIS_MAX) return VS_ERR_CAPACITY;
 
   // 1. carriers of all frames (Section 3.3: C = mean of the frame's tokens), parked until they have a slot
   PoolArgs pa;
@@ -912,7 +910,7 @@ int vs_frame_prefill_chunk(vs_stream* h, int32_t stream_id, const void* hidden, 
     ba.chunk_first_frame = bp.frame_id[0];
     ba.chunk_l1 = l1;
     ba.pre_scores = nullptr; ba.pre_stride = 0;
-  ba.j0 = 0; ba.j1 = D.M; ba.commit = 1;
+    ba.j0 = 0; ba.j1 = D.M; ba.commit = 1;
     const bool any_full = D.M > 0 && bp.count[F - 1] == D.M;
     if (planned) {
       // the updates score against their incoming carrier only (or not at all): every cosine of the
@@ -993,8 +991,8 @@ int vs_frame_prefill_chunk(vs_stream* h, int32_t stream_id, const void* hidden, 
       aa.out_fp32 = D.out_fp32;
       aa.h_in = D.residual ? h_in : nullptr;
       aa.h_out = D.residual ? h->at<bf16>(lo.hbuf[cur ^ 1]) : nullptr;
-    aa.h_out_region = (cur ^ 1) ? DR_HBUF1 : DR_HBUF0;
-    if (D.use_rmsnorm && l + 1 < D.L) { aa.ss_out = h->at<float>(lo.row_ss); aa.next_gain = h->gain[l + 1]; aa.xn_out = h->at<bf16>(lo.xn); }
+      aa.h_out_region = (cur ^ 1) ? DR_HBUF1 : DR_HBUF0;
+      if (D.use_rmsnorm && l + 1 < D.L) { aa.ss_out = h->at<float>(lo.row_ss); aa.next_gain = h->gain[l + 1]; aa.xn_out = h->at<bf16>(lo.xn); }
       if (D.d_ff > 0) {
         // full decoder block: the attention rows (bf16) feed the output projection; the residual comes there
         aa.out = h->at<void>(lo.obuf); aa.out_fp32 = 0;

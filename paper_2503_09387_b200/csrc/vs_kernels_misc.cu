@@ -330,7 +330,7 @@ cudaError_t launch_chunk_scores(const BankUpdateArgs& a, const BatchParams& bp, 
 // written once, after the last frame.  (Walking the streaming update's global arrays frame by frame took 6 us a frame, longer
 // than the projection it runs beside; this way it is about 1 us.)  The embeddings move into their slots with the K/V rows.
 __global__ void __launch_bounds__(256, 8) chunk_plan_kernel(BankUpdateArgs a, BatchParams bp) {   // <= 32 registers: fits beside a projection CTA
-  extern __shared__ unsigned short axis[];           // [M] carriers in temporal order (M + 1 + F <= 8192)
+  extern __shared__ unsigned short axis[];           // [M] carriers in temporal order (M + 1 + F <= CHUNK_AXIS_MAX)
   __shared__ double red_s[2][8];
   __shared__ int red_i[2][8];
   __shared__ int slot_of[VS_MAX_BATCH], victim[VS_MAX_BATCH];

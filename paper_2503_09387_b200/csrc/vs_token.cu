@@ -22,10 +22,12 @@
 // Attention: a unit = (token row, KV head, share of the keys) per CTA, all query heads of the group as the 8 columns
 // of S^T = K Q^T and O^T = V^T P^T (see decode_attn_kernel, whose arithmetic this is); the last unit of a row and head to
 // finish combines the shares in order.
-// The whole grid is resident (one CTA per SM, checked at launch), so every wait ends; all are bounded: on expiry the CTA
+// The whole grid is resident (one CTA per SM; that an SM holds one is checked when a handle is made), so every wait ends; all are bounded: on expiry the CTA
 // raises its abort flag, every later wait returns at once, copies in flight are awaited (bounded) and the status is set.
-// (Before: two launches per layer for rows <= 4 -- 11.5 us a layer at the Qwen2-7B shape where the matrix takes 5.1 us of
-// HBM time -- and five for a full decoder layer, 110 us against 71 us.)
+// Where this kernel is taken, and what the launches cost there: token_step_pays.  (At the Qwen2-7B shape one row costs 90 us a full
+// layer, 92 by launches, where its weights take 71 us of HBM time.  Through the attention layers alone it is 16.5 us a layer against
+// 11.4 by the two launches, which is why these still run there: the weights take 5, and two phases a layer leave nothing to hide
+// their waits behind.)
 #include "vs_common.cuh"
 
 namespace vs {
@@ -389,12 +391,12 @@ __global__ void __launch_bounds__(kThreads, 1) token_kernel(const __grid_constan
   uint8_t* ctl = u_base + kUnion + (size_t)NT * 8 * (D / 2) * 8;
   uint4 (*q_s)[kHeads][D / 8] = reinterpret_cast<uint4 (*)[kHeads][D / 8]>(ctl);          // [hi | lo][8][D / 8]
   float2 (*st_ml)[kHeads] = reinterpret_cast<float2 (*)[kHeads]>(ctl + 2 * kHeads * D * 2);
-  float* rsc_s = reinterpret_cast<float*>(ctl + 2 * kHeads * D * 2 + kCW * kHeads * 8);   // [32] row scales
-  float* sum_s = rsc_s + 32;                                                             // [8]
-  unsigned long long* best_s = reinterpret_cast<unsigned long long*>(sum_s + 8);         // [32] greedy-choice keys
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(best_s + 32);
+  float* rsc_s = reinterpret_cast<float*>(ctl + 2 * kHeads * D * 2 + kCW * kHeads * 8);   // [16] row scales
+  float* sum_s = rsc_s + TOK_MAX_ROWS;                                                   // [8]
+  unsigned long long* best_s = reinterpret_cast<unsigned long long*>(sum_s + 8);         // [16] greedy-choice keys
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(best_s + TOK_MAX_ROWS);
   int* bcast = const_cast<int*>(abort_flag) + 1;
-  const uint32_t bars = smem_u32(best_s + 34);
+  const uint32_t bars = smem_u32(best_s + TOK_MAX_ROWS + 2);
   auto full = [&](int s) { return bars + 8u * (uint32_t)s; };                     // the weights' bytes and the 32 lanes that bring the token rows
   auto empty = [&](int s) { return bars + 8u * (uint32_t)(kMaxStages + s); };
   const uint32_t rs_bar = bars + 8u * (uint32_t)(2 * kMaxStages);
@@ -410,7 +412,7 @@ __global__ void __launch_bounds__(kThreads, 1) token_kernel(const __grid_constan
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
-  if (tid < 32) best_s[tid] = 0ull;
+  if (tid < TOK_MAX_ROWS) best_s[tid] = 0ull;
   __syncthreads();
   // Every role walks the phases in order (one loop with the phase as a variable: a copy of the code per phase did not fit
   // the instruction cache).
@@ -481,20 +483,13 @@ __global__ void __launch_bounds__(kThreads, 1) token_kernel(const __grid_constan
         if (!__all_sync(0xffffffffu, mbar_wait(empty(slot), par, abort_flag))) return;
         const uint32_t dst = ring + slot * stage_bytes + kStageW;
         const int k0 = kk * KS;
-        constexpr int CH = KS / 8;                 // 16-byte pieces of a row's slab
-        if (CH == 64) {
-          const bool in0 = k0 + lane * 8 < p.K, in1 = k0 + 256 + lane * 8 < p.K;
+        static_assert(KS == 512, "two 16-byte pieces of a row's slab a lane");
+        const bool in0 = k0 + lane * 8 < p.K, in1 = k0 + 256 + lane * 8 < p.K;
 #pragma unroll 1
-          for (int r = 0; r < rows; ++r) {
-            const bf16* src = x + (size_t)r * p.K + k0 + lane * 8;
-            if (in0) cp_async16(dst + (uint32_t)r * RS + lane * 16, src);
-            if (in1) cp_async16(dst + (uint32_t)r * RS + 512 + lane * 16, src + 256);
-          }
-        } else {
-          const bool in0 = k0 + lane * 8 < p.K;
-#pragma unroll 4
-          for (int r = 0; r < rows; ++r)
-            if (in0) cp_async16(dst + (uint32_t)r * RS + lane * 16, x + (size_t)r * p.K + k0 + lane * 8);
+        for (int r = 0; r < rows; ++r) {
+          const bf16* src = x + (size_t)r * p.K + k0 + lane * 8;
+          if (in0) cp_async16(dst + (uint32_t)r * RS + lane * 16, src);
+          if (in1) cp_async16(dst + (uint32_t)r * RS + 512 + lane * 16, src + 256);
         }
         cp_async_arrive(full(slot));
         if (++kk == p.kst) kk = 0;
@@ -1048,8 +1043,15 @@ cudaError_t launch_shape(TokArgs a, const BatchParams& bp, int n_sms, cudaStream
 }
 template <int D>
 cudaError_t init_head() {
-  cudaError_t e = cudaFuncSetAttribute(token_kernel<D, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynSmem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(token_kernel<D, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynSmem);
+  cudaError_t e = cudaSuccess;
+  auto fits = [&](auto kernel) {       // one CTA of it on an SM
+    int n = 0;
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynSmem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kThreads, kMaxDynSmem);
+    if (e == cudaSuccess && n < 1) e = cudaErrorInvalidConfiguration;
+  };
+  fits(token_kernel<D, 1>);
+  fits(token_kernel<D, 2>);
   return e;
 }
 }  // namespace
