@@ -154,7 +154,7 @@ def test_block_in_chunks_and_carriers_only_forward_through_the_checked_build(che
 
 
 def test_qwen_shape_through_the_checked_build(checked_library):
-    """The kernels' full-size launch shapes (K split over four CTAs, 176-column token tiles, clusters of two in the
+    """The kernels' full-size launch shapes (K split over four CTAs, 176-column token tiles, clusters of four in the
     attention, the matrix-vector projection and the split decode attention) with every workspace store checked:
     one Qwen2-7B-shaped attention layer, bank of 4 so that frames evict; then one layer with RMSNorm, the decoder
     block (d_ff 1024) and the language-model head."""

@@ -246,7 +246,7 @@ def test_chunked_prefill_long_run_with_many_evictions():
 
 def test_chunked_prefill_qwen_shape():
     """One layer at the Qwen2-7B shape, 8 frames per call, 24 frames: the projection of a chunk is a
-    1360-row GEMM (six token tiles, no K split)."""
+    1360-row GEMM (CTA pairs, eight token tiles, no K split)."""
     w = synth.workload("layer", n_frames=24, bank_capacity=16)
     p = Pair(w, max_chunk_frames=8)
     p.text([0], [w.prefix_hidden()], "prefix")
@@ -284,7 +284,7 @@ def test_carriers_only_forward_small():
 
 
 def test_carriers_only_forward_qwen_shape():
-    """64 carriers at the Qwen2-7B shape: a 64-row projection (K split) and a 128-key attention."""
+    """64 carriers at the Qwen2-7B shape: a 64-row projection (K split) and an attention over 128 keys."""
     w = synth.workload("layer", n_frames=70, bank_capacity=64)
     p = Pair(w)
     p.text([0], [w.prefix_hidden()], "prefix")
@@ -577,7 +577,7 @@ def test_deep_stream_all_512_frames_bookkeeping():
 def test_long_key_axis_at_the_qwen_shape():
     """One layer at the Qwen2-7B shape with the 28-layer workload's bank of 512: 511 frames fill the
     bank (the oracle projects their carrier rows only), then three frames in full -- 64 + 511 / 512 +
-    170 = 745 / 746 keys, six key tiles, the last two evicting -- the 32-token question and 8 answer
+    170 = 745 / 746 keys, thirteen key tiles, the last two evicting -- the 32-token question and 8 answer
     tokens (split-KV decode over 609 keys and more)."""
     w = synth.workload("deep", n_layers=1, use_rmsnorm=0, residual=0, n_frames=514, decode_tokens=8)
     p = Pair(w, max_text=w.question_len + w.decode_tokens)
@@ -986,9 +986,9 @@ def test_non_finite_carrier_keeps_the_bank_bookkeeping_in_range():
 
 
 def test_very_large_bank_and_the_chunk_limit():
-    """A bank of 2100 carriers (a key axis of 17 and more 128-key tiles in the prefill attention, split decode over
+    """A bank of 2100 carriers (a key axis of 33 and more key tiles in the prefill attention, split decode over
     2100 keys): filled by frames whose layers the oracle skips, then ten full frames that evict; and the limit of
-    the chunk call's victim bitmap (bank capacity + 1 + frames per call <= 8192)."""
+    the chunk call's bank axis (bank capacity + 1 + frames per call <= 8192)."""
     w = synth.workload("long", d_model=128, n_q_heads=2, n_kv_heads=1, head_dim=64, tokens_per_frame=3, n_frames=2110,
                        bank_capacity=2100, prefix_len=5, question_len=4, decode_tokens=2)
     p = Pair(w, max_text=8)
