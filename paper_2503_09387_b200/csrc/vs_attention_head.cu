@@ -15,6 +15,7 @@
 // alone waits there, combines and writes the row -- no global scratch, no atomics, no polling; the
 // co-scheduled cluster is what guarantees that the barrier completes.
 #include "vs_common.cuh"
+#include "vs_ptx.cuh"
 
 namespace vs {
 
@@ -25,17 +26,9 @@ constexpr int kDecWarps = kDecThreads / 32;
 constexpr int kBatch = 8;     // keys a lane group loads before computing
 constexpr int kMaxCluster = 8;  // portable cluster size: most key splits of one (stream, query head)
 
-__device__ __forceinline__ uint32_t map_shared_rank(uint32_t addr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
 __device__ __forceinline__ void st_shared_cluster_f32(uint32_t addr, float v) {
   asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
 }
-__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_arrive_release() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait_acquire() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 // One CTA = one query head x one key split x one stream.  The heads of a KV group read the
 // same K/V rows from L2; spreading them over CTAs keeps every SM's instruction stream short,

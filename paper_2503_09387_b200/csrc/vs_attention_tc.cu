@@ -27,6 +27,7 @@
 // last S is there, which the first phase of the cluster's barrier tells).
 // All mbarrier waits are bounded.
 #include "vs_common.cuh"
+#include "vs_ptx.cuh"
 #include "vs_bank_update.cuh"
 
 namespace vs {
@@ -36,60 +37,11 @@ namespace {
 constexpr int kKeys = ATTN_KEY_BOX;   // keys per tile = key rows per bulk tensor copy
 constexpr int kRows = 128;       // MMA M
 constexpr int kTok = 16;         // query tokens per CTA
-constexpr unsigned long long kWaitLimitNs = 400ull * 1000ull * 1000ull;
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid) {
-  const int n = valid ? 16 : 0;   // 0 source bytes: the destination is zero-filled
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 __device__ __forceinline__ void fence_async_proxy() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-  return ok != 0;
-}
-// Bounded wait: spins on try_wait (which itself blocks for a short hardware-defined time) and
-// consults the clock only every 1024 failed polls.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-  uint32_t spins = 0;
-  unsigned long long t0 = 0;
-  while (!mbar_try_wait(bar, parity)) {
-    if ((++spins & 1023u) == 0u) {
-      if (*abort_flag) return false;
-      const unsigned long long now = global_ns();
-      if (t0 == 0) t0 = now;
-      else if (now - t0 > kWaitLimitNs) { *abort_flag = 1; return false; }
-    }
-  }
-  return true;
-}
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* tm, int x, int y, int z, uint32_t bar) {
   asm volatile(
       "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
@@ -118,9 +70,6 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t addr, uint32_t lbo, uint3
 __device__ __forceinline__ uint32_t make_idesc(int n, int b_mn) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)b_mn << 16) | ((uint32_t)(n >> 3) << 17) |
          ((uint32_t)(kRows >> 4) << 24);
-}
-__device__ __forceinline__ void umma_commit(uint32_t bar, uint32_t elected) {
-  asm volatile("{\n\t.reg .pred e;\n\tsetp.ne.u32 e, %1, 0;\n\t@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar), "r"(elected) : "memory");
 }
 __device__ __forceinline__ void umma_ss(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t accumulate, uint32_t elected) {
   asm volatile(
@@ -175,13 +124,6 @@ __device__ __forceinline__ float ex2_approx(float x) {
 }
 
 // ---- thread-block cluster: the key splits of one (row tile, KV head, batch entry) -----------------------
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ uint32_t map_shared_rank(uint32_t addr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
 // to a peer's shared memory, counted in bytes on a barrier of the peer's
 __device__ __forceinline__ void st_async_f2(uint32_t addr, float2 v, uint32_t bar) {
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];"
@@ -375,7 +317,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
   VS_STAMP(bp, 2, 1);
 
   __syncwarp();
-  if (nsplit > 1 && warp >= 4) cluster_arrive();   // (first phase; the softmax threads' arrival is the one that means something)
+  if (nsplit > 1 && warp >= 4) cluster_arrive_release();   // (first phase; the softmax threads' arrival is the one that means something)
   float m_run = -INFINITY, l_run = 0.f;      // softmax threads: m_run in the log2 domain (score * scale_log2e), the reference of P and O
   bool ok = true;
   if (warp == kLoaderWarp) {
@@ -512,7 +454,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
       ok = mbar_wait(bar_s(t & 1), (uint32_t)(t >> 1) & 1u, abort_flag) && ok;
       tc_fence_after();
       // (the last S: nothing will read this CTA's query again, its peers may store rows there)
-      if (nsplit > 1 && t == n_tiles - 1) { __syncwarp(); cluster_arrive(); }
+      if (nsplit > 1 && t == n_tiles - 1) { __syncwarp(); cluster_arrive_release(); }
       float sc[kKeys];
       const uint32_t ts = tmem + 64u * (uint32_t)(t & 1) + lane_base;
       tmem_ld32(ts, sc);
@@ -601,9 +543,9 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
     cp_async_commit();
   }
   if (nsplit > 1) {
-    if (warp < 4 && n_tiles == 0) cluster_arrive();
+    if (warp < 4 && n_tiles == 0) cluster_arrive_release();
     if (tid == 0) mbar_arrive_expect_tx(bar_recv, (uint32_t)((nsplit - 1) * G * my_tok * (kRowBytes + 8)));
-    cluster_wait();                 // every peer's query is dead, and its barriers exist
+    cluster_wait_acquire();                 // every peer's query is dead, and its barriers exist
   }
   const int gg = tid >> 4, tk = tid & 15, owner = nsplit == 1 ? 0 : tk / tok_per;      // softmax threads: their row
   if (warp < 4) {
@@ -688,7 +630,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
       }
     }
     __syncthreads();
-    if (nsplit > 1) cluster_arrive();   // this CTA has what it waited for
+    if (nsplit > 1) cluster_arrive_release();   // this CTA has what it waited for
     VS_STAMP(bp, 2, 3);
     // Half a warp per row (lane: units u and, with D = 128, u + 16), two heads of a token side by side, one pair at a time: this
     // code runs once per CTA, and its size -- four rows unrolled: 25 KB -- cost more than the latency that unrolling hides.  The
@@ -801,7 +743,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
   }
   // every CTA of the cluster has what it waited for: nobody's shared memory goes away while a copy may be reading it
   __syncwarp();
-  if (nsplit > 1) cluster_wait();
+  if (nsplit > 1) cluster_wait_acquire();
   tc_fence_before();
   __syncthreads();
   if (warp == kIssuerWarp) {

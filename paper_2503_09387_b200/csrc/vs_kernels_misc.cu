@@ -2,6 +2,7 @@
 //   carrier aggregation (Section 3.3: C = (1/N) sum_i E_i), RoPE table, RMSNorm, eviction
 //   scoring and bank commit (Section 3.3, memory mechanism).
 #include "vs_common.cuh"
+#include "vs_ptx.cuh"
 #include "vs_bank_update.cuh"
 
 namespace vs {
@@ -227,6 +228,7 @@ cudaError_t launch_lm_norm(const void* h, int h_fp32, const bf16* gain, bf16* xn
   return launch_pdl(lm_norm_kernel, dim3(rows), dim3(256), 0, st, h, h_fp32, gain, xn, row_ss, parts, d, dr);
 }
 
+
 // Greedy choice.  (value, index) pairs are compared as "larger value, else equal value and lower
 // index"; a NaN is never larger, so it loses to every number, and a row without any number above
 // -inf gives token 0.  grid = (slices, rows): every block reduces its slice of the row and offers
@@ -234,12 +236,6 @@ cudaError_t launch_lm_norm(const void* h, int h_fp32, const bf16* gain, bf16* xn
 // bits mapped monotonically to an unsigned word on top, the complemented index below -- and the
 // block that arrives last (a ticket per row) turns the key back into the token and clears key and
 // ticket for the next call.
-__device__ __forceinline__ unsigned long long argmax_key(float v, int i) {
-  const uint32_t b = __float_as_uint(v);
-  const uint32_t ordered = (b & 0x80000000u) ? ~b : (b | 0x80000000u);     // ascending with v (no NaN gets here)
-  return ((unsigned long long)ordered << 32) | (uint32_t)(0x7fffffff - i);
-}
-
 __global__ void __launch_bounds__(256) argmax_rows_kernel(const float* __restrict__ logits, int32_t* __restrict__ token,
                                                           unsigned long long* __restrict__ keys, int* __restrict__ tickets, int vocab, DebugRef dr) {
   pdl_wait();

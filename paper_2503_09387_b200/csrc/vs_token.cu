@@ -29,6 +29,7 @@
 // 11.4 by the two launches, which is why these still run there.  Stamps of such a layer: 5.4 us from the projection's input being
 // known to its last store, about 4 for the attention, the other 7 until counters are seen, twice a layer.)
 #include "vs_common.cuh"
+#include "vs_ptx.cuh"
 
 namespace vs {
 
@@ -41,36 +42,11 @@ constexpr int kKeysPerTile = 16;
 constexpr int kHeads = 8;
 constexpr int kMaxStages = 12;
 constexpr int kCntStride = 32;                    // counters lie a cache line apart
-constexpr unsigned long long kWaitLimitNs = 400ull * 1000ull * 1000ull;
 enum { PH_QKV = 0, PH_ATT, PH_WO, PH_GU, PH_DN, PH_LM };
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-  return ok != 0;
-}
 // Bounded; false (at once) when it expired or another role of the CTA already gave up.  (Out of line, like what else runs
 // once a phase: a layer's code has to fit the instruction cache.)
-__device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+__device__ __noinline__ bool stage_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
   uint32_t spins = 0;
   unsigned long long t0 = 0;
   while (!mbar_try_wait(bar, parity)) {
@@ -83,8 +59,8 @@ __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volat
   }
   return true;
 }
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-  return mbar_try_wait(bar, parity) || mbar_wait_slow(bar, parity, abort_flag);
+__device__ __forceinline__ bool stage_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  return mbar_try_wait(bar, parity) || stage_wait_slow(bar, parity, abort_flag);
 }
 __device__ __forceinline__ int ld_acquire(const int* p) {
   int v;
@@ -126,9 +102,6 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* tm,
       "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
       ::"r"(dst), "l"(tm), "r"(x), "r"(y), "r"(z), "r"(w), "r"(bar) : "memory");
 }
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
 // this thread's arrival, once the copies it has issued so far have landed
 __device__ __forceinline__ void cp_async_arrive(uint32_t bar) {
   asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
@@ -143,30 +116,10 @@ __device__ __forceinline__ uint4 lds128(uint32_t addr) {
   asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
   return v;
 }
-__device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-__device__ __forceinline__ uint32_t transpose_8x8(uint32_t v) {
-  uint32_t r;
-  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(r) : "r"(v));
-  return r;
-}
-__device__ __forceinline__ uint32_t pack2(float lo, float hi) {
-  const __nv_bfloat162 t = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<const uint32_t*>(&t);
-}
 __device__ __forceinline__ float2 unpack2(uint32_t w) { return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w)); }
-__device__ __forceinline__ uint32_t word(const uint4& v, int i) { return i == 0 ? v.x : (i == 1 ? v.y : (i == 2 ? v.z : v.w)); }
 __device__ __forceinline__ float ld_bf16_cg(const bf16* p) {
   const unsigned short u = __ldcg(reinterpret_cast<const unsigned short*>(p));
   return __uint_as_float((uint32_t)u << 16);
-}
-// see argmax_rows_kernel: orders like "larger value, else lower index"
-__device__ __forceinline__ unsigned long long argmax_key(float v, int i) {
-  const uint32_t b = __float_as_uint(v);
-  const uint32_t ordered = (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-  return ((unsigned long long)ordered << 32) | (uint32_t)(0x7fffffff - i);
 }
 
 #ifdef VS_TRACE
@@ -439,7 +392,7 @@ __global__ void __launch_bounds__(kThreads, 1) token_kernel(const __grid_constan
         int tile = p.s0 / p.kst, kk = p.s0 - tile * p.kst;
 #pragma unroll 1
         for (int s = p.s0; s < p.s1; ++s, ++n) {
-          if (!mbar_wait(empty(slot), par, abort_flag)) return;
+          if (!stage_wait(empty(slot), par, abort_flag)) return;
           const uint32_t dst = ring + slot * stage_bytes;
           const int kb = kk * (KS / 64);           // (blocks past the end of a row read as zeros)
           mbar_arrive_expect_tx(full(slot), kStageW);
@@ -480,7 +433,7 @@ __global__ void __launch_bounds__(kThreads, 1) token_kernel(const __grid_constan
       int kk = p.s0 % p.kst;
 #pragma unroll 1
       for (int s = p.s0; s < p.s1; ++s) {
-        if (!__all_sync(0xffffffffu, mbar_wait(empty(slot), par, abort_flag))) return;
+        if (!__all_sync(0xffffffffu, stage_wait(empty(slot), par, abort_flag))) return;
         const uint32_t dst = ring + slot * stage_bytes + kStageW;
         const int k0 = kk * KS;
         static_assert(KS == 512, "two 16-byte pieces of a row's slab a lane");
@@ -607,7 +560,7 @@ __global__ void __launch_bounds__(kThreads, 1) token_kernel(const __grid_constan
 #pragma unroll 1
       for (int s = p.s0; s < p.s1; ++s) {
         const int len = min(KS, p.K - kk * KS);
-        mbar_wait(full(slot), par, abort_flag);
+        stage_wait(full(slot), par, abort_flag);
         if (warp == 0 && kind == PH_QKV && s == p.s0) TOK_STAMP(1, l);
         if (warp == 0 && kind == PH_QKV && s == p.s1 - 1) TOK_STAMP(2, l);
         const bool part_ends = kk + 1 == p.kst || s + 1 == p.s1;
@@ -658,7 +611,7 @@ __global__ void __launch_bounds__(kThreads, 1) token_kernel(const __grid_constan
           acc[i][0] = 0.f; acc[i][1] = 0.f; acc[i][2] = 0.f; acc[i][3] = 0.f;
         }
         compute_bar();
-        if (normed) mbar_wait(rs_bar, rs_parity, abort_flag);
+        if (normed) stage_wait(rs_bar, rs_parity, abort_flag);
         if (item < ITEMS) {
           float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
