@@ -1,7 +1,7 @@
 // Decode attention, one CTA per query head: the variant for few streams (see vs_attention.cu for the grouped one).  There
 // the step is a chain of latencies -- a key range's scores, the merges, the store -- and 28 short chains beat four that do
 // seven heads each (11.5 against 13.1 us per layer of the 28-layer token step at the Qwen2-7B shape, bank 512); reading K and V once
-// per head costs nothing while they are few.
+// per head costs nothing while they are few.  It stores single elements, so it also serves an `out` that is not aligned for more.
 // (Section 3.3, decoding phase; Eq. 1 per head with grouped KV heads): one
 // query token per stream attends over [prompt prefix | carrier bank | text of the turn].  No
 // visual-token K/V exists at this point -- only carriers.
