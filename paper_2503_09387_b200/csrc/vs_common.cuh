@@ -374,6 +374,8 @@ struct AttnArgs {
   const int32_t* free_slot;      // free slot of stream s at free_slot[s * free_slot_stride]
   int free_slot_stride;
   int Hq, Hkv, D, slots, M;
+  int G;                         // Hq / Hkv; with the reciprocals (see divide) set by the launch
+  uint32_t rcp_split, rcp_rt, rcp_hkv;
   float scale_log2e;
   // CTAs that share the key tiles of one (row tile, KV head, batch entry): a thread-block cluster of 1 .. 8
   // whose members each take a contiguous run of key tiles and combine through distributed shared memory

@@ -761,7 +761,7 @@ int vs_frame_prefill(vs_stream* h, const int32_t* stream_ids, int32_t n_active, 
     aa.out = last ? out_final : (D.residual ? nullptr : h->at<void>(lo.obuf));
     aa.out_fp32 = D.out_fp32;
     aa.h_in = D.residual ? h_in : nullptr;
-    aa.h_out = D.residual ? h->at<bf16>(lo.hbuf[cur ^ 1]) : nullptr;
+    aa.h_out = D.residual && !last ? h->at<bf16>(lo.hbuf[cur ^ 1]) : nullptr;
     aa.h_out_region = (cur ^ 1) ? DR_HBUF1 : DR_HBUF0;
     if (D.use_rmsnorm && l + 1 < D.L) { aa.ss_out = h->at<float>(lo.row_ss); aa.next_gain = h->gain[l + 1]; aa.xn_out = h->at<bf16>(lo.xn); }
     if (D.d_ff > 0) {
@@ -990,7 +990,7 @@ int vs_frame_prefill_chunk(vs_stream* h, int32_t stream_id, const void* hidden, 
       aa.out = (last || !D.residual) ? layer_out : nullptr;
       aa.out_fp32 = D.out_fp32;
       aa.h_in = D.residual ? h_in : nullptr;
-      aa.h_out = D.residual ? h->at<bf16>(lo.hbuf[cur ^ 1]) : nullptr;
+      aa.h_out = D.residual && !last ? h->at<bf16>(lo.hbuf[cur ^ 1]) : nullptr;
       aa.h_out_region = (cur ^ 1) ? DR_HBUF1 : DR_HBUF0;
       if (D.use_rmsnorm && l + 1 < D.L) { aa.ss_out = h->at<float>(lo.row_ss); aa.next_gain = h->gain[l + 1]; aa.xn_out = h->at<bf16>(lo.xn); }
       if (D.d_ff > 0) {
@@ -1091,10 +1091,11 @@ int vs_bank_forward(vs_stream* h, int32_t stream_id, void* out, void* cuda_strea
     seg_stored(aa.seg[0], h->tm_prefix_k, h->tm_prefix_v, 0, l, D);
     seg_step(aa.seg[1], h->tm_step_k, h->tm_step_v, 3, rows);
     aa.n_seg = 2;
-    aa.out = (l == D.L - 1) ? out : (D.residual ? nullptr : h->at<void>(lo.obuf));
+    const bool last = l == D.L - 1;
+    aa.out = last ? out : (D.residual ? nullptr : h->at<void>(lo.obuf));
     aa.out_fp32 = D.out_fp32;
     aa.h_in = D.residual ? h_in : nullptr;
-    aa.h_out = D.residual ? h->at<bf16>(lo.hbuf[cur ^ 1]) : nullptr;
+    aa.h_out = D.residual && !last ? h->at<bf16>(lo.hbuf[cur ^ 1]) : nullptr;
     aa.h_out_region = (cur ^ 1) ? DR_HBUF1 : DR_HBUF0;
     if (D.use_rmsnorm && l + 1 < D.L) { aa.ss_out = h->at<float>(lo.row_ss); aa.next_gain = h->gain[l + 1]; aa.xn_out = h->at<bf16>(lo.xn); }
     if (D.d_ff > 0) {
@@ -1229,7 +1230,7 @@ int vs_decode_step(vs_stream* h, const int32_t* stream_ids, int32_t n_active, co
     rc = run_projection(h, l, src, rows, fa, bp, st);
     if (rc != VS_OK) return rc;
 
-    bf16* h_out = D.residual ? h->at<bf16>(lo.hbuf[next_buf]) : nullptr;
+    bf16* h_out = D.residual && l + 1 < D.L ? h->at<bf16>(lo.hbuf[next_buf]) : nullptr;
     const int h_out_region = next_buf ? DR_HBUF1 : DR_HBUF0;
     const float scale_log2e = (float)(1.4426950408889634 / std::sqrt((double)D.D));
     if (T == 1) {

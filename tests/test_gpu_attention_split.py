@@ -3,11 +3,12 @@ asked of the library), groups whose rows fill the exchange area and reach out of
 rows or none."""
 import ctypes as C
 
+import numpy as np
 import pytest
 import torch
 
 from paper_2503_09387_b200 import binding, synth
-from tests.parity import Pair
+from tests.parity import Pair, errors, to_dev, to_f64
 
 pytestmark = pytest.mark.gpu
 
@@ -58,4 +59,33 @@ def test_the_cluster_sizes_in_use(G, D, sizes):
             at[s] += T
     assert used == sizes
     p.check_bank(0)
+    p.close()
+
+
+# rows that no cluster shares (many streams), to the least aligned address that is taken; heads that leave softmax warps idle, several layers' residual
+@pytest.mark.parametrize("G,D,L,out_dtype", [(7, 128, 2, 1), (8, 128, 1, 0), (1, 128, 2, 0), (3, 64, 2, 1), (8, 64, 1, 0)])
+def test_rows_without_peers(G, D, L, out_dtype):
+    # (chained layers: flipped roundings of the stored rows reach the next layer's scores, whose size grows with the width -- 7168 wide, one row of
+    # the second layer was 5.1e-2 off at a relative RMS of 4.7e-3.  So no wider than 2688, and 2e-2 * sqrt(L), as the deep chain's test has it.)
+    S, Hkv = 60, 3
+    d = G * Hkv * D
+    w = synth.workload("deep", n_layers=L, d_model=d, n_q_heads=G * Hkv, n_kv_heads=Hkv, head_dim=D, tokens_per_frame=17, n_frames=0, bank_capacity=1,
+                       prefix_len=3, question_len=0, decode_tokens=0, n_streams=S, frame_model="iid", seed=71)
+    p = Pair(w, with_gain=True, max_prefix=160, max_step_tokens=128, out_dtype=out_dtype)
+    at = 0
+    for i, T in enumerate((2, 63, 64, 18)):                   # one to three tiles of keys, ragged row tiles
+        assert _cluster_size(G, D, S * Hkv * ((T + 15) // 16), (at + 63) // 64 + (T + 63) // 64) == 1
+        x = [synth.normal_bf16(w.seed, synth.TAG_QUESTION, (T, d), 1.0, offset=(i * S + s) * 128 * d) for s in range(S)]
+        big = torch.empty(S * T * d + 64, dtype=p.gpu.out_torch_dtype, device="cuda")
+        out = big[4:4 + S * T * d].view(S, T, d)              # 16 bytes (fp32) or 8 (bf16) off
+        p.gpu.decode_step(list(range(S)), to_dev(np.stack(x)), out=out)
+        got = to_f64(out)
+        for s in (0, S - 1):
+            want = p.ora[s].text_step(synth.bf16_bits_to_f64(x[s]))
+            # beside the arithmetic's 2e-2 * sqrt(L): with two or three keys a row is nearly one V row, whose stored elements may have been
+            # rounded to the other neighbour, a unit, at most 2^-7 of the largest |v|, apart; half a unit for rounding to a bf16 output
+            max_abs, rel_rms = errors(got[s], want)
+            tol = 2e-2 * L ** 0.5 + (2.0 ** -7 + (0 if out_dtype else 2.0 ** -8)) * np.max(np.abs(want))
+            assert max_abs <= tol and rel_rms <= 1e-2, (T, s, max_abs, tol, rel_rms)
+        at += T
     p.close()
