@@ -51,19 +51,19 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(DecodeArgs 
 
   // what follows from the parameters alone comes before the wait on the stream's earlier kernels
   const int split = blockIdx.x, hkv = blockIdx.y, b = blockIdx.z;
-  const int sid = bp.stream_id[b];
+  const int sid = bp.entry[b].stream_id;
   const int G = a.Hq / a.Hkv;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = lane >> 2, t4 = lane & 3;
-  const int count = bp.count[b];
+  const int count = bp.entry[b].count;
   const bool bank_full = (a.M > 0 && count == a.M);
   // first phase of the cluster's barrier: "this CTA runs", so that nobody writes into the shared memory of a
   // CTA that has not started; everyone arrives here and waits only just before its remote writes
   if (a.nsplit > 1) cluster_arrive_relaxed();
 
   int P, NB, TL;
-  if (a.to_prefix) { P = bp.prefix_len[b] + 1; NB = 0; TL = 0; }
-  else { P = bp.prefix_len[b]; NB = (a.M == 0) ? 0 : (bank_full ? a.M + 1 : count); TL = bp.text_len[b] + 1; }
+  if (a.to_prefix) { P = bp.entry[b].prefix_len + 1; NB = 0; TL = 0; }
+  else { P = bp.entry[b].prefix_len; NB = (a.M == 0) ? 0 : (bank_full ? a.M + 1 : count); TL = bp.entry[b].text_len + 1; }
   const int Lv = P + NB + TL;
   const int begin = (int)(((long long)Lv * split) / a.nsplit);
   const int end = (int)(((long long)Lv * (split + 1)) / a.nsplit);

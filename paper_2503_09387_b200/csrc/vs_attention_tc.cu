@@ -289,9 +289,9 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
   const int id = (int)blockIdx.x - ((int)blockIdx.x >= a.bank_pos ? a.bank_grid : 0), id2 = divide(id, nsplit, a.rcp_split);
   const int split = id - id2 * nsplit, id3 = divide(id2, n_rt, a.rcp_rt), rt = id2 - id3 * n_rt, b = divide(id3, a.Hkv, a.rcp_hkv);
   const int hkv = id3 - b * a.Hkv, r0 = rt * kTok;
-  const int sid = bp.stream_id[b];
+  const int sid = bp.entry[b].stream_id;
   const int G = a.G;
-  const int count = a.chunk_mode ? a.chunk_count0 : bp.count[b];
+  const int count = a.chunk_mode ? a.chunk_count0 : bp.entry[b].count;
   const bool bank_full = (a.M > 0 && count == a.M);
 
   // the virtual key axis: segments end to end, each starting on a multiple of kKeys keys
@@ -301,10 +301,10 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
   for (int s = 0; s < 4; ++s) {
     int len = 0, kind = -1;
     if (s < a.n_seg) {
-      kind = a.seg[s].kind;
-      if (kind == 0) len = bp.prefix_len[b];
+      kind = a.seg_kind[s];
+      if (kind == 0) len = bp.entry[b].prefix_len;
       else if (kind == 1) { len = (a.M == 0) ? 0 : (bank_full ? a.M + 1 : count); bank_len = len; }
-      else if (kind == 2) len = bp.text_len[b];
+      else if (kind == 2) len = bp.entry[b].text_len;
       else if (kind == 4) len = (a.M == 0) ? 0 : b;                     // carriers of the chunk's frames before this one
       else len = min(rps, r0 + kTok);                                   // later keys are visible to no row of this tile
     }

@@ -268,10 +268,10 @@ __device__ __forceinline__ void bank_update_block(const BankUpdateArgs& a, const
                                                   uint32_t scratch_bytes) {
   const int tid = threadIdx.x;
   const bool on = tid < NT;
-  const int sid = bp.stream_id[b];
+  const int sid = bp.entry[b].stream_id;
   StreamMeta* meta = a.meta + sid;
   const bool meta_ok = VS_STORE_OK(bp, DR_META, meta, sizeof(StreamMeta));
-  if (!a.commit && (a.M == 0 || bp.count[b] < a.M)) return;           // nothing to score
+  if (!a.commit && (a.M == 0 || bp.entry[b].count < a.M)) return;           // nothing to score
   if (a.M == 0) {
     if (block == 0 && tid == 0 && meta_ok) { meta->frames_seen += 1; meta->last_victim_frame = -1; }
     return;
@@ -279,7 +279,7 @@ __device__ __forceinline__ void bank_update_block(const BankUpdateArgs& a, const
   int32_t* order = a.order + (size_t)sid * a.slots;
   int32_t* slot_frame = a.slot_frame + (size_t)sid * a.slots;
   int64_t* slot_pos = a.slot_pos + (size_t)sid * a.slots;
-  const int count = bp.count[b];
+  const int count = bp.entry[b].count;
   const int incoming = (a.incoming_emb != nullptr) ? meta->free_slot : a.step_slot[sid];
   // chunked prefill, a launch per frame: the incoming embedding is read from where it is parked and moved into its slot
   // by whoever commits
@@ -294,12 +294,12 @@ __device__ __forceinline__ void bank_update_block(const BankUpdateArgs& a, const
       if (tid == 0 && VS_STORE_OK(bp, DR_CHUNK_VICTIM, a.record_victim + b, 4)) a.record_victim[b] = -1;
     }
   };
-  const int64_t carrier_pos = bp.pos_base[b] + bp.rows_per_stream - 1;
+  const int64_t carrier_pos = bp.entry[b].pos_base + bp.rows_per_stream - 1;
   if (count < a.M) {
     if (block == 0) adopt();
     if (block == 0 && tid == 0) {
       if (VS_STORE_OK(bp, DR_ORDER, order + count, 4)) order[count] = incoming;
-      if (VS_STORE_OK(bp, DR_SLOT_FRAME, slot_frame + incoming, 4)) slot_frame[incoming] = (int32_t)bp.frame_id[b];
+      if (VS_STORE_OK(bp, DR_SLOT_FRAME, slot_frame + incoming, 4)) slot_frame[incoming] = (int32_t)bp.entry[b].frame_id;
       if (VS_STORE_OK(bp, DR_SLOT_POS, slot_pos + incoming, 8)) slot_pos[incoming] = carrier_pos;
       if (meta_ok) {
         meta->count = count + 1;
@@ -381,11 +381,11 @@ __device__ __forceinline__ void bank_update_block(const BankUpdateArgs& a, const
   if (tid == 0) {
     if (VS_STORE_OK(bp, DR_ORDER, order + count - 1, 4)) order[count - 1] = incoming;
     if (VS_STORE_OK(bp, DR_SLOT_FRAME, slot_frame + victim_slot, 4)) slot_frame[victim_slot] = -1;
-    if (VS_STORE_OK(bp, DR_SLOT_FRAME, slot_frame + incoming, 4)) slot_frame[incoming] = (int32_t)bp.frame_id[b];
+    if (VS_STORE_OK(bp, DR_SLOT_FRAME, slot_frame + incoming, 4)) slot_frame[incoming] = (int32_t)bp.entry[b].frame_id;
     if (VS_STORE_OK(bp, DR_SLOT_POS, slot_pos + incoming, 8)) slot_pos[incoming] = carrier_pos;
     if (a.log_cap > 0) {
       int32_t* e = a.evict_log + ((size_t)sid * a.log_cap + (meta->log_count % a.log_cap)) * 2;
-      if (VS_STORE_OK(bp, DR_EVICT_LOG, e, 8)) { e[0] = (int32_t)bp.frame_id[b]; e[1] = victim_frame; }
+      if (VS_STORE_OK(bp, DR_EVICT_LOG, e, 8)) { e[0] = (int32_t)bp.entry[b].frame_id; e[1] = victim_frame; }
     }
     meta->log_count += 1;
     meta->evictions += 1;

@@ -29,15 +29,20 @@ struct StreamMeta {
 };
 
 // ---- per-call description of the listed streams (passed by value to kernels) -----------
+// One listed stream.  (Side by side: a block finds all it needs to know in one line of the constant cache, which is cold when a
+// kernel starts.)
+struct BatchEntry {
+  int32_t stream_id;
+  int32_t count;                       // carriers in the bank before this step (host mirror)
+  int32_t prefix_len;
+  int32_t text_len;                    // tail length before this step
+  int64_t pos_base;                    // position id of the step's first token
+  int64_t frame_id;                    // frames_seen before this step
+};
 struct BatchParams {
   int32_t n_active;
   int32_t rows_per_stream;             // N + 1 for a frame step, T for a text step
-  int32_t stream_id[VS_MAX_BATCH];
-  int32_t count[VS_MAX_BATCH];         // carriers in the bank before this step (host mirror)
-  int32_t prefix_len[VS_MAX_BATCH];
-  int32_t text_len[VS_MAX_BATCH];      // tail length before this step
-  int64_t pos_base[VS_MAX_BATCH];      // position id of the step's first token
-  int64_t frame_id[VS_MAX_BATCH];      // frames_seen before this step
+  BatchEntry entry[VS_MAX_BATCH];
 #ifdef VS_TRACE
   unsigned long long* trace;           // timeline log of a -DVS_TRACE build, or null
   unsigned trace_seq;                  // sequence number of the launch
@@ -347,19 +352,34 @@ struct BankUpdateArgs {
 constexpr int ATTN_KEY_BOX = 64;   // key rows per bulk tensor copy; segments start on multiples of it on the key axis
 struct AttnSegment {
   CUtensorMap tk, tv;
-  int kind;                      // 0 prefix, 1 bank, 2 tail (earlier tokens of the turn), 3 this step's rows (causal),
-                                 // 4 carriers of the chunk's earlier frames (entry b sees b of them)
   int rows_per_batch;            // row coordinate of batch entry b's first key: b * rows_per_batch
   int z0, z_per_stream;          // Z coordinate = z0 + stream id * z_per_stream + KV head
 };
 struct AttnArgs {
+  // what a block needs to know first, side by side (see BatchEntry)
+  int seg_kind[4];               // of the segments below: 0 prefix, 1 bank, 2 tail (earlier tokens of the turn), 3 this step's rows (causal),
+                                 // 4 carriers of the chunk's earlier frames (entry b sees b of them)
+  int n_seg;
+  // CTAs that share the key tiles of one (row tile, KV head, batch entry): a thread-block cluster of 1 .. 8
+  // whose members each take a contiguous run of key tiles and combine through distributed shared memory
+  int nsplit;
+  // frame steps: the bank update (it needs the carrier embeddings only) is done by bank_grid CTAs of the grid (a multiple
+  // of nsplit; 0: none) from bank_pos (another) on, bank_ctas of them for each listed stream
+  int bank_grid, bank_pos, bank_ctas;
+  int Hq, Hkv, D, slots, M;
+  int G;                         // Hq / Hkv; with the reciprocals (see divide) set by the launch
+  uint32_t rcp_split, rcp_rt, rcp_hkv;
+  // chunk of frames in ONE launch (entry b = frame b): the bank segment is the bank as it was
+  // before the chunk (chunk_count0 carriers) for every frame; what frame b must not see -- the slot
+  // that was free, and whoever the updates of frames 0 .. b-1 evicted (chunk_victim) -- is masked
+  int chunk_mode, chunk_count0;
+  float scale_log2e;
+  const int32_t* chunk_victim;
   const bf16* q;                 // [rows][Hq*D]
   const bf16* q_lo;
   const bf16* q_tiled;           // or: the query as the projection's GEMM leaves it for this kernel, one block per
                                  // (batch entry, 16-token row tile, KV head): [hi | lo][128 rows = g * 16 + token][D],
                                  // 128-byte swizzled like the MMA operand, fetched by one bulk copy
-  AttnSegment seg[4];
-  int n_seg;
   void* out;                     // [rows][Hq*D], bf16 or fp32
   int out_fp32;
   int out_region;                // checked build: the workspace region that out lies in, or -1 (the caller's buffer)
@@ -373,22 +393,8 @@ struct AttnArgs {
   int h_out_region;              // checked build: which residual buffer h_out is (DR_HBUF0 / DR_HBUF1)
   const int32_t* free_slot;      // free slot of stream s at free_slot[s * free_slot_stride]
   int free_slot_stride;
-  int Hq, Hkv, D, slots, M;
-  int G;                         // Hq / Hkv; with the reciprocals (see divide) set by the launch
-  uint32_t rcp_split, rcp_rt, rcp_hkv;
-  float scale_log2e;
-  // CTAs that share the key tiles of one (row tile, KV head, batch entry): a thread-block cluster of 1 .. 8
-  // whose members each take a contiguous run of key tiles and combine through distributed shared memory
-  int nsplit;
-  // frame steps: the bank update (it needs the carrier embeddings only) is done by bank_grid CTAs of the grid (a multiple
-  // of nsplit; 0: none) from bank_pos (another) on, bank_ctas of them for each listed stream
   BankUpdateArgs bank;
-  int bank_grid, bank_pos, bank_ctas;
-  // chunk of frames in ONE launch (entry b = frame b): the bank segment is the bank as it was
-  // before the chunk (chunk_count0 carriers) for every frame; what frame b must not see -- the slot
-  // that was free, and whoever the updates of frames 0 .. b-1 evicted (chunk_victim) -- is masked
-  int chunk_mode, chunk_count0;
-  const int32_t* chunk_victim;
+  AttnSegment seg[4];
 };
 // chunked prefill: the bank update of one frame as a launch of its own (it precedes the projection)
 cudaError_t launch_bank_update(const BankUpdateArgs& a, const BatchParams& bp, bool full, cudaStream_t st);

@@ -219,7 +219,7 @@ __device__ __forceinline__ void finish_row(const ProjectionOut& o, const BatchPa
       *reinterpret_cast<uint2*>(f + half) = w2;
     }
     const int b = row / rps, tt = row - b * rps;
-    const int sid = bp.stream_id[b];
+    const int sid = bp.entry[b].stream_id;
     bf16* dst = nullptr;
     if (o.mode == 0) {
       if (tt == rps - 1 && o.M > 0) {
@@ -227,7 +227,7 @@ __device__ __forceinline__ void finish_row(const ProjectionOut& o, const BatchPa
         dst = (is_k ? o.bank_k : o.bank_v) + (((size_t)sid * o.Hkv + hkv) * o.slots + slot) * D + k0;
       }
     } else if (o.mode != 3) {
-      const int tb = (o.mode == 1) ? bp.prefix_len[b] : bp.text_len[b];
+      const int tb = (o.mode == 1) ? bp.entry[b].prefix_len : bp.entry[b].text_len;
       dst = (is_k ? o.text_k : o.text_v) + (((size_t)sid * o.Hkv + hkv) * o.text_cap + tb + tt) * D + k0;
     }
     // (the carrier row goes to the bank, text rows to the prefix or the tail)

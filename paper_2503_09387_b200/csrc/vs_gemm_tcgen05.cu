@@ -195,7 +195,7 @@ qkv_gemm_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant_
     const int row = n0 + t_begin + (te >> 4);
     if ((m0 + hl * p.o.D + k0) / p.o.D < p.o.Hq + p.o.Hkv && (te >> 4) < slice && row < p.rows) {
       const int b = row / bp.rows_per_stream;
-      const double pos = (double)(bp.pos_base[b] + (row - b * bp.rows_per_stream));
+      const double pos = (double)(bp.entry[b].pos_base + (row - b * bp.rows_per_stream));
       double sn, cs;
       float r[8];
 #pragma unroll

@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(kThreads, 2) qkv_gemv_kernel(const bf16* __res
     fb = fr / bp.rows_per_stream; ftt = fr - fb * bp.rows_per_stream;
     if (rotate) {
       double sn, cs;
-      sincos((double)(bp.pos_base[fb] + ftt) * o.inv_freq[k0], &sn, &cs);
+      sincos((double)(bp.entry[fb].pos_base + ftt) * o.inv_freq[k0], &sn, &cs);
       rc = (float)cs; rsn = (float)sn;
     }
   }
@@ -242,8 +242,8 @@ __global__ void __launch_bounds__(kThreads, 2) qkv_gemv_kernel(const bf16* __res
       const int hkv = is_k ? hs - o.Hq : hs - o.Hq - o.Hkv;
       bf16* f = (is_k ? o.kf : o.vf) + (size_t)row * o.Hkv * D + (size_t)hkv * D + k0;
       if (VS_STORE_OK(bp, is_k ? DR_KF : DR_VF, f, 2) && VS_STORE_OK(bp, is_k ? DR_KF : DR_VF, f + half, 2)) { f[0] = o1; f[half] = o2; }
-      const int sid = bp.stream_id[fb];
-      const int tb = (o.mode == 1) ? bp.prefix_len[fb] : bp.text_len[fb];
+      const int sid = bp.entry[fb].stream_id;
+      const int tb = (o.mode == 1) ? bp.entry[fb].prefix_len : bp.entry[fb].text_len;
       bf16* dst = (is_k ? o.text_k : o.text_v) + (((size_t)sid * o.Hkv + hkv) * o.text_cap + tb + ftt) * D + k0;
       const int dreg = (o.mode == 1) ? (is_k ? DR_PREFIX_K : DR_PREFIX_V) : (is_k ? DR_TAIL_K : DR_TAIL_V);
       if (VS_STORE_OK(bp, dreg, dst, 2) && VS_STORE_OK(bp, dreg, dst + half, 2)) { dst[0] = o1; dst[half] = o2; }

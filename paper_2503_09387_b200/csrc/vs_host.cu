@@ -297,12 +297,16 @@ int attn_split(const vs_stream* h, const BatchParams& bp, const int* key_len, in
 }
 
 // segments of the attention's key axis
-void seg_stored(AttnSegment& sg, const CUtensorMap& k, const CUtensorMap& v, int kind, int layer, const Dims& D) {
-  sg.tk = k; sg.tv = v; sg.kind = kind; sg.rows_per_batch = 0;
+void seg_stored(AttnArgs& aa, int i, const CUtensorMap& k, const CUtensorMap& v, int kind, int layer, const Dims& D) {
+  AttnSegment& sg = aa.seg[i];
+  aa.seg_kind[i] = kind;
+  sg.tk = k; sg.tv = v; sg.rows_per_batch = 0;
   sg.z0 = layer * D.S * D.Hkv; sg.z_per_stream = D.Hkv;
 }
-void seg_step(AttnSegment& sg, const CUtensorMap& k, const CUtensorMap& v, int kind, int rows_per_batch) {
-  sg.tk = k; sg.tv = v; sg.kind = kind; sg.rows_per_batch = rows_per_batch; sg.z0 = 0; sg.z_per_stream = 0;
+void seg_step(AttnArgs& aa, int i, const CUtensorMap& k, const CUtensorMap& v, int kind, int rows_per_batch) {
+  AttnSegment& sg = aa.seg[i];
+  aa.seg_kind[i] = kind;
+  sg.tk = k; sg.tv = v; sg.rows_per_batch = rows_per_batch; sg.z0 = 0; sg.z_per_stream = 0;
 }
 
 // launches the linear layer described by `g` (all but the tiling) on `src` [rows][K]
@@ -686,13 +690,13 @@ int vs_frame_prefill(vs_stream* h, const int32_t* stream_ids, int32_t n_active, 
   bool any_full = false;
   for (int i = 0; i < n_active; ++i) {
     const HostStream& s = h->hs[stream_ids[i]];
-    bp.stream_id[i] = stream_ids[i];
-    bp.count[i] = (int32_t)(s.frames_seen < D.M ? s.frames_seen : D.M);
-    bp.prefix_len[i] = (int32_t)s.prefix_len;
-    bp.text_len[i] = 0;
-    bp.pos_base[i] = s.next_pos;
-    bp.frame_id[i] = s.frames_seen;
-    if (D.M > 0 && bp.count[i] == D.M) any_full = true;
+    bp.entry[i].stream_id = stream_ids[i];
+    bp.entry[i].count = (int32_t)(s.frames_seen < D.M ? s.frames_seen : D.M);
+    bp.entry[i].prefix_len = (int32_t)s.prefix_len;
+    bp.entry[i].text_len = 0;
+    bp.entry[i].pos_base = s.next_pos;
+    bp.entry[i].frame_id = s.frames_seen;
+    if (D.M > 0 && bp.entry[i].count == D.M) any_full = true;
   }
   const int rows = n_active * (N + 1);
   StreamMeta* meta = h->at<StreamMeta>(lo.meta);
@@ -752,9 +756,9 @@ int vs_frame_prefill(vs_stream* h, const int32_t* stream_ids, int32_t n_active, 
     AttnArgs aa;
     std::memset(&aa, 0, sizeof(aa));
     aa.q = fa.q; aa.q_lo = fa.q_lo; aa.q_tiled = fa.q_tiled;
-    seg_stored(aa.seg[0], h->tm_prefix_k, h->tm_prefix_v, 0, l, D);
-    seg_stored(aa.seg[1], h->tm_bank_k, h->tm_bank_v, 1, l, D);
-    seg_step(aa.seg[2], h->tm_step_k, h->tm_step_v, 3, N + 1);
+    seg_stored(aa, 0, h->tm_prefix_k, h->tm_prefix_v, 0, l, D);
+    seg_stored(aa, 1, h->tm_bank_k, h->tm_bank_v, 1, l, D);
+    seg_step(aa, 2, h->tm_step_k, h->tm_step_v, 3, N + 1);
     aa.n_seg = 3;
     const bool last = (l == D.L - 1);
     // a layer whose rows only feed the residual stream stores no output rows
@@ -785,8 +789,8 @@ int vs_frame_prefill(vs_stream* h, const int32_t* stream_ids, int32_t n_active, 
     {
       int kl[3] = {0, 0, N + 1};
       for (int i = 0; i < n_active; ++i) {
-        const int bl = D.M == 0 ? 0 : (bp.count[i] == D.M ? D.M + 1 : bp.count[i]);
-        if (bp.prefix_len[i] + bl > kl[0] + kl[1]) { kl[0] = bp.prefix_len[i]; kl[1] = bl; }
+        const int bl = D.M == 0 ? 0 : (bp.entry[i].count == D.M ? D.M + 1 : bp.entry[i].count);
+        if (bp.entry[i].prefix_len + bl > kl[0] + kl[1]) { kl[0] = bp.entry[i].prefix_len; kl[1] = bl; }
       }
       aa.nsplit = attn_split(h, bp, kl, 3, aa.bank_ctas * n_active);
     }
@@ -841,19 +845,19 @@ int vs_frame_prefill_chunk(vs_stream* h, int32_t stream_id, const void* hidden, 
   bp.rows_per_stream = N + 1;
   for (int j = 0; j < F; ++j) {
     const int64_t seen = hs.frames_seen + j;
-    bp.stream_id[j] = stream_id;
-    bp.count[j] = (int32_t)(seen < D.M ? seen : D.M);
-    bp.prefix_len[j] = (int32_t)hs.prefix_len;
-    bp.text_len[j] = 0;
-    bp.pos_base[j] = hs.next_pos + (int64_t)j * (N + 1);
-    bp.frame_id[j] = seen;
+    bp.entry[j].stream_id = stream_id;
+    bp.entry[j].count = (int32_t)(seen < D.M ? seen : D.M);
+    bp.entry[j].prefix_len = (int32_t)hs.prefix_len;
+    bp.entry[j].text_len = 0;
+    bp.entry[j].pos_base = hs.next_pos + (int64_t)j * (N + 1);
+    bp.entry[j].frame_id = seen;
   }
   auto one_frame = [&](int j) {
     BatchParams b1;
     VS_BP_INIT(h, b1);
     b1.n_active = 1; b1.rows_per_stream = N + 1;
-    b1.stream_id[0] = bp.stream_id[j]; b1.count[0] = bp.count[j]; b1.prefix_len[0] = bp.prefix_len[j];
-    b1.pos_base[0] = bp.pos_base[j]; b1.frame_id[0] = bp.frame_id[j];
+    b1.entry[0].stream_id = bp.entry[j].stream_id; b1.entry[0].count = bp.entry[j].count; b1.entry[0].prefix_len = bp.entry[j].prefix_len;
+    b1.entry[0].pos_base = bp.entry[j].pos_base; b1.entry[0].frame_id = bp.entry[j].frame_id;
     return b1;
   };
   const int rows = F * (N + 1);
@@ -862,7 +866,7 @@ int vs_frame_prefill_chunk(vs_stream* h, int32_t stream_id, const void* hidden, 
   int32_t* chunk_victim = h->at<int32_t>(lo.chunk_victim);
   // the bank as every frame of the chunk finds it on its key axis: the carriers that were there
   // before the chunk (all M + 1 slots once the bank is full)
-  const int count0 = bp.count[0];
+  const int count0 = bp.entry[0].count;
   const int l1 = (D.M > 0 && count0 == D.M) ? D.M + 1 : count0;
   // refused on the bank's capacity, not on its fill, so that a stream does not run into the limit only once its bank is full
   if ((D.M > 0 ? D.M + 1 : 0) + F > CHUNK_AXIS_MAX) return VS_ERR_CAPACITY;
@@ -907,11 +911,11 @@ int vs_frame_prefill_chunk(vs_stream* h, int32_t stream_id, const void* hidden, 
     ba.slot_pos = h->at<int64_t>(lo.slot_pos); ba.evict_log = h->at<int32_t>(lo.evict_log);
     ba.scores = h->at<double>(lo.scores);
     ba.d = D.d; ba.slots = D.slots; ba.M = D.M; ba.policy = D.evict_policy; ba.log_cap = D.log_cap;
-    ba.chunk_first_frame = bp.frame_id[0];
+    ba.chunk_first_frame = bp.entry[0].frame_id;
     ba.chunk_l1 = l1;
     ba.pre_scores = nullptr; ba.pre_stride = 0;
     ba.j0 = 0; ba.j1 = D.M; ba.commit = 1;
-    const bool any_full = D.M > 0 && bp.count[F - 1] == D.M;
+    const bool any_full = D.M > 0 && bp.entry[F - 1].count == D.M;
     if (planned) {
       // the updates score against their incoming carrier only (or not at all): every cosine of the
       // chunk in one launch, then all F updates in turn by one block
@@ -930,7 +934,7 @@ int vs_frame_prefill_chunk(vs_stream* h, int32_t stream_id, const void* hidden, 
         ba.record_slot = chunk_slot + j;
         ba.record_victim = chunk_victim + j;
         const BatchParams b1 = one_frame(j);
-        VS_LAUNCH(h, bst, KC_COMMIT, launch_bank_update(ba, b1, D.M > 0 && b1.count[0] == D.M, bst));
+        VS_LAUNCH(h, bst, KC_COMMIT, launch_bank_update(ba, b1, D.M > 0 && b1.entry[0].count == D.M, bst));
       }
     }
   }
@@ -982,10 +986,10 @@ int vs_frame_prefill_chunk(vs_stream* h, int32_t stream_id, const void* hidden, 
       AttnArgs aa;
       std::memset(&aa, 0, sizeof(aa));
       aa.q = fa.q; aa.q_lo = fa.q_lo; aa.q_tiled = fa.q_tiled;
-      seg_stored(aa.seg[0], h->tm_prefix_k, h->tm_prefix_v, 0, l, D);
-      seg_stored(aa.seg[1], h->tm_bank_k, h->tm_bank_v, 1, l, D);
-      seg_step(aa.seg[2], tm_carr_k, tm_carr_v, 4, 0);
-      seg_step(aa.seg[3], h->tm_step_k, h->tm_step_v, 3, N + 1);
+      seg_stored(aa, 0, h->tm_prefix_k, h->tm_prefix_v, 0, l, D);
+      seg_stored(aa, 1, h->tm_bank_k, h->tm_bank_v, 1, l, D);
+      seg_step(aa, 2, tm_carr_k, tm_carr_v, 4, 0);
+      seg_step(aa, 3, h->tm_step_k, h->tm_step_v, 3, N + 1);
       aa.n_seg = 4;
       aa.out = (last || !D.residual) ? layer_out : nullptr;
       aa.out_fp32 = D.out_fp32;
@@ -1001,7 +1005,7 @@ int vs_frame_prefill_chunk(vs_stream* h, int32_t stream_id, const void* hidden, 
       aa.free_slot = chunk_slot; aa.free_slot_stride = 0;
       aa.chunk_mode = 1; aa.chunk_count0 = count0; aa.chunk_victim = chunk_victim;
       {
-        const int kl[4] = {bp.prefix_len[0], D.M == 0 ? 0 : l1, D.M == 0 ? 0 : F - 1, N + 1};
+        const int kl[4] = {bp.entry[0].prefix_len, D.M == 0 ? 0 : l1, D.M == 0 ? 0 : F - 1, N + 1};
         aa.nsplit = attn_split(h, bp, kl, 4, 0);
       }
       aa.Hq = D.Hq; aa.Hkv = D.Hkv; aa.D = D.D; aa.slots = D.slots; aa.M = D.M;
@@ -1051,9 +1055,9 @@ int vs_bank_forward(vs_stream* h, int32_t stream_id, void* out, void* cuda_strea
   VS_BP_INIT(h, bp);
   bp.n_active = 1;
   bp.rows_per_stream = count;
-  bp.stream_id[0] = stream_id;
-  bp.prefix_len[0] = (int32_t)hs.prefix_len;
-  bp.pos_base[0] = hs.prefix_len;
+  bp.entry[0].stream_id = stream_id;
+  bp.entry[0].prefix_len = (int32_t)hs.prefix_len;
+  bp.entry[0].pos_base = hs.prefix_len;
   const int rows = count;
   VS_LAUNCH(h, st, KC_OTHER, launch_gather_carriers(h->at<bf16>(lo.emb), h->at<int32_t>(lo.order), h->at<bf16>(lo.hbuf[0]),
                                                     stream_id, D.slots, D.d, count, debug_ref(h), st));
@@ -1088,8 +1092,8 @@ int vs_bank_forward(vs_stream* h, int32_t stream_id, void* out, void* cuda_strea
     AttnArgs aa;
     std::memset(&aa, 0, sizeof(aa));
     aa.q = fa.q; aa.q_lo = fa.q_lo; aa.q_tiled = fa.q_tiled;
-    seg_stored(aa.seg[0], h->tm_prefix_k, h->tm_prefix_v, 0, l, D);
-    seg_step(aa.seg[1], h->tm_step_k, h->tm_step_v, 3, rows);
+    seg_stored(aa, 0, h->tm_prefix_k, h->tm_prefix_v, 0, l, D);
+    seg_step(aa, 1, h->tm_step_k, h->tm_step_v, 3, rows);
     aa.n_seg = 2;
     const bool last = l == D.L - 1;
     aa.out = last ? out : (D.residual ? nullptr : h->at<void>(lo.obuf));
@@ -1105,7 +1109,7 @@ int vs_bank_forward(vs_stream* h, int32_t stream_id, void* out, void* cuda_strea
     aa.free_slot = h->at<int32_t>(lo.step_slot); aa.free_slot_stride = 0;
     aa.Hq = D.Hq; aa.Hkv = D.Hkv; aa.D = D.D; aa.slots = D.slots; aa.M = 0;      // no bank segment on this key axis
     {
-      const int kl[2] = {bp.prefix_len[0], rows};
+      const int kl[2] = {bp.entry[0].prefix_len, rows};
       aa.nsplit = attn_split(h, bp, kl, 2, 0);
     }
     aa.scale_log2e = (float)(1.4426950408889634 / std::sqrt((double)D.D));
@@ -1152,13 +1156,13 @@ int vs_decode_step(vs_stream* h, const int32_t* stream_ids, int32_t n_active, co
   int max_keys = 0;
   for (int i = 0; i < n_active; ++i) {
     const HostStream& s = h->hs[stream_ids[i]];
-    bp.stream_id[i] = stream_ids[i];
-    bp.count[i] = (int32_t)(s.frames_seen < D.M ? s.frames_seen : D.M);
-    bp.prefix_len[i] = (int32_t)s.prefix_len;
-    bp.text_len[i] = (int32_t)s.text_len;
-    bp.pos_base[i] = to_prefix ? s.next_pos : s.next_pos + s.text_len;
-    bp.frame_id[i] = s.frames_seen;
-    const int keys = (int)s.prefix_len + bp.count[i] + 1 + (int)s.text_len + T;
+    bp.entry[i].stream_id = stream_ids[i];
+    bp.entry[i].count = (int32_t)(s.frames_seen < D.M ? s.frames_seen : D.M);
+    bp.entry[i].prefix_len = (int32_t)s.prefix_len;
+    bp.entry[i].text_len = (int32_t)s.text_len;
+    bp.entry[i].pos_base = to_prefix ? s.next_pos : s.next_pos + s.text_len;
+    bp.entry[i].frame_id = s.frames_seen;
+    const int keys = (int)s.prefix_len + bp.entry[i].count + 1 + (int)s.text_len + T;
     if (keys > max_keys) max_keys = keys;
   }
   const int rows = n_active * T;
@@ -1270,19 +1274,19 @@ int vs_decode_step(vs_stream* h, const int32_t* stream_ids, int32_t n_active, co
       std::memset(&aa, 0, sizeof(aa));
       aa.q = fa.q; aa.q_lo = fa.q_lo; aa.q_tiled = fa.q_tiled;
       int ns = 0;
-      seg_stored(aa.seg[ns++], h->tm_prefix_k, h->tm_prefix_v, 0, l, D);
+      seg_stored(aa, ns++, h->tm_prefix_k, h->tm_prefix_v, 0, l, D);
       if (!to_prefix) {
-        seg_stored(aa.seg[ns++], h->tm_bank_k, h->tm_bank_v, 1, l, D);
-        seg_stored(aa.seg[ns++], h->tm_tail_k, h->tm_tail_v, 2, l, D);
+        seg_stored(aa, ns++, h->tm_bank_k, h->tm_bank_v, 1, l, D);
+        seg_stored(aa, ns++, h->tm_tail_k, h->tm_tail_v, 2, l, D);
       }
-      seg_step(aa.seg[ns++], h->tm_step_k, h->tm_step_v, 3, T);
+      seg_step(aa, ns++, h->tm_step_k, h->tm_step_v, 3, T);
       aa.n_seg = ns;
       {
         int kl[4] = {0, 0, 0, T};
         for (int i = 0; i < n_active; ++i) {
-          const int bl = (to_prefix || D.M == 0) ? 0 : (bp.count[i] == D.M ? D.M + 1 : bp.count[i]);
-          const int tl = to_prefix ? 0 : bp.text_len[i];
-          if (bp.prefix_len[i] + bl + tl > kl[0] + kl[1] + kl[2]) { kl[0] = bp.prefix_len[i]; kl[1] = bl; kl[2] = tl; }
+          const int bl = (to_prefix || D.M == 0) ? 0 : (bp.entry[i].count == D.M ? D.M + 1 : bp.entry[i].count);
+          const int tl = to_prefix ? 0 : bp.entry[i].text_len;
+          if (bp.entry[i].prefix_len + bl + tl > kl[0] + kl[1] + kl[2]) { kl[0] = bp.entry[i].prefix_len; kl[1] = bl; kl[2] = tl; }
         }
         aa.nsplit = attn_split(h, bp, kl, 4, 0);
       }
@@ -1327,7 +1331,7 @@ int vs_reset_stream(vs_stream* h, const int32_t* stream_ids, int32_t n_active, v
   BatchParams bp;
   VS_BP_INIT(h, bp);
   bp.n_active = n_active;
-  for (int i = 0; i < n_active; ++i) bp.stream_id[i] = stream_ids[i];
+  for (int i = 0; i < n_active; ++i) bp.entry[i].stream_id = stream_ids[i];
   VS_LAUNCH(h, st, KC_OTHER, launch_reset(h->at<StreamMeta>(h->lo.meta), h->at<int32_t>(h->lo.slot_frame), D.slots, bp, st));
   for (int i = 0; i < n_active; ++i) h->hs[stream_ids[i]] = HostStream();
   h->last_stream = st;

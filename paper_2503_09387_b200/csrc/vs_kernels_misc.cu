@@ -26,9 +26,9 @@ __device__ __forceinline__ bf16 f64_to_bf16_rne(double x) {
 __global__ void __launch_bounds__(256) pool_kernel(PoolArgs a, BatchParams bp, int pool_blocks) {
   // what depends on the parameters alone comes before the wait on the stream's earlier kernels
   const int b = blockIdx.y;
-  const int sid = bp.stream_id[b];
+  const int sid = bp.entry[b].stream_id;
   const int N = a.N, d = a.d;
-  const long long pos0 = bp.pos_base[b];
+  const long long pos0 = bp.entry[b].pos_base;
   VS_STAMP(bp, 0, 0);
   if ((int)blockIdx.x >= pool_blocks) {
     pdl_wait();
@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(256) rope_table_kernel(RopeArgs a, BatchParams
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= T * half) return;
   const int r = idx / half, k = idx - r * half;
-  const double ang = (double)(bp.pos_base[b] + r) * a.inv_freq[k];
+  const double ang = (double)(bp.entry[b].pos_base + r) * a.inv_freq[k];
   double s, c;
   sincos(ang, &s, &c);
   float2* rp = a.rope + ((size_t)b * T + r) * half + k;
@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(128, 8) chunk_scores_kernel(BankUpdateArgs a, 
   const int b = blockIdx.y, lane = threadIdx.x & 31;
   const int c = blockIdx.x * 4 + (threadIdx.x >> 5);
   if (c >= a.chunk_l1 + b) return;                                 // uniform over the warp
-  const int sid = bp.stream_id[b];
+  const int sid = bp.entry[b].stream_id;
   const bf16* va = (c < a.chunk_l1) ? a.emb + ((size_t)sid * a.slots + c) * a.d : emb_stage + (size_t)(c - a.chunk_l1) * a.d;
   double dot, na, nb;
   warp_dot_norms<16>(va, emb_stage + (size_t)b * a.d, a.d, lane, dot, na, nb);
@@ -333,7 +333,7 @@ __global__ void __launch_bounds__(256, 8) chunk_plan_kernel(BankUpdateArgs a, Ba
   pdl_wait();
   pdl_launch_dependents();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int F = bp.n_active, sid = bp.stream_id[0], l1 = a.chunk_l1;
+  const int F = bp.n_active, sid = bp.entry[0].stream_id, l1 = a.chunk_l1;
   StreamMeta* meta = a.meta + sid;
   const bool meta_ok = VS_STORE_OK(bp, DR_META, meta, sizeof(StreamMeta));
   int32_t* order = a.order + (size_t)sid * a.slots;
@@ -343,7 +343,7 @@ __global__ void __launch_bounds__(256, 8) chunk_plan_kernel(BankUpdateArgs a, Ba
     if (tid == 0 && meta_ok) { meta->frames_seen += F; meta->last_victim_frame = -1; }
     return;
   }
-  int count = bp.count[0], free_slot = meta->free_slot;
+  int count = bp.entry[0].count, free_slot = meta->free_slot;
   for (int i = tid; i < count; i += 256) axis[i] = (unsigned short)order[i];
   __syncthreads();
   int evicted = 0;
@@ -411,7 +411,7 @@ __global__ void __launch_bounds__(256, 8) chunk_plan_kernel(BankUpdateArgs a, Ba
       const int n = evicted - (F - tid);
       if (evicted - n <= a.log_cap) {
         int32_t* e = a.evict_log + ((size_t)sid * a.log_cap + ((first_log + n) % a.log_cap)) * 2;
-        if (VS_STORE_OK(bp, DR_EVICT_LOG, e, 8)) { e[0] = (int32_t)bp.frame_id[tid]; e[1] = my_victim_frame; }
+        if (VS_STORE_OK(bp, DR_EVICT_LOG, e, 8)) { e[0] = (int32_t)bp.entry[tid].frame_id; e[1] = my_victim_frame; }
       }
     }
   }
@@ -421,8 +421,8 @@ __global__ void __launch_bounds__(256, 8) chunk_plan_kernel(BankUpdateArgs a, Ba
     const int c = axis[i], sl = (c < l1) ? c : slot_of[c - l1];
     if (VS_STORE_OK(bp, DR_ORDER, order + i, 4)) order[i] = sl;
     if (c >= l1) {
-      if (VS_STORE_OK(bp, DR_SLOT_FRAME, slot_frame + sl, 4)) slot_frame[sl] = (int32_t)bp.frame_id[c - l1];
-      if (VS_STORE_OK(bp, DR_SLOT_POS, slot_pos + sl, 8)) slot_pos[sl] = bp.pos_base[c - l1] + bp.rows_per_stream - 1;
+      if (VS_STORE_OK(bp, DR_SLOT_FRAME, slot_frame + sl, 4)) slot_frame[sl] = (int32_t)bp.entry[c - l1].frame_id;
+      if (VS_STORE_OK(bp, DR_SLOT_POS, slot_pos + sl, 8)) slot_pos[sl] = bp.entry[c - l1].pos_base + bp.rows_per_stream - 1;
     }
   }
   if (tid == 0 && meta_ok) {
@@ -497,7 +497,7 @@ cudaError_t launch_poison(void* p, size_t bytes, cudaStream_t st) {
 // because nothing reads a slot that the metadata does not list
 __global__ void reset_kernel(StreamMeta* meta, int32_t* slot_frame, int slots, BatchParams bp) {
   pdl_wait();
-  const int sid = bp.stream_id[blockIdx.x];
+  const int sid = bp.entry[blockIdx.x].stream_id;
   for (int i = threadIdx.x; i < slots; i += blockDim.x)
     if (VS_STORE_OK(bp, DR_SLOT_FRAME, slot_frame + (size_t)sid * slots + i, 4)) slot_frame[(size_t)sid * slots + i] = -1;
   if (threadIdx.x == 0 && VS_STORE_OK(bp, DR_META, meta + sid, sizeof(StreamMeta))) {

@@ -248,8 +248,8 @@ __device__ __forceinline__ void finish_item(const TokArgs& a, const BatchParams&
         const int hkv = is_k ? hs - a.Hq : hs - a.Hq - a.Hkv;
         bf16* f = (is_k ? a.kf : a.vf) + ((size_t)row * a.Hkv + hkv) * D + k0;
         if (VS_STORE_OK(bp, is_k ? DR_KF : DR_VF, f, 2) && VS_STORE_OK(bp, is_k ? DR_KF : DR_VF, f + half, 2)) { f[0] = o1; f[half] = o2; }
-        const int b = row / rps, tt = row - b * rps, sid = bp.stream_id[b];
-        const int tb = a.to_prefix ? bp.prefix_len[b] : bp.text_len[b], cap = a.to_prefix ? a.maxP : a.maxT;
+        const int b = row / rps, tt = row - b * rps, sid = bp.entry[b].stream_id;
+        const int tb = a.to_prefix ? bp.entry[b].prefix_len : bp.entry[b].text_len, cap = a.to_prefix ? a.maxP : a.maxT;
         bf16* base = a.to_prefix ? (is_k ? a.prefix_k : a.prefix_v) + (size_t)l * a.ls_prefix : (is_k ? a.tail_k : a.tail_v) + (size_t)l * a.ls_tail;
         bf16* dst = base + (((size_t)sid * a.Hkv + hkv) * cap + tb + tt) * D + k0;
         const int dreg = a.to_prefix ? (is_k ? DR_PREFIX_K : DR_PREFIX_V) : (is_k ? DR_TAIL_K : DR_TAIL_V);
@@ -495,7 +495,7 @@ __global__ void __launch_bounds__(kThreads, 1) token_kernel(const __grid_constan
       for (int i = tid; i < rows * (D / 2); i += kCT) {
         const int row = i / (D / 2), k = i - row * (D / 2), b = row / rps;
         double sn, cs;
-        sincos((double)(bp.pos_base[b] + (row - b * rps)) * a.inv_freq[k], &sn, &cs);
+        sincos((double)(bp.entry[b].pos_base + (row - b * rps)) * a.inv_freq[k], &sn, &cs);
         rope_s[i] = make_float2((float)cs, (float)sn);
       }
     pdl_wait();
@@ -663,11 +663,11 @@ __global__ void __launch_bounds__(kThreads, 1) token_kernel(const __grid_constan
       Unit x;
       const int split = u % a.nsplit, rh = u / a.nsplit;
       x.hkv = rh % a.Hkv; x.row = rh / a.Hkv;
-      const int b = x.row / rps, tt = x.row - b * rps, sid = bp.stream_id[b];
-      const bool bank_full = a.M > 0 && bp.count[b] == a.M;
+      const int b = x.row / rps, tt = x.row - b * rps, sid = bp.entry[b].stream_id;
+      const bool bank_full = a.M > 0 && bp.entry[b].count == a.M;
       int NB, TL;
-      if (a.to_prefix) { x.P = bp.prefix_len[b] + tt + 1; NB = 0; TL = 0; }
-      else { x.P = bp.prefix_len[b]; NB = (a.M == 0) ? 0 : (bank_full ? a.M + 1 : bp.count[b]); TL = bp.text_len[b] + tt + 1; }
+      if (a.to_prefix) { x.P = bp.entry[b].prefix_len + tt + 1; NB = 0; TL = 0; }
+      else { x.P = bp.entry[b].prefix_len; NB = (a.M == 0) ? 0 : (bank_full ? a.M + 1 : bp.entry[b].count); TL = bp.entry[b].text_len + tt + 1; }
       x.PB = x.P + NB;
       const int Lv = x.PB + TL;
       x.fresh = Lv - tt - 1;
