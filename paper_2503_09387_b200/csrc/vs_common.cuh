@@ -442,6 +442,7 @@ struct DecodeArgs {
   float scale_log2e;
 };
 cudaError_t launch_decode_attention_heads(const DecodeArgs& a, const BatchParams& bp, cudaStream_t st);   // a CTA per query head
+cudaError_t decode_attention_init();     // opt-in shared memory attribute, once per process/device
 cudaError_t launch_decode_attention(const DecodeArgs& a, const BatchParams& bp, cudaStream_t st);
 
 // A step of up to TOK_MAX_ROWS token rows through all layers, or the language-model head of as many rows: one persistent

@@ -600,7 +600,7 @@ int vs_create_stream(const vs_config* cfg, const vs_weights* weights, void* work
     h->gain_f = static_cast<const bf16*>(weights->norm_f_w);
     if (encode_2d(h, &h->tm_lm, weights->w_lm, (uint64_t)D.d, (uint64_t)D.vocab, GEMM_BLOCK_M) != VS_OK) return fail(VS_ERR_CUDA);
   }
-  if (pair_gemm_init() != cudaSuccess || qkv_gemm_init() != cudaSuccess || qkv_gemv_init() != cudaSuccess || token_step_init() != cudaSuccess || prefill_attention_tc_init() != cudaSuccess) return fail(VS_ERR_CUDA);
+  if (pair_gemm_init() != cudaSuccess || qkv_gemm_init() != cudaSuccess || qkv_gemv_init() != cudaSuccess || token_step_init() != cudaSuccess || prefill_attention_tc_init() != cudaSuccess || decode_attention_init() != cudaSuccess) return fail(VS_ERR_CUDA);
   h->n_pairs = pair_gemm_max_pairs();
   if (h->n_pairs < 1) return fail(VS_ERR_CUDA);
   for (int sp = 2; sp <= ATTN_MAX_SPLIT; ++sp) h->attn_clusters[sp] = 2 * prefill_attention_max_clusters(D.D, sp);
