@@ -22,8 +22,8 @@
 // (Section 3.2: only the carrier keeps its K/V), text rows are appended to the prefix or to the
 // turn's tail.
 //
-// Per CTA: 6 or 18 warps.  Warp 0 lane 0 = TMA producer, warp 1 = TMEM allocator + MMA issuer
-// (lane 0), warps 2.. = epilogue, 4 or 16 of them (tcgen05.ld of the 32-lane quarter that
+// Per CTA: 6, 10 or 18 warps.  Warp 0 lane 0 = TMA producer, warp 1 = TMEM allocator + MMA issuer
+// (lane 0), warps 2.. = epilogue, 4, 8 or 16 of them (tcgen05.ld of the 32-lane quarter that
 // warp % 4 allows; with 16, four warps per quarter take every fourth block of 16 columns).
 // Every mbarrier wait is bounded; on expiry the CTA raises an abort flag, records
 // VS_ERR_DEVICE_TIMEOUT, lets in-flight copies land, frees its tensor memory and exits.
@@ -37,6 +37,10 @@ using namespace gemm;
 
 constexpr int kMaxEpiWarps = 16;                 // 4 per scheduler: the epilogue is bound by instruction latency
 constexpr int kMaxThreads = 64 + 32 * kMaxEpiWarps;
+// Up to 16 rows without a table: ten warps of 80 registers and six stages, so that a CTA of the decode attention (eight warps of 128
+// registers, 106 KB) fits beside this one and has its first keys when the projection is done.  (Sixteen finishing warps of 96, eight stages:
+// 16 streams of 1150 keys 26.6 us, 25.7 this way.)
+constexpr int kFewBound = 768, kFewWarps = 8, kFewStages = 6;   // (threads that would fill the register file at 80 each)
 // Instruction descriptor, kind::f16: D = fp32, A = B = bf16, both K-major, M = 128, N = n.
 __device__ __forceinline__ uint32_t make_idesc(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(GEMM_BLOCK_M >> 4) << 24);
@@ -68,7 +72,7 @@ __device__ __forceinline__ int ld_acquire_gpu(const int* p) {
 __host__ __device__ inline int first_block(int r, int n_blk, int ksplit) { return (r * n_blk + ksplit - 1) / ksplit; }
 
 template <bool kOwnRope>   // no RoPE table, every finishing thread derives the rotation of its one row
-__global__ void __launch_bounds__(kMaxThreads, 1)
+__global__ void __launch_bounds__(kOwnRope ? kFewBound : kMaxThreads, 1)
 qkv_gemm_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_x,
                 const __grid_constant__ CUtensorMap tm_w2, KernelParams p, BatchParams bp) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -373,9 +377,11 @@ cudaError_t launch_qkv_gemm(const GemmArgs& a, const BatchParams& bp, cudaStream
   if (a.tile_n < 16 || a.tile_n > 256 || (a.tile_n & 15) || 128 % a.out.D != 0) return cudaErrorInvalidValue;
   p.xchg = a.xchg;
   p.flags = a.flags;
+  const bool own_rope = a.out.rope == nullptr && a.out.mode < 4;
   const int stage_bytes = kStageABytes + a.tile_n * 128, most_kb = (p.total_kb + a.ksplit - 1) / a.ksplit;
   int stages = (kMaxDynSmem - 3072) / stage_bytes;
-  if (stages > 8) stages = 8;
+  const int most = own_rope ? kFewStages : 8;
+  if (stages > most) stages = most;
   if (stages > most_kb) stages = most_kb;
   if (stages < 1) return cudaErrorInvalidValue;
   p.stages = stages;
@@ -390,15 +396,15 @@ cudaError_t launch_qkv_gemm(const GemmArgs& a, const BatchParams& bp, cudaStream
   p.data_bytes = (uint32_t)data;
   const size_t smem = 1024 + data + 16 * stages + 64 + 1024;     // + the slice's RMSNorm row scales
   if (smem > (size_t)kMaxDynSmem) return cudaErrorInvalidValue;
-  // a step of few rows is finished by 4 warps; others by 16, which overlap one another's latency
-  const int threads = 64 + 32 * (a.rows <= 8 ? 4 : kMaxEpiWarps);
+  // a step of few rows is finished by 4 or 8 warps; others by 16, which overlap one another's latency
+  const int threads = 64 + 32 * (a.rows <= 8 ? 4 : (own_rope ? kFewWarps : kMaxEpiWarps));
   // without a RoPE table every finishing thread must have at most one row
-  if (a.out.rope == nullptr && a.out.mode < 4 && (a.out.inv_freq == nullptr || a.rows > 2 * (threads / 32 - 2))) return cudaErrorInvalidValue;
+  if (own_rope && (a.out.inv_freq == nullptr || a.rows > 2 * (threads / 32 - 2))) return cudaErrorInvalidValue;
   const dim3 grid((a.E_out + GEMM_BLOCK_M - 1) / GEMM_BLOCK_M, a.n_tiles, a.ksplit);
   // the CTAs of a K split wait for one another: the whole grid has to be resident at once (a CTA an SM always fits)
   if (a.ksplit > 1 && (a.xchg == nullptr || a.flags == nullptr || (long long)grid.x * grid.y * grid.z > a.n_sms ||
                        (long long)grid.x * grid.y * grid.z > GEMM_XCHG_CTAS)) return cudaErrorInvalidValue;
-  if (a.out.rope == nullptr && a.out.mode < 4) return launch_pdl(qkv_gemm_kernel<true>, grid, dim3(threads), smem, st, a.tm_w, a.tm_x, a.tm_w2, p, bp);
+  if (own_rope) return launch_pdl(qkv_gemm_kernel<true>, grid, dim3(threads), smem, st, a.tm_w, a.tm_x, a.tm_w2, p, bp);
   return launch_pdl(qkv_gemm_kernel<false>, grid, dim3(threads), smem, st, a.tm_w, a.tm_x, a.tm_w2, p, bp);
 }
 
