@@ -308,6 +308,7 @@ struct GemmArgs {
   int* flags;                    // [m_tiles*n_tiles][ksplit], zero between launches
   int n_sms;
   int* status;
+  int beside_attention;          // CTAs of the prefill attention that runs right ahead of or behind this launch, or 0
 };
 struct Tiling { int tile_n, n_tiles, ksplit, pairs; };
 Tiling choose_tiles(int K, int E, int n_sms, int max_pairs, int rows, bool own_rope);

@@ -41,6 +41,17 @@ constexpr int kMaxThreads = 64 + 32 * kMaxEpiWarps;
 // registers, 106 KB) fits beside this one and has its first keys when the projection is done.  (Sixteen finishing warps of 96, eight stages:
 // 16 streams of 1150 keys 26.6 us, 25.7 this way.)
 constexpr int kFewBound = 768, kFewWarps = 8, kFewStages = 6;   // (threads that would fill the register file at 80 each)
+// The same beside the prefill attention (ten warps of 96 registers, 113 KB): whether a projection of 17 to 48 rows, or the W_o behind the
+// attention, leaves room for one of its CTAs, which then has its set-up and first keys behind it when the projection is done, as this
+// block has its first weights when the attention is.  The price is depth, five stages of weights for eight, which a step whose attention
+// takes few SMs had on all others anyway.  Whole steps of 8 layers over 128 to 830 keys, us without and with: 48 rows 195 to 208 / 190 to
+// 197; 32 rows 183 / 182 to 185 over few keys (up to 48 attention CTAs), 194 / 190 over many; 20 rows 176 / 182; 64 rows, four stages,
+// 193 / 203.  Where K leaves no more stages anyway it costs nothing: 6 small layers of 30 rows 123 / 119.5.
+constexpr int kSlimSmem = 113 * 1024;
+inline bool goes_beside_attention(const GemmArgs& a, int most_kb, int slim_stages) {
+  return a.beside_attention > 0 && a.rows <= 48 &&
+         (most_kb <= slim_stages || a.rows > 32 || (a.rows > 24 && 8 * a.beside_attention >= 3 * a.n_sms));
+}
 // Instruction descriptor, kind::f16: D = fp32, A = B = bf16, both K-major, M = 128, N = n.
 __device__ __forceinline__ uint32_t make_idesc(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(GEMM_BLOCK_M >> 4) << 24);
@@ -380,6 +391,9 @@ cudaError_t launch_qkv_gemm(const GemmArgs& a, const BatchParams& bp, cudaStream
   const bool own_rope = a.out.rope == nullptr && a.out.mode < 4;
   const int stage_bytes = kStageABytes + a.tile_n * 128, most_kb = (p.total_kb + a.ksplit - 1) / a.ksplit;
   int stages = (kMaxDynSmem - 3072) / stage_bytes;
+  const int slim_stages = (kSlimSmem - 3072) / stage_bytes;
+  const bool slim = !own_rope && goes_beside_attention(a, most_kb, slim_stages);
+  if (slim) stages = slim_stages;
   const int most = own_rope ? kFewStages : 8;
   if (stages > most) stages = most;
   if (stages > most_kb) stages = most_kb;
@@ -397,7 +411,7 @@ cudaError_t launch_qkv_gemm(const GemmArgs& a, const BatchParams& bp, cudaStream
   const size_t smem = 1024 + data + 16 * stages + 64 + 1024;     // + the slice's RMSNorm row scales
   if (smem > (size_t)kMaxDynSmem) return cudaErrorInvalidValue;
   // a step of few rows is finished by 4 or 8 warps; others by 16, which overlap one another's latency
-  const int threads = 64 + 32 * (a.rows <= 8 ? 4 : (own_rope ? kFewWarps : kMaxEpiWarps));
+  const int threads = 64 + 32 * (a.rows <= 8 ? 4 : (own_rope || slim ? kFewWarps : kMaxEpiWarps));
   // without a RoPE table every finishing thread must have at most one row
   if (own_rope && (a.out.inv_freq == nullptr || a.rows > 2 * (threads / 32 - 2))) return cudaErrorInvalidValue;
   const dim3 grid((a.E_out + GEMM_BLOCK_M - 1) / GEMM_BLOCK_M, a.n_tiles, a.ksplit);
