@@ -60,18 +60,22 @@ __device__ __forceinline__ void bias_of(const ProjectionOut& o, const Place& pl,
   }
 }
 
+// What a launch does with a finished row, known when the code is compiled: the projection (modes 0 to 3), or mode 4, 5 or 6.  (One
+// kernel with all of them: the code of a row is run once or twice a launch, so what lies between its parts is fetched for nothing.)
+enum Finish { FIN_PROJECT = 0, FIN_RESIDUAL = 4, FIN_SWIGLU = 5, FIN_LOGITS = 6 };
 // What the finishing of a token row reads from global memory, asked for ahead of the arithmetic.
 struct FinishIn { float4 ra, rb; uint2 r1, r2; };
+template <int kFin>
 __device__ __forceinline__ FinishIn finish_in(const ProjectionOut& o, const Place& pl, int E_out, int m0e, int row) {
   FinishIn in;
   in.ra = in.rb = make_float4(1.f, 0.f, 1.f, 0.f);
   in.r1 = in.r2 = make_uint2(0u, 0u);
-  if (pl.rotate) {
+  if (kFin == FIN_PROJECT && pl.rotate) {
     const float2* rp = o.rope + (size_t)row * (o.D >> 1) + pl.k0;
     in.ra = *reinterpret_cast<const float4*>(rp);
     in.rb = *reinterpret_cast<const float4*>(rp + 2);
   }
-  if (o.mode == 4 && o.lin_res != nullptr) {
+  if (kFin == FIN_RESIDUAL && o.lin_res != nullptr) {
     const bf16* rp = o.lin_res + (size_t)row * E_out + m0e + pl.f1;
     in.r1 = *reinterpret_cast<const uint2*>(rp);
     in.r2 = *reinterpret_cast<const uint2*>(rp + (pl.f2 - pl.f1));
@@ -80,6 +84,7 @@ __device__ __forceinline__ FinishIn finish_in(const ProjectionOut& o, const Plac
 }
 
 // a1, a2: the summed products of the row's four pairs.  te & 15 == threadIdx.x & 15 within the half warp that shares the row.
+template <int kFin>
 __device__ __forceinline__ void finish_row(const ProjectionOut& o, const BatchParams& bp, const Place& pl, int E_out, int m0e, int row,
                                            const float4& a1, const float4& a2, float rsc, const float (&bb1)[4], const float (&bb2)[4],
                                            const FinishIn& in, int te) {
@@ -87,7 +92,7 @@ __device__ __forceinline__ void finish_row(const ProjectionOut& o, const BatchPa
   float x1[4] = {a1.x, a1.y, a1.z, a1.w}, x2[4] = {a2.x, a2.y, a2.z, a2.w};
 #pragma unroll
   for (int i = 0; i < 4; ++i) { x1[i] = fmaf(x1[i], rsc, bb1[i]); x2[i] = fmaf(x2[i], rsc, bb2[i]); }
-  if (pl.rotate) {
+  if (kFin == FIN_PROJECT && pl.rotate) {
     const float cs[4] = {in.ra.x, in.ra.z, in.rb.x, in.rb.z}, sn[4] = {in.ra.y, in.ra.w, in.rb.y, in.rb.w};
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -96,7 +101,7 @@ __device__ __forceinline__ void finish_row(const ProjectionOut& o, const BatchPa
       x1[i] = y1; x2[i] = y2;
     }
   }
-  if (o.mode == 5) {
+  if constexpr (kFin == FIN_SWIGLU) {
     // SwiGLU: features f1.. are gate rows, f2 = f1 + 64.. the matching up rows
     __align__(8) bf16 av[4];
 #pragma unroll
@@ -105,14 +110,14 @@ __device__ __forceinline__ void finish_row(const ProjectionOut& o, const BatchPa
     if (VS_STORE_OK(bp, o.lin_out_region, dst, 8)) *reinterpret_cast<uint2*>(dst) = *reinterpret_cast<const uint2*>(av);
     return;
   }
-  if (o.mode == 6) {
+  if constexpr (kFin == FIN_LOGITS) {
     // plain linear layer, rows kept in fp32 (logits of the vocabulary projection); the buffer is the caller's
     float* fo = static_cast<float*>(o.final_out) + (size_t)row * E_out + m0e;
     *reinterpret_cast<float4*>(fo + f1) = make_float4(x1[0], x1[1], x1[2], x1[3]);
     *reinterpret_cast<float4*>(fo + f2) = make_float4(x2[0], x2[1], x2[2], x2[3]);
     return;
   }
-  if (o.mode == 4) {
+  if constexpr (kFin == FIN_RESIDUAL) {
     // linear layer + residual; the rows as stored (bf16) also give the next RMSNorm its statistics
     const size_t c1 = (size_t)row * E_out + m0e + f1, c2 = (size_t)row * E_out + m0e + f2;
     if (o.lin_res != nullptr) {

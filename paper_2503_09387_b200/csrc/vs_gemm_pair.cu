@@ -71,7 +71,7 @@ struct PairParams {
 struct Tile { int m0, n0; };
 
 // The epilogue warps of one CTA: every tile's 128 x tile_n accumulator, in the order the issuer fills them.
-template <typename TileFn>
+template <int kFin, typename TileFn>
 __device__ __forceinline__ void epilogue_role(const PairParams& p, const BatchParams& bp, uint32_t tmem, float* staging, float* rsc_all,
                                               volatile int* abort_flag, uint32_t acc_full0, uint32_t acc_empty0, int warp, int lane, int pair,
                                               int n_pairs, int n_items, TileFn tile) {
@@ -108,7 +108,7 @@ __device__ __forceinline__ void epilogue_role(const PairParams& p, const BatchPa
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
         const int row = t.n0 + (c0 + u) * 16 + (te >> 4);
-        if (pl.on && row < p.rows) in[u] = finish_in(p.o, pl, p.E_out, t.m0, row);
+        if (pl.on && row < p.rows) in[u] = finish_in<kFin>(p.o, pl, p.E_out, t.m0, row);
       }
       float* st = staging + buf * (kChunk * kPitch);
       buf ^= 1;
@@ -135,12 +135,13 @@ __device__ __forceinline__ void epilogue_role(const PairParams& p, const BatchPa
         const float4 a1 = *reinterpret_cast<const float4*>(st + tok * kPitch + pl.f1);
         const float4 a2 = *reinterpret_cast<const float4*>(st + tok * kPitch + pl.f2);
         // RMSNorm's row scale commutes with the projection: applied here, in fp32
-        finish_row(p.o, bp, pl, p.E_out, t.m0, row, a1, a2, p.o.row_ss != nullptr ? rsc_s[c0 * 16 + tok] : 1.f, bb1, bb2, in[u], te);
+        finish_row<kFin>(p.o, bp, pl, p.E_out, t.m0, row, a1, a2, p.o.row_ss != nullptr ? rsc_s[c0 * 16 + tok] : 1.f, bb1, bb2, in[u], te);
       }
     }
   }
 }
 
+template <int kFin>
 __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
 pair_gemm_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_x,
                  const __grid_constant__ CUtensorMap tm_w2, const __grid_constant__ PairParams p, const __grid_constant__ BatchParams bp) {
@@ -200,7 +201,7 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant
       auto load_w = [&](const Tile& t, int kb, int s) {
         const uint32_t dst = base + (uint32_t)s * stage_bytes, bar = map_shared_rank(full_bar(s), 0u);
         if (rank == 0) mbar_arrive_expect_tx(full_bar(s), 2u * stage_bytes);      // the bytes of both CTAs
-        if (p.o.mode == 5) {
+        if constexpr (kFin == FIN_SWIGLU) {
           // a 128-row tile = 64 rows of the gate matrix, then the same 64 rows of the up matrix
           tma_load_2d_pair(dst, &tm_w, kb * GEMM_BLOCK_K, t.m0 >> 1, bar);
           tma_load_2d_pair(dst + kStageABytes / 2, &tm_w2, kb * GEMM_BLOCK_K, t.m0 >> 1, bar);
@@ -274,7 +275,7 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant
     }
   } else {
     pdl_wait();
-    epilogue_role(p, bp, tmem, staging, rsc_s, abort_flag, acc_full(0), acc_empty(0), warp, lane, pair, n_pairs, n_items, tile);
+    epilogue_role<kFin>(p, bp, tmem, staging, rsc_s, abort_flag, acc_full(0), acc_empty(0), warp, lane, pair, n_pairs, n_items, tile);
   }
 
   tcgen05_fence_before();
@@ -290,9 +291,25 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant
 
 size_t fixed_smem(int stages) { return 1024 + kStagingBytes + 2 * 256 * 4 + 16 * (size_t)stages + 64; }
 
+using Kernel = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const PairParams, const BatchParams);
+Kernel kernel_of(int mode) {
+  switch (mode) {
+    case FIN_RESIDUAL: return pair_gemm_kernel<FIN_RESIDUAL>;
+    case FIN_SWIGLU: return pair_gemm_kernel<FIN_SWIGLU>;
+    case FIN_LOGITS: return pair_gemm_kernel<FIN_LOGITS>;
+    default: return pair_gemm_kernel<FIN_PROJECT>;
+  }
+}
+
 }  // namespace
 
-cudaError_t pair_gemm_init() { return cudaFuncSetAttribute(pair_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem); }
+cudaError_t pair_gemm_init() {
+  for (int mode : {(int)FIN_PROJECT, (int)FIN_RESIDUAL, (int)FIN_SWIGLU, (int)FIN_LOGITS}) {
+    const cudaError_t e = cudaFuncSetAttribute((const void*)kernel_of(mode), cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
 
 // CTA pairs of this kernel that can be resident at once on the current device; 0 if the query fails
 int pair_gemm_max_pairs() {
@@ -303,7 +320,7 @@ int pair_gemm_max_pairs() {
   attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr; cfg.numAttrs = 1;
   int pairs = 0;
-  if (cudaOccupancyMaxActiveClusters(&pairs, pair_gemm_kernel, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
+  if (cudaOccupancyMaxActiveClusters(&pairs, kernel_of(FIN_PROJECT), &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
   return pairs;
 }
 
@@ -328,7 +345,7 @@ cudaError_t launch_pair_gemm(const GemmArgs& a, int max_pairs, const BatchParams
   while (cols < a.tile_n) cols <<= 1;
   p.acc_cols = cols;
   const int items = p.m_tiles * p.n_tiles, pairs = items < max_pairs ? items : max_pairs;
-  return launch_pdl(pair_gemm_kernel, dim3(2 * pairs), dim3(kThreads), (size_t)stages * stage_bytes + fixed_smem(stages), st, a.tm_w, a.tm_x, a.tm_w2, p, bp);
+  return launch_pdl(kernel_of(a.out.mode), dim3(2 * pairs), dim3(kThreads), (size_t)stages * stage_bytes + fixed_smem(stages), st, a.tm_w, a.tm_x, a.tm_w2, p, bp);
 }
 
 }  // namespace vs

@@ -82,7 +82,7 @@ __device__ __forceinline__ int ld_acquire_gpu(const int* p) {
 // first token block (of n_blk) that share r of a K split owns
 __host__ __device__ inline int first_block(int r, int n_blk, int ksplit) { return (r * n_blk + ksplit - 1) / ksplit; }
 
-template <bool kOwnRope>   // no RoPE table, every finishing thread derives the rotation of its one row
+template <int kFin, bool kOwnRope>   // kOwnRope: no RoPE table, every finishing thread derives the rotation of its one row
 __global__ void __launch_bounds__(kOwnRope ? kFewBound : kMaxThreads, 1)
 qkv_gemm_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_x,
                 const __grid_constant__ CUtensorMap tm_w2, KernelParams p, BatchParams bp) {
@@ -133,7 +133,7 @@ qkv_gemm_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant_
     const int s = kb % p.stages, kx = (kb0 + kb) * GEMM_BLOCK_K;
     const uint32_t a_dst = base + (uint32_t)s * stage_bytes;
     mbar_arrive_expect_tx(full_bar(s), stage_bytes);
-    if (p.o.mode == 5) {
+    if constexpr (kFin == FIN_SWIGLU) {
       // a 128-row tile = 64 rows of the gate matrix, then the same 64 rows of the up matrix
       tma_load_2d(a_dst, &tm_w, kx, m0 >> 1, full_bar(s));
       tma_load_2d(a_dst + kStageABytes / 2, &tm_w2, kx, m0 >> 1, full_bar(s));
@@ -328,7 +328,7 @@ qkv_gemm_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant_
           }
         }
         if (!kOwnRope || !pl.rotate) {
-          R.in = finish_in(p.o, pl, p.E_out, m0, row);
+          R.in = finish_in<kFin>(p.o, pl, p.E_out, m0, row);
         } else {                         // the thread's only row (the launch checks it)
           R.in.ra = own_ra; R.in.rb = own_rb;
         }
@@ -346,7 +346,7 @@ qkv_gemm_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant_
             a2.x += R.v2[r].x; a2.y += R.v2[r].y; a2.z += R.v2[r].z; a2.w += R.v2[r].w;
           }
         }
-        finish_row(p.o, bp, pl, p.E_out, m0, row, a1, a2, R.rsc, bb1, bb2, R.in, te);
+        finish_row<kFin>(p.o, bp, pl, p.E_out, m0, row, a1, a2, R.rsc, bb1, bb2, R.in, te);
       };
       // four warps per scheduler overlap one another's load latency; a thread holds one row at a time
 #pragma unroll 1
@@ -367,11 +367,25 @@ qkv_gemm_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant_
   VS_STAMP(bp, 1, 15);
 }
 
+using Kernel = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, KernelParams, BatchParams);
+Kernel kernel_of(int mode, bool own_rope) {
+  switch (mode) {
+    case FIN_RESIDUAL: return qkv_gemm_kernel<FIN_RESIDUAL, false>;
+    case FIN_SWIGLU: return qkv_gemm_kernel<FIN_SWIGLU, false>;
+    case FIN_LOGITS: return qkv_gemm_kernel<FIN_LOGITS, false>;
+    default: return own_rope ? qkv_gemm_kernel<FIN_PROJECT, true> : qkv_gemm_kernel<FIN_PROJECT, false>;
+  }
+}
+
 }  // namespace
 
 cudaError_t qkv_gemm_init() {
-  const cudaError_t e = cudaFuncSetAttribute(qkv_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
-  return e != cudaSuccess ? e : cudaFuncSetAttribute(qkv_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
+  for (int mode : {(int)FIN_PROJECT, (int)FIN_RESIDUAL, (int)FIN_SWIGLU, (int)FIN_LOGITS})
+    for (bool own_rope : {false, true}) {
+      const cudaError_t e = cudaFuncSetAttribute((const void*)kernel_of(mode, own_rope), cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
+      if (e != cudaSuccess) return e;
+    }
+  return cudaSuccess;
 }
 
 cudaError_t launch_qkv_gemm(const GemmArgs& a, const BatchParams& bp, cudaStream_t st) {
@@ -418,8 +432,7 @@ cudaError_t launch_qkv_gemm(const GemmArgs& a, const BatchParams& bp, cudaStream
   // the CTAs of a K split wait for one another: the whole grid has to be resident at once (a CTA an SM always fits)
   if (a.ksplit > 1 && (a.xchg == nullptr || a.flags == nullptr || (long long)grid.x * grid.y * grid.z > a.n_sms ||
                        (long long)grid.x * grid.y * grid.z > GEMM_XCHG_CTAS)) return cudaErrorInvalidValue;
-  if (own_rope) return launch_pdl(qkv_gemm_kernel<true>, grid, dim3(threads), smem, st, a.tm_w, a.tm_x, a.tm_w2, p, bp);
-  return launch_pdl(qkv_gemm_kernel<false>, grid, dim3(threads), smem, st, a.tm_w, a.tm_x, a.tm_w2, p, bp);
+  return launch_pdl(kernel_of(a.out.mode, own_rope), grid, dim3(threads), smem, st, a.tm_w, a.tm_x, a.tm_w2, p, bp);
 }
 
 }  // namespace vs
