@@ -10,10 +10,11 @@
 // (One CTA per tile of 256 rows, epilogue after the main loop: 0.88 PFLOP/s on the 2720 rows of a 16-frame chunk through full
 // decoder layers; this kernel 1.2, power-capped clocks included.)
 //
-// The epilogue (8 warps) takes 32 tokens at a time through shared memory, so that a thread finishes both elements of four
+// The epilogue (16 warps; with 8, two tokens a thread and chunk, five streams of 121 rows took 259 us for 6 layers, now 250, a full-model
+// frame 4.11 and 4.09 ms) takes 32 tokens at a time through shared memory, so that a thread finishes both elements of four
 // rotation pairs of a token and stores 8-byte pieces.
-// Per CTA 10 warps.  Warp 0 lane 0 = TMA loader (weights are constant: a launch's first stages of them are requested before the
-// wait on the stream's earlier kernels), warp 1 = TMEM allocator, its lane 0 in the pair's first CTA the MMA issuer, warps 2..9
+// Per CTA 18 warps.  Warp 0 lane 0 = TMA loader (weights are constant: a launch's first stages of them are requested before the
+// wait on the stream's earlier kernels), warp 1 = TMEM allocator, its lane 0 in the pair's first CTA the MMA issuer, warps 2..17
 // the epilogue (tcgen05.ld of the 32-lane quarter that warp % 4 allows).  Every wait is bounded; on expiry the CTA raises an
 // abort flag, records VS_ERR_DEVICE_TIMEOUT, lets in-flight copies land, frees its tensor memory and exits.
 // No copy is multicast: the halves each CTA loads are its own.
@@ -25,7 +26,7 @@ namespace {
 
 using namespace gemm;
 
-constexpr int kEpiWarps = 8;
+constexpr int kEpiWarps = 16;
 constexpr int kEpiThreads = kEpiWarps * 32;
 constexpr int kThreads = 64 + kEpiThreads;
 constexpr int kChunk = 32;                                      // tokens the epilogue stages at a time
@@ -62,6 +63,11 @@ __device__ __forceinline__ void umma_commit_pair(uint32_t bar, uint32_t elected)
                ::"r"(bar), "h"((uint16_t)3), "r"(elected) : "memory");
 }
 
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(taddr) : "memory");
+}
+
 struct PairParams {
   ProjectionOut o;
   int* status;
@@ -75,10 +81,10 @@ template <int kFin, typename TileFn>
 __device__ __forceinline__ void epilogue_role(const PairParams& p, const BatchParams& bp, uint32_t tmem, float* staging, float* rsc_all,
                                               volatile int* abort_flag, uint32_t acc_full0, uint32_t acc_empty0, int warp, int lane, int pair,
                                               int n_pairs, int n_items, TileFn tile) {
-  const int te = (int)threadIdx.x - 64;                  // 0 .. 255
-  const int quarter = warp & 3, second = (warp - 2) >> 2;  // TMEM lanes this warp may read; which 16 tokens of a chunk
-  auto epi_bar = [] { asm volatile("bar.sync 1, 256;" ::: "memory"); };
-  static_assert(kEpiThreads == 256, "the named barrier above counts 256 threads");
+  const int te = (int)threadIdx.x - 64;                  // 0 .. 511
+  const int quarter = warp & 3, eighth = (warp - 2) >> 2;  // TMEM lanes this warp may read; which 8 tokens of a chunk
+  auto epi_bar = [] { asm volatile("bar.sync 1, 512;" ::: "memory"); };
+  static_assert(kEpiThreads == 512 && kChunk == 32, "the named barrier above counts 512 threads, half a warp to a token");
   int j = 0, buf = 0;
 #pragma unroll 1
   for (int i = pair; i < n_items; i += n_pairs, ++j) {
@@ -104,21 +110,19 @@ __device__ __forceinline__ void epilogue_role(const PairParams& p, const BatchPa
     VS_STAMP_BY(bp, 1, 2, 64);        // accumulator complete
 #pragma unroll 1
     for (int c0 = 0; c0 < n_blk; c0 += 2) {              // 32 tokens at a time, two staging buffers
-      FinishIn in[2];
-#pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const int row = t.n0 + (c0 + u) * 16 + (te >> 4);
-        if (pl.on && row < p.rows) in[u] = finish_in<kFin>(p.o, pl, p.E_out, t.m0, row);
-      }
+      const int tok = te >> 4, row = t.n0 + c0 * 16 + tok;
+      const bool mine = pl.on && c0 + (tok >> 4) < n_blk && row < p.rows;
+      FinishIn in;
+      if (mine) in = finish_in<kFin>(p.o, pl, p.E_out, t.m0, row);
       float* st = staging + buf * (kChunk * kPitch);
       buf ^= 1;
-      if (c0 + second < n_blk && ok) {
-        uint32_t r[16];
-        tmem_ld16(tm + (uint32_t)((c0 + second) * 16), r);
+      if (c0 + (eighth >> 1) < n_blk && ok) {
+        uint32_t r[8];
+        tmem_ld8(tm + (uint32_t)(c0 * 16 + eighth * 8), r);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        float* d = st + (16 * second) * kPitch + quarter * 32 + lane;
+        float* d = st + (8 * eighth) * kPitch + quarter * 32 + lane;
 #pragma unroll
-        for (int k = 0; k < 16; ++k) d[k * kPitch] = __uint_as_float(r[k]);
+        for (int k = 0; k < 8; ++k) d[k * kPitch] = __uint_as_float(r[k]);
       }
       if (c0 + 2 >= n_blk) {
         // this warp has read its last part of the accumulator: once all have, the issuer may fill it again
@@ -128,14 +132,11 @@ __device__ __forceinline__ void epilogue_role(const PairParams& p, const BatchPa
       }
       // (one barrier a chunk: the buffer written next is the one read a chunk ago, which every thread has left by the barrier)
       epi_bar();
-#pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const int tok = 16 * u + (te >> 4), row = t.n0 + c0 * 16 + tok;
-        if (!pl.on || c0 + u >= n_blk || row >= p.rows || *abort_flag) continue;
+      if (mine && !*abort_flag) {
         const float4 a1 = *reinterpret_cast<const float4*>(st + tok * kPitch + pl.f1);
         const float4 a2 = *reinterpret_cast<const float4*>(st + tok * kPitch + pl.f2);
         // RMSNorm's row scale commutes with the projection: applied here, in fp32
-        finish_row<kFin>(p.o, bp, pl, p.E_out, t.m0, row, a1, a2, p.o.row_ss != nullptr ? rsc_s[c0 * 16 + tok] : 1.f, bb1, bb2, in[u], te);
+        finish_row<kFin>(p.o, bp, pl, p.E_out, t.m0, row, a1, a2, p.o.row_ss != nullptr ? rsc_s[c0 * 16 + tok] : 1.f, bb1, bb2, in, te);
       }
     }
   }
