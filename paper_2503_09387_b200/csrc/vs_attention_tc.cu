@@ -233,10 +233,14 @@ struct Exchange {
   __host__ __device__ uint32_t staged(int i) const { return (uint32_t)(L::kCtl - (staged_rows() - i) * kRowBytes); }
 };
 
-template <int D>
+// What a launch stores, known when the code is compiled: rows (fp32 or bf16), or the residual stream that they are added to.
+enum Stored { ST_ROWS_FP32, ST_ROWS_BF16, ST_RESIDUAL };
+template <int D, int kStored>
 __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const __grid_constant__ AttnArgs a,
                                                                           const __grid_constant__ BatchParams bp, int* status) {
   extern __shared__ __align__(1024) uint8_t gbase[];
+  constexpr bool residual = kStored == ST_RESIDUAL, rows_out = !residual, rows_fp32 = kStored == ST_ROWS_FP32;
+  const bool sums = residual && a.ss_out != nullptr;
   using L = Smem<D>;
   constexpr int CPR = D / 8, NS = L::kStages;
   const uint32_t base = smem_u32(gbase);
@@ -633,7 +637,6 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
     // side.  (Through shared memory, half a warp to a row: 5.5 us a CTA.)
     if (soft) {
       constexpr int NB = D / 64;
-      const bool res = a.h_out != nullptr;
       size_t at[2];
       bool on[2];
 #pragma unroll
@@ -644,7 +647,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
       for (int c = 0; c < NB; ++c)
 #pragma unroll
         for (int i = 0; i < 16; ++i)
-          hv[c][i] = (res && on[i & 1]) ? *reinterpret_cast<const uint32_t*>(a.h_in + at[i & 1] + 64 * c + 8 * (i >> 1)) : 0u;
+          hv[c][i] = (residual && on[i & 1]) ? *reinterpret_cast<const uint32_t*>(a.h_in + at[i & 1] + 64 * c + 8 * (i >> 1)) : 0u;
       ok = wait_o() && ok;
       __syncwarp();
       tc_fence_after();
@@ -663,8 +666,8 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
           if (!on[r]) continue;
           const float v0 = v[2 * i] * inv[r], v1 = v[2 * i + 1] * inv[r];
           const size_t e = at[r] + 64 * c + 8 * (i >> 1);
-          if (a.out != nullptr) {                                        // (null: a layer whose rows only feed the residual stream)
-            if (a.out_fp32) {
+          if constexpr (rows_out) {
+            if constexpr (rows_fp32) {
               float* o = static_cast<float*>(a.out) + e;
               if (VS_STORE_OK(bp, a.out_region, o, 8)) *reinterpret_cast<float2*>(o) = make_float2(v0, v1);
             } else {
@@ -672,11 +675,11 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
               if (VS_STORE_OK(bp, a.out_region, o, 4)) *reinterpret_cast<uint32_t*>(o) = pack2(v0, v1);
             }
           }
-          if (res) {
+          if constexpr (residual) {
             const float2 h = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&hv[c][i]));
             const uint32_t w = pack2(h.x + v0, h.y + v1);
             if (VS_STORE_OK(bp, a.h_out_region, a.h_out + e, 4)) *reinterpret_cast<uint32_t*>(a.h_out + e) = w;
-            if (a.ss_out != nullptr) {
+            if (sums) {
               // RMSNorm of the next layer: its statistics are those of the rows as stored (bf16)
               const float2 s = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w));
               ss[r] += s.x * s.x + s.y * s.y;
@@ -690,7 +693,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
           }
         }
       }
-      if (a.ss_out != nullptr) {
+      if (sums) {
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
           ss[r] += __shfl_xor_sync(0xffffffffu, ss[r], 1);
@@ -712,7 +715,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
       r.at = row0 + (size_t)(split * tok_per + r.tl) * tok_step + (size_t)r.g * D + 4 * u;
       return r;
     };
-    auto load_res = [&](const Row& r) { return (a.h_out != nullptr && r.on) ? *reinterpret_cast<const uint2*>(a.h_in + r.at) : make_uint2(0u, 0u); };
+    auto load_res = [&](const Row& r) { return (residual && r.on) ? *reinterpret_cast<const uint2*>(a.h_in + r.at) : make_uint2(0u, 0u); };
     __syncwarp();
     if (soft && n_tiles == 0) cluster_arrive_release();
     if (tid == 0) mbar_arrive_expect_tx(bar_recv, (uint32_t)((nsplit - 1) * G * my_tok * (kRowBytes + 8)));
@@ -827,20 +830,20 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
         ss[k] = 0.f;
         if (!rw[k].on) continue;
         const size_t e = rw[k].at;
-        if (a.out != nullptr) {                                        // (null: a layer whose rows only feed the residual stream)
-          if (a.out_fp32) {
+        if constexpr (rows_out) {
+          if constexpr (rows_fp32) {
             if (VS_STORE_OK(bp, a.out_region, static_cast<float*>(a.out) + e, 16)) *reinterpret_cast<float4*>(static_cast<float*>(a.out) + e) = v[k];
           } else {
             const uint2 w = make_uint2(pack2(v[k].x, v[k].y), pack2(v[k].z, v[k].w));
             if (VS_STORE_OK(bp, a.out_region, static_cast<bf16*>(a.out) + e, 8)) *reinterpret_cast<uint2*>(static_cast<bf16*>(a.out) + e) = w;
           }
         }
-        if (a.h_out != nullptr) {
+        if constexpr (residual) {
           const float2 h0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&h[k].x));
           const float2 h1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&h[k].y));
           const uint2 w = make_uint2(pack2(h0.x + v[k].x, h0.y + v[k].y), pack2(h1.x + v[k].z, h1.y + v[k].w));
           if (VS_STORE_OK(bp, a.h_out_region, a.h_out + e, 8)) *reinterpret_cast<uint2*>(a.h_out + e) = w;
-          if (a.ss_out != nullptr) {
+          if (sums) {
             // RMSNorm of the next layer: its statistics are those of the rows as stored (bf16)
             const float2 s0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w.x)), s1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w.y));
             ss[k] = (s0.x * s0.x + s0.y * s0.y) + (s1.x * s1.x + s1.y * s1.y);
@@ -855,7 +858,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
           }
         }
       }
-      if (a.ss_out != nullptr) {
+      if (sums) {
 #pragma unroll
         for (int k = 0; k < U; ++k) {
 #pragma unroll
@@ -865,7 +868,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
       }
     }
   }
-  if (a.ss_out != nullptr) {
+  if (sums) {
     // the token's sum of squares over this KV head's query heads, in head order; the projection adds the KV heads' parts in
     // order
     __syncthreads();
@@ -893,17 +896,27 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
   VS_STAMP(bp, 2, 15);
 }
 
+using Kernel = void (*)(const AttnArgs, const BatchParams, int*);
+template <int D>
+Kernel kernel_of(Stored what) {
+  return what == ST_RESIDUAL ? prefill_attn_tc_kernel<D, ST_RESIDUAL> : what == ST_ROWS_FP32 ? prefill_attn_tc_kernel<D, ST_ROWS_FP32> : prefill_attn_tc_kernel<D, ST_ROWS_BF16>;
+}
+template <int D>
+cudaError_t init() {
+  for (Stored what : {ST_ROWS_FP32, ST_ROWS_BF16, ST_RESIDUAL}) {
+    const void* k = reinterpret_cast<const void*>(kernel_of<D>(what));
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<D>::kTotal);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100);   // two CTAs an SM
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 }  // namespace
 
 cudaError_t prefill_attention_tc_init() {
-  cudaError_t e = cudaSuccess;
-  const void* k[2] = {reinterpret_cast<const void*>(prefill_attn_tc_kernel<128>), reinterpret_cast<const void*>(prefill_attn_tc_kernel<64>)};
-  const int bytes[2] = {Smem<128>::kTotal, Smem<64>::kTotal};
-  for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
-    e = cudaFuncSetAttribute(k[i], cudaFuncAttributeMaxDynamicSharedMemorySize, bytes[i]);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k[i], cudaFuncAttributePreferredSharedMemoryCarveout, 100);   // two CTAs an SM
-  }
-  return e;
+  const cudaError_t e = init<128>();
+  return e != cudaSuccess ? e : init<64>();
 }
 
 // The byte ranges of an Exchange in CTA `split`, as (begin, end) pairs for a check on the host: the rows it finishes, the peers' pairs,
@@ -958,8 +971,10 @@ cudaError_t launch_prefill_attention_tc(const AttnArgs& args, const BatchParams&
   attr[1].val.clusterDim.x = a.nsplit; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = a.nsplit > 1 ? 2 : 1;
-  if (a.D == 128) { cfg.dynamicSmemBytes = Smem<128>::kTotal; return cudaLaunchKernelEx(&cfg, prefill_attn_tc_kernel<128>, a, bp, status); }
-  if (a.D == 64) { cfg.dynamicSmemBytes = Smem<64>::kTotal; return cudaLaunchKernelEx(&cfg, prefill_attn_tc_kernel<64>, a, bp, status); }
+  if ((a.out != nullptr) == (a.h_out != nullptr)) return cudaErrorInvalidValue;      // rows, or the residual stream (the last layer's rows have no next)
+  const Stored what = a.h_out != nullptr ? ST_RESIDUAL : (a.out_fp32 ? ST_ROWS_FP32 : ST_ROWS_BF16);
+  if (a.D == 128) { cfg.dynamicSmemBytes = Smem<128>::kTotal; return cudaLaunchKernelEx(&cfg, kernel_of<128>(what), a, bp, status); }
+  if (a.D == 64) { cfg.dynamicSmemBytes = Smem<64>::kTotal; return cudaLaunchKernelEx(&cfg, kernel_of<64>(what), a, bp, status); }
   return cudaErrorInvalidValue;
 }
 
@@ -976,8 +991,8 @@ int prefill_attention_max_clusters(int head_dim, int s) {
   attr[0].val.clusterDim.x = s; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr; cfg.numAttrs = 1;
   int clusters = 0;
-  const cudaError_t e = head_dim == 128 ? cudaOccupancyMaxActiveClusters(&clusters, prefill_attn_tc_kernel<128>, &cfg)
-                                        : cudaOccupancyMaxActiveClusters(&clusters, prefill_attn_tc_kernel<64>, &cfg);
+  const cudaError_t e = head_dim == 128 ? cudaOccupancyMaxActiveClusters(&clusters, kernel_of<128>(ST_RESIDUAL), &cfg)
+                                        : cudaOccupancyMaxActiveClusters(&clusters, kernel_of<64>(ST_RESIDUAL), &cfg);
   if (e != cudaSuccess) { cudaGetLastError(); return 0; }
   return clusters;
 }
