@@ -153,6 +153,9 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(DecodeArgs 
     for (int r = 0; r < 4; ++r)
 #pragma unroll
       for (int c = 0; c < VC; ++c) vr[r][c] = lds128(stage + (uint32_t)((2 * KC + r * VC + c) * 512));
+    // The next copies go over these pieces: nothing else orders an asynchronous copy behind loads that have merely been issued.  (16 streams
+    // of 1150 keys, projection included: 24.4 us, 25.5 without the fence; with the copies issued after the MMAs instead 27.3.)
+    __threadfence_block();
   };
   const bool early = warp + kDecWarps < n_tiles && begin + (warp + kDecWarps + 1) * kTileKeys <= own_v;
   if (early) fetch_tile(begin + (warp + kDecWarps) * kTileKeys);
