@@ -47,7 +47,9 @@ constexpr int kFewBound = 768, kFewWarps = 8, kFewStages = 6;   // (threads that
 // takes few SMs had on all others anyway.  Whole steps of 8 layers over 128 to 830 keys, us without and with: 48 rows 195 to 208 / 190 to
 // 197; 32 rows 183 / 182 to 185 over few keys (up to 48 attention CTAs), 194 / 190 over many; 20 rows 176 / 182; 64 rows, four stages,
 // 193 / 203.  Where K leaves no more stages anyway it costs nothing: 6 small layers of 30 rows 123 / 119.5.
-constexpr int kSlimSmem = 113 * 1024;
+// Registers: the launch bound of twice its threads leaves this form at most half of the register file, as the attention's two blocks an SM do.
+constexpr int kSlimSmem = 113 * 1024, kSlimThreads = 64 + 32 * kFewWarps, kBound = 2 * kSlimThreads;
+static_assert(kBound >= kMaxThreads, "every form of the launch");
 inline bool goes_beside_attention(const GemmArgs& a, int most_kb, int slim_stages) {
   return a.beside_attention > 0 && a.rows <= 48 &&
          (most_kb <= slim_stages || a.rows > 32 || (a.rows > 24 && 8 * a.beside_attention >= 3 * a.n_sms));
@@ -83,7 +85,7 @@ __device__ __forceinline__ int ld_acquire_gpu(const int* p) {
 __host__ __device__ inline int first_block(int r, int n_blk, int ksplit) { return (r * n_blk + ksplit - 1) / ksplit; }
 
 template <int kFin, bool kOwnRope>   // kOwnRope: no RoPE table, every finishing thread derives the rotation of its one row
-__global__ void __launch_bounds__(kOwnRope ? kFewBound : kMaxThreads, 1)
+__global__ void __launch_bounds__(kOwnRope ? kFewBound : kBound, 1)
 qkv_gemm_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_x,
                 const __grid_constant__ CUtensorMap tm_w2, KernelParams p, BatchParams bp) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
