@@ -808,6 +808,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
     // F4 lanes per row, U rows of a lane side by side: their loads are all on their way before the first sum
 #pragma unroll 1
     for (int jb = warp * RPW; jb < my_rows; jb += U * kWarps * RPW) {
+      const Row first = row_of(jb);
       Row rw[U];
       float4 v[U];
       uint2 h[U];
@@ -816,7 +817,8 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
         rw[k] = row_of(jb + hv + k * kWarps * RPW);
         h[k] = jb == warp * RPW ? h_first[k] : load_res(rw[k]);
         v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (!rw[k].on) { rw[k].g = 0; rw[k].tl = 0; }
+        // (a place without a row goes along with the warp's first one: another warp's weights may be giving way to its sums already)
+        if (!rw[k].on) { rw[k].g = first.g; rw[k].tl = first.tl; }
       }
 #pragma unroll 1
       for (int s = 0; s < nsplit; ++s)
