@@ -196,8 +196,8 @@ struct Smem {
   static constexpr int kQBytes = kRows * D * 2;           // one of hi / lo
   static constexpr int kKVBytes = kKeys * D * 2;          // a K or V tile
   static constexpr int kStages = D == 128 ? 3 : 6;
-  static constexpr int kQ = 0;                            // [hi | lo]; at the end fp32 rows (see Exchange)
-  static constexpr int kRing = 2 * kQBytes;               // [stage] K or V tile; at the end rows or, without a cluster, residual input
+  static constexpr int kQ = 0;                            // [hi | lo]; in a cluster, at the end, fp32 rows (see Exchange)
+  static constexpr int kRing = 2 * kQBytes;               // [stage] K or V tile; in a cluster, at the end, rows on their way to peers
   static constexpr int kCtl = kRing + kStages * kKVBytes; // barriers, tmem slot, abort flag
   static constexpr int kPairs = kCtl + 80 + 16 * kStages;               // (max, denominator) of the peers' parts; weights; sums of squares
   static constexpr int kPairRows = D == 128 ? 108 : 128;  // (as many as two CTAs an SM leave room for)
@@ -206,7 +206,8 @@ struct Smem {
 };
 
 // Where a row tile's rows lie in the shared memory of CTA `split` of its cluster once the CTA's key tiles are done: byte offsets.
-// The tile has n_tok tokens; CTA s finishes tokens s * tok_per ..., tok_per of them or what is left (without a cluster: all).
+// The tile has n_tok tokens; CTA s finishes tokens s * tok_per ..., tok_per of them or what is left.  (Without a cluster a CTA finishes
+// all of them out of its threads' registers, and nothing but the sums of squares has a place here.)
 // Where the query was: the rows of its tokens, [CTA they come from][head][token].  At the top of the ring, on into the query's place
 // where the ring does not hold them all: the rows that are on their way to the peers.  The peers' (max, denominator) pairs have a place
 // of their own.  (With the pairs behind the rows a group of eight heads could not be split at all: its 128 rows fill the query's place.)
@@ -932,11 +933,11 @@ void prefill_attention_ranges(int head_dim, int group, int nsplit, int n_tok, in
   auto fill = [&](auto ex, int q_end, int total) {
     const int n = ex.my_tok, row = ex.kRowBytes, first = split == 0 ? 1 : 0, last = split == nsplit - 1 ? nsplit - 2 : nsplit - 1, staged = ex.staged_rows();
     for (int i = 0; i < 8; ++i) r[i] = 0;
-    if (n > 0) {
+    if (n > 0) { r[6] = (int)ex.stats(0, 0); r[7] = (int)ex.stats(group - 1, n - 1) + 4; }
+    if (n > 0 && nsplit > 1) {
       r[0] = (int)ex.row(0, 0, 0); r[1] = (int)ex.row(nsplit - 1, group - 1, n - 1) + row;
-      r[6] = (int)ex.stats(0, 0); r[7] = (int)ex.stats(group - 1, n - 1) + 4;
+      r[2] = (int)ex.pair(split, first, 0, 0); r[3] = (int)ex.pair(split, last, group - 1, n - 1) + 8;
     }
-    if (n > 0 && nsplit > 1) { r[2] = (int)ex.pair(split, first, 0, 0); r[3] = (int)ex.pair(split, last, group - 1, n - 1) + 8; }
     if (staged > 0) { r[4] = (int)ex.staged(0); r[5] = (int)ex.staged(staged - 1) + row; }
     r[8] = q_end; r[9] = total;
   };

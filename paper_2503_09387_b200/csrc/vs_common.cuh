@@ -380,7 +380,7 @@ struct AttnArgs {
   const bf16* q_lo;
   const bf16* q_tiled;           // or: the query as the projection's GEMM leaves it for this kernel, one block per
                                  // (batch entry, 16-token row tile, KV head): [hi | lo][128 rows = g * 16 + token][D],
-                                 // 128-byte swizzled like the MMA operand, fetched by one bulk copy
+                                 // 128-byte swizzled like the MMA operand, fetched by bulk copies, two for each 64 dims
   void* out;                     // [rows][Hq*D], bf16 or fp32
   int out_fp32;
   int out_region;                // checked build: the workspace region that out lies in, or -1 (the caller's buffer)

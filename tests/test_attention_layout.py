@@ -42,6 +42,9 @@ def test_nothing_lies_over_rows_on_their_way(lib, D):
                     assert not any(_meet(r["staged"], r[k]) for k in ("rows", "pairs", "sums")), what
                     assert not _meet(r["rows"], r["pairs"]) and not _meet(r["rows"], r["sums"]), what
                     assert r["rows"][1] <= ring, what                         # the ring may still be in use when they come
+                    if n == 1:                                                # no peers: rows leave from registers, only sums have a place
+                        assert r["rows"] == r["pairs"] == r["staged"] == (0, 0), what
+                        assert r["sums"][1] - r["sums"][0] == 4 * ((G - 1) * 16 + n_tok), what
 
 
 @pytest.mark.parametrize("D", [64, 128])
