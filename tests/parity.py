@@ -99,7 +99,8 @@ class Pair:
     def __init__(self, w: synth.Workload, n_streams: Optional[int] = None, max_step_tokens: int = 64,
                  evict_policy: int = 0, agg_mode: int = 0, with_bias: bool = False, with_gain: bool = False,
                  max_tokens_per_frame: Optional[int] = None, max_prefix: Optional[int] = None,
-                 max_text: Optional[int] = None, out_dtype: int = 1, max_chunk_frames: int = 1, d_ff: int = 0, vocab: int = 0):
+                 max_text: Optional[int] = None, out_dtype: int = 1, max_chunk_frames: int = 1, d_ff: int = 0, vocab: int = 0,
+                 n_oracles: Optional[int] = None):
         self.w = w
         S = n_streams or w.n_streams
         self.S = S
@@ -146,7 +147,7 @@ class Pair:
         self.ora: List[vo.OracleStream] = [
             vo.OracleStream(ocfg, [f64(b) for b in wbits],
                             [f64(b) for b in bbits] if bbits else None,
-                            [f64(b) for b in gbits] if gbits else None, oblk) for _ in range(S)]
+                            [f64(b) for b in gbits] if gbits else None, oblk) for _ in range(n_oracles or S)]
         self.worst = [0.0, 0.0]
         self.d_ff = d_ff
 
