@@ -809,17 +809,17 @@ __global__ void __launch_bounds__(kAttnThreads, 2) prefill_attn_tc_kernel(const 
     // F4 lanes per row, U rows of a lane side by side: their loads are all on their way before the first sum
 #pragma unroll 1
     for (int jb = warp * RPW; jb < my_rows; jb += U * kWarps * RPW) {
-      const Row first = row_of(jb);
       Row rw[U];
       float4 v[U];
       uint2 h[U];
 #pragma unroll
       for (int k = 0; k < U; ++k) {
-        rw[k] = row_of(jb + hv + k * kWarps * RPW);
+        // (a place without a row goes along with the warp's first one: another warp's weights may be giving way to its sums already)
+        const int j = jb + hv + k * kWarps * RPW;
+        rw[k] = row_of(j < my_rows ? j : jb);
+        rw[k].on = j < my_rows;
         h[k] = jb == warp * RPW ? h_first[k] : load_res(rw[k]);
         v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-        // (a place without a row goes along with the warp's first one: another warp's weights may be giving way to its sums already)
-        if (!rw[k].on) { rw[k].g = first.g; rw[k].tl = first.tl; }
       }
 #pragma unroll 1
       for (int s = 0; s < nsplit; ++s)
