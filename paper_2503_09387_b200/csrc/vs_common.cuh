@@ -296,6 +296,9 @@ struct ProjectionOut {
   const bf16* next_gain; bf16* xn_out;   // mode 4 with ss_out: xn_out = bf16(stored row * next_gain), or null
 };
 
+// The prefill attention that runs right ahead of a linear layer (W_o) or behind it (the projection): its CTAs (0: none, or no room is
+// to be left for it) and the key tiles of one; and whether the layer is one of a full decoder layer.
+struct BesideAttention { int ctas, tiles, full, ahead; };
 struct GemmArgs {
   CUtensorMap tm_w2;             // mode 5: the up matrix (tm_w is then the gate matrix, both with boxes of 64 rows)
   CUtensorMap tm_w;              // [E_out, d] bf16, box 64 x 128, 128-byte swizzle
@@ -308,9 +311,12 @@ struct GemmArgs {
   int* flags;                    // [m_tiles*n_tiles][ksplit], zero between launches
   int n_sms;
   int* status;
-  int beside_attention;          // CTAs of the prefill attention that runs right ahead of or behind this launch, or 0
+  BesideAttention beside;
 };
 struct Tiling { int tile_n, n_tiles, ksplit, pairs; };
+// Whether a few-row linear layer of `blocks` CTAs leaves room for those of the attention beside it: K blocks of a CTA and the ring
+// stages that it keeps if it does.
+bool leaves_room_for_attention(BesideAttention att, int rows, int blocks, int most_kb, int slim_stages, int n_sms);
 Tiling choose_tiles(int K, int E, int n_sms, int max_pairs, int rows, bool own_rope);
 cudaError_t launch_qkv_gemm(const GemmArgs& a, const BatchParams& bp, cudaStream_t st);
 cudaError_t qkv_gemm_init();     // opt-in shared memory attribute, once per process/device

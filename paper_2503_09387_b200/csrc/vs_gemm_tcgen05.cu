@@ -42,18 +42,11 @@ constexpr int kMaxThreads = 64 + 32 * kMaxEpiWarps;
 // 16 streams of 1150 keys 26.6 us, 25.7 this way.)
 constexpr int kFewBound = 768, kFewWarps = 8, kFewStages = 6;   // (threads that would fill the register file at 80 each)
 // The same beside the prefill attention (ten warps of 96 registers, 113 KB): whether a projection of 17 to 48 rows, or the W_o behind the
-// attention, leaves room for one of its CTAs, which then has its set-up and first keys behind it when the projection is done, as this
-// block has its first weights when the attention is.  The price is depth, five stages of weights for eight, which a step whose attention
-// takes few SMs had on all others anyway.  Whole steps of 8 layers over 128 to 830 keys, us without and with: 48 rows 195 to 208 / 190 to
-// 197; 32 rows 183 / 182 to 185 over few keys (up to 48 attention CTAs), 194 / 190 over many; 20 rows 176 / 182; 64 rows, four stages,
-// 193 / 203.  Where K leaves no more stages anyway it costs nothing: 6 small layers of 30 rows 123 / 119.5.
+// attention, leaves room for one of its CTAs (leaves_room_for_attention), which then has its set-up and first keys behind it when the
+// projection is done, as this block has its first weights when the attention is.  The price is depth, five stages of weights for eight.
 // Registers: the launch bound of twice its threads leaves this form at most half of the register file, as the attention's two blocks an SM do.
 constexpr int kSlimSmem = 113 * 1024, kSlimThreads = 64 + 32 * kFewWarps, kBound = 2 * kSlimThreads;
 static_assert(kBound >= kMaxThreads, "every form of the launch");
-inline bool goes_beside_attention(const GemmArgs& a, int most_kb, int slim_stages) {
-  return a.beside_attention > 0 && a.rows <= 48 &&
-         (most_kb <= slim_stages || a.rows > 32 || (a.rows > 24 && 8 * a.beside_attention >= 3 * a.n_sms));
-}
 // Instruction descriptor, kind::f16: D = fp32, A = B = bf16, both K-major, M = 128, N = n.
 __device__ __forceinline__ uint32_t make_idesc(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(GEMM_BLOCK_M >> 4) << 24);
@@ -381,6 +374,28 @@ Kernel kernel_of(int mode, bool own_rope) {
 
 }  // namespace
 
+// Whole steps, us without / with room, attention layers alone unless a full layer is named; keys before the question:
+// * more than 48 rows: four stages and less, 64 rows 193 / 203; where K leaves no more stages than the room it costs nothing (8 layers of
+//   width 1024, 17 to 48 rows: 0.5 to 3.5 % gained).
+// * 33 to 48 rows gain (width 3584, 6 layers, one stream, 33 rows over 64 keys 1.3 %, over 1200 6.8 %; groups of eight 7 to 11 %), 25 to 32
+//   where the attention takes three eighths of the SMs: it pays by its keys.  With a key tile to a CTA and a projection on nine tenths of
+//   the SMs they lose: 4 x 8 rows over 64 keys 3.5 %, 25 rows 2.1 %, width 2560 2 x 13 rows 4 %; with two tiles 25 rows gain 0.9 %, with
+//   three 3.1.  Projections on fewer SMs gain with one too (width 2048, 25 rows 7 %; 4096, 4 x 7 rows 3 %).
+// * where a CTA's share of K is longer than the eight stages, an attention of so many CTAs that, with the projection's, there are
+//   1.7 to an SM does not wait in the room but takes it: width 3584, 4 x 12 rows over 700 keys lose 5.1 %, 5 x 9 8.3 %, 12 x 4 3.4 %, 2 x 17
+//   2.7 % (144 + 128 or more), one stream of 48 (144 + 96) gains 4.6 %; width 4096, 12 x 4 lose 4.5 % (120 + 192), 8 x 4 gain 2.7 (120 + 128).
+// * there a full layer's W_o loses by itself (3 layers: 28 rows 321.4 / 324.2, 40 rows 321.7 / 326.5), and its projection gains with 144 + 64
+//   (28 rows 321.4 / 317.1) and not with 144 + 96 (40 rows 321.7 / 326.5).
+// Found the other way: width 3584, 6 x 8 rows over 64 keys (144 + 96) lose 3.0 %, 3 x 11 1.8.
+bool leaves_room_for_attention(BesideAttention att, int rows, int blocks, int most_kb, int slim_stages, int n_sms) {
+  if (att.ctas <= 0 || rows > 48) return false;
+  if (most_kb <= slim_stages) return true;
+  if (most_kb > 8 && (att.ahead || 20 * (att.ctas + blocks) > (att.full ? 29 : 34) * n_sms)) return false;
+  if (rows > 32) return true;
+  if (!att.full && att.tiles < 2 && 10 * blocks > 9 * n_sms) return false;
+  return rows > 24 && 8 * att.ctas >= 3 * n_sms;
+}
+
 cudaError_t qkv_gemm_init() {
   for (int mode : {(int)FIN_PROJECT, (int)FIN_RESIDUAL, (int)FIN_SWIGLU, (int)FIN_LOGITS})
     for (bool own_rope : {false, true}) {
@@ -408,7 +423,8 @@ cudaError_t launch_qkv_gemm(const GemmArgs& a, const BatchParams& bp, cudaStream
   const int stage_bytes = kStageABytes + a.tile_n * 128, most_kb = (p.total_kb + a.ksplit - 1) / a.ksplit;
   int stages = (kMaxDynSmem - 3072) / stage_bytes;
   const int slim_stages = (kSlimSmem - 3072) / stage_bytes;
-  const bool slim = !own_rope && goes_beside_attention(a, most_kb, slim_stages);
+  const int blocks = (a.E_out + GEMM_BLOCK_M - 1) / GEMM_BLOCK_M * a.n_tiles * a.ksplit;
+  const bool slim = !own_rope && leaves_room_for_attention(a.beside, a.rows, blocks, most_kb, slim_stages, a.n_sms);
   if (slim) stages = slim_stages;
   const int most = own_rope ? kFewStages : 8;
   if (stages > most) stages = most;

@@ -288,12 +288,16 @@ int ensure_step_maps(vs_stream* h, int rows) {
   return VS_OK;
 }
 
+int key_tiles(const int* key_len, int n_len) {
+  int n = 0;
+  for (int i = 0; i < n_len; ++i) n += (key_len[i] + ATTN_KEY_BOX - 1) / ATTN_KEY_BOX;
+  return n;
+}
+
 // CTAs that share the key tiles of a row tile (see attention_split), for the longest key axis among the listed entries, whose
 // segments have key_len[i] keys
 int attn_split(const vs_stream* h, const BatchParams& bp, const int* key_len, int n_len, int bank_ctas) {
-  int key_tiles = 0;
-  for (int i = 0; i < n_len; ++i) key_tiles += (key_len[i] + ATTN_KEY_BOX - 1) / ATTN_KEY_BOX;
-  return attention_split(h->dm.D, h->dm.G, (bp.rows_per_stream + 15) / 16 * h->dm.Hkv * bp.n_active, key_tiles, bank_ctas, h->n_sms, h->attn_clusters);
+  return attention_split(h->dm.D, h->dm.G, (bp.rows_per_stream + 15) / 16 * h->dm.Hkv * bp.n_active, key_tiles(key_len, n_len), bank_ctas, h->n_sms, h->attn_clusters);
 }
 
 // segments of the attention's key axis
@@ -367,9 +371,9 @@ static_assert(KC_OTHER + 1 == VS_N_KERNEL_CLASSES, "kernel class table");
   } while (0)
 
 // QKV projection of `rows` token rows read from `src` ([rows][d] bf16) for layer l, finished
-// rows written as `po` says.  attn_ctas: of the prefill attention that reads them, where the launch may leave room for them.
+// rows written as `po` says.  beside: the prefill attention that reads them.
 int run_projection(vs_stream* h, int l, const bf16* src, int rows, const ProjectionOut& po, const BatchParams& bp,
-                   cudaStream_t st, int attn_ctas) {
+                   cudaStream_t st, BesideAttention beside) {
   const Dims& D = h->dm;
   if (po.rope == nullptr && qkv_gemv_supported(po, rows, D.d) && (reinterpret_cast<uintptr_t>(src) & 15u) == 0) {
     // a text step of a few rows: bound by reading W once, done on the CUDA cores
@@ -378,7 +382,7 @@ int run_projection(vs_stream* h, int l, const bf16* src, int rows, const Project
   }
   GemmArgs g;
   g.tm_w = h->tm_w[l]; g.tm_w2 = h->tm_w[l];
-  g.out = po; g.beside_attention = attn_ctas;
+  g.out = po; g.beside = beside;
   return launch_linear(h, g, src, rows, D.d, D.E_out, bp, st);
 }
 
@@ -399,9 +403,9 @@ int launch_linear(vs_stream* h, GemmArgs& g, const bf16* src, int rows, int K, i
 // One linear layer of the rest of the decoder block on the tensor cores: rows x K times W[E][K]^T, finished as
 // `po` says (mode 4: + residual; mode 5: SwiGLU of a gate / up pair, E = 2 * d_ff).
 int run_linear(vs_stream* h, const CUtensorMap& tm_w, const CUtensorMap& tm_w2, const bf16* src, int rows, int K, int E,
-               ProjectionOut po, const BatchParams& bp, cudaStream_t st, int attn_ctas = 0) {
+               ProjectionOut po, const BatchParams& bp, cudaStream_t st, BesideAttention beside = {}) {
   GemmArgs g;
-  g.beside_attention = attn_ctas;
+  g.beside = beside;
   g.tm_w = tm_w; g.tm_w2 = tm_w2;
   po.Hq = 0; po.Hkv = 0; po.D = 128; po.slots = 0; po.text_cap = 0; po.M = 0; po.norm_inline = 0;
   g.out = po;
@@ -413,7 +417,7 @@ int run_linear(vs_stream* h, const CUtensorMap& tm_w, const CUtensorMap& tm_w2, 
 // h2 = h1 + act W_down^T -> hbuf[0] (and `final_out` on the last layer).  Each stored tensor leaves its RMSNorm
 // statistics (and, with a gain vector, its gained copy) for the projection that reads it next.
 int run_block_rest(vs_stream* h, int l, int rows, const bf16* h_in, const bf16* a_rows, void* final_out, const BatchParams& bp,
-                   cudaStream_t st, int attn_ctas) {
+                   cudaStream_t st, BesideAttention beside) {
   const Dims& D = h->dm;
   const Layout& lo = h->lo;
   bf16* h1 = h->at<bf16>(lo.hbuf[1]);
@@ -425,7 +429,7 @@ int run_block_rest(vs_stream* h, int l, int rows, const bf16* h_in, const bf16* 
   // W_o
   po.mode = 4; po.lin_out = h1; po.lin_res = h_in; po.lin_out_region = DR_HBUF1;
   if (D.use_rmsnorm) { po.ss_out = ss2; po.ss_out_parts = D.ss_parts; po.next_gain = h->gain2[l]; po.xn_out = h->at<bf16>(lo.xn); }
-  int rc = run_linear(h, h->tm_wo[l], h->tm_wo[l], a_rows, rows, D.d, D.d, po, bp, st, attn_ctas);
+  int rc = run_linear(h, h->tm_wo[l], h->tm_wo[l], a_rows, rows, D.d, D.d, po, bp, st, beside);
   if (rc != VS_OK) return rc;
   // gate and up with the SwiGLU epilogue
   std::memset(&po, 0, sizeof(po));
@@ -751,7 +755,7 @@ int vs_frame_prefill(vs_stream* h, const int32_t* stream_ids, int32_t n_active, 
     fa.text_k = nullptr; fa.text_v = nullptr;
     fa.free_slot = h->at<int32_t>(lo.step_slot); fa.free_slot_stride = 1;
     fa.Hq = D.Hq; fa.Hkv = D.Hkv; fa.D = D.D; fa.slots = D.slots; fa.text_cap = 0; fa.mode = 0; fa.M = D.M;
-    rc = run_projection(h, l, src, rows, fa, bp, st, 0);
+    rc = run_projection(h, l, src, rows, fa, bp, st, {});
     if (rc != VS_OK) return rc;
 
     AttnArgs aa;
@@ -776,9 +780,12 @@ int vs_frame_prefill(vs_stream* h, const int32_t* stream_ids, int32_t n_active, 
     }
     aa.free_slot = h->at<int32_t>(lo.step_slot); aa.free_slot_stride = 1;
     // the bank update (Section 3.3, memory mechanism: evict if full, then append) rides in the attention launches: each layer's
-    // scores a share of the bank, the last one's commits.  Five rows to a CTA (a row per warp) while the CTAs are few; at most one
-    // CTA for every two SMs, or for every SM where the attention comes in waves anyway: scoring is fp64 arithmetic and runs
-    // beside the tensor work of the SM's other CTA, but must not take the slots that the attention's clusters need
+    // scores a share of the bank, the last one's commits.  Five rows to a CTA (it scores four to a warp, side by side) while the CTAs are
+    // few; at most one CTA for every two SMs, or for every SM where the attention comes in waves anyway: scoring runs beside the tensor
+    // work of the SM's other CTA, but must not take the slots that the attention's clusters need.  Against the best of 2 to 40 rows
+    // (28 / 4 heads): through 6 layers, and through one with banks of 32, 64 or 1024 rows or eight streams, at most 3 % slower; through one
+    // layer fewer CTAs gain where a bank of 256 or 512 costs the attention a cluster size: 256 rows 35.8 us, 31.3 with eight to a CTA,
+    // 512 rows 37.5 and 32.8 with twenty, four streams of 256 48.5 and 45.6 with twenty; 64 rows lose 1.2 by twenty, 1024 rows 0.3
     if (any_full || last) {
       aa.bank = ba;
       aa.bank.j0 = (int)((int64_t)D.M * l / D.L); aa.bank.j1 = (int)((int64_t)D.M * (l + 1) / D.L); aa.bank.commit = last ? 1 : 0;
@@ -809,7 +816,7 @@ int vs_frame_prefill(vs_stream* h, const int32_t* stream_ids, int32_t n_active, 
     VS_LAUNCH(h, st, KC_PREFILL_ATTN, launch_prefill_attention_tc(aa, bp, h->at<int>(lo.status), st));
     if (D.d_ff > 0) {
       // h2 lands in hbuf[0] again: the layer input of every layer is hbuf[0]
-      rc = run_block_rest(h, l, rows, h_in, h->at<bf16>(lo.obuf), last ? out_final : nullptr, bp, st, 0);
+      rc = run_block_rest(h, l, rows, h_in, h->at<bf16>(lo.obuf), last ? out_final : nullptr, bp, st, {});
       if (rc != VS_OK) return rc;
     } else if (D.residual) cur ^= 1;
   }
@@ -975,7 +982,7 @@ int vs_frame_prefill_chunk(vs_stream* h, int32_t stream_id, const void* hidden, 
     fa.bank_v = h->at<bf16>(lo.bank_v) + (size_t)l * layer_stride_bank(D);
     fa.free_slot = chunk_slot; fa.free_slot_stride = 0;
     fa.Hq = D.Hq; fa.Hkv = D.Hkv; fa.D = D.D; fa.slots = D.slots; fa.text_cap = 0; fa.mode = 3; fa.M = D.M;
-    rc = run_projection(h, l, src, rows, fa, bp, st, 0);
+    rc = run_projection(h, l, src, rows, fa, bp, st, {});
     if (rc != VS_OK) return rc;
 
     const bool last = (l == D.L - 1);
@@ -1026,7 +1033,7 @@ int vs_frame_prefill_chunk(vs_stream* h, int32_t stream_id, const void* hidden, 
     }
     if (D.d_ff > 0) {
       // h2 lands in hbuf[0] again: the layer input of every layer is hbuf[0]
-      rc = run_block_rest(h, l, rows, h_in, h->at<bf16>(lo.obuf), (last && out != nullptr) ? out : nullptr, bp, st, 0);
+      rc = run_block_rest(h, l, rows, h_in, h->at<bf16>(lo.obuf), (last && out != nullptr) ? out : nullptr, bp, st, {});
       if (rc != VS_OK) return rc;
     } else if (D.residual) cur ^= 1;
   }
@@ -1087,7 +1094,7 @@ int vs_bank_forward(vs_stream* h, int32_t stream_id, void* out, void* cuda_strea
     fa.q_tiled = h->at<bf16>(lo.q_tiled);
     fa.free_slot = h->at<int32_t>(lo.step_slot); fa.free_slot_stride = 0;
     fa.Hq = D.Hq; fa.Hkv = D.Hkv; fa.D = D.D; fa.slots = D.slots; fa.text_cap = 0; fa.mode = 3; fa.M = D.M;
-    rc = run_projection(h, l, src, rows, fa, bp, st, 0);
+    rc = run_projection(h, l, src, rows, fa, bp, st, {});
     if (rc != VS_OK) return rc;
 
     AttnArgs aa;
@@ -1117,7 +1124,7 @@ int vs_bank_forward(vs_stream* h, int32_t stream_id, void* out, void* cuda_strea
     aa.out_region = rows_region(h, aa.out);
     VS_LAUNCH(h, st, KC_PREFILL_ATTN, launch_prefill_attention_tc(aa, bp, h->at<int>(lo.status), st));
     if (D.d_ff > 0) {
-      rc = run_block_rest(h, l, rows, h_in, h->at<bf16>(lo.obuf), (l == D.L - 1) ? out : nullptr, bp, st, 0);
+      rc = run_block_rest(h, l, rows, h_in, h->at<bf16>(lo.obuf), (l == D.L - 1) ? out : nullptr, bp, st, {});
       if (rc != VS_OK) return rc;
     } else if (D.residual) cur ^= 1;
   }
@@ -1194,7 +1201,8 @@ int vs_decode_step(vs_stream* h, const int32_t* stream_ids, int32_t n_active, co
   }
 
   if (T > 1 && ensure_step_maps(h, rows) != VS_OK) return VS_ERR_CUDA;
-  int key_split = 0, attn_ctas = 0;          // of the prefill attention, which a step of several tokens takes
+  int key_split = 0;                         // of the prefill attention, which a step of several tokens takes
+  BesideAttention beside = {0, 0, D.d_ff > 0, 0};
   if (T > 1) {
     int kl[4] = {0, 0, 0, T};
     for (int i = 0; i < n_active; ++i) {
@@ -1203,7 +1211,8 @@ int vs_decode_step(vs_stream* h, const int32_t* stream_ids, int32_t n_active, co
       if (bp.entry[i].prefix_len + bl + tl > kl[0] + kl[1] + kl[2]) { kl[0] = bp.entry[i].prefix_len; kl[1] = bl; kl[2] = tl; }
     }
     key_split = attn_split(h, bp, kl, 4, 0);
-    attn_ctas = (T + 15) / 16 * D.Hkv * n_active * key_split;
+    beside.ctas = (T + 15) / 16 * D.Hkv * n_active * key_split;
+    beside.tiles = (key_tiles(kl, 4) + key_split - 1) / key_split;
   }
   const bf16* h_in = static_cast<const bf16*>(hidden);
   int next_buf = 0;
@@ -1243,7 +1252,7 @@ int vs_decode_step(vs_stream* h, const int32_t* stream_ids, int32_t n_active, co
     fa.free_slot = &meta->free_slot; fa.free_slot_stride = (int)(sizeof(StreamMeta) / sizeof(int32_t));
     fa.Hq = D.Hq; fa.Hkv = D.Hkv; fa.D = D.D; fa.slots = D.slots;
     fa.text_cap = to_prefix ? D.maxP : D.maxT; fa.mode = to_prefix ? 1 : 2; fa.M = D.M;
-    rc = run_projection(h, l, src, rows, fa, bp, st, attn_ctas);
+    rc = run_projection(h, l, src, rows, fa, bp, st, beside);
     if (rc != VS_OK) return rc;
 
     bf16* h_out = D.residual && l + 1 < D.L ? h->at<bf16>(lo.hbuf[next_buf]) : nullptr;
@@ -1310,7 +1319,7 @@ int vs_decode_step(vs_stream* h, const int32_t* stream_ids, int32_t n_active, co
       VS_LAUNCH(h, st, KC_PREFILL_ATTN, launch_prefill_attention_tc(aa, bp, h->at<int>(lo.status), st));
     }
     if (D.d_ff > 0) {
-      rc = run_block_rest(h, l, rows, h_in, h->at<bf16>(lo.obuf), (l == D.L - 1) ? out : nullptr, bp, st, attn_ctas);
+      rc = run_block_rest(h, l, rows, h_in, h->at<bf16>(lo.obuf), (l == D.L - 1) ? out : nullptr, bp, st, {beside.ctas, beside.tiles, 1, 1});
       if (rc != VS_OK) return rc;
       h_in = h->at<bf16>(lo.hbuf[0]);
     } else if (D.residual) { h_in = h_out; next_buf ^= 1; }

@@ -77,3 +77,22 @@ def test_current_stream_with_and_without_torchs_private_call():
         b = binding.StreamBatch.__new__(binding.StreamBatch)
         b.handle, b.torch, b.device, b.device_index, b._raw_stream = None, public, 3, 3, raw
         assert b._stream() == want
+
+
+class _Beside(C.Structure):
+    _fields_ = [(n, C.c_int) for n in ("ctas", "tiles", "full", "ahead")]
+
+
+# (attention CTAs, key tiles of one, full layer, W_o), rows, blocks of the layer, K blocks of one, stages kept -> room left?  Shapes measured both ways.
+@pytest.mark.parametrize("att,rows,blocks,kb,stages,room", [
+    ((96, 3, 0, 0), 48, 144, 14, 5, True), ((96, 1, 0, 0), 33, 144, 14, 5, True), ((64, 2, 0, 0), 25, 144, 14, 5, True),
+    ((64, 1, 0, 0), 25, 144, 14, 5, False), ((64, 1, 0, 0), 32, 144, 14, 5, False), ((64, 1, 0, 0), 25, 128, 8, 5, True),      # few keys
+    ((128, 2, 0, 0), 48, 144, 14, 5, False), ((160, 3, 0, 0), 45, 144, 14, 5, False), ((256, 2, 0, 0), 32, 144, 14, 5, False), # many streams
+    ((128, 2, 0, 0), 32, 120, 22, 5, True), ((192, 2, 0, 0), 48, 120, 22, 5, False), ((256, 2, 0, 0), 48, 128, 8, 5, True),
+    ((64, 1, 1, 0), 28, 144, 14, 5, True), ((96, 2, 1, 0), 40, 144, 14, 5, False), ((96, 2, 1, 1), 40, 140, 12, 5, False),     # full layers
+    ((48, 2, 0, 0), 24, 144, 14, 5, False), ((64, 2, 0, 0), 49, 144, 14, 5, False), ((0, 0, 0, 0), 40, 144, 14, 5, False),
+    ((256, 1, 1, 1), 17, 140, 4, 5, True)])
+def test_room_beside_the_attention(lib, att, rows, blocks, kb, stages, room):
+    f = lib._ZN2vs25leaves_room_for_attentionENS_15BesideAttentionEiiiii
+    f.argtypes, f.restype = [_Beside] + [C.c_int] * 5, C.c_bool
+    assert f(_Beside(*att), rows, blocks, kb, stages, 148) == room
