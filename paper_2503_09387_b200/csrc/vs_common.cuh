@@ -314,6 +314,7 @@ struct GemmArgs {
   BesideAttention beside;
 };
 struct Tiling { int tile_n, n_tiles, ksplit, pairs; };
+int few_row_linear_registers();          // of a thread, the most
 // Whether a few-row linear layer of `blocks` CTAs leaves room for those of the attention beside it: K blocks of a CTA and the ring
 // stages that it keeps if it does.
 bool leaves_room_for_attention(BesideAttention att, int rows, int blocks, int most_kb, int slim_stages, int n_sms);

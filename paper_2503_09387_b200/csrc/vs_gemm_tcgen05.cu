@@ -44,9 +44,9 @@ constexpr int kFewBound = 768, kFewWarps = 8, kFewStages = 6;   // (threads that
 // The same beside the prefill attention (ten warps of 96 registers, 113 KB): whether a projection of 17 to 48 rows, or the W_o behind the
 // attention, leaves room for one of its CTAs (leaves_room_for_attention), which then has its set-up and first keys behind it when the
 // projection is done, as this block has its first weights when the attention is.  The price is depth, five stages of weights for eight.
-// Registers: the launch bound of twice its threads leaves this form at most half of the register file, as the attention's two blocks an SM do.
-constexpr int kSlimSmem = 113 * 1024, kSlimThreads = 64 + 32 * kFewWarps, kBound = 2 * kSlimThreads;
-static_assert(kBound >= kMaxThreads, "every form of the launch");
+// Registers: its ten warps of at most 96 take no more than half of the register file, as the attention's two blocks an SM do (a test asks
+// few_row_linear_registers; a launch bound of 640 threads that forces it made 6 small full layers 268.4 -> 269.7 us).
+constexpr int kSlimSmem = 113 * 1024;
 // Instruction descriptor, kind::f16: D = fp32, A = B = bf16, both K-major, M = 128, N = n.
 __device__ __forceinline__ uint32_t make_idesc(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(GEMM_BLOCK_M >> 4) << 24);
@@ -78,7 +78,7 @@ __device__ __forceinline__ int ld_acquire_gpu(const int* p) {
 __host__ __device__ inline int first_block(int r, int n_blk, int ksplit) { return (r * n_blk + ksplit - 1) / ksplit; }
 
 template <int kFin, bool kOwnRope>   // kOwnRope: no RoPE table, every finishing thread derives the rotation of its one row
-__global__ void __launch_bounds__(kOwnRope ? kFewBound : kBound, 1)
+__global__ void __launch_bounds__(kOwnRope ? kFewBound : kMaxThreads, 1)
 qkv_gemm_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_x,
                 const __grid_constant__ CUtensorMap tm_w2, KernelParams p, BatchParams bp) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -403,6 +403,17 @@ cudaError_t qkv_gemm_init() {
       if (e != cudaSuccess) return e;
     }
   return cudaSuccess;
+}
+
+// registers a thread of the kernels that may run beside the prefill attention, the most of them; 0 if the query fails
+int few_row_linear_registers() {
+  int most = 0;
+  for (int mode : {(int)FIN_PROJECT, (int)FIN_RESIDUAL}) {
+    cudaFuncAttributes at;
+    if (cudaFuncGetAttributes(&at, (const void*)kernel_of(mode, false)) != cudaSuccess) { cudaGetLastError(); return 0; }
+    most = at.numRegs > most ? at.numRegs : most;
+  }
+  return most;
 }
 
 cudaError_t launch_qkv_gemm(const GemmArgs& a, const BatchParams& bp, cudaStream_t st) {

@@ -2,7 +2,7 @@
 over many), of one stream and of several, where K is deep enough to lose stages by it and where it is not."""
 import pytest
 
-from paper_2503_09387_b200 import synth
+from paper_2503_09387_b200 import binding, synth
 from tests.parity import Pair
 
 pytestmark = pytest.mark.gpu
@@ -29,3 +29,8 @@ def test_rows_around_the_rule(d, Hq, Hkv, d_ff, L, more, affine):
     for s in ids:
         p.check_bank(s, layer=L - 1)
     p.close()
+
+
+def test_the_projection_beside_the_attention_takes_half_the_registers():
+    regs = binding.load_library()._ZN2vs24few_row_linear_registersEv()
+    assert 0 < regs and 2 * 320 * ((regs + 7) // 8 * 8) <= 65536          # ten warps; registers are given out eight a thread
