@@ -63,9 +63,10 @@ __device__ __forceinline__ void bank_cp_async16(void* dst, const void* src) {
 // Scores bank rows j0 .. j1 - 1 against the incoming carrier (policy 0), four rows to a warp: a lane's sum is a chain of d / 32
 // dependent fp64 operations, 9 clocks each at best, and every element costs a conversion of 9 to 14; four rows side by side fill
 // the one with the other.  The rows stream through shared memory, 512 elements of each at a time, two chunks ahead; the incoming carrier is
-// widened to fp64 once per block.  What bounds it is the conversion of the rows' elements, an instruction at a sixteenth of the fp32
-// rate, in this form: the fixed order is that of the sums, and asks for no particular way from bf16 to fp64.  Same sums in the
-// same order as warp_dot_norms.  (One row a warp, staged whole: 16 banks of 1024 rows added 50 us to a batched frame step.)
+// widened to fp64 once per block.  No one unit bounds it: of a frame step of 16 full banks of 1024 rows, 230 us, this loop's arithmetic and
+// loads are 23; without the conversions it takes 224.6, without the rows' own norms 228.2, without either 221.6, so most of it is the chain of
+// loads from shared memory and sums.  (Conversions by integer operations: 265 against 273 us of a longer such step, more instructions.)  Same
+// sums in the same order as warp_dot_norms.  (One row a warp, staged whole: 16 banks of 1024 rows added 50 us to a batched frame step.)
 constexpr int kScoreRows = 4, kScoreChunk = 512, kScoreStages = 3, kScoreWarpBytes = kScoreRows * kScoreStages * kScoreChunk * 2;
 __device__ __forceinline__ int staged_warps(int d, uint32_t bytes) {
   const int left = (int)bytes - d * 8;

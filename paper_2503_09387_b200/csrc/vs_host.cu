@@ -18,11 +18,14 @@ using namespace vs;
 namespace vs {
 
 // CTAs to spread the key tiles of each of row_ctas row tiles over (one cluster).  All must be resident at once, beside bank_ctas for
-// the bank update (39 of those behind 264 of 296 made a frame step of three streams 61 us a layer, not 50).  Cost in key tiles (about
-// 1.7 us each when the CTA has its SM alone), fitted to frames, clips, carriers and questions of 2 to 13 tiles: two CTAs an SM make a
-// tile longer, a row tile's row stores cost three, shared by the CTAs of the cluster -- also by those that have no key tile (45
-// rows of two tiles: 27 us a layer split in two, 25 in eight) --, the exchange a half, and nearly every SM taken 0.4: the next
-// linear layer's CTAs then find no room to wait in, with their weights.  clusters[s]: clusters of s CTAs that run at once.
+// the bank update (39 of those behind 264 of 296 made a frame step of three streams 61 us a layer, not 50).  Cost in key tiles, fitted to
+// frames, clips, carriers and questions of 2 to 13 tiles when a row tile's stores took 5.5 us: two CTAs an SM make a tile longer, the
+// stores cost three, shared by the CTAs of the cluster, also by those that have no key tile, the exchange a half, and nearly every SM
+// taken 0.4: the next linear layer's CTAs then find no room to wait in, with their weights.  Without a cluster the stores take 2.8 us
+// now, so short key axes are split further than pays.  Against the best size that runs, over 52 calls each (frames, clips, carriers,
+// questions of 2 to 192 rows and 40 to 1000 keys; whole steps of 6 and 8 layers): 28 / 4 heads of 128 dims 1.0 % slower on average, at
+// most 7.7 (101 carriers 158 us, 147 in four); 16 / 4 heads of 64 dims 1.9 %, at most 15 (101 carriers 136 us in eight, 118 in one).
+// clusters[s]: clusters of s CTAs that run at once.
 int attention_split(int head_dim, int group, int row_ctas, int key_tiles, int bank_ctas, int n_sms, const int* clusters) {
   int best = 1;
   double cost = 1e30;
@@ -38,12 +41,14 @@ int attention_split(int head_dim, int group, int row_ctas, int key_tiles, int ba
 
 // Tiling of a linear layer: CTAs with 128 weight rows each and K cut into ksplit shares (few rows), or CTA pairs with 256
 // (many), and the token columns of a tile.  The choice minimises the clocks of the waves' main loops plus what their epilogues
-// add.  The main loops run at the operands' rate from L2, about 47 bytes a clock of an SM (the MMAs need less: 2 clocks a token
-// column): a 64-element block of K is (128 + tile_n) * 128 bytes to a CTA, (128 + tile_n / 2) * 128 to a CTA of a pair.  A tile's
-// epilogue costs 900 clocks and 14 a column, in a pair kernel only the last one counts, with 3100 clocks for the longer start;
+// add.  The main loops are booked at 47 bytes of operands a clock of an SM (the MMAs need less: 2 clocks a token column; a rate
+// fitted, not a bound: 40 % fewer bytes by another way of splitting did not shorten a few-row layer): a 64-element block of K is
+// (128 + tile_n) * 128 bytes to a CTA, (128 + tile_n / 2) * 128 to a CTA of a pair.  A tile's epilogue costs 900 clocks and 14 a column, in a pair kernel only the last one counts, with 3100 clocks for the longer start;
 // a K split 1000 and 3.5 a column more (partial tiles through L2, a flag), and it needs its whole grid resident at once.
-// Fitted to whole steps of 17 to 1280 rows at the shapes of two backbones, K 1024 to 18944: the chosen tiling is 0.3 % slower
-// than the best one on average (a split costed at 5000 clocks whatever its tile left 1.2 %, at K = 18944 and 480 rows 10 %).
+// Fitted to whole steps of 17 to 1280 rows at the shapes of two backbones, K 1024 to 18944, before the finishing of rows was rebuilt.
+// Since then, against the best of every split and four token tilings, over the four layers of a full decoder at 11 sizes of 24 to 1360
+// rows: at K 3584 and 18944 0.6 % slower on average, at most 7.8 (K 18944, 512 rows, two decoder layers 525 us, 487 with two tiles of
+// 256 split in two), at K 1024 and 4096 0.8 %, at most 12 (24 rows, E 1536, six layers 294 us, 263 split in five).
 Tiling choose_tiles(int K, int E, int n_sms, int max_pairs, int rows, bool own_rope) {
   const int kb = K / GEMM_BLOCK_K, resident = n_sms < GEMM_XCHG_CTAS ? n_sms : GEMM_XCHG_CTAS;
   const int nt_min = (rows + 255) / 256;
@@ -450,18 +455,19 @@ size_t layer_stride_bank(const Dims& D) { return (size_t)D.S * D.Hkv * D.slots *
 size_t layer_stride_prefix(const Dims& D) { return (size_t)D.S * D.Hkv * D.maxP * D.D; }
 size_t layer_stride_tail(const Dims& D) { return (size_t)D.S * D.Hkv * D.maxT * D.D; }
 
-// Whether a step of n_active x T rows goes to the persistent kernel.  Both sides measured (us, persistent against launches layer by
-// layer); the number of keys moves them alike (64 to 1024 carriers).
+// Whether a step of n_active x T rows goes to the persistent kernel.  Both sides measured (us, persistent / launches layer by layer, over
+// 500 keys); the number of keys moves them alike (64 to 1024 carriers).
 // Full layers and the head, up to 8 rows (at 16 the slabs leave the ring too few stages: 3 layers at the Qwen2-7B shape 362 against
-// 344).  Where a layer's projection holds 223 KB for every SM (that shape, 2 layers): one row 181 against 184, eight 199 against 213.
-// Narrower layers hide less of the phases' synchronisation behind weights, and single tokens of several streams, whose launches are
-// the cheapest (matrix-vector kernel, attention by head), go there from three rows on: 6 layers of width 1536 (42 KB an SM) 237
-// against 242 for two streams, 260 against 246 for four, 300 against 272 for eight; 1024 (21 KB) 168 / 181, 188 / 179, 227 / 210;
-// 2048 (85 KB) 272 / 263, 287 / 268, 330 / 295.  One stream's several tokens stay: 239 / 273 for two, 302 / 306 for eight at 1536.
-// Attention alone: steps of several tokens up to 16 rows (8 layers over 564 keys: width 1024 79 / 84 for two tokens, 82 / 118 for
-// five; 2048 108 / 113, 101 / 148; 3584 138 / 132, 129 / 174; 16 rows 192 / 206, 32 rows 842 against 770 for 28 layers) and single
-// tokens of more streams than the matrix-vector kernel takes (8 streams 180 / 251, 16 209 / 249), in a stack; one to four single
-// tokens are faster by launches (28 layers 463 against 352), and so are two to four rows in a single layer (19.4 against 17.7).
+// 344, before the launches gained).  Where a layer's projection holds 223 KB for every SM (that shape, 3 layers): one row 273 / 277,
+// eight 296 / 302.  Narrower layers hide less of the phases' synchronisation behind weights, and single tokens of several streams, whose
+// launches are the cheapest (matrix-vector kernel, attention by head), go there from three rows on: 6 layers of width 1536 (42 KB an SM)
+// 207 / 211 for two streams, 217 / 209 for three, 259 / 238 for eight; 1024 (21 KB) 175 / 193, 183 / 195, four 194 / 193, eight 230 / 226;
+// 2048 (85 KB) 253 / 258, 257 / 263, 268 / 267, 311 / 299.  One stream's several tokens stay: 202 / 234 for two, 265 / 261 for eight at
+// 1536.  Attention alone: steps of several tokens up to 16 rows (8 layers: width 1024 75 / 88 for two tokens, 83 / 127 for five, 103 / 129
+// for 16; 2048 105 / 107, 102 / 148, 135 / 155; 3584 134 / 134, 130 / 181, 159 / 195; 32 rows and 28 layers 842 / 770) and single tokens of
+// more streams than the matrix-vector kernel takes (3584: 8 streams 152 / 167, 16 169 / 193), in a stack; one to four single tokens are
+// faster by launches (140 / 91, 136 / 114), and so are two to four rows in a single layer (16.2 / 14.0; width 1024 11.6 / 12.5).  In a single
+// layer 12 to 16 rows of several tokens lose up to 12 % (16 rows 21.3 / 20.3, width 2048 18.9 / 16.9).
 // And not where a layer's projection holds less than 16 KB for every SM: there is then no weight stream to hide the
 // synchronisation behind.
 // wide: the rows' address takes four elements at a time; else the kernel takes what no other can store, a full layer's rows.
@@ -1269,11 +1275,12 @@ int vs_decode_step(vs_stream* h, const int32_t* stream_ids, int32_t n_active, co
       da.meta = meta;
       da.Hq = D.Hq; da.Hkv = D.Hkv; da.D = D.D; da.slots = D.slots; da.M = D.M; da.maxP = D.maxP; da.maxT = D.maxT;
       // A CTA per query head, or per KV head (K and V read once per group).  The first for one stream, and for two to four in groups of
-      // more than four where its CTAs, two to an SM, take no more than seven eighths of the places: its chains are shorter (8 layers,
-      // head size 128, us against by KV head: groups of seven, two streams, 246 keys 94 / 117; of six, three streams, 166 keys
-      // 88 / 98; of five, three streams, 246 keys 83 / 89; of five, four streams, 166 keys 90 / 86 is the one found the other
-      // way; groups of four: 61 either way or 8 % slower).  Beyond that its clusters no longer all fit (256 CTAs in clusters of four
-      // 146 / 147, 288 of 296: 120 / 100).  There short contexts are written by the CTA directly, longer ones split over a cluster of
+      // more than four where its CTAs, two to an SM, take no more than seven eighths of the places: its chains are shorter (128 tokens
+      // through 8 layers, head size 128, us a token against by KV head: groups of seven, one stream of 1000 keys and the tail 102 / 130,
+      // two of 246 93 / 118; of six, three streams of 166 64 / 68; of five, three of 246 83 / 96; of eight, two of 246 147 / 158).
+      // Beyond that its clusters no longer all fit (groups of seven, two streams of 440 keys 128 / 121, three of 246 129 / 118; of five, four of
+      // 166 113 / 94).  Groups of four, head size 64: three streams of 166 63 / 58; one stream is the one found the other way (80 keys
+      // 53.5 / 51.7, 440 keys 60.7 / 56.4, 1000 keys 61.0 / 62.5).  There short contexts are written by the CTA directly, longer ones split over a cluster of
       // 2, 4 or 8 CTAs (a CTA then walks about 64 to 128 keys)
       int ns = (max_keys <= 96) ? 1 : (max_keys <= 192 ? 2 : (max_keys <= 448 ? 4 : 8));
       const bool by_head = n_active == 1 || !wide || (n_active <= 4 && D.G > 4 && 4LL * ns * D.Hq * n_active <= 7LL * h->n_sms);
